@@ -13,10 +13,19 @@
 // converted to int64 with 2^-32 resolution, normalised by their log-sum-exp,
 // children below tau are dropped, the h_max largest are kept (ties by
 // index), the kept ones are listed in index order and their log-weights
-// renormalised.  The log-sum-exp is summed differently (FP64 exponentials
-// here, FP32 exponentials with compensated sums there), so the two agree up
-// to its rounding: a child whose normalised weight lies within that rounding
-// of tau may land on either side of the cut.
+// renormalised.  The log-sum-exp is summed differently (exponentials to
+// 2^-55 here, FP32 exponentials with compensated sums there), so the two
+// agree up to its rounding: a child whose normalised weight lies within that
+// rounding of tau may land on either side of the cut.
+//
+// What bounds it: at a million children the 8 MB of log-weights stay in L2,
+// so a pass is a few microseconds and the cost is the FP64 pipe (about two
+// operations a clock on an SM) and the number of launches.  Therefore the
+// keys and the exponentials are formed in integer arithmetic (fx_exp), and
+// what one block has to decide between two passes is done by the last block
+// of the first (five launches instead of twelve).  Measured, 10^6 children,
+// h_max 20000: 413 us with an FP64 exponential per child and per kept child
+// in one block (twelve launches), 64 us with these.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -38,22 +47,29 @@ constexpr size_t kOffBlkM = 0;                                   // long long[kM
 constexpr size_t kOffBlkS = kOffBlkM + 8 * kMaxBlocks;           // double[kMaxBlocks]
 constexpr size_t kOffBlkGt = kOffBlkS + 8 * kMaxBlocks;          // uint32[kMaxBlocks]
 constexpr size_t kOffBlkEq = kOffBlkGt + 4 * kMaxBlocks;         // uint32[kMaxBlocks]
-constexpr size_t kOffHist = kOffBlkEq + 4 * kMaxBlocks;          // uint32[kBinsS]
+constexpr size_t kOffHist = kOffBlkEq + 4 * kMaxBlocks;          // uint32[kBinsS], then the boundary list
 constexpr size_t kOffScal = kOffHist + 4 * kBinsS;               // Scal
 constexpr size_t kScratchBytes = kOffScal + 256;
 // the size glmb.h states for the scratch array
 static_assert(kScratchBytes == 41216, "scratch size changed: update glmb.h");
+// keys of the boundary bin that fit in the histogram's place
+constexpr unsigned kListS = kBinsS / 2;
+// up to this many children the boundary bin of the first histogram is listed
+// and finished by one block; beyond it the bin outgrows the list, and each
+// digit takes a histogram pass over the children
+constexpr long long kListN = 1LL << 22;
 
 struct SelScal {
-  unsigned done;        // last-block counter
-  unsigned pad;
+  unsigned done[3];     // last-block counters (histogram, boundary list, count)
+  unsigned n_list;      // keys in the boundary list (may exceed kListS)
   double lse;           // log-sum-exp over valid children
+  double lse_kept;      // log-sum-exp of the kept log-weights less lse
   long long thr;        // fixed-point threshold
+  long long top;        // largest key
   long long prefix;     // radix prefix
   long long need;       // elements still needed at the boundary key
   long long bound;      // boundary key
   long long mode;       // 0 running, 1 keep all candidates, 2 nothing valid
-  long long n_kept;
 };
 
 __device__ __align__(256) unsigned char g_select_scratch[kScratchBytes];
@@ -64,175 +80,224 @@ struct Ptrs {
   unsigned* blk_gt;
   unsigned* blk_eq;
   unsigned* hist;
+  long long* list;
   SelScal* sc;
 };
 
 __host__ __device__ inline Ptrs ptrs_of(unsigned char* base) {
   return Ptrs{(long long*)(base + kOffBlkM), (double*)(base + kOffBlkS), (unsigned*)(base + kOffBlkGt),
-              (unsigned*)(base + kOffBlkEq), (unsigned*)(base + kOffHist), (SelScal*)(base + kOffScal)};
+              (unsigned*)(base + kOffBlkEq), (unsigned*)(base + kOffHist), (long long*)(base + kOffHist),
+              (SelScal*)(base + kOffScal)};
 }
 
+// The log-weight times 2^32, rounded to nearest (ties to even), from its
+// bits: the FP64 conversion runs at a small fraction of the integer rate.
+// Log-weights outside (-2^30, 2^30) -- -inf, +inf and NaN among them -- mark
+// children without weight; inside, every key is below 2^62 in magnitude, so
+// the difference of two keys cannot overflow.
 __device__ __forceinline__ long long key_of(double lw) {
-  // log-weights outside (-2^30, 2^30) -- -inf, +inf and NaN among them --
-  // mark children without weight; inside, every key is below 2^62 in
-  // magnitude, so the difference of two keys cannot overflow
-  if (!(lw > -1073741824.0 && lw < 1073741824.0)) return kKeyInvalid;
-  return __double2ll_rn(lw * 4294967296.0);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(lw);
+  const int e = (int)((b >> 52) & 0x7FFull);
+  if (e >= 1023 + 30) return kKeyInvalid;
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;   // |lw| = m 2^(e - 1075)
+  const int r = 1043 - e;   // right shift that leaves |lw| 2^32 (subnormals give 0 too)
+  unsigned long long v;
+  if (r <= 0) {
+    v = m << -r;
+  } else if (r > 54) {
+    v = 0ull;
+  } else {
+    v = m >> r;
+    const unsigned long long rem = m << (64 - r);   // the part dropped, as a fraction of 2^64
+    v += (rem > 0x8000000000000000ull || (rem == 0x8000000000000000ull && (v & 1ull))) ? 1ull : 0ull;
+  }
+  return (b >> 63) ? -(long long)v : (long long)v;
 }
 
+// 2^(-j/64) as 63-bit fractions, from exp's Taylor series at compile time
+struct Exp2Tab {
+  unsigned long long v[64];
+  constexpr Exp2Tab() : v{} {
+    for (int j = 0; j < 64; ++j) {
+      const double x = -0.69314718055994530942 * j / 64.0;
+      double t = 1.0, s = 0.0;
+      for (int k = 24; k >= 1; --k) s = (s + 1.0) * x / k;   // x (1 + x/2 (1 + x/3 (...)))
+      t += s;
+      v[j] = (unsigned long long)(t * 9223372036854775808.0);
+    }
+  }
+};
+__device__ const Exp2Tab kExp2Tab{};
+// the block's copy (lanes read different entries); every kernel that forms
+// exponentials fills it first
+__device__ __forceinline__ unsigned long long* exp_tab() {
+  __shared__ unsigned long long t[64];
+  return t;
+}
+__device__ __forceinline__ void load_exp_tab() {
+  if (threadIdx.x < 64) exp_tab()[threadIdx.x] = kExp2Tab.v[threadIdx.x];
+  __syncthreads();
+}
+
+// exp(-d 2^-32) 2^58 for d >= 0, to about 2^-51 of its value, in integer
+// arithmetic: d log2(e) = i + j/64 + r, then the table's 2^(-j/64) times the
+// Taylor polynomial of 2^-r (z = r ln 2 < 0.011, six terms: z^7/7! < 2^-57).
+__device__ __forceinline__ unsigned long long fx_exp(unsigned long long d) {
+  if (d >= (42ull << 32)) return 0ull;                         // below 2^-60
+  constexpr unsigned long long kLog2e = 0x5C551D94AE0BF85Eull; // log2(e) 2^62
+  constexpr unsigned long long kLn2 = 0xB17217F7D1CF79ACull;   // ln(2) 2^64
+  const unsigned long long y = __umul64hi(d << 25, kLog2e);    // 2^-55 units
+  const int i = (int)(y >> 55), j = (int)(y >> 49) & 63;
+  const unsigned long long z = __umul64hi((y & 0x1FFFFFFFFFFFFull) << 9, kLn2);   // z 2^64
+  // 1 - z (1 - z (1/2 - z (1/6 - z (1/24 - z (1/120 - z/720))))), the inner
+  // terms in 32 bits (z 2^32 < 2^26), the outer ones scaled by 2^63
+  const uint32_t zh = (uint32_t)(z >> 32);
+  uint32_t q = 35791394u - __umulhi(zh, 5965232u);             // (1/120 - z/720) 2^32
+  q = 178956971u - __umulhi(zh, q);                            // 1/24
+  q = 715827883u - __umulhi(zh, q);                            // 1/6
+  unsigned long long p = 0x4000000000000000ull - __umul64hi(z, (unsigned long long)q << 31);
+  p = 0x8000000000000000ull - __umul64hi(z, p);
+  p = 0x8000000000000000ull - __umul64hi(z, p);
+  const unsigned long long t = __umul64hi(p, exp_tab()[j]);   // 2^62 scale
+  const int s = 4 + i;
+  return (t + (1ull << (s - 1))) >> s;
+}
+constexpr double kExpInv = 3.4694469519536141888e-18;          // 2^-58
+
+__device__ __forceinline__ long long warp_max_ll(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+  return v;
+}
+template <typename T>
+__device__ __forceinline__ T warp_sum_of(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+// inclusive scan over a warp
+template <typename T>
+__device__ __forceinline__ T warp_incl(T x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+// The maximum and the sum of exp(key - maximum) over a block's (m, s) pairs
+// (a pair with m = kKeyInvalid is empty), in every thread.
 struct LseS {
   long long m;
   double s;
 };
-__device__ __forceinline__ LseS comb(LseS a, LseS b) {
-  if (a.m == kKeyInvalid) return b;
-  if (b.m == kKeyInvalid) return a;
-  if (a.m >= b.m) return {a.m, a.s + b.s * exp((double)(b.m - a.m) * kFxInv)};
-  return {b.m, b.s + a.s * exp((double)(a.m - b.m) * kFxInv)};
-}
-__device__ LseS block_comb(LseS v) {
+__device__ LseS block_lse(LseS v) {
   __shared__ long long sm[32];
   __shared__ double ss[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    v = comb(v, LseS{__shfl_xor_sync(0xFFFFFFFFu, v.m, o), __shfl_xor_sync(0xFFFFFFFFu, v.s, o)});
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  const long long wm = warp_max_ll(v.m);
+  if (lane == 0) sm[w] = wm;
   __syncthreads();
-  if (lane == 0) { sm[w] = v.m; ss[w] = v.s; }
+  const long long M = warp_max_ll(lane < nw ? sm[lane] : kKeyInvalid);
+  const double r = v.m == kKeyInvalid ? 0.0
+                   : v.m == M         ? v.s
+                                      : v.s * ((double)fx_exp((unsigned long long)(M - v.m)) * kExpInv);
+  const double ws = warp_sum_of(r);
+  if (lane == 0) ss[w] = ws;
   __syncthreads();
-  if (w == 0) {
-    v = lane < nw ? LseS{sm[lane], ss[lane]} : LseS{kKeyInvalid, 0.0};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      v = comb(v, LseS{__shfl_xor_sync(0xFFFFFFFFu, v.m, o), __shfl_xor_sync(0xFFFFFFFFu, v.s, o)});
-  }
-  return v;
+  return LseS{M, warp_sum_of(lane < nw ? ss[lane] : 0.0)};
 }
 
 __device__ __forceinline__ void chunk_of(long long n, long long& lo, long long& hi) {
   const long long per = (n + gridDim.x - 1) / gridDim.x;
-  lo = (long long)blockIdx.x * per;
-  hi = lo + per < n ? lo + per : n;
+  lo = min(n, (long long)blockIdx.x * per);
+  hi = min(n, lo + per);
 }
 
-// the previous call's contents are cleared here
-__global__ void sel_init(unsigned char* base, int h_max) {
+// Pass 1: per-block maximum and sum of exponentials.  Each warp takes eight
+// keys per lane at a time and sums them against its running maximum, so only
+// a new maximum costs FP64 work.  Block 0 clears what the later passes count
+// in (the previous call's contents).
+__global__ void __launch_bounds__(kThreads) sel_lse(const double* __restrict__ lw, long long n, int h_max,
+                                                    unsigned char* base) {
+  load_exp_tab();
+  pdl_enter();
   Ptrs p = ptrs_of(base);
-  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) p.hist[b] = 0u;
-  if (threadIdx.x == 0) {
-    p.sc->done = 0u;
-    p.sc->need = h_max;
-    p.sc->prefix = 0;
-    p.sc->bound = 0;
-    p.sc->mode = 0;
-    p.sc->n_kept = 0;
+  if (blockIdx.x == 0) {
+    for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) p.hist[b] = 0u;
+    if (threadIdx.x == 0) {
+      p.sc->done[0] = p.sc->done[1] = p.sc->done[2] = 0u;
+      p.sc->n_list = 0u;
+      p.sc->need = h_max;
+      p.sc->prefix = 0;
+      p.sc->bound = 0;
+      p.sc->mode = 0;
+    }
   }
-}
-
-__global__ void sel_lse(const double* __restrict__ lw, long long n, double log_tau,
-                        unsigned char* base) {
-  __shared__ bool last;
-  Ptrs p = ptrs_of(base);
   long long lo, hi;
   chunk_of(n, lo, hi);
   LseS v{kKeyInvalid, 0.0};
-  for (long long j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-    const long long k = key_of(lw[j]);
-    if (k != kKeyInvalid) v = comb(v, LseS{k, 1.0});
+  constexpr int kU = 8;
+  for (long long j0 = lo; j0 < hi; j0 += kU * kThreads) {
+    double x[kU];
+    long long k[kU], m = v.m;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const long long j = j0 + u * kThreads + threadIdx.x;
+      x[u] = j < hi ? lw[j] : -INFINITY;
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      k[u] = key_of(x[u]);
+      m = max(m, k[u]);
+    }
+    m = warp_max_ll(m);
+    if (m == kKeyInvalid) continue;
+    if (m != v.m) {
+      if (v.m != kKeyInvalid) v.s *= (double)fx_exp((unsigned long long)(m - v.m)) * kExpInv;
+      v.m = m;
+    }
+    unsigned long long s = 0ull;   // at most 8 terms of 2^58
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (k[u] != kKeyInvalid) s += fx_exp((unsigned long long)(m - k[u]));
+    if (s) v.s += (double)s * kExpInv;
   }
-  v = block_comb(v);
+  v = block_lse(v);
   if (threadIdx.x == 0) {
     p.blk_m[blockIdx.x] = v.m;
     p.blk_s[blockIdx.x] = v.s;
-    __threadfence();
-    last = atomicAdd(&p.sc->done, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  LseS u{kKeyInvalid, 0.0};
-  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
-    u = comb(u, LseS{((volatile long long*)p.blk_m)[b], ((volatile double*)p.blk_s)[b]});
-  u = block_comb(u);
-  if (threadIdx.x == 0) {
-    p.sc->done = 0u;
-    if (u.m == kKeyInvalid || !(u.s > 0.0)) {
-      p.sc->lse = -INFINITY;
-      p.sc->thr = LLONG_MAX;
-      p.sc->mode = 2;
-    } else {
-      p.sc->lse = (double)u.m * kFxInv + log(u.s);
-      p.sc->thr = (long long)ceil((p.sc->lse + log_tau) * 4294967296.0);
-    }
   }
 }
 
-__global__ void sel_hist(const double* __restrict__ lw, long long n, int shift, unsigned char* base) {
-  __shared__ unsigned hist[kBinsS];
-  Ptrs p = ptrs_of(base);
-  if (p.sc->mode != 0) return;
-  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) hist[b] = 0;
-  __syncthreads();
-  const long long thr = p.sc->thr;
-  const unsigned long long prefix = (unsigned long long)p.sc->prefix;
-  long long lo, hi;
-  chunk_of(n, lo, hi);
-  for (long long j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-    const long long k = key_of(lw[j]);
-    if (k == kKeyInvalid || k < thr) continue;
-    const unsigned long long v = (unsigned long long)(k - thr);
-    if ((v >> (shift + kDigitS)) != prefix) continue;
-    atomicAdd(&hist[(v >> shift) & (kBinsS - 1)], 1u);
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x)
-    if (hist[b]) atomicAdd(&p.hist[b], hist[b]);
-}
-
-// one block of kBinsS / 4 threads; thread t owns bins [4t, 4t + 4)
-__global__ void sel_find(int shift, int first, unsigned char* base) {
+// Boundary digit of histogram h (kBinsS bins, shared memory) by a block of
+// kBinsS / 4 threads: the digit and the elements still needed in its bin;
+// `all`: the whole histogram is within `need`.
+struct Digit {
+  int digit;
+  long long need;
+  bool all;
+};
+__device__ Digit find_digit(const unsigned* h, long long need) {
   __shared__ unsigned wsum[32];
-  Ptrs p = ptrs_of(base);
+  __shared__ int s_digit;
+  __shared__ long long s_need;
   const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
-  const bool running = p.sc->mode == 0;
-  const long long need = p.sc->need;
   unsigned b4[4], mine = 0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    b4[k] = p.hist[4 * t + k];
+    b4[k] = h[4 * t + k];
     mine += b4[k];
-    p.hist[4 * t + k] = 0;
   }
-  unsigned x = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
-  }
+  const unsigned x = warp_incl(mine);
   if (lane == 31) wsum[wp] = x;
   __syncthreads();
-  if (wp == 0) {
-    unsigned s = wsum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-      if (lane >= o) s += y;
-    }
-    wsum[lane] = s;
-  }
-  __syncthreads();
-  if (!running) return;
-  const unsigned incl = x + (wp > 0 ? wsum[wp - 1] : 0u);
-  const unsigned total = wsum[31];
-  const unsigned above = total - incl, upto = above + mine;
-  if (first && (long long)total <= need) {
-    if (t == 0) {
-      p.sc->mode = 1;
-      p.sc->bound = p.sc->thr - 1;
-      p.sc->need = 0;
-    }
-    return;
-  }
+  const unsigned ws = warp_incl(wsum[lane]);
+  const unsigned total = __shfl_sync(0xFFFFFFFFu, ws, 31);
+  const unsigned before = __shfl_sync(0xFFFFFFFFu, ws, max(wp - 1, 0));
+  const unsigned above = total - x - (wp > 0 ? before : 0u), upto = above + mine;
   if ((long long)above < need && (long long)upto >= need) {
     unsigned cum = above;
     int b = 3;
@@ -240,9 +305,151 @@ __global__ void sel_find(int shift, int first, unsigned char* base) {
       if ((long long)(cum + b4[b]) >= need) break;
       cum += b4[b];
     }
-    p.sc->prefix = (p.sc->prefix << kDigitS) | (4 * t + b);
-    p.sc->need = need - cum;
-    if (shift == 0) p.sc->bound = p.sc->thr + p.sc->prefix;
+    s_digit = 4 * t + b;
+    s_need = need - cum;
+  }
+  __syncthreads();
+  const Digit d{s_digit, s_need, (long long)total <= need};
+  __syncthreads();
+  return d;
+}
+
+// true in every thread of the grid's last block to get here
+__device__ bool last_block(unsigned* done) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Pass 2 (and, for large n, once per further digit): histogram of the digit
+// of `width` bits at `shift` of the keys at or above the threshold that share the prefix; the
+// last block finds the boundary digit.  On the first digit every block forms
+// the log-sum-exp and the threshold from pass 1's partials (the same in all).
+__global__ void __launch_bounds__(1024) sel_hist(const double* __restrict__ lw, long long n, int shift, int width, int first,
+                                                 int nblk_lse, double log_tau, unsigned char* base) {
+  load_exp_tab();
+  pdl_enter();
+  __shared__ unsigned hist[kBinsS];
+  __shared__ long long s_thr;
+  Ptrs p = ptrs_of(base);
+  if (p.sc->mode != 0) return;
+  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) hist[b] = 0;
+  if (first) {
+    const int b = threadIdx.x;   // one partial per thread (kMaxBlocks = blockDim)
+    const LseS u = block_lse(b < nblk_lse ? LseS{p.blk_m[b], p.blk_s[b]} : LseS{kKeyInvalid, 0.0});
+    const bool none = u.m == kKeyInvalid || !(u.s > 0.0);
+    if (threadIdx.x == 0) {
+      double lse = -INFINITY;
+      long long thr = LLONG_MAX;
+      if (!none) {
+        lse = (double)u.m * kFxInv + log(u.s);
+        thr = (long long)ceil((lse + log_tau) * 4294967296.0);
+      }
+      s_thr = thr;
+      if (blockIdx.x == 0) {
+        p.sc->lse = lse;
+        p.sc->thr = thr;
+        p.sc->top = u.m;
+      }
+    }
+  } else if (threadIdx.x == 0) {
+    s_thr = p.sc->thr;
+  }
+  __syncthreads();
+  const long long thr = s_thr;
+  const unsigned long long prefix = (unsigned long long)p.sc->prefix;
+  long long lo, hi;
+  chunk_of(n, lo, hi);
+#pragma unroll 4
+  for (long long j = lo + threadIdx.x; j < hi; j += blockDim.x) {
+    const long long k = key_of(lw[j]);
+    if (k == kKeyInvalid || k < thr) continue;
+    const unsigned long long v = (unsigned long long)(k - thr);
+    if ((v >> (shift + width)) != prefix) continue;
+    atomicAdd(&hist[(v >> shift) & ((1u << width) - 1u)], 1u);
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x)
+    if (hist[b]) atomicAdd(&p.hist[b], hist[b]);
+  if (!last_block(&p.sc->done[0])) return;
+  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) {
+    hist[b] = __ldcg(&p.hist[b]);
+    p.hist[b] = 0u;
+  }
+  __syncthreads();
+  const long long need = p.sc->need;
+  const Digit d = find_digit(hist, need);
+  if (threadIdx.x != 0) return;
+  p.sc->done[0] = 0u;
+  if (thr == LLONG_MAX) {
+    p.sc->mode = 2;
+  } else if (first && d.all) {
+    p.sc->mode = 1;
+    p.sc->bound = thr - 1;
+    p.sc->need = 0;
+  } else {
+    const long long pre = (long long)((prefix << width) | (unsigned)d.digit);
+    p.sc->prefix = pre;
+    p.sc->need = d.need;
+    if (shift == 0) p.sc->bound = thr + pre;
+  }
+}
+
+// Pass 3 (n <= kListN): the keys of the boundary bin are listed, and the last
+// block finds the boundary key among them digit by digit in shared memory.  A
+// bin that outgrows the list (many equal or nearly equal keys) is read from
+// the children again by that block.
+__global__ void __launch_bounds__(1024) sel_boundary(const double* __restrict__ lw, long long n, int shift,
+                                                     unsigned char* base) {
+  pdl_enter();
+  __shared__ unsigned hist[kBinsS];
+  Ptrs p = ptrs_of(base);
+  if (p.sc->mode != 0) return;
+  const long long thr = p.sc->thr;
+  unsigned long long prefix = (unsigned long long)p.sc->prefix;
+  const int lane = threadIdx.x & 31;
+  long long lo, hi;
+  chunk_of(n, lo, hi);
+  for (long long j0 = lo; j0 < hi; j0 += blockDim.x) {
+    const long long j = j0 + threadIdx.x;
+    const long long k = j < hi ? key_of(lw[j]) : kKeyInvalid;
+    const bool in = k != kKeyInvalid && k >= thr && ((unsigned long long)(k - thr) >> shift) == prefix;
+    const unsigned bal = __ballot_sync(0xFFFFFFFFu, in);
+    if (!bal) continue;
+    unsigned at = 0;
+    if (lane == __ffs(bal) - 1) at = atomicAdd(&p.sc->n_list, (unsigned)__popc(bal));
+    at = __shfl_sync(0xFFFFFFFFu, at, __ffs(bal) - 1) + __popc(bal & ((1u << lane) - 1u));
+    if (in && at < kListS) p.list[at] = k;
+  }
+  if (!last_block(&p.sc->done[1])) return;
+  const unsigned nl = __ldcg(&p.sc->n_list);
+  const bool listed = nl <= kListS;
+  const long long total = listed ? (long long)nl : n;
+  long long need = p.sc->need;
+  for (int above = shift; above > 0;) {
+    const int width = min(kDigitS, above), sh = above - width;
+    for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) hist[b] = 0u;
+    __syncthreads();
+    for (long long j = threadIdx.x; j < total; j += blockDim.x) {
+      const long long k = listed ? __ldcg(&p.list[j]) : key_of(lw[j]);
+      if (k == kKeyInvalid || k < thr) continue;
+      const unsigned long long v = (unsigned long long)(k - thr);
+      if ((v >> above) != prefix) continue;
+      atomicAdd(&hist[(v >> sh) & ((1u << width) - 1u)], 1u);
+    }
+    __syncthreads();
+    const Digit d = find_digit(hist, need);
+    prefix = (prefix << width) | (unsigned)d.digit;
+    need = d.need;
+    above = sh;
+  }
+  if (threadIdx.x == 0) {
+    p.sc->need = need;
+    p.sc->bound = thr + (long long)prefix;
   }
 }
 
@@ -253,94 +460,110 @@ __device__ __forceinline__ void keep_kind(long long k, const SelScal& s, bool& g
   else if (k == s.bound && s.need > 0) eq = true;
 }
 
-__global__ void sel_count(const double* __restrict__ lw, long long n, unsigned char* base) {
-  __shared__ unsigned cg, ce;
+// Pass 4: per-block counts above and at the boundary, and the sum of
+// exp(key - largest key) above it; the last block turns the counts into
+// offsets and forms the kept children's log-sum-exp (the largest key is
+// always kept).
+__global__ void __launch_bounds__(kThreads) sel_count(const double* __restrict__ lw, long long n, int h_max,
+                                                      int* n_out, unsigned char* base) {
+  load_exp_tab();
+  pdl_enter();
+  __shared__ unsigned long long wc[kThreads / 32];
+  __shared__ double wd[kThreads / 32];
   Ptrs p = ptrs_of(base);
-  if (threadIdx.x == 0) { cg = 0; ce = 0; }
-  __syncthreads();
   const SelScal s = *p.sc;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  constexpr int kWarps = kThreads / 32;
   long long lo, hi;
   chunk_of(n, lo, hi);
-  unsigned g = 0, e = 0;
-  for (long long j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-    bool gt, eq;
-    keep_kind(key_of(lw[j]), s, gt, eq);
-    g += gt;
-    e += eq;
+  unsigned long long c = 0;   // above | at << 32
+  double sum = 0.0;
+  constexpr int kU = 4;
+  for (long long j0 = lo; j0 < hi; j0 += kU * kThreads) {
+    unsigned long long f = 0ull;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const long long j = j0 + u * kThreads + threadIdx.x;
+      const long long k = j < hi ? key_of(lw[j]) : kKeyInvalid;
+      bool gt, eq;
+      keep_kind(k, s, gt, eq);
+      c += (gt ? 1ull : 0ull) + (eq ? 1ull << 32 : 0ull);
+      if (gt) f += fx_exp((unsigned long long)(s.top - k));
+    }
+    if (f) sum += (double)f * kExpInv;
   }
-  if (g) atomicAdd(&cg, g);
-  if (e) atomicAdd(&ce, e);
+  c = warp_sum_of(c);
+  sum = warp_sum_of(sum);
+  if (lane == 0) {
+    wc[wp] = c;
+    wd[wp] = sum;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    p.blk_gt[blockIdx.x] = cg;
-    p.blk_eq[blockIdx.x] = ce;
+    for (int w = 1; w < kWarps; ++w) {
+      c += wc[w];
+      sum += wd[w];
+    }
+    p.blk_gt[blockIdx.x] = (unsigned)(c & 0xFFFFFFFFull);
+    p.blk_eq[blockIdx.x] = (unsigned)(c >> 32);
+    p.blk_s[blockIdx.x] = sum;
   }
-}
-
-// exclusive offsets of the per-block counts (one block), total kept
-__global__ void sel_offsets(int nblk, int h_max, int* n_out, unsigned char* base) {
-  __shared__ unsigned long long carry;
-  Ptrs p = ptrs_of(base);
-  if (threadIdx.x == 0) carry = 0;
+  if (!last_block(&p.sc->done[2])) return;
+  // exclusive offsets over the blocks, four per thread
+  unsigned long long v[4], mine = 0;
+  sum = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const unsigned b = 4 * threadIdx.x + q;
+    v[q] = b < gridDim.x ? ((unsigned long long)__ldcg(&p.blk_eq[b]) << 32) | __ldcg(&p.blk_gt[b]) : 0ull;
+    if (b < gridDim.x) sum += __ldcg(&p.blk_s[b]);
+    mine += v[q];
+  }
+  const unsigned long long x = warp_incl(mine);
+  sum = warp_sum_of(sum);
+  if (lane == 31) wc[wp] = x;
+  if (lane == 0) wd[wp] = sum;
   __syncthreads();
-  for (int b0 = 0; b0 < nblk; b0 += blockDim.x) {
-    const int b = b0 + threadIdx.x;
-    unsigned long long v = b < nblk ? ((unsigned long long)p.blk_eq[b] << 32) | p.blk_gt[b] : 0ULL;
-    // block inclusive scan of packed (eq, gt) counts
-    __shared__ unsigned long long ws[32];
-    unsigned long long x = v;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  unsigned long long excl = x - mine, total = 0;
+  for (int w = 0; w < kWarps; ++w) {
+    if (w < wp) excl += wc[w];
+    total += wc[w];
+  }
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[wp] = x;
-    __syncthreads();
-    if (wp == 0) {
-      unsigned long long s = lane < (int)((blockDim.x + 31) >> 5) ? ws[lane] : 0ULL;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-        if (lane >= o) s += y;
-      }
-      ws[lane] = s;
-    }
-    __syncthreads();
-    const unsigned long long excl = carry + (wp > 0 ? ws[wp - 1] : 0ULL) + x - v;
-    if (b < nblk) {
-      p.blk_gt[b] = (unsigned)(excl & 0xFFFFFFFFULL);
+  for (int q = 0; q < 4; ++q) {
+    const unsigned b = 4 * threadIdx.x + q;
+    if (b < gridDim.x) {
+      p.blk_gt[b] = (unsigned)(excl & 0xFFFFFFFFull);
       p.blk_eq[b] = (unsigned)(excl >> 32);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) carry += ws[((blockDim.x + 31) >> 5) - 1];
-    __syncthreads();
+    excl += v[q];
   }
   if (threadIdx.x == 0) {
-    const long long gt = (long long)(carry & 0xFFFFFFFFULL), eq = (long long)(carry >> 32);
-    long long kept = p.sc->mode == 2 ? 0 : gt + (eq < p.sc->need ? eq : p.sc->need);
+    const long long gt = (long long)(total & 0xFFFFFFFFull), eq = (long long)(total >> 32);
+    long long kept = s.mode == 2 ? 0 : gt + min(eq, s.need);
     if (kept > h_max) kept = h_max;
-    p.sc->n_kept = kept;
     *n_out = (int)kept;
+    for (int w = 1; w < kWarps; ++w) sum += wd[w];
+    if (s.mode == 0 && s.need > 0)
+      sum += (double)min(eq, s.need) * ((double)fx_exp((unsigned long long)(s.top - s.bound)) * kExpInv);
+    p.sc->lse_kept = kept > 0 ? ((double)s.top * kFxInv - s.lse) + log(sum) : 0.0;
   }
 }
 
-// kept children in index order; log-weights normalised over all children
-__global__ void sel_write(const double* __restrict__ lw, long long n, int h_max, long long* idx_out,
-                          double* lw_out, unsigned char* base) {
-  __shared__ unsigned wg[kThreads / 32], we[kThreads / 32];
-  __shared__ unsigned run_g, run_e;
+// Pass 5: kept children in index order, their log-weights normalised over
+// all children and then over the kept ones
+__global__ void __launch_bounds__(kThreads) sel_write(const double* __restrict__ lw, long long n, int h_max,
+                                                      long long* idx_out, double* lw_out, unsigned char* base) {
+  pdl_enter();
+  __shared__ unsigned wg[2][kThreads / 32], we[2][kThreads / 32];
   Ptrs p = ptrs_of(base);
   const SelScal s = *p.sc;
   long long lo, hi;
   chunk_of(n, lo, hi);
-  if (threadIdx.x == 0) {
-    run_g = p.blk_gt[blockIdx.x];
-    run_e = p.blk_eq[blockIdx.x];
-  }
-  __syncthreads();
+  unsigned run_g = p.blk_gt[blockIdx.x], run_e = p.blk_eq[blockIdx.x];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  for (long long base_j = lo; base_j < hi; base_j += blockDim.x) {
+  int par = 0;
+  for (long long base_j = lo; base_j < hi; base_j += kThreads, par ^= 1) {
     const long long j = base_j + threadIdx.x;
     bool gt = false, eq = false;
     long long k = kKeyInvalid;
@@ -349,59 +572,40 @@ __global__ void sel_write(const double* __restrict__ lw, long long n, int h_max,
       keep_kind(k, s, gt, eq);
     }
     const unsigned bg = __ballot_sync(0xFFFFFFFFu, gt), be = __ballot_sync(0xFFFFFFFFu, eq);
-    if (lane == 0) { wg[wp] = __popc(bg); we[wp] = __popc(be); }
+    if (lane == 0) { wg[par][wp] = __popc(bg); we[par][wp] = __popc(be); }
     __syncthreads();
     unsigned og = run_g, oe = run_e;
-    for (int w = 0; w < wp; ++w) { og += wg[w]; oe += we[w]; }
+    for (int w = 0; w < kThreads / 32; ++w) {
+      if (w < wp) { og += wg[par][w]; oe += we[par][w]; }
+      run_g += wg[par][w];
+      run_e += we[par][w];
+    }
     og += __popc(bg & ((1u << lane) - 1u));
     oe += __popc(be & ((1u << lane) - 1u));
     if (gt || (eq && (long long)oe < s.need)) {
       const long long pos = (long long)og + ((long long)oe < s.need ? (long long)oe : s.need);
       if (pos < h_max) {
         idx_out[pos] = j;
-        lw_out[pos] = (double)k * kFxInv - s.lse;
+        lw_out[pos] = ((double)k * kFxInv - s.lse) - s.lse_kept;
       }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { run_g += wg[w]; run_e += we[w]; }
-    }
-    __syncthreads();
   }
 }
 
-// renormalise the kept log-weights (one block)
-__global__ void sel_renorm(double* lw_out, unsigned char* base) {
-  __shared__ double red[32];
-  __shared__ double s_m, s_l;
-  Ptrs p = ptrs_of(base);
-  const long long n = p.sc->n_kept;
-  double m = -INFINITY;
-  for (long long j = threadIdx.x; j < n; j += blockDim.x) m = fmax(m, lw_out[j]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double g = -INFINITY;
-    for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) g = fmax(g, red[w]);
-    s_m = g;
-  }
-  __syncthreads();
-  double sum = 0.0;
-  for (long long j = threadIdx.x; j < n; j += blockDim.x) sum += exp(lw_out[j] - s_m);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double S = 0.0;
-    for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) S += red[w];
-    s_l = s_m + log(S);
-  }
-  __syncthreads();
-  for (long long j = threadIdx.x; j < n; j += blockDim.x) lw_out[j] -= s_l;
+// a launch whose blocks may start while the previous kernel of the stream
+// finishes (every kernel waits for it in pdl_enter)
+template <typename... KArgs, typename... Args>
+void launch_sel(void (*k)(KArgs...), int grid, int block, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
 // device address of the scratch array, looked up once per device
@@ -434,22 +638,28 @@ extern "C" glmb_status glmb_select_top_static(const double* logw_dev, int64_t n,
   const glmb_status st = scratch_for_current_device(&base);
   if (st != GLMB_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  const int nblk = (int)(n == 0 ? 1 : std::min<long long>((n + kThreads - 1) / kThreads, kMaxBlocks));
+  // blocks of the passes whose partials are kept per block, and of the
+  // passes with a histogram per block (one of 1024 threads per SM: each
+  // block adds its bins to global memory once)
+  const int nblk = (int)(n == 0 ? 1 : std::min<long long>((n + 4 * kThreads - 1) / (4 * kThreads), kMaxBlocks));
+  const int hblk = (int)std::max<long long>(1, std::min<long long>((n + 1023) / 1024, 152));
   const double log_tau = std::log(tau);
   const double vmax = std::max(1.0, -log_tau) * 4294967296.0 + 2.0;
   const int nbits = std::max(1, (int)std::ceil(std::log2(vmax)));
-  const int passes = (nbits + kDigitS - 1) / kDigitS;
-  sel_init<<<1, 256, 0, s>>>(base, h_max);
-  sel_lse<<<nblk, kThreads, 0, s>>>(logw_dev, n, log_tau, base);
-  for (int q = 0; q < passes; ++q) {
-    const int shift = (passes - 1 - q) * kDigitS;
-    sel_hist<<<nblk, kThreads, 0, s>>>(logw_dev, n, shift, base);
-    sel_find<<<1, kBinsS / 4, 0, s>>>(shift, q == 0, base);
+  // digits from the top of the nbits bits of key - threshold
+  const int width = std::min(kDigitS, nbits), top = nbits - width;
+  launch_sel(sel_lse, nblk, kThreads, s, logw_dev, n, h_max, base);
+  launch_sel(sel_hist, hblk, 1024, s, logw_dev, n, top, width, 1, nblk, log_tau, base);
+  if (n <= kListN) {
+    if (top > 0) launch_sel(sel_boundary, hblk, 1024, s, logw_dev, n, top, base);
+  } else {
+    for (int above = top; above > 0;) {
+      const int w = std::min(kDigitS, above);
+      above -= w;
+      launch_sel(sel_hist, hblk, 1024, s, logw_dev, n, above, w, 0, nblk, log_tau, base);
+    }
   }
-  sel_count<<<nblk, kThreads, 0, s>>>(logw_dev, n, base);
-  sel_offsets<<<1, 1024, 0, s>>>(nblk, h_max, n_out_dev, base);
-  sel_write<<<nblk, kThreads, 0, s>>>(logw_dev, n, h_max, (long long*)idx_out_dev, logw_out_dev,
-                                      base);
-  sel_renorm<<<1, 1024, 0, s>>>(logw_out_dev, base);
+  launch_sel(sel_count, nblk, kThreads, s, logw_dev, n, h_max, n_out_dev, base);
+  launch_sel(sel_write, nblk, kThreads, s, logw_dev, n, h_max, (long long*)idx_out_dev, logw_out_dev, base);
   return cudaGetLastError() == cudaSuccess ? GLMB_OK : GLMB_E_CUDA;
 }
