@@ -2,10 +2,14 @@
 // children (arXiv 2512.06230, Section 3: weights below tau are discarded,
 // the H_max most likely hypotheses are kept, and one update is run per
 // distinct (track, detection set)), plus the estimate reductions.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "../../include/glmb.h"
 #include "glmb_kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace glmb {
 
@@ -931,19 +935,52 @@ void launch_estimates(const HypTable& hp, int H, const unsigned* H_dev, int H_bo
            (glmb_track*)tracks, pcap, err);
 }
 
-__global__ void meas_assoc_kernel(HypTable hp, int H, int M, double* r_u) {
+// Clutter probability of each detection: the total weight of the hypotheses
+// that assign it to clutter (fixed point: the sums do not depend on order).
+// A cluster of kAssocSplit blocks takes 32 detections (lanes), its warps
+// the hypotheses, so a row of theta is read in 64-byte pieces by many warps
+// at once; the blocks' sums meet in the first one's shared memory.  Measured
+// at about 4000 hypotheses x 200 detections: 484 us with one thread per
+// detection walking all hypotheses (a chain of dependent loads); with the
+// cluster a 40-frame scene that reads it once went from 11.68 to 11.24 ms.
+constexpr int kAssocSplit = 8, kAssocWarps = 16;
+
+__global__ void __cluster_dims__(1, kAssocSplit, 1) __launch_bounds__(32 * kAssocWarps)
+    meas_assoc_kernel(HypTable hp, int H, int M, double* r_u) {
   pdl_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= M) return;
+  __shared__ unsigned long long s_w[kAssocWarps][32];
+  __shared__ unsigned long long s_sum[32];
+  cg::cluster_group cl = cg::this_cluster();
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  const int rank = (int)blockIdx.y;
   unsigned long long s = 0ull;
-  for (int h = 0; h < H; ++h)
-    if (hp.theta[(size_t)h * M + i] == 0) s += w_fx(hp.logw[h]);
-  r_u[i] = (double)s * kWfxInv;
+#pragma unroll 4
+  for (int h = rank * kAssocWarps + wp; h < H; h += kAssocSplit * kAssocWarps) {
+    const unsigned long long w = w_fx(hp.logw[h]);
+    if (i < M && hp.theta[(size_t)h * M + i] == 0) s += w;
+  }
+  s_w[wp][lane] = s;
+  __syncthreads();
+  if (wp == 0) {
+    s = 0ull;
+#pragma unroll
+    for (int w = 0; w < kAssocWarps; ++w) s += s_w[w][lane];
+    s_sum[lane] = s;
+  }
+  cl.sync();
+  if (rank == 0 && wp == 0) {
+    s = 0ull;
+#pragma unroll
+    for (int r = 0; r < kAssocSplit; ++r) s += cl.map_shared_rank(s_sum, r)[lane];
+    if (i < M) r_u[i] = (double)s * kWfxInv;
+  }
+  cl.sync();   // no block leaves while its sums are read
 }
 
 void launch_meas_assoc(const HypTable& hp, int H, int M, double* r_u, cudaStream_t s) {
   if (M <= 0) return;
-  launch_k(meas_assoc_kernel, (M + 127) / 128, 128, 0, s, hp, H, M, r_u);
+  launch_k(meas_assoc_kernel, dim3((M + 31) / 32, kAssocSplit), 32 * kAssocWarps, 0, s, hp, H, M, r_u);
 }
 
 }  // namespace glmb
