@@ -2172,7 +2172,7 @@ glmb_status glmb_mlp_forward(const float* params, const float* X, int64_t n, flo
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   const long long tiles = (n + 127) / 128;
-  const int grid = (int)std::max(1LL, std::min(tiles, 4LL * n_sm));
+  const int grid = (int)std::max(1LL, std::min(tiles, 2LL * n_sm));
   launch_gate_forward_rows(params, X, n, logit, err, grid, (cudaStream_t)stream);
   return cudaGetLastError() == cudaSuccess ? GLMB_OK : GLMB_E_CUDA;
 }
@@ -2181,15 +2181,13 @@ glmb_status glmb_mlp_backward(const float* params, const float* X, const float* 
                               float* grad, double* loss, uint32_t* err, void* stream) {
   if (n < 0 || !params || !grad || !loss || !err || (n > 0 && (!X || !y || !wt))) return GLMB_E_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
-  if (cudaMemsetAsync(grad, 0, GLMB_GATE_NPARAM * sizeof(float), s) != cudaSuccess ||
-      cudaMemsetAsync(loss, 0, sizeof(double), s) != cudaSuccess)
-    return GLMB_E_CUDA;
-  if (n == 0) return GLMB_OK;
+  launch_gate_zero(grad, loss, s);
+  if (n == 0) return cudaGetLastError() == cudaSuccess ? GLMB_OK : GLMB_E_CUDA;
   int dev = 0, n_sm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   const long long tiles = (n + 127) / 128;
-  launch_gate_train(params, X, y, wt, n, grad, loss, err, (int)std::max(1LL, std::min(tiles, (long long)n_sm)), s);
+  launch_gate_train(params, X, y, wt, n, grad, loss, err, (int)std::max(1LL, std::min(tiles, 2LL * n_sm)), s);
   return cudaGetLastError() == cudaSuccess ? GLMB_OK : GLMB_E_CUDA;
 }
 

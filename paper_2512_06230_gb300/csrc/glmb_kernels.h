@@ -271,6 +271,8 @@ void launch_gate_forward_rows(const float* P, const float* X, long long n, float
 void launch_gate_forward_table(const float* P, float thr, const Model& md, const CompTable& ct,
                                const PairTable& full, const FrameDev* fs, float* logit, uint8_t* keep,
                                unsigned* err, int grid, cudaStream_t s);
+// zeroes grad and *loss
+void launch_gate_zero(float* grad, double* loss, cudaStream_t s);
 // adds the gradient of sum wt (softplus(z) - y z) to grad and the loss to *loss
 void launch_gate_train(const float* P, const float* X, const float* y, const float* wt, long long n,
                        float* grad, double* loss, unsigned* err, int grid, cudaStream_t s);
