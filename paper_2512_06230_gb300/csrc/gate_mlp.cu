@@ -325,17 +325,6 @@ __device__ __forceinline__ void write_input(unsigned char* a0, int m, const floa
   st_core8(a0, core_off(m, 8, 2), v + 8);
 }
 
-// component of pair p: the c with ptr[c] <= p < ptr[c + 1]
-__device__ __forceinline__ int pair_comp(const uint32_t* __restrict__ ptr, int T, uint32_t p) {
-  int lo = 0, hi = T;  // invariant ptr[lo] <= p < ptr[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(ptr + mid) <= p) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
-
 }  // namespace
 
 // the gate's raw features of pair p: d^2 (recovered from log C and log det
@@ -395,12 +384,10 @@ __global__ void __launch_bounds__(kTile * kFwdGroups, 2) gate_forward_kernel(con
   volatile int* flag = reinterpret_cast<int*>(sm + FLay::FLAG) + group;
   const uint32_t mbar = smem_u32(sm + FLay::MBAR) + 8u * (uint32_t)group;
   long long n = g.n;
-  int T = 0;
   if (kTable) {
     // a table that overflowed its capacity (the frame is abandoned) is
     // scored only up to the capacity
-    T = g.fs->T;
-    n = min((long long)g.pt.ptr[T], g.pt.cap_pairs);
+    n = min((long long)*g.pt.total, g.pt.cap_pairs);
   }
   const long long tiles = (n + kTile - 1) / kTile;
   if ((long long)blockIdx.x >= tiles) return;
@@ -425,8 +412,7 @@ __global__ void __launch_bounds__(kTile * kFwdGroups, 2) gate_forward_kernel(con
   const long long first = blockIdx.x + (long long)gridDim.x * group, stride = (long long)gridDim.x * kFwdGroups;
   auto features = [&](long long row, float (&f)[kIn]) {
     if (kTable) {
-      const int c = pair_comp(g.pt.ptr, T, (uint32_t)row);
-      pair_features(g.md, g.ct, g.pt, *g.fs, (uint32_t)row, c, f);
+      pair_features(g.md, g.ct, g.pt, *g.fs, (uint32_t)row, (int)g.pt.comp[row], f);
     } else {
 #pragma unroll
       for (int j = 0; j < kIn; ++j) f[j] = __ldg(g.X + row * kIn + j);
@@ -853,35 +839,18 @@ __global__ void gate_adam_kernel(float* __restrict__ P, const float* __restrict_
 __global__ void gate_features_kernel(Model md, CompTable ct, PairTable pt, const FrameDev* __restrict__ fs,
                                      float* __restrict__ X, long long cap) {
   pdl_enter();
-  const int T = fs->T;
-  const long long n = min((long long)pt.ptr[T], cap);
+  const long long n = min((long long)*pt.total, cap);
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n;
        p += (long long)gridDim.x * blockDim.x) {
     float f[kIn];
-    pair_features(md, ct, pt, *fs, (uint32_t)p, pair_comp(pt.ptr, T, (uint32_t)p), f);
+    pair_features(md, ct, pt, *fs, (uint32_t)p, (int)pt.comp[p], f);
     for (int j = 0; j < kIn; ++j) X[p * kIn + j] = f[j];
   }
 }
 
-// kept pairs per component (warp per component)
-__global__ void gate_count_kernel(PairTable full, const uint8_t* __restrict__ keep, PairTable gated,
-                                  const FrameDev* __restrict__ fs) {
-  pdl_enter();
-  const int T = fs->T, lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < T; c += nw) {
-    const uint32_t cap = (uint32_t)full.cap_pairs;
-    const uint32_t lo = min(full.ptr[c], cap), hi = min(full.ptr[c + 1], cap);
-    unsigned k = 0;
-    for (uint32_t j = lo + lane; j < hi; j += 32) k += keep[j];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) k += __shfl_xor_sync(0xFFFFFFFFu, k, off);
-    if (lane == 0) gated.cnt[c] = k;
-  }
-}
-
-// stable compaction of the kept pairs into the gated table, and the death
-// probability (reading R2) over the pairs that remain
+// stable compaction of the kept pairs into the gated table (a warp per
+// component counts its kept pairs, takes their place and copies them), and
+// the death probability (reading R2) over the pairs that remain
 __global__ void gate_compact_kernel(Model md, CompTable ct, PairTable full, const uint8_t* __restrict__ keep,
                                     PairTable gated, const FrameDev* __restrict__ fs) {
   pdl_enter();
@@ -889,8 +858,18 @@ __global__ void gate_compact_kernel(Model md, CompTable ct, PairTable full, cons
   const int nw = (gridDim.x * blockDim.x) >> 5;
   const size_t cf = (size_t)full.cap_pairs, cg = (size_t)gated.cap_pairs;
   for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < T; c += nw) {
-    const uint32_t lo = min(full.ptr[c], (uint32_t)cf), hi = min(full.ptr[c + 1], (uint32_t)cf);
-    uint32_t out = gated.ptr[c];
+    const uint32_t lo = min(full.ptr[c], (uint32_t)cf), hi = min(lo + full.cnt[c], (uint32_t)cf);
+    unsigned kept = 0;
+    for (uint32_t j = lo + lane; j < hi; j += 32) kept += keep[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xFFFFFFFFu, kept, o);
+    uint32_t out = 0;
+    if (lane == 0) {
+      out = kept ? atomicAdd(gated.total, kept) : 0u;
+      gated.cnt[c] = kept;
+      gated.ptr[c] = out;
+    }
+    out = __shfl_sync(0xFFFFFFFFu, out, 0);
     float lm = -INFINITY, ls = 0.f;
     bool any = false;
     for (uint32_t j0 = lo; j0 < hi; j0 += 32) {
@@ -901,6 +880,7 @@ __global__ void gate_compact_kernel(Model md, CompTable ct, PairTable full, cons
       if (k && q < cg) {
         const float lc = full.logC[j];
         gated.meas[q] = full.meas[j];
+        gated.comp[q] = (uint32_t)c;
         gated.logC[q] = lc;
         gated.q[q] = full.q[j];
         for (int a = 0; a < dz; ++a) gated.e[a * cg + q] = full.e[a * cf + j];
@@ -959,7 +939,7 @@ __global__ void gate_usage_kernel(HypTable par, HypTable out, CompTable A, CompT
       if (t == 0 || t > nt) continue;
       const int c = kc[t - 1];
       if (c < 0) continue;
-      uint32_t lo = pt.ptr[c], hi = pt.ptr[c + 1];
+      uint32_t lo = pt.ptr[c], hi = lo + pt.cnt[c];
       const uint32_t end = hi;
       while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
@@ -1048,9 +1028,8 @@ void launch_gate_features(const Model& md, const CompTable& ct, const PairTable&
 }
 
 void launch_gate_compact(const Model& md, const CompTable& ct, const PairTable& full, const uint8_t* keep,
-                         const PairTable& gated, const FrameDev* fs, bool count, int grid, cudaStream_t s) {
-  if (count) launch_k(gate_count_kernel, grid, 256, 0, s, full, keep, gated, fs);
-  else launch_k(gate_compact_kernel, grid, 256, 0, s, md, ct, full, keep, gated, fs);
+                         const PairTable& gated, const FrameDev* fs, int grid, cudaStream_t s) {
+  launch_k(gate_compact_kernel, grid, 256, 0, s, md, ct, full, keep, gated, fs);
 }
 
 void launch_gate_usage(const HypTable& par, const HypTable& out, const CompTable& A, const CompTable& B,

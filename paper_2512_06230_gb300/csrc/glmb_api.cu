@@ -115,11 +115,11 @@ struct glmb_handle {
   uint32_t* gc_flag = nullptr;
   uint32_t* gc_newpos = nullptr;
   // frame results, one device block copied back in one piece:
-  // [scalars (S_N)][prune counters (8)][estimates], mirrored in pinned host
-  // memory up to the end of the estimate records
+  // [estimates][prune counters (8)][scalars (S_N)], mirrored in pinned host
+  // memory; the frame inputs follow it (in_bytes below)
   unsigned* d_scal = nullptr;
   unsigned* h_scal = nullptr;
-  size_t res_off_cnt = 0, res_off_est = 0;
+  size_t res_off_cnt = 0, res_off_scal = 0;
   // estimates: [nb (16 B)][pmf][tracks][done], mirrored on the host up to
   // est_off_end (the start of done); `done` holds the component bound and
   // the block counter of the existence sums, est_rcomp their per-component
@@ -143,13 +143,18 @@ struct glmb_handle {
   bool ev_pending[kNumStages] = {};
   double stage_ms[kNumStages] = {};
   long long stage_calls[kNumStages] = {};
-  // frame inputs, one device block [sizes][births][detections] that a frame
-  // graph fills with one copy from its pinned image; the host block is
-  // [sizes slot 0][the device block's image, whose sizes are slot 1]
-  // (slot 0: glmb_predict, slot 1: glmb_update and glmb_step)
+  // frame inputs, after the results in the same device block:
+  // [scalars][sizes][detections][births].  A frame graph fills them with one
+  // copy from their pinned image, which zeroes the frame's scalars as well;
+  // the births are copied with it for the particle model (each particle reads
+  // its component's record) and read from the pinned image by the table kernel
+  // otherwise.  The host block is [zero scalars, sizes of slot 0][image: zero
+  // scalars, sizes of slot 1, detections, births] (slot 0: glmb_predict, slot
+  // 1: glmb_update and glmb_step).
   size_t in_off_births = 0, in_off_Z = 0;
+  unsigned char* h_in = nullptr;   // the image
   FrameDev* d_fs = nullptr;
-  FrameDev* h_fs = nullptr;
+  FrameDev* h_fs[2] = {nullptr, nullptr};
   // shared-memory plan of the expansion: exact slot maximum (from the last
   // prune), estimated pair maximum (from earlier frames; redone if exceeded)
   int alive_max = 0;
@@ -289,37 +294,41 @@ void free_all(glmb_handle* h) {
 size_t round_up64(size_t x) { return (x + 63) / 64 * 64; }
 
 // The frame's input and result blocks (layouts at their handle fields).
+constexpr size_t kScalBytes = 64;   // S_N scalars, before the sizes
+static_assert(S_N * sizeof(unsigned) == kScalBytes, "scalar block");
 bool alloc_io(glmb_handle* h) {
-  const size_t fs = sizeof(FrameDev);
-  h->in_off_births = round_up64(fs);
-  h->in_off_Z = h->in_off_births + round_up64((size_t)h->cap_births * kBirthRec * sizeof(double));
-  const size_t in_bytes = h->in_off_Z + (size_t)h->cap_meas * h->md.dz * sizeof(float);
-  unsigned char *din = nullptr, *hin = nullptr;
-  if (!dalloc(h, &din, (long long)in_bytes) || !halloc(h, &hin, (long long)(fs + in_bytes))) return false;
-  h->d_fs = reinterpret_cast<FrameDev*>(din);
-  h->d_births = reinterpret_cast<double*>(din + h->in_off_births);
-  h->d_Z = reinterpret_cast<float*>(din + h->in_off_Z);
-  h->h_fs = reinterpret_cast<FrameDev*>(hin);
-  h->h_births = reinterpret_cast<double*>(hin + fs + h->in_off_births);
-  h->h_Z = reinterpret_cast<float*>(hin + fs + h->in_off_Z);
-
   const size_t pcap = (size_t)h->max_tracks + 1;
   h->est_off_pmf = 16;
   h->est_off_tr = h->est_off_pmf + 8 * pcap;
   h->est_off_end = h->est_off_tr + sizeof(glmb_track) * pcap;
   h->est_off_done = h->est_off_end;
-  h->res_off_cnt = round_up64(S_N * sizeof(unsigned));
-  h->res_off_est = h->res_off_cnt + 64;
-  unsigned char *dres = nullptr, *hres = nullptr;
-  if (!dalloc(h, &dres, (long long)(h->res_off_est + h->est_off_done + 16)) ||
-      !halloc(h, &hres, (long long)(h->res_off_est + h->est_off_end)))
+  h->res_off_cnt = round_up64(h->est_off_done + 16);
+  h->res_off_scal = h->res_off_cnt + 64;
+  // offsets from the scalars
+  const size_t fs = kScalBytes + round_up64(sizeof(FrameDev));
+  h->in_off_Z = fs;
+  h->in_off_births = fs + round_up64((size_t)h->cap_meas * h->md.dz * sizeof(float));
+  const size_t in_bytes = h->in_off_births + (size_t)h->cap_births * kBirthRec * sizeof(double);
+  unsigned char *d = nullptr, *hin = nullptr, *hres = nullptr;
+  if (!dalloc(h, &d, (long long)(h->res_off_scal + in_bytes)) || !halloc(h, &hin, (long long)(fs + in_bytes)) ||
+      !halloc(h, &hres, (long long)(h->res_off_scal + kScalBytes)))
     return false;
-  h->d_scal = reinterpret_cast<unsigned*>(dres);
-  h->pw.counts = reinterpret_cast<unsigned*>(dres + h->res_off_cnt);
-  h->d_est = dres + h->res_off_est;
-  h->h_scal = reinterpret_cast<unsigned*>(hres);
+  h->d_est = d;
+  h->pw.counts = reinterpret_cast<unsigned*>(d + h->res_off_cnt);
+  unsigned char* in = d + h->res_off_scal;
+  h->d_scal = reinterpret_cast<unsigned*>(in);
+  h->d_fs = reinterpret_cast<FrameDev*>(in + kScalBytes);
+  h->d_Z = reinterpret_cast<float*>(in + h->in_off_Z);
+  h->d_births = reinterpret_cast<double*>(in + h->in_off_births);
+  std::memset(hin, 0, fs + h->in_off_Z);
+  h->h_fs[0] = reinterpret_cast<FrameDev*>(hin + kScalBytes);
+  h->h_in = hin + fs;
+  h->h_fs[1] = reinterpret_cast<FrameDev*>(h->h_in + kScalBytes);
+  h->h_Z = reinterpret_cast<float*>(h->h_in + h->in_off_Z);
+  h->h_births = reinterpret_cast<double*>(h->h_in + h->in_off_births);
+  h->h_est = hres;
   h->h_cnt = reinterpret_cast<unsigned*>(hres + h->res_off_cnt);
-  h->h_est = hres + h->res_off_est;
+  h->h_scal = reinterpret_cast<unsigned*>(hres + h->res_off_scal);
   return true;
 }
 
@@ -626,7 +635,7 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
             alloc_hyps(h, h->hyps[0]) && alloc_hyps(h, h->hyps[1]) &&
             alloc_io(h) && dalloc(h, &h->est_rcomp, h->cap_comp + h->max_tracks + 1) &&
             dalloc(h, &h->pt.cnt, h->cap_comp + 1) && dalloc(h, &h->pt.ptr, h->cap_comp + 1) &&
-            dalloc(h, &h->pt.meas, h->cap_pairs) && dalloc(h, &h->pt.logC, h->cap_pairs) &&
+            dalloc(h, &h->pt.meas, h->cap_pairs) && dalloc(h, &h->pt.comp, h->cap_pairs) && dalloc(h, &h->pt.logC, h->cap_pairs) &&
             dalloc(h, &h->pt.q, h->cap_pairs) && dalloc(h, &h->pt.e, h->cap_pairs * dz) &&
             dalloc(h, &h->pt.dthr, h->cap_comp) && dalloc(h, &h->pt.dprob, h->cap_comp) &&
             dalloc(h, &h->pt.logdetS, h->cap_comp) &&
@@ -663,6 +672,8 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
     return GLMB_E_OOM;
   }
   h->pt.cap_pairs = h->cap_pairs;
+  h->pt.total = h->d_scal + S_K;
+  h->pt_full.total = h->d_scal + S_KFULL;
   cudaMemsetAsync(h->pw.blk_done, 0, 4 * sizeof(unsigned), h->stream);
   cudaMemsetAsync(h->pw.hist, 0, 4096 * sizeof(unsigned), h->stream);
   if (set_initial(h) != GLMB_OK) {
@@ -781,10 +792,10 @@ glmb_status stage_detections(glmb_handle* h, const float* Z, int M, int z_is_dev
   return GLMB_OK;
 }
 
-// frame sizes to the device (pinned slot -> d_fs; by this call, or by the
-// frame graph when copy is false)
+// frame sizes to the device, and the frame's scalars to zero (pinned slot ->
+// d_scal, d_fs; by this call, or by the frame graph when copy is false)
 glmb_status upload_sizes(glmb_handle* h, int slot, bool copy = true) {
-  FrameDev& f = h->h_fs[slot];
+  FrameDev& f = *h->h_fs[slot];
   f = FrameDev{};
   f.n_comp = h->n_comp;
   f.nb = h->nb;
@@ -793,7 +804,9 @@ glmb_status upload_sizes(glmb_handle* h, int slot, bool copy = true) {
   f.H = h->H;
   f.frame = h->frame;
   f.Z = h->z_dev;
-  if (copy) CU(cudaMemcpyAsync(h->d_fs, &f, sizeof f, cudaMemcpyHostToDevice, h->stream));
+  if (copy)
+    CU(cudaMemcpyAsync(h->d_scal, reinterpret_cast<unsigned char*>(&f) - kScalBytes, kScalBytes + sizeof f,
+                       cudaMemcpyHostToDevice, h->stream));
   return GLMB_OK;
 }
 
@@ -814,32 +827,37 @@ glmb_status enqueue_predict(glmb_handle* h, const Plan& p) {
   return GLMB_OK;
 }
 
-glmb_status enqueue_table(glmb_handle* h, const Plan& p) {
+// fuse: the table kernel predicts the components it gates (a frame graph
+// without enqueue_predict), from the pinned birth records
+glmb_status enqueue_table(glmb_handle* h, const Plan& p, bool fuse = false) {
   const CompTable& B = h->comps[1 - h->cur];
-  const int T = h->T_work, dz = h->md.dz;
-  const long long cap = p.fixed ? h->cap_comp : std::max(T, 1);
-  CU(cudaMemsetAsync(h->d_scal, 0, S_N * sizeof(unsigned), h->stream));
+  const int T = h->T_work;
   prof_begin(h, kStageTable);
   const int gt = p.fixed ? 4 * h->n_sm : std::max(1, std::min((T * 32 + 255) / 256, 16 * h->n_sm));
   // with the gate pruning, the Mahalanobis-gated table goes to pt_full and
   // the gate compacts the pairs it keeps into pt
   const bool prune = h->gate_mode == GLMB_GATE_PRUNE;
   const PairTable& P0 = prune ? h->pt_full : h->pt;
-  launch_table_count(h->md, B, P0, h->d_fs, h->d_scal + S_ERR, gt, h->stream);   // also checks Z is finite
-  scan_u32(P0.cnt, P0.ptr, &h->d_fs->T, 1, cap, h->d_scal + (prune ? S_KFULL : S_K), true, h->scan_tmp32,
-           h->scan_cap32, h->d_scal + S_ERR, h->stream);
-  launch_table_write(h->md, B, P0, h->d_fs, h->d_scal + S_FP64, h->d_scal + S_ERR, gt,
-                     h->stream);
+  TableArgs ta{};
+  ta.md = h->md;
+  ta.src = h->comps[h->cur];
+  ta.ct = B;
+  ta.pt = P0;
+  ta.fs = h->d_fs;
+  ta.births = fuse ? h->h_births : h->d_births;
+  ta.fuse = fuse ? 1 : 0;
+  ta.n_fp64 = h->d_scal + S_FP64;
+  ta.err = h->d_scal + S_ERR;
+  ta.hkeys = h->hkeys;
+  ta.upd_slot = h->upd_slot;
+  ta.n_upd_prev = h->d_hprev;
+  ta.cap_upd = (int)h->cap_upd;
+  launch_table(ta, h->cap_meas, gt, h->stream);   // also checks Z is finite
   if (h->md.particle) launch_particle_logc(h->md, h->pm, B, P0, h->d_fs, gt, h->stream);
   if (h->gate_mode != GLMB_GATE_OFF) {
     launch_gate_forward_table(h->gate_params, h->gate_thr, h->md, B, P0, h->d_fs, h->gate_logit,
                               prune ? h->gate_keep : nullptr, h->d_scal + S_ERR, 2 * h->n_sm, h->stream);
-    if (prune) {
-      launch_gate_compact(h->md, B, P0, h->gate_keep, h->pt, h->d_fs, true, gt, h->stream);
-      scan_u32(h->pt.cnt, h->pt.ptr, &h->d_fs->T, 1, cap, h->d_scal + S_K, true, h->scan_tmp32, h->scan_cap32,
-               h->d_scal + S_ERR, h->stream);
-      launch_gate_compact(h->md, B, P0, h->gate_keep, h->pt, h->d_fs, false, gt, h->stream);
-    }
+    if (prune) launch_gate_compact(h->md, B, P0, h->gate_keep, h->pt, h->d_fs, gt, h->stream);
   }
   h->gate_mode_frame = h->gate_mode;
   // the largest slot and pair counts per parent are recorded by the
@@ -1017,9 +1035,6 @@ glmb_status enqueue_prune(glmb_handle* h, const Plan& p) {
                     h->cap_entries, s);
   }
   prof_end(h, kStageSelect);
-  // the update hash table: only the slots the last materialisation filled
-  // are cleared (the whole table is cleared after a frame that failed)
-  launch_hash_reset(h->hkeys, h->upd_slot, h->d_hprev, (int)h->cap_upd, h->d_scal + S_NUPD, 2 * h->n_sm, s);
   const long long capT = p.fixed ? h->cap_comp : std::max(h->T_work, 1);
   ExpandArgs a = expand_args(h, p, true);
   a.surv_idx = h->pw.surv_idx;
@@ -1176,9 +1191,10 @@ glmb_status exact_maxima(glmb_handle* h, unsigned& max_T, unsigned& max_K) {
 // the frame's counters (and, with estimates, the estimate block) to pinned
 // host memory, on the stream
 glmb_status enqueue_results(glmb_handle* h, bool with_est) {
-  // scalars and counters (and the estimates) in one copy of the result block
-  const size_t bytes = with_est ? h->res_off_est + h->est_off_end : h->res_off_cnt + 8 * sizeof(unsigned);
-  CU(cudaMemcpyAsync(h->h_scal, h->d_scal, bytes, cudaMemcpyDeviceToHost, h->stream));
+  // counters and scalars (after the estimates) in one copy of the result block
+  const size_t from = with_est ? 0 : h->res_off_cnt;
+  CU(cudaMemcpyAsync(h->h_est + from, h->d_est + from, h->res_off_scal + kScalBytes - from, cudaMemcpyDeviceToHost,
+                     h->stream));
   return GLMB_OK;
 }
 
@@ -1268,6 +1284,42 @@ glmb_status finish_frame(glmb_handle* h, bool copies_enqueued = false, bool est_
   ++h->gen;
   if (est_enqueued) h->est_gen = h->gen;
   return GLMB_OK;
+}
+
+extern "C++" {
+// Pairs of table P in table order (component, then detection): their storage
+// positions, and the CSR offsets by component.
+glmb_status pair_order(glmb_handle* h, const PairTable& P, std::vector<uint32_t>& csr, std::vector<uint32_t>& at) {
+  const int T = h->T_work;
+  unsigned K32 = 0;
+  CU(cudaMemcpy(&K32, P.total, sizeof K32, cudaMemcpyDeviceToHost));
+  std::vector<uint32_t> cnt(std::max(T, 1)), ptr(std::max(T, 1));
+  if (T > 0) {
+    CU(cudaMemcpy(cnt.data(), P.cnt, (size_t)T * 4, cudaMemcpyDeviceToHost));
+    CU(cudaMemcpy(ptr.data(), P.ptr, (size_t)T * 4, cudaMemcpyDeviceToHost));
+  }
+  csr.assign((size_t)T + 1, 0u);
+  at.clear();
+  at.reserve(K32);
+  for (int c = 0; c < T; ++c) {
+    for (uint32_t j = 0; j < cnt[c]; ++j) at.push_back(ptr[c] + j);
+    csr[c + 1] = (uint32_t)at.size();
+  }
+  return GLMB_OK;
+}
+
+// rows of `width` device elements at the storage positions `at`, in that
+// order, `stride` elements apart in out (positions beyond the n stored rows,
+// of a table that overflowed, give zeros)
+template <typename T>
+glmb_status gather_pairs(glmb_handle* h, T* out, int stride, const T* src, int width, const std::vector<uint32_t>& at,
+                         long long n) {
+  std::vector<T> col((size_t)n * width);
+  CU(cudaMemcpy(col.data(), src, col.size() * sizeof(T), cudaMemcpyDeviceToHost));
+  for (size_t k = 0; k < at.size(); ++k)
+    for (int a = 0; a < width; ++a) out[k * stride + a] = at[k] < n ? col[(size_t)at[k] * width + a] : T(0);
+  return GLMB_OK;
+}
 }
 
 }  // namespace
@@ -1439,12 +1491,21 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
       const auto t_cap = std::chrono::steady_clock::now();
       CU(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
       h->capturing = true;
-      // sizes, births and host detections in one copy of the input block
-      cudaMemcpyAsync(h->d_fs, &h->h_fs[1],
-                      h->in_off_Z + (size_t)std::min(q.M, h->cap_meas) * h->md.dz * sizeof(float),
-                      cudaMemcpyHostToDevice, h->stream);
-      enqueue_predict(h, q);
-      enqueue_table(h, q);
+      // zero scalars, sizes and host detections (and the particle model's
+      // births) in one copy of the input block
+      const size_t in_bytes =
+          h->md.particle ? h->in_off_births + (size_t)h->cap_births * kBirthRec * sizeof(double)
+                         : h->in_off_Z + (size_t)std::min(q.M, h->cap_meas) * h->md.dz * sizeof(float);
+      cudaMemcpyAsync(h->d_scal, h->h_in, in_bytes, cudaMemcpyHostToDevice, h->stream);
+      // (a profiled prediction stage runs the prediction on its own)
+      const bool fuse = !h->md.particle && !(h->prof_mask & (1u << kStagePredict));
+      if (!fuse) {
+        if (!h->md.particle)
+          cudaMemcpyAsync(h->d_births, h->h_births, (size_t)h->cap_births * kBirthRec * sizeof(double),
+                          cudaMemcpyHostToDevice, h->stream);
+        enqueue_predict(h, q);
+      }
+      enqueue_table(h, q, fuse);
       enqueue_expand(h, q, true);
       enqueue_prune(h, q);
       if (h->step_estimates)
@@ -1609,7 +1670,7 @@ glmb_status glmb_get_info(glmb_handle* h, glmb_info* info) {
   info->n_pairs = h->n_pairs;
   if (h->have_update) {
     uint32_t K32 = 0;
-    CU(cudaMemcpy(&K32, h->pt.ptr + h->T_work, sizeof K32, cudaMemcpyDeviceToHost));
+    CU(cudaMemcpy(&K32, h->pt.total, sizeof K32, cudaMemcpyDeviceToHost));
     info->n_pairs = K32;
   }
   info->n_pairs_pregate = h->gate_mode_frame == GLMB_GATE_PRUNE ? h->n_pairs_pregate : info->n_pairs;
@@ -2007,22 +2068,21 @@ glmb_status glmb_get_pairs(glmb_handle* h, uint32_t* comp_ptr, uint32_t* meas, f
   if (!h->have_update) return fail(h, GLMB_E_STATE, "get_pairs: no update");
   CU(cudaStreamSynchronize(h->stream));
   const int T = h->T_work, dz = h->md.dz;
-  uint32_t K32 = 0;
-  CU(cudaMemcpy(&K32, h->pt.ptr + T, sizeof K32, cudaMemcpyDeviceToHost));
-  const long long K = std::min<long long>(K32, h->cap_pairs);
+  std::vector<uint32_t> csr, at;
+  glmb_status st = pair_order(h, h->pt, csr, at);
+  if (st != GLMB_OK) return st;
+  const long long K = std::min<long long>((long long)at.size(), h->cap_pairs);
   *n_pairs = K;
   if (T + 1 > cap_comp || K > cap_pairs) return fail(h, GLMB_E_CAPACITY, "get_pairs: caps");
-  if (comp_ptr) CU(cudaMemcpy(comp_ptr, h->pt.ptr, (size_t)(T + 1) * 4, cudaMemcpyDeviceToHost));
+  if (comp_ptr) std::memcpy(comp_ptr, csr.data(), (size_t)(T + 1) * 4);
+  at.resize(K);
   if (K == 0) return GLMB_OK;
-  if (meas) CU(cudaMemcpy(meas, h->pt.meas, (size_t)K * 4, cudaMemcpyDeviceToHost));
-  if (logC) CU(cudaMemcpy(logC, h->pt.logC, (size_t)K * 4, cudaMemcpyDeviceToHost));
-  if (q) CU(cudaMemcpy(q, h->pt.q, (size_t)K * 4, cudaMemcpyDeviceToHost));
+  if (meas && (st = gather_pairs(h, meas, 1, h->pt.meas, 1, at, K)) != GLMB_OK) return st;
+  if (logC && (st = gather_pairs(h, logC, 1, h->pt.logC, 1, at, K)) != GLMB_OK) return st;
+  if (q && (st = gather_pairs(h, q, 1, h->pt.q, 1, at, K)) != GLMB_OK) return st;
   if (e)
-    for (int a = 0; a < dz; ++a) {
-      std::vector<float> col(K);
-      CU(cudaMemcpy(col.data(), h->pt.e + (size_t)a * h->cap_pairs, (size_t)K * 4, cudaMemcpyDeviceToHost));
-      for (long long j = 0; j < K; ++j) e[j * dz + a] = col[j];
-    }
+    for (int a = 0; a < dz; ++a)
+      if ((st = gather_pairs(h, e + a, dz, h->pt.e + (size_t)a * h->cap_pairs, 1, at, K)) != GLMB_OK) return st;
   return GLMB_OK;
 }
 
@@ -2072,7 +2132,7 @@ glmb_status glmb_set_gate(glmb_handle* h, const float* params, float threshold, 
   if (mode == GLMB_GATE_PRUNE && !h->pt_full.ptr) {
     PairTable& F = h->pt_full;
     if (!(dalloc(h, &F.cnt, h->cap_comp + 1) && dalloc(h, &F.ptr, h->cap_comp + 1) &&
-          dalloc(h, &F.meas, h->cap_pairs) && dalloc(h, &F.logC, h->cap_pairs) && dalloc(h, &F.q, h->cap_pairs) &&
+          dalloc(h, &F.meas, h->cap_pairs) && dalloc(h, &F.comp, h->cap_pairs) && dalloc(h, &F.logC, h->cap_pairs) && dalloc(h, &F.q, h->cap_pairs) &&
           dalloc(h, &F.e, h->cap_pairs * dz) && dalloc(h, &F.dthr, h->cap_comp) &&
           dalloc(h, &F.dprob, h->cap_comp))) {
       F.ptr = nullptr;
@@ -2111,16 +2171,17 @@ glmb_status glmb_gate_features(glmb_handle* h, float* X, int64_t cap, int64_t* n
   if (!h->have_update) return fail(h, GLMB_E_STATE, "gate_features: no update");
   CU(cudaStreamSynchronize(h->stream));
   const PairTable& P0 = pregate_table(h);
-  uint32_t K32 = 0;
-  CU(cudaMemcpy(&K32, P0.ptr + h->T_work, sizeof K32, cudaMemcpyDeviceToHost));
-  *n = K32;
-  if ((int64_t)K32 > cap) return fail(h, GLMB_E_CAPACITY, "gate_features: %u pairs, cap %lld", K32, (long long)cap);
-  if (K32 == 0) return GLMB_OK;
+  std::vector<uint32_t> csr, at;
+  glmb_status st = pair_order(h, P0, csr, at);
+  if (st != GLMB_OK) return st;
+  *n = (int64_t)at.size();
+  if (*n > cap)
+    return fail(h, GLMB_E_CAPACITY, "gate_features: %lld pairs, cap %lld", (long long)*n, (long long)cap);
+  if (*n == 0) return GLMB_OK;
   if (!h->gate_X && !dalloc(h, &h->gate_X, h->cap_pairs * 5)) return fail(h, GLMB_E_OOM, "gate_features: scratch");
   launch_gate_features(h->md, h->comps[1 - h->cur], P0, h->d_fs, h->gate_X, h->cap_pairs, 2 * h->n_sm, h->stream);
-  CU(cudaMemcpyAsync(X, h->gate_X, (size_t)K32 * 5 * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
-  return GLMB_OK;
+  return gather_pairs(h, X, 5, h->gate_X, 5, at, std::min<long long>(*n, h->cap_pairs));
 }
 
 glmb_status glmb_gate_logits(glmb_handle* h, float* logit, int64_t cap, int64_t* n) {
@@ -2128,12 +2189,13 @@ glmb_status glmb_gate_logits(glmb_handle* h, float* logit, int64_t cap, int64_t*
   if (!h->have_update || h->gate_mode_frame == GLMB_GATE_OFF)
     return fail(h, GLMB_E_STATE, "gate_logits: no update with the gate on");
   CU(cudaStreamSynchronize(h->stream));
-  uint32_t K32 = 0;
-  CU(cudaMemcpy(&K32, pregate_table(h).ptr + h->T_work, sizeof K32, cudaMemcpyDeviceToHost));
-  *n = K32;
-  if ((int64_t)K32 > cap) return fail(h, GLMB_E_CAPACITY, "gate_logits: cap");
-  if (K32) CU(cudaMemcpy(logit, h->gate_logit, (size_t)K32 * sizeof(float), cudaMemcpyDeviceToHost));
-  return GLMB_OK;
+  std::vector<uint32_t> csr, at;
+  glmb_status st = pair_order(h, pregate_table(h), csr, at);
+  if (st != GLMB_OK) return st;
+  *n = (int64_t)at.size();
+  if (*n > cap) return fail(h, GLMB_E_CAPACITY, "gate_logits: cap");
+  if (*n == 0) return GLMB_OK;
+  return gather_pairs(h, logit, 1, h->gate_logit, 1, at, std::min<long long>(*n, h->cap_pairs));
 }
 
 glmb_status glmb_gate_usage(glmb_handle* h, uint8_t* used, int64_t cap_pairs, uint8_t* hyp_flag, int cap_h,
@@ -2143,8 +2205,10 @@ glmb_status glmb_gate_usage(glmb_handle* h, uint8_t* used, int64_t cap_pairs, ui
     return fail(h, GLMB_E_STATE, "gate_usage: no pruned frame");
   if (h->gate_mode_frame == GLMB_GATE_PRUNE) return fail(h, GLMB_E_STATE, "gate_usage: the gate pruned the table");
   CU(cudaStreamSynchronize(h->stream));
-  uint32_t K32 = 0;
-  CU(cudaMemcpy(&K32, h->pt.ptr + h->T_work, sizeof K32, cudaMemcpyDeviceToHost));
+  std::vector<uint32_t> csr, at;
+  glmb_status st = pair_order(h, h->pt, csr, at);
+  if (st != GLMB_OK) return st;
+  const uint32_t K32 = (uint32_t)at.size();
   *n_pairs = K32;
   *n_hyp = h->H;
   if ((used && (int64_t)K32 > cap_pairs) || (hyp_flag && h->H > cap_h))
@@ -2158,9 +2222,9 @@ glmb_status glmb_gate_usage(glmb_handle* h, uint8_t* used, int64_t cap_pairs, ui
   launch_gate_usage(h->hyps[h->par_buf], h->hyps[h->hcur], h->comps[h->cur], h->comps[1 - h->cur], h->pw.surv_idx,
                     h->H, h->cfg.h_up, h->theta_M, h->pt, h->d_fs, score ? h->gate_logit : nullptr, h->gate_thr,
                     h->gate_used, h->gate_hflag, capT, std::max(1, std::min(h->H, 8 * h->n_sm)), h->stream);
-  if (used && K32) CU(cudaMemcpyAsync(used, h->gate_used, K32, cudaMemcpyDeviceToHost, h->stream));
   if (hyp_flag && h->H) CU(cudaMemcpyAsync(hyp_flag, h->gate_hflag, (size_t)h->H, cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
+  if (used && K32) return gather_pairs(h, used, 1, h->gate_used, 1, at, std::min<long long>(K32, h->cap_pairs));
   return GLMB_OK;
 }
 

@@ -101,9 +101,13 @@ struct CompTable {
 };
 
 struct PairTable {
-  uint32_t* cnt;          // [comp] gated count (count pass)
-  uint32_t* ptr;          // [comp + 1] CSR offsets
+  // component c's gated pairs, in detection order, at [ptr[c], ptr[c] + cnt[c]);
+  // the components' pieces lie in the order they were taken (from *total)
+  uint32_t* cnt;          // [comp]
+  uint32_t* ptr;          // [comp]
+  unsigned* total;        // pairs taken so far (zero at the frame's start)
   uint32_t* meas;         // [pair]
+  uint32_t* comp;         // [pair] its component
   float* logC;            // [pair] log Eq. 2 entry
   float* q;               // [pair] e^T R^-1 e
   float* e;               // [dz][cap_pairs]

@@ -37,12 +37,27 @@ inline void launch_k(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
 // appended at dst[n_comp..) (births_dev: per birth [r, mean[6], cov[36]] FP64)
 void launch_predict(const Model& md, const CompTable& src, const CompTable& dst, const FrameDev* fs,
                     const double* births_dev, int grid, cudaStream_t s);
-// detections: fs->Z ([M][dz] floats on the device); the count kernel also
-// sets kErrInput in *err when a detection coordinate is not finite
-void launch_table_count(const Model& md, const CompTable& ct, const PairTable& pt,
-                        const FrameDev* fs, unsigned* err, int grid, cudaStream_t s);
-void launch_table_write(const Model& md, const CompTable& ct, const PairTable& pt,
-                        const FrameDev* fs, unsigned* n_fp64, unsigned* err, int grid, cudaStream_t s);
+// the gated table (and, with fuse, the prediction and births of the working
+// table before it); detections: fs->Z ([M][dz] floats on the device), whose
+// coordinates are checked finite (kErrInput in *err); *pt.total, *n_fp64 and
+// *err are zero before; also clears the update hash table's slots that the
+// last materialisation filled
+struct TableArgs {
+  Model md;
+  CompTable src, ct;      // state table (fuse), working table
+  PairTable pt;
+  const FrameDev* fs;
+  const double* births;   // birth records (fuse; device or pinned host memory)
+  int fuse;
+  int words;              // set by launch_table
+  unsigned* n_fp64;
+  unsigned* err;
+  unsigned long long* hkeys;
+  const uint32_t* upd_slot;
+  const unsigned* n_upd_prev;
+  int cap_upd;
+};
+void launch_table(TableArgs a, int cap_meas, int grid, cudaStream_t s);
 void launch_parent_stats(const HypTable& hp, const FrameDev* fs, const PairTable& pt,
                          unsigned* max_T, unsigned* max_K, int grid, cudaStream_t s);
 
@@ -185,11 +200,6 @@ int expand_warp_best_cta(int dz, int materialize, int T, int max_warps, int smem
 // whether a kernel of a captured graph takes the frame's Philox key in its
 // ExpandArgs (the draw and warp kernels)
 bool expand_kernel_takes_key(const void* fn);
-// clears the hash slots of the n_prev updates recorded in upd_slot (the
-// previous materialisation's), instead of clearing the whole table, and
-// zeroes the insert counter n_cur
-void launch_hash_reset(unsigned long long* hkeys, const uint32_t* upd_slot, const unsigned* n_prev, int cap_upd,
-                       unsigned* n_cur, int grid, cudaStream_t s);
 struct PruneWork;
 // marks duplicate children (status 2, key dropped), one block per parent
 // and writes the log-sum-exp partial of its unique children per block
@@ -278,13 +288,14 @@ void launch_gate_train(const float* P, const float* X, const float* y, const flo
                        float* grad, double* loss, unsigned* err, int grid, cudaStream_t s);
 void launch_gate_adam(float* P, const float* G, float* m, float* v, int t, float lr, float b1, float b2,
                       float eps, cudaStream_t s);
-// raw features of the pairs of table pt into X (at most cap rows)
+// raw features of the pairs of table pt into X (at most cap rows, where the
+// pairs lie)
 void launch_gate_features(const Model& md, const CompTable& ct, const PairTable& pt, const FrameDev* fs,
                           float* X, long long cap, int grid, cudaStream_t s);
-// count = true: kept pairs per component into gated.cnt; false: stable
-// compaction into gated (whose ptr is the scan of cnt) and death probabilities
+// the pairs of `full` that the gate kept, compacted into gated (component by
+// component, in detection order), and the death probabilities
 void launch_gate_compact(const Model& md, const CompTable& ct, const PairTable& full, const uint8_t* keep,
-                         const PairTable& gated, const FrameDev* fs, bool count, int grid, cudaStream_t s);
+                         const PairTable& gated, const FrameDev* fs, int grid, cudaStream_t s);
 // pairs of table pt used by the H_new retained hypotheses `out` (children
 // surv[j] of parents `par`; A the new state's components, B the predicted
 // ones; capT >= the largest retained track count), and per retained

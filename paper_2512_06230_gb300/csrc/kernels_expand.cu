@@ -534,8 +534,9 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   __syncthreads();
   for (int t = tid; t < T; t += nthr) {
     const uint32_t c = s_comp[t];
-    for (uint32_t j = pt.ptr[c], je = pt.ptr[c + 1]; j < je; ++j) atomicAdd(&s_rowfill[pt.meas[j]], 1u);
-    s_srow[t] = (pt.ptr[c + 1] > pt.ptr[c] && s_dthr[t] > 0u) ? 1 : 0;
+    const uint32_t n = pt.cnt[c], j0 = pt.ptr[c];
+    for (uint32_t j = j0; j < j0 + n; ++j) atomicAdd(&s_rowfill[pt.meas[j]], 1u);
+    s_srow[t] = (n && s_dthr[t] > 0u) ? 1 : 0;
   }
   __syncthreads();
   // exclusive scan of the row counts over the block: each thread a
@@ -579,7 +580,7 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   if (s_wsum[7]) return;
   for (int t = tid; t < T; t += nthr) {
     const uint32_t c = s_comp[t];
-    for (uint32_t j = pt.ptr[c], je = pt.ptr[c + 1]; j < je; ++j) {
+    for (uint32_t j = pt.ptr[c], je = j + pt.cnt[c]; j < je; ++j) {
       const uint32_t i = pt.meas[j];
       const uint32_t pos = atomicAdd(&s_rowfill[i], 1u);
       s_cslot[pos] = (uint16_t)t;
@@ -1846,20 +1847,6 @@ __global__ void __launch_bounds__(128) dedup_kernel(const FrameDev* __restrict__
     part_sum[blockIdx.x] = t;
     part_cnt[blockIdx.x] = c;
   }
-}
-
-__global__ void hash_reset_kernel(unsigned long long* hkeys, const uint32_t* __restrict__ upd_slot,
-                                  const unsigned* __restrict__ n_prev, int cap_upd, unsigned* n_cur) {
-  pdl_enter();
-  if (blockIdx.x == 0 && threadIdx.x == 0) *n_cur = 0u;   // this frame's insert counter
-  const unsigned n = min(*n_prev, (unsigned)cap_upd);
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    hkeys[upd_slot[i]] = 0ull;
-}
-
-void launch_hash_reset(unsigned long long* hkeys, const uint32_t* upd_slot, const unsigned* n_prev, int cap_upd,
-                       unsigned* n_cur, int grid, cudaStream_t s) {
-  launch_k(hash_reset_kernel, grid, 256, 0, s, hkeys, upd_slot, n_prev, cap_upd, n_cur);
 }
 
 void launch_dedup(const FrameDev* fs, int HU, long long* child_key, const unsigned long long* child_hash,

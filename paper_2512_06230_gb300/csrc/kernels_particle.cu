@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(256) particle_logc_kernel(Model md, PartModel 
   const float r0 = (float)pm.Rinv[0], r1 = (float)(pm.Rinv[1] + pm.Rinv[2]), r3 = (float)pm.Rinv[3];
   const float lc0 = (float)(pm.log_pd - pm.lnorm);
   for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < T; c += nwarps) {
-    const unsigned k0 = pt.ptr[c], k1 = min(pt.ptr[c + 1], cap_p);
+    const unsigned k0 = min(pt.ptr[c], cap_p), k1 = min(k0 + pt.cnt[c], cap_p);
     const double mx = (double)ct.mhi[c], my = (double)ct.mhi[(size_t)ct.cap + c];
     float ox[kRegP], oy[kRegP], ow[kRegP];
 #pragma unroll
