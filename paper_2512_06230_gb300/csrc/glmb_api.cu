@@ -123,7 +123,7 @@ struct glmb_handle {
   // estimates: [nb (16 B)][pmf][tracks][done], mirrored on the host up to
   // est_off_end (the start of done); `done` holds the component bound and
   // the block counter of the existence sums, est_rcomp their per-component
-  // sums followed by the per-track sums (all left zeroed by the kernels)
+  // sums (all left zeroed by the kernels)
   unsigned char* d_est = nullptr;
   unsigned long long* est_rcomp = nullptr;
   unsigned char* h_est = nullptr;
@@ -633,7 +633,7 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
   const long long scan_n = std::max(h->cap_comp, h->cap_children);
   bool ok = alloc_comps(h, h->comps[0], h->cap_comp, dx) && alloc_comps(h, h->comps[1], h->cap_comp, dx) &&
             alloc_hyps(h, h->hyps[0]) && alloc_hyps(h, h->hyps[1]) &&
-            alloc_io(h) && dalloc(h, &h->est_rcomp, h->cap_comp + h->max_tracks + 1) &&
+            alloc_io(h) && dalloc(h, &h->est_rcomp, h->cap_comp) &&
             dalloc(h, &h->pt.cnt, h->cap_comp + 1) && dalloc(h, &h->pt.ptr, h->cap_comp + 1) &&
             dalloc(h, &h->pt.meas, h->cap_pairs) && dalloc(h, &h->pt.comp, h->cap_pairs) && dalloc(h, &h->pt.logC, h->cap_pairs) &&
             dalloc(h, &h->pt.q, h->cap_pairs) && dalloc(h, &h->pt.e, h->cap_pairs * dz) &&
@@ -1187,26 +1187,40 @@ glmb_status exact_maxima(glmb_handle* h, unsigned& max_T, unsigned& max_K) {
   return GLMB_OK;
 }
 
-// frame result: commit, abandon, or redo with exact maxima; `done` on return
-// the frame's counters (and, with estimates, the estimate block) to pinned
-// host memory, on the stream
-glmb_status enqueue_results(glmb_handle* h, bool with_est) {
-  // counters and scalars (after the estimates) in one copy of the result block
-  const size_t from = with_est ? 0 : h->res_off_cnt;
-  CU(cudaMemcpyAsync(h->h_est + from, h->d_est + from, h->res_off_scal + kScalBytes - from, cudaMemcpyDeviceToHost,
-                     h->stream));
+// the frame's counters and scalars to pinned host memory, on the stream (a
+// frame with its estimates has them written by the estimates' kernel)
+glmb_status enqueue_results(glmb_handle* h) {
+  CU(cudaMemcpyAsync(h->h_cnt, h->pw.counts, 64 + kScalBytes, cudaMemcpyDeviceToHost, h->stream));
   return GLMB_OK;
 }
 
-// estimates of table (Y, A) with Y's hypothesis count on the device
-// (H_dev) or on the host
+// estimates of table (Y, A) with Y's hypothesis count on the device (H_dev:
+// a frame's own estimates, written with its counters and scalars straight to
+// the pinned result block) or on the host
 void enqueue_estimates(glmb_handle* h, const HypTable& Y, const CompTable& A, const unsigned* H_dev, int H) {
-  const int pcap = h->max_tracks + 1;
   prof_begin(h, kStageEstimates);
   unsigned* work = reinterpret_cast<unsigned*>(h->d_est + h->est_off_done);   // [cmax, done]
-  launch_estimates(Y, H, H_dev, H_dev ? h->cap_h : H, A, h->md.dx, (double*)(h->d_est + h->est_off_pmf), pcap,
-                   (int*)h->d_est, h->est_rcomp, h->est_rcomp + h->cap_comp, h->d_est + h->est_off_tr, work,
-                   work + 1, h->n_sm, H_dev ? h->d_scal + S_ERR : nullptr, h->stream);
+  unsigned char* to = H_dev ? h->h_est : h->d_est;
+  EstArgs a{};
+  a.hp = Y;
+  a.H_host = H;
+  a.H_dev = H_dev;
+  a.ct = A;
+  a.dx = h->md.dx;
+  a.pmf = (double*)(to + h->est_off_pmf);
+  a.pcap = h->max_tracks + 1;
+  a.nb = (int*)h->d_est;
+  a.r_comp = h->est_rcomp;
+  a.cmax = work;
+  a.done = work + 1;
+  a.out = (glmb_track*)(to + h->est_off_tr);
+  if (H_dev) {
+    a.err = h->d_scal + S_ERR;
+    a.res_dev = h->pw.counts;   // the counters, then the scalars
+    a.res_host = h->h_cnt;
+    a.nb_host = (int*)h->h_est;
+  }
+  launch_estimates(a, H_dev ? h->cap_h : H, h->n_sm, h->stream);
   prof_end(h, kStageEstimates);
 }
 
@@ -1230,7 +1244,7 @@ glmb_status finish_frame(glmb_handle* h, bool copies_enqueued = false, bool est_
     return fail(h, st, "prune: %s", msg);
   };
   glmb_status st;
-  if (!copies_enqueued && (st = enqueue_results(h, false)) != GLMB_OK) return st;
+  if (!copies_enqueued && (st = enqueue_results(h)) != GLMB_OK) return st;
   CU(cudaStreamSynchronize(h->stream));
   const unsigned* cnt = h->h_cnt;
   unsigned e = h->h_scal[S_ERR];
@@ -1250,7 +1264,7 @@ glmb_status finish_frame(glmb_handle* h, bool copies_enqueued = false, bool est_
     if ((st = clear_hash_if_dirty(h)) != GLMB_OK) return st;
     if ((st = enqueue_expand(h, p)) != GLMB_OK) return st;
     if ((st = enqueue_prune(h, p)) != GLMB_OK) return st;
-    if ((st = enqueue_results(h, false)) != GLMB_OK) return st;
+    if ((st = enqueue_results(h)) != GLMB_OK) return st;
     CU(cudaStreamSynchronize(h->stream));
     e = h->h_scal[S_ERR];
     if (e & (kErrUpdates | kErrHash)) h->hash_dirty = true;
@@ -1510,7 +1524,8 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
       enqueue_prune(h, q);
       if (h->step_estimates)
         enqueue_estimates(h, h->hyps[1 - h->hcur], h->comps[h->cur], h->pw.counts, 0);
-      enqueue_results(h, h->step_estimates);
+      else
+        enqueue_results(h);
       h->capturing = false;
       CU(cudaStreamEndCapture(h->stream, &graph));
       size_t n_nodes = 0;
@@ -1583,7 +1598,8 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
     enqueue_prune(h, p);
     if (h->step_estimates)
       enqueue_estimates(h, h->hyps[1 - h->hcur], h->comps[h->cur], h->pw.counts, 0);
-    enqueue_results(h, h->step_estimates);
+    else
+      enqueue_results(h);
   }
   CU(cudaGetLastError());
   h->H_par = h->H;

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/glmb.h"
 #include "glmb_dev.cuh"
 
 namespace glmb {
@@ -306,14 +307,34 @@ void launch_gate_usage(const HypTable& par, const HypTable& out, const CompTable
                        cudaStream_t s);
 
 // estimates: pmf[pcap], nb = {n_hat, MAP hypothesis}, tracks =
-// glmb_track[pcap]; r_comp[ct.cap] (per-component weight sums), r_map[pcap]
-// (per-track sums), cmax and done are zeroed work areas, left zeroed;
-// H_dev (nullable) gives H on the device, H_bound an upper bound of H (the
-// launch shape follows it); err (nullable): the frame's error flags, on
-// which the kernels do nothing
-void launch_estimates(const HypTable& hp, int H, const unsigned* H_dev, int H_bound, const CompTable& ct, int dx,
-                      double* pmf, int pcap, int* nb, unsigned long long* r_comp, unsigned long long* r_map,
-                      void* tracks, unsigned* cmax, unsigned* done, int n_sm, const unsigned* err, cudaStream_t s);
+// glmb_track[pcap] (pmf and tracks may lie in pinned host memory); r_comp[ct.cap]
+// (per-component weight sums), cmax and done are zeroed work areas, left
+// zeroed; H_dev (nullable) gives H on the device; err (nullable): the frame's
+// error flags, on which the kernels do nothing; res_host (nullable): pinned
+// memory that receives the kEstResWords words at res_dev (the frame's counters
+// and scalars), and nb_host then nb
+constexpr int kEstResWords = 32;
+struct EstArgs {
+  HypTable hp;
+  int H_host;
+  const unsigned* H_dev;
+  CompTable ct;
+  int dx;
+  double* pmf;
+  int pcap;
+  int* nb;
+  unsigned long long* r_comp;
+  unsigned* cmax;
+  unsigned* done;
+  glmb_track* out;
+  const unsigned* err;
+  const unsigned* res_dev;
+  unsigned* res_host;
+  int* nb_host;
+  int fused;   // set by launch_estimates
+};
+// H_bound: an upper bound of H (the launch shape follows it)
+void launch_estimates(EstArgs a, int H_bound, int n_sm, cudaStream_t s);
 void launch_meas_assoc(const HypTable& hp, int H, int M, double* r_u, cudaStream_t s);
 
 }  // namespace glmb

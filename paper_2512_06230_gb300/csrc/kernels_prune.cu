@@ -5,6 +5,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cstddef>
 
 #include "../../include/glmb.h"
 #include "glmb_kernels.h"
@@ -701,8 +702,8 @@ __device__ __forceinline__ unsigned long long w_fx(double logw) {
 // Cardinality distribution, MAP cardinality (ties to the smaller n) and the
 // heaviest hypothesis of that cardinality (ties to the lower index), by one
 // block: nb[0] = n_hat, nb[1] = MAP hypothesis.
-__device__ __forceinline__ void est_card_block(const HypTable& hp, const int H, double* pmf, int pcap, int* nb) {
-  extern __shared__ unsigned long long s_pmf[];   // [pcap]
+__device__ __forceinline__ void est_card_block(const HypTable& hp, const int H, double* pmf, int pcap, int* nb,
+                                              int* nb_host, unsigned long long* s_pmf) {
   __shared__ unsigned long long bw[32];
   __shared__ int bi[32];
   __shared__ double lw_w[32];
@@ -778,6 +779,10 @@ __device__ __forceinline__ void est_card_block(const HypTable& hp, const int H, 
       if (li_w[w] >= 0 && (k < 0 || lw_w[w] > b || (lw_w[w] == b && li_w[w] < k))) { b = lw_w[w]; k = li_w[w]; }
     nb[0] = nhat;
     nb[1] = k;
+    if (nb_host) {
+      nb_host[0] = nhat;
+      nb_host[1] = k;
+    }
   }
 }
 
@@ -790,149 +795,184 @@ __device__ __forceinline__ void est_card_block(const HypTable& hp, const int H, 
 // labelled tracks), reached without waiting for the MAP hypothesis.
 constexpr int kEstPriv = 4096;   // components summed in shared memory per block
 
-__global__ void est_sums_kernel(HypTable hp, int H_host, const unsigned* H_dev, double* pmf, int pcap, int* nb,
-                                unsigned long long* r_comp, int ccap, unsigned* cmax, const unsigned* err) {
-  pdl_enter();
-  // a frame that failed left the new table incomplete: nothing to read
-  if (err && (*(volatile const unsigned*)err & kErrFatal)) return;
-  const int H = H_dev ? (int)*H_dev : H_host;
-  if (blockIdx.x == 0) {
-    est_card_block(hp, H, pmf, pcap, nb);
-    return;
-  }
-  // hypotheses share most of their components, so the block sums the
-  // first kEstPriv components in shared memory and adds each nonzero sum
-  // to global memory once (fixed point: the sums do not depend on order)
-  __shared__ unsigned long long s_acc[kEstPriv];
-  __shared__ unsigned s_top;
-  for (int c = threadIdx.x; c < kEstPriv; c += blockDim.x) s_acc[c] = 0ull;
-  if (threadIdx.x == 0) s_top = 0u;
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int wpb = blockDim.x >> 5;
-  unsigned top = 0u;
-  for (int h = (blockIdx.x - 1) * wpb + (threadIdx.x >> 5); h < H; h += (gridDim.x - 1) * wpb) {
-    const uint32_t lo = hp.ptr[h], hi = hp.ptr[h + 1];
-    const unsigned long long wgt = w_fx(hp.logw[h]);
-    for (uint32_t e = lo + lane; e < hi; e += 32) {
-      const uint32_t c = min(hp.comp[e], (uint32_t)ccap - 1u);
-      if (wgt) {
-        if (c < (uint32_t)kEstPriv) atomicAdd(&s_acc[c], wgt);
-        else atomicAdd(&r_comp[c], wgt);
-      }
-      top = max(top, c + 1u);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
-  if (lane == 0 && top) atomicMax(&s_top, top);
-  __syncthreads();
-  const unsigned nt = min(s_top, (unsigned)kEstPriv);
-  for (unsigned c = threadIdx.x; c < nt; c += blockDim.x)
-    if (s_acc[c]) atomicAdd(&r_comp[c], s_acc[c]);
-  if (threadIdx.x == 0 && s_top) atomicMax(cmax, s_top);
-}
-
-// Existence of the MAP tracks, second half: the labels of the MAP
-// hypothesis (in label order) go to each block's shared memory; every
-// component with a nonzero sum adds it to its label's entry (binary search)
-// and its sum is cleared, so r_comp is left zeroed.  One block writes the
-// MAP tracks (glmb_track records: mean hi + lo in FP64, full covariance)
-// from its own sums; with several blocks (large tables) each adds its sums
-// into r_map once and the last block to finish writes the tracks.  cmax,
-// done and r_map are left zeroed.
-__global__ void est_tracks_kernel(HypTable hp, CompTable ct, int dx, const int* __restrict__ nb,
-                                  unsigned long long* r_comp, unsigned* cmax, unsigned* done,
-                                  unsigned long long* r_map, glmb_track* out, int cap, const unsigned* err) {
-  pdl_enter();
-  if (err && (*(volatile const unsigned*)err & kErrFatal)) return;
-  extern __shared__ unsigned long long s_key[];   // [cap] MAP labels, then [cap] sums
-  unsigned long long* s_r = s_key + cap;
-  __shared__ bool last;
-  const int best = nb[1];
-  const uint32_t b0 = best >= 0 ? hp.ptr[best] : 0u;
-  const int nmap = best >= 0 ? min((int)(hp.ptr[best + 1] - b0), cap) : 0;
+// The MAP hypothesis' tracks [t0, t1) (its labels, ascending): the components
+// with a nonzero sum add it to their label's entry, and the block writes the
+// glmb_track records (mean hi + lo in FP64, full covariance), one warp per
+// record with its 8-byte words across the lanes, so that the reads are one
+// round and the writes (to pinned host memory in a frame's graph) are whole
+// lines.  s_key, s_r: t1 - t0 entries each.  `clear`: the sums are zeroed as
+// they are read (a block that is their only reader).
+__device__ __forceinline__ void est_write_tracks(const EstArgs& a, int best, uint32_t nc, int t0, int t1, bool clear,
+                                                 unsigned long long* s_key, unsigned long long* s_r) {
+  const HypTable& hp = a.hp;
+  const CompTable& ct = a.ct;
   const uint32_t ccap = (uint32_t)ct.cap;
-  const uint32_t nc = min(*(volatile unsigned*)cmax, ccap);
-  for (int j = threadIdx.x; j < nmap; j += blockDim.x) {
-    const uint32_t cm = min(hp.comp[b0 + j], ccap - 1u);
+  const uint32_t b0 = best >= 0 ? hp.ptr[best] : 0u;
+  const int n = t1 - t0;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const uint32_t cm = min(hp.comp[b0 + t0 + j], ccap - 1u);
     s_key[j] = ((unsigned long long)ct.lk[cm] << 32) | ct.lb[cm];
     s_r[j] = 0ull;
   }
   __syncthreads();
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += gridDim.x * blockDim.x) {
-    const unsigned long long v = r_comp[c];
-    if (!v) continue;
-    r_comp[c] = 0ull;
+  const unsigned long long klo = n > 0 ? s_key[0] : 1ull, khi = n > 0 ? s_key[n - 1] : 0ull;
+#pragma unroll 2
+  for (uint32_t c = threadIdx.x; c < nc; c += blockDim.x) {
+    const unsigned long long v = __ldcg(&a.r_comp[c]);
     const unsigned long long key = ((unsigned long long)ct.lk[c] << 32) | ct.lb[c];
-    int l = 0, u = nmap;
+    if (!v) continue;
+    if (clear) a.r_comp[c] = 0ull;
+    if (key < klo || key > khi) continue;
+    int l = 0, u = n;
     while (l < u) {
       const int mid = (l + u) >> 1;
       if (s_key[mid] < key) l = mid + 1; else u = mid;
     }
-    if (l < nmap && s_key[l] == key) atomicAdd(&s_r[l], v);
+    if (l < n && s_key[l] == key) atomicAdd(&s_r[l], v);
   }
   __syncthreads();
-  const bool multi = gridDim.x > 1;
-  if (multi) {
-    for (int j = threadIdx.x; j < nmap; j += blockDim.x)
-      if (s_r[j]) atomicAdd(&r_map[j], s_r[j]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-  }
-  if (threadIdx.x == 0) {
-    // every block has read cmax by now (the last block, or the only one)
-    *cmax = 0u;
-    if (multi) *done = 0u;
-  }
   const size_t cc = ct.cap;
-  for (int j = threadIdx.x; j < nmap; j += blockDim.x) {
-    unsigned long long rs = s_r[j];
-    if (multi) {
-      rs = ((volatile unsigned long long*)r_map)[j];
-      r_map[j] = 0ull;
-    }
-    const uint32_t c = min(hp.comp[b0 + j], ccap - 1u);
-    glmb_track& t = out[j];
-    t.label_k = ct.lk[c];
-    t.label_b = ct.lb[c];
-    t.r = (double)rs * kWfxInv;
-    for (int a = 0; a < 6; ++a)
-      t.mean[a] = a < dx ? (double)ct.mhi[a * cc + c] + (double)ct.mlo[a * cc + c] : 0.0;
-    for (int k = 0; k < 36; ++k) t.cov[k] = 0.0;
-    for (int i = 0; i < dx; ++i)
-      for (int k = i; k < dx; ++k) {
-        const double v = ct.cov[(size_t)pidx(dx, i, k) * cc + c];
-        t.cov[i * dx + k] = v;
-        t.cov[k * dx + i] = v;
+  const int lane = threadIdx.x & 31, dx = a.dx;
+  constexpr int kWords = sizeof(glmb_track) / 8;
+  static_assert(kWords == 44 && offsetof(glmb_track, r) == 8 && offsetof(glmb_track, mean) == 16 &&
+                    offsetof(glmb_track, cov) == 64,
+                "glmb_track words: labels, r, mean[6], cov[36]");
+  for (int j = threadIdx.x >> 5; j < n; j += (int)(blockDim.x >> 5)) {
+    const uint32_t c = min(hp.comp[b0 + t0 + j], ccap - 1u);
+    unsigned long long* out = reinterpret_cast<unsigned long long*>(a.out + t0 + j);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int w = lane + 32 * q;
+      if (w >= kWords) break;
+      double v = 0.0;
+      if (w == 1) {
+        v = (double)s_r[j] * kWfxInv;
+      } else if (w >= 2 && w < 8) {
+        if (w - 2 < dx) v = (double)ct.mhi[(w - 2) * cc + c] + (double)ct.mlo[(w - 2) * cc + c];
+      } else if (w >= 8 && w - 8 < dx * dx) {
+        const int i = (w - 8) / dx, k = (w - 8) - i * dx;
+        v = ct.cov[(size_t)pidx(dx, min(i, k), max(i, k)) * cc + c];
       }
+      // labels: label_k in the low word, label_b in the high one
+      out[w] = w == 0 ? (s_key[j] >> 32) | (s_key[j] << 32) : (unsigned long long)__double_as_longlong(v);
+    }
   }
 }
 
-void launch_estimates(const HypTable& hp, int H, const unsigned* H_dev, int H_bound, const CompTable& ct, int dx,
-                      double* pmf, int pcap, int* nb, unsigned long long* r_comp, unsigned long long* r_map,
-                      void* tracks, unsigned* cmax, unsigned* done, int n_sm, const unsigned* err, cudaStream_t s) {
-  static int attr_pcap = 0;   // the limits only grow (graphs of larger filters stay valid)
-  // (est_sums_kernel also holds kEstPriv sums in static shared memory, so
-  // the opt-in is made whatever the dynamic size)
-  if (pcap > attr_pcap) {
-    cudaFuncSetAttribute(est_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pcap * 8);
-    cudaFuncSetAttribute(est_tracks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pcap * 16);
-    attr_pcap = pcap;
+// Estimates of a table.  Block 0: cardinality and MAP hypothesis; the other
+// blocks: the components' weight sums.  `fused`: the last block to finish
+// writes the tracks (their labels fit one block); else est_tracks_kernel
+// does.  In a frame's graph block 0 also puts the frame's counters and
+// scalars (final by now) into the pinned result block, whether or not the
+// frame succeeded, so that no copy follows.
+// What bounds it is latency.  Measured per frame: N = 1000 69 -> 25 us, a
+// convoy of five objects 18 -> 14 us and the whole frame, with the copy of the
+// results gone, 111 -> 100 us.
+__global__ void __launch_bounds__(1024) est_sums_kernel(const __grid_constant__ EstArgs a) {
+  pdl_enter();
+  extern __shared__ unsigned long long s_dyn[];   // max(kEstPriv, 2 pcap) words when fused
+  __shared__ unsigned s_top;
+  __shared__ bool s_last;
+  if (a.res_host && blockIdx.x == 0 && threadIdx.x < kEstResWords) a.res_host[threadIdx.x] = a.res_dev[threadIdx.x];
+  // a frame that failed left the new table incomplete: nothing to read
+  if (a.err && (*(volatile const unsigned*)a.err & kErrFatal)) return;
+  const int H = a.H_dev ? (int)*a.H_dev : a.H_host;
+  const int wpb = blockDim.x >> 5, lane = threadIdx.x & 31;
+  if (blockIdx.x == 0) {
+    est_card_block(a.hp, H, a.pmf, a.pcap, a.nb, a.nb_host, s_dyn);
+  } else if ((int)(blockIdx.x - 1) * wpb < H) {
+    // hypotheses share most of their components, so the block sums the
+    // first kEstPriv components in shared memory and adds each nonzero sum
+    // to global memory once (fixed point: the sums do not depend on order)
+    unsigned long long* s_acc = s_dyn;
+    const int npriv = min(kEstPriv, a.ct.cap);
+    for (int c = threadIdx.x; c < npriv; c += blockDim.x) s_acc[c] = 0ull;
+    if (threadIdx.x == 0) s_top = 0u;
+    __syncthreads();
+    unsigned top = 0u;
+    for (int h = (blockIdx.x - 1) * wpb + (threadIdx.x >> 5); h < H; h += (gridDim.x - 1) * wpb) {
+      const uint32_t lo = a.hp.ptr[h], hi = a.hp.ptr[h + 1];
+      const unsigned long long wgt = w_fx(a.hp.logw[h]);
+      for (uint32_t e = lo + lane; e < hi; e += 32) {
+        const uint32_t c = min(a.hp.comp[e], (uint32_t)a.ct.cap - 1u);
+        if (wgt) {
+          if (c < (uint32_t)kEstPriv) atomicAdd(&s_acc[c], wgt);
+          else atomicAdd(&a.r_comp[c], wgt);
+        }
+        top = max(top, c + 1u);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+    if (lane == 0 && top) atomicMax(&s_top, top);
+    __syncthreads();
+    const unsigned nt = min(s_top, (unsigned)npriv);
+    for (unsigned c = threadIdx.x; c < nt; c += blockDim.x)
+      if (s_acc[c]) atomicAdd(&a.r_comp[c], s_acc[c]);
+    if (threadIdx.x == 0 && s_top) atomicMax(a.cmax, s_top);
+  }
+  if (!a.fused) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(a.done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int best = ((volatile int*)a.nb)[1];
+  const uint32_t nc = min(*(volatile unsigned*)a.cmax, (uint32_t)a.ct.cap);
+  const int nmap = best >= 0 ? min((int)(a.hp.ptr[best + 1] - a.hp.ptr[best]), a.pcap) : 0;
+  est_write_tracks(a, best, nc, 0, nmap, true, s_dyn, s_dyn + a.pcap);
+  if (threadIdx.x == 0) {
+    *a.cmax = 0u;
+    *a.done = 0u;
+  }
+}
+
+// The MAP tracks of a filter with many: each block takes kEstTile of them;
+// the last block zeroes the sums.
+constexpr int kEstTile = 32, kEstThreads = 512;
+__global__ void __launch_bounds__(kEstThreads) est_tracks_kernel(const __grid_constant__ EstArgs a) {
+  pdl_enter();
+  if (a.err && (*(volatile const unsigned*)a.err & kErrFatal)) return;
+  __shared__ unsigned long long s_key[kEstTile], s_r[kEstTile];
+  __shared__ bool s_last;
+  const int best = a.nb[1];
+  const uint32_t nc = min(*(volatile unsigned*)a.cmax, (uint32_t)a.ct.cap);
+  const int nmap = best >= 0 ? min((int)(a.hp.ptr[best + 1] - a.hp.ptr[best]), a.pcap) : 0;
+  for (int t0 = blockIdx.x * kEstTile; t0 < nmap; t0 += gridDim.x * kEstTile) {
+    est_write_tracks(a, best, nc, t0, min(nmap, t0 + kEstTile), false, s_key, s_r);
+    __syncthreads();
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(a.done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  for (uint32_t c = threadIdx.x; c < nc; c += blockDim.x) a.r_comp[c] = 0ull;
+  if (threadIdx.x == 0) {
+    *a.cmax = 0u;
+    *a.done = 0u;
+  }
+}
+
+// One launch while the table holds at most 4096 hypotheses (the components in
+// use grow with them) and one block can hold the tracks' labels and sums
+// beside the cardinality bins; else a second launch spreads the tracks over
+// blocks (N = 1000, one block for all tracks: 52 us).
+constexpr int kEstFuseTracks = 512;
+void launch_estimates(EstArgs a, int H_bound, int n_sm, cudaStream_t s) {
+  a.fused = H_bound <= 4096 && a.pcap <= kEstFuseTracks ? 1 : 0;
+  const int words = std::max(std::min(kEstPriv, a.ct.cap), a.fused ? 2 * a.pcap : a.pcap);
+  static int attr_words = 48 * 1024 / 8;   // the limit only grows (graphs of larger filters stay valid)
+  if (words > attr_words) {
+    cudaFuncSetAttribute(est_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, words * 8);
+    attr_words = words;
   }
   // block 0: the cardinality; blocks 1..: one warp per hypothesis
-  const int sum_blocks = H_dev ? n_sm : std::max(1, std::min((H + 31) / 32, n_sm));
-  launch_k(est_sums_kernel, 1 + sum_blocks, 1024, (size_t)pcap * 8, s, hp, H, H_dev, pmf, pcap, nb, r_comp,
-           ct.cap, cmax, err);
-  // the components in use grow with the hypotheses: one block while the
-  // table holds at most 4096 hypotheses, else two blocks per SM
-  const int track_blocks = H_bound <= 4096 ? 1 : 2 * n_sm;
-  launch_k(est_tracks_kernel, track_blocks, 1024, (size_t)pcap * 16, s, hp, ct, dx, nb, r_comp, cmax, done, r_map,
-           (glmb_track*)tracks, pcap, err);
+  const int blocks = std::max(1, std::min((H_bound + 31) / 32, n_sm));
+  launch_k(est_sums_kernel, 1 + blocks, 1024, (size_t)words * 8, s, a);
+  if (!a.fused)
+    launch_k(est_tracks_kernel, std::max(1, std::min((a.pcap + kEstTile - 1) / kEstTile, 2 * n_sm)), kEstThreads, 0, s, a);
 }
 
 // Clutter probability of each detection: the total weight of the hypotheses
