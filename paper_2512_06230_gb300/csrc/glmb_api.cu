@@ -25,8 +25,8 @@ enum { kStagePredict = 0, kStageTable, kStageExpand, kStageSelect, kStageMat, kS
        kStageEstimates, kNumStages };
 
 // device scalar slots
-enum { S_ERR = 0, S_FP64 = 1, S_MAXT = 2, S_MAXK = 3, S_NUPD = 4, S_NKEEP = 5, S_K = 6, S_REDO = 7, S_STAGE = 8, S_KFULL = 9,
-       S_N = 16 };
+enum { S_ERR = 0, S_FP64 = 1, S_MAXT = 2, S_MAXK = 3, S_NUPD = 4, S_NKEEP = 5, S_K = 6, S_REDO = 7, S_STAGE = 8, S_NOTE = 9,
+       S_KFULL = 10, S_N = 16 };
 
 }  // namespace
 
@@ -103,6 +103,7 @@ struct glmb_handle {
   unsigned char* img = nullptr;
   size_t img_alloc = 0;
   uint32_t* redo_list = nullptr;
+  unsigned char* notes = nullptr;
   PruneWork pw{};
   unsigned long long* hkeys = nullptr;
   uint32_t* hvals = nullptr;
@@ -644,6 +645,7 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
             dalloc(h, &h->child_hash, h->cap_children) &&
             dalloc(h, &h->child_alive, h->cap_children) &&
             dalloc(h, &h->redo_list, h->cap_children) &&
+            dalloc(h, &h->notes, h->cap_children * (long long)expand_note_bytes()) &&
             dalloc(h, &h->pw.blk_max, 4097) && dalloc(h, &h->pw.blk_sum, 4097) &&
             dalloc(h, &h->pw.blk_done, 4) && dalloc(h, &h->pw.lse, 2) && dalloc(h, &h->pw.thr, 1) &&
             dalloc(h, &h->pw.part_max, kMaxLseParts) && dalloc(h, &h->pw.part_sum, kMaxLseParts) &&
@@ -882,6 +884,8 @@ ExpandArgs expand_args(glmb_handle* h, const Plan& p, bool mat) {
   a.warp_all = p.thread ? 0 : 1;
   a.redo_list = h->redo_list;
   a.redo_count = h->d_scal + S_REDO;
+  a.notes = h->notes;
+  a.note_count = h->d_scal + S_NOTE;
   a.stage_next = h->d_scal + S_STAGE;
   a.materialize = mat ? 1 : 0;
   a.err = h->d_scal + S_ERR;
@@ -968,18 +972,12 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
   const int st_grid = p.fixed ? st_ctas * n_sm : std::max(1, std::min(h->H, st_ctas * n_sm));
   // draws: one thread per child over the frame's children in order
   // (persistent grid)
-  // CTAs of 256 threads, or smaller ones when the frame's children would
-  // not give every SM two of them (the mid scene's 32 000 children fill
-  // only 125 CTAs of 256)
-  int d_thr = h->tune.draw_threads;
-  if (d_thr <= 0) {
-    const long long kids = (long long)h->H * h_up;
-    d_thr = 256;
-    while (d_thr > 64 && kids < 2LL * n_sm * d_thr) d_thr >>= 1;
-  }
-  const int d_smem = expand_draw_smem(d_thr);
+  const int d_thr = h->tune.draw_threads > 0 ? h->tune.draw_threads : 256;
+  // the chunk records of a CTA's parents in shared memory when two CTAs fit
+  a.draw_staged = 2 * (expand_draw_smem(d_thr, h_up, p.T, p.M, true) + 1024) <= h->smem_per_sm ? 1 : 0;
+  const int d_smem = expand_draw_smem(d_thr, h_up, p.T, p.M, a.draw_staged != 0);
   const int d_ctas = std::max(1, expand_occupancy(a, ExpandKernel::kDraw, d_thr, d_smem));
-  const long long d_need = ((long long)h->H * h_up + d_thr - 1) / d_thr;
+  const long long d_need = ((long long)h->H * h_up + 63) / 64;   // (a CTA takes fewer than d_thr children when they are few)
   const int d_grid = p.fixed ? d_ctas * n_sm : (int)std::max(1LL, std::min(d_need, (long long)d_ctas * n_sm));
   // warp kernel: the overflow list, or every child
   int wg = p.wg;
@@ -989,7 +987,7 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
   a.warp_group = wg;
   const int w_ctas = std::max(1, expand_occupancy(a, ExpandKernel::kWarp, w_thr, w_smem));
   int w_grid = w_ctas * n_sm;
-  if (p.thread) w_grid = n_sm;
+  if (p.thread) w_grid = std::min(w_ctas, 2) * n_sm;
   else if (!p.fixed)
     w_grid = (int)std::max(1LL, std::min(((long long)h->H * h_up + p.Gw - 1) / p.Gw, (long long)w_grid));
   h->exp_smem = p.thread ? img : w_smem;
@@ -999,7 +997,7 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
   h->exp_plan[2] = p.M;
   h->exp_plan[3] = p.thread ? d_thr : w_thr;
   prof_begin(h, kStageExpand);
-  if (!scal_zeroed) CU(cudaMemsetAsync(h->d_scal + S_REDO, 0, 2 * sizeof(unsigned), s));   // S_REDO, S_STAGE
+  if (!scal_zeroed) CU(cudaMemsetAsync(h->d_scal + S_REDO, 0, 3 * sizeof(unsigned), s));   // S_REDO, S_STAGE, S_NOTE
   launch_expand_kernel(a, ExpandKernel::kStage, st_grid, st_thr, st_smem, s);
   if (p.thread) launch_expand_kernel(a, ExpandKernel::kDraw, d_grid, d_thr, d_smem, s);
   launch_expand_kernel(a, ExpandKernel::kWarp, w_grid, w_thr, w_smem, s);

@@ -198,24 +198,33 @@ __device__ __forceinline__ PhiloxRun philox_run(uint32_t c0, uint32_t c1, uint32
 // Where the key is a per-thread value (an out-of-line function's argument),
 // philox_at_rk forms them per call instead, so they take no registers
 // across the caller's loop.
-__device__ __forceinline__ uint4 philox_at(const PhiloxRun& p, uint32_t cc, uint2 k) {
+__device__ __forceinline__ uint2 mul_wide(uint32_t a, uint32_t b) {   // (low, high) word of the product
+  const unsigned long long p = (unsigned long long)a * b;
+  return make_uint2((uint32_t)p, (uint32_t)(p >> 32));
+}
+
+// The call's product that depends on the chunk alone (w2 holds c0 and the
+// key only): children of one parent drawn together form it once.
+__device__ __forceinline__ uint2 philox_chunk(const PhiloxRun& p, uint32_t cc) {
+  return mul_wide(0xCD9E8D57u, p.w2 ^ cc);                  // round 2, second product
+}
+__device__ __forceinline__ uint4 philox_at(const PhiloxRun& p, uint2 D, uint2 k) {
   constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
-  const uint32_t w2 = p.w2 ^ cc;
-  const uint32_t hiD = __umulhi(M1, w2), loD = M1 * w2;     // round 2, second product
-  const uint32_t y0 = hiD ^ p.y0;
-  const uint32_t hiE = __umulhi(M0, y0), loE = M0 * y0;     // round 3, first product
-  uint4 c = make_uint4(loD ^ p.z0, p.z1, hiE ^ p.z2, loE);
+  const uint2 E = mul_wide(M0, D.y ^ p.y0);                 // round 3, first product
+  uint4 c = make_uint4(D.x ^ p.z0, p.z1, E.y ^ p.z2, E.x);
   k.x += 3u * 0x9E3779B9u;
   k.y += 3u * 0xBB67AE85u;
 #pragma unroll
   for (int r = 3; r < 10; ++r) {
-    const uint32_t hi0 = __umulhi(M0, c.x), lo0 = M0 * c.x;
-    const uint32_t hi1 = __umulhi(M1, c.z), lo1 = M1 * c.z;
-    c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
+    const uint2 m0 = mul_wide(M0, c.x), m1 = mul_wide(M1, c.z);
+    c = make_uint4(m1.y ^ c.y ^ k.x, m1.x, m0.y ^ c.w ^ k.y, m0.x);
     k.x += 0x9E3779B9u;
     k.y += 0xBB67AE85u;
   }
   return c;
+}
+__device__ __forceinline__ uint4 philox_at(const PhiloxRun& p, uint32_t cc, uint2 k) {
+  return philox_at(p, philox_chunk(p, cc), k);
 }
 
 __device__ __forceinline__ uint4 philox_at_rk(const PhiloxRun& p, uint32_t cc, uint2 k) {

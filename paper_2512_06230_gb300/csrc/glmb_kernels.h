@@ -134,9 +134,12 @@ struct ExpandArgs {
   unsigned char* img;
   long long img_stride;
   int stage_smem;         // staged in shared memory (else in the image itself)
+  int draw_staged;        // thread-per-child draw: the parents' chunk records go to shared memory first
   int warp_all;           // warp kernel: every child of every parent (else the overflow list)
   uint32_t* redo_list;    // children the draw kernel could not take
   unsigned* redo_count;
+  unsigned char* notes;   // children with noted rows (expand_note_bytes each)
+  unsigned* note_count;
   unsigned* stage_next;   // staging: next parent to take (zero at the launch)
   int stage_tail;         // staging in global memory: what it keeps in shared memory (expand_stage_tail_bytes)
   int warp_group;         // warp kernel: warps per child (1, 2, 4 or 8; a CTA holds whole groups)
@@ -182,7 +185,8 @@ int expand_image_bytes(int dz, int T_max, int K_max, int M);
 // array; the image in shared memory takes mode 0)
 int expand_stage_tail_bytes(int dz, int T_plan, int K_plan, int M_plan, int mode);
 // shared memory of a draw-kernel CTA of `threads` threads
-int expand_draw_smem(int threads);
+size_t expand_note_bytes();
+int expand_draw_smem(int threads, int h_up, int T_plan, int M_plan, bool staged);
 // shared memory of a warp-kernel CTA of `warps` warps
 int expand_warp_smem(int dz, int materialize, int T_max, int warps, int grp = 0);
 enum class ExpandKernel { kStage, kDraw, kWarp, kMatPrep };

@@ -21,8 +21,10 @@
 //             with a dead candidate fall back to the FP32 normalised row of
 //             C'_k); deaths and rows that leave the reference are listed in
 //             shared memory; the child's log-weight is the reference score
-//             plus the tabulated changes, or, when a slot is met twice, the
-//             exact rescoring of every met slot (stage 3), in fixed point;
+//             plus its deviations' changes (finish_notes, in the warp
+//             kernel's launch, for the few children that have any), or, when
+//             a slot is met twice, the exact rescoring of every met slot
+//             (stage 3), in fixed point;
 //   warp      one warp per child, rows split over the lanes and per-slot sums
 //             in shared memory: children whose lists overflow the draw
 //             kernel's, every child when parents are too few to fill
@@ -47,7 +49,7 @@ struct Lay {
   int scal;
   int row, rowbl, seref, sqref, termref, hwref, deadd;
   int rowrk, rch, rowoff, rowfill, roww0, rowthr0;
-  int comp, dthr, logp, log1mp, mref, refnew, hph, dpc;
+  int comp, dthr, logp, log1mp, mref, refnew, hph, dpc, dth;
   int cthr, ceidx, cw, ce, cq, cslot;
   int ninfref, dninf, srow;
   int total;
@@ -114,6 +116,7 @@ __host__ __device__ inline Lay make_lay(int dz, int T, int K, int M) {
   L.refnew = b.take(4LL * T);
   L.hph = b.take(4LL * NP * T);             // H P H^T of each slot (packed)
   L.dpc = b.take(4LL * (T / 4 + 2));        // chunks of 4 slots that can die
+  L.dth = b.take(16LL * (T / 4 + 2));       // their slots' largest dying words (see the chunk lists)
   L.cthr = b.take(4LL * K);
   L.ceidx = b.take(4LL * K);
   L.cw = b.take(4LL * K);
@@ -436,6 +439,7 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   int* s_mref = in_tail ? at<int>(tb, TS.mref) : at<int>(sm, L.mref);
   float* s_hph = at<float>(sm, L.hph);
   uint32_t* s_dpc = at<uint32_t>(sm, L.dpc);
+  uint4* s_dth = at<uint4>(sm, L.dth);
   uint32_t* s_cthr = at<uint32_t>(sm, L.cthr);
   uint32_t* s_ceidx = in_tail ? at<uint32_t>(tb, TS.ceidx) : at<uint32_t>(sm, L.ceidx);
   float* s_cw = at<float>(sm, L.cw);
@@ -821,13 +825,21 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   {
     const int nch = (T + 3) >> 2;
     for (int cc = tid; cc < nch; cc += nthr) {
-      uint32_t mask = 0;
+      // u < threshold, on the whole word: word <= (threshold << 8) - 1 (a
+      // slot that cannot die keeps 0, which the mask bit sorts out)
+      uint32_t mask = 0, top[4];
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
         const int t = 4 * cc + b;
-        if (t < T && s_dthr[t] > 0u) mask |= 1u << b;
+        const uint32_t dt = t < T ? s_dthr[t] : 0u;
+        if (dt > 0u) mask |= 1u << b;
+        top[b] = dt > 0u ? (dt << 8) - 1u : 0u;
       }
-      if (mask) s_dpc[atomicAdd(&s_wsum[0], 1u)] = ((uint32_t)cc << 4) | mask;
+      if (mask) {
+        const uint32_t x = atomicAdd(&s_wsum[0], 1u);
+        s_dpc[x] = ((uint32_t)cc << 4) | mask;
+        s_dth[x] = make_uint4(top[0], top[1], top[2], top[3]);
+      }
     }
   }
   __syncthreads();
@@ -1014,9 +1026,9 @@ __device__ __noinline__ TermOut single_deviation(const Model* md, const View* vp
 
 template <int DZ>
 __device__ __noinline__ SlowSum slow_rows(const Model* md, const PairTable* pt, const unsigned char* img,
-                                          const int Tp, const int Kp, const int Mp, const uint16_t* s_slow,
-                                          const int nslow, const int stride, const unsigned long long bloom,
-                                          const uint32_t n, const uint2 key) {
+                                          const int Tp, const int Kp, const int Mp, const uint16_t* rows,
+                                          const int nslow, const unsigned long long bloom, const uint32_t n,
+                                          const uint2 key) {
   constexpr int kE = 2 * 24;
   const Lay L = make_lay(DZ, Tp, Kp, Mp);
   const View v = make_view(img, L, *pt);
@@ -1039,7 +1051,7 @@ __device__ __noinline__ SlowSum slow_rows(const Model* md, const PairTable* pt, 
   unsigned long long metm = 0ull;
   bool twice = false;
   for (int q = 0; q < nslow; ++q) {
-    const int i = s_slow[q * stride];
+    const int i = rows[q];
     const uint4 rr = philox_at_rk(pr, (uint32_t)i >> 2, key);
     const uint32_t k = word_of(rr, i & 3) >> 8;
     const uint4 R = v.row[i];
@@ -1185,58 +1197,92 @@ constexpr int kDrawSlow = 24;
 // kind of per-thread list, after the noted rows); a child with more
 // regenerates its death draws instead.
 constexpr int kDrawDead = 8;
-// chunks per iteration of the draw loop's rows: three (1) or one (0)
-constexpr int kDrawPairs = 1;
+// Chunks per iteration of the draw loops: independent Philox chains in
+// flight (rows: 2 or 4 measured the same as 3 within 1 %).
+constexpr int kDrawDeaths = 2, kDrawRows = 3;
 
-// Draws child n of the parent staged at img.  The chunk loop only tests the
-// reference intervals and notes the rows that need more (their uniform is
-// regenerated afterwards), so it holds nothing but its own state in
-// registers.  Slots its deviations meet more than once are rescored exactly
-// (slow_rows).  Returns false when the child must be drawn by the warp
-// kernel: more noted rows than the list holds.
+// What the chunk loops read of a parent, staged in shared memory beside the
+// other parents of a CTA's children: offsets from the parent's part.
+struct DrawRec {
+  int rch, dth, dpc, total;
+};
+__host__ __device__ inline DrawRec make_draw_rec(int T, int M) {
+  DrawRec R;
+  Bump b;
+  R.rch = b.take(48LL * ((M + 3) / 4 + 1));
+  R.dth = b.take(16LL * (T / 4 + 2));
+  R.dpc = b.take(4LL * (T / 4 + 2));
+  R.total = b.off;
+  return R;
+}
+// A child whose chunk loop noted rows: what finish_notes needs beside the
+// child's partial sums (child_key, child_hash, child_alive).
+struct DrawNote {
+  uint32_t child;
+  uint16_t n_rows;
+  int16_t dninf;
+  unsigned long long bloom;
+  uint16_t rows[kDrawSlow];
+};
+size_t expand_note_bytes() { return sizeof(DrawNote); }
+// parents that `threads` consecutive children can belong to
+__host__ __device__ inline int draw_parents(int threads, int h_up) { return (threads - 1) / h_up + 2; }
+
+template <int N>
+struct Int {
+  static constexpr int value = N;
+};
+
+// Draws child n of the parent staged at img; rch, dth and dpc are the
+// parent's arrays of these names (in shared memory, or the image's).  The
+// chunk loops only test the thresholds and intervals and note the slots that
+// die and the rows that need more (their uniform is regenerated afterwards),
+// so they hold nothing but their own state in registers.  Slots its
+// deviations meet more than once are rescored exactly (slow_rows).  A child
+// with more noted rows than the list holds is left to the warp kernel (the
+// redo list).
 template <int DZ>
-__device__ __forceinline__ bool thread_child(const ExpandArgs& a, const unsigned char* img, const Lay& L,
-                                             const int h, const int n, const uint2 key, uint16_t* s_slow,
-                                             uint16_t* s_dead) {
+__device__ __forceinline__ void thread_child(const ExpandArgs& a, const unsigned char* img, const Lay& L, const int h,
+                                             const int n, const uint2 key, uint16_t* s_slow, uint16_t* s_dead,
+                                             const RowChunk* rch, const uint4* dth, const uint32_t* dpc) {
   const Model& md = a.md;
   const Scal& sc = *at<Scal>(img, L.scal);
+  const int bd = (int)blockDim.x;
   unsigned long long bloom = 0ull;
   int nd = 0;
   {
     // stage 1: deaths; only their bloom (slots with candidate rows) is kept
     // through the chunk loop, their score and key changes are summed after
-    const uint32_t* dpc = at<uint32_t>(img, L.dpc);
-    const uint32_t* dthr = at<uint32_t>(img, L.dthr);
     const uint8_t* srow = at<uint8_t>(img, L.srow);
     const PhiloxRun pd = philox_run((uint32_t)sc.uid, (uint32_t)(sc.uid >> 32), 2u * (uint32_t)n, key);
     const int ndpc = sc.ndpc;
-    auto test_deaths = [&](uint32_t ent, const uint4& r) {
-      const uint32_t cc = ent >> 4, mask = ent & 15u;
-      const uint4 th = *reinterpret_cast<const uint4*>(dthr + 4 * cc);
+    // N chunks: N independent Philox chains in flight
+    auto chunks = [&](int x, auto nn) {
+      constexpr int N = decltype(nn)::value;
+      uint32_t e[N];
+      uint4 r[N];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const uint32_t thb = b == 0 ? th.x : b == 1 ? th.y : b == 2 ? th.z : th.w;
-        if (((mask >> b) & 1u) && (word_of(r, b) >> 8) < thb) {
-          const uint32_t t = 4u * cc + (uint32_t)b;
-          if (nd < kDrawDead) s_dead[nd * (int)blockDim.x] = (uint16_t)t;
-          ++nd;
-          if (srow[t]) bloom |= 1ull << (t & 63u);
+      for (int u = 0; u < N; ++u) e[u] = dpc[x + u];
+#pragma unroll
+      for (int u = 0; u < N; ++u) r[u] = philox_at(pd, e[u] >> 4, key);
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const uint4 th = dth[x + u];
+        if (r[u].x <= th.x || r[u].y <= th.y || r[u].z <= th.z || r[u].w <= th.w) {
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            if (word_of(r[u], b) <= word_of(th, b) && ((e[u] >> b) & 1u)) {
+              const uint32_t t = 4u * (e[u] >> 4) + (uint32_t)b;
+              if (nd < kDrawDead) s_dead[nd * bd] = (uint16_t)t;
+              ++nd;
+              if (srow[t]) bloom |= 1ull << (t & 63u);
+            }
         }
       }
     };
-    // two chunks per iteration: two independent Philox chains in flight
     int x = 0;
-    for (; x + 1 < ndpc; x += 2) {
-      const uint32_t e0 = dpc[x], e1 = dpc[x + 1];
-      const uint4 r0 = philox_at(pd, e0 >> 4, key);
-      const uint4 r1 = philox_at(pd, e1 >> 4, key);
-      test_deaths(e0, r0);
-      test_deaths(e1, r1);
-    }
-    if (x < ndpc) {
-      const uint32_t e = dpc[x];
-      test_deaths(e, philox_at(pd, e >> 4, key));
-    }
+    for (; x + kDrawDeaths <= ndpc; x += kDrawDeaths) chunks(x, Int<kDrawDeaths>());
+    for (; x < ndpc; ++x) chunks(x, Int<1>());
   }
   // stage 2: one categorical draw per detection row with candidates; rows
   // outside their reference interval, or whose candidates' bloom meets the
@@ -1244,138 +1290,207 @@ __device__ __forceinline__ bool thread_child(const ExpandArgs& a, const unsigned
   int nslow = 0;
   {
     const PhiloxRun pr = philox_run((uint32_t)sc.uid, (uint32_t)(sc.uid >> 32), 2u * (uint32_t)n + 1u, key);
-    const RowChunk* rch = at<RowChunk>(img, L.rch);
+    const unsigned long long* rowbl = at<unsigned long long>(img, L.rowbl);
+    const uint32_t blo = (uint32_t)bloom, bhi = (uint32_t)(bloom >> 32);
     const int nrca = sc.nrca;
-    // the interval tests of chunk x with its four words r
-    auto test_chunk = [&](int x, uint32_t cc, const uint4& r) {
-      const uint4 hd = rch[x].head, base = rch[x].base, span = rch[x].span;
-      const uint32_t hit = ((((unsigned long long)hd.w << 32) | hd.z) & bloom) ? hd.y : 0u;
-      // bit b: row 4 cc + b left its reference interval
-      uint32_t out = 0u;
+    auto chunks = [&](int x, auto nn) {
+      constexpr int N = decltype(nn)::value;
+      uint4 r[N];
 #pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if (word_of(r, b) - word_of(base, b) > word_of(span, b)) out |= 1u << b;
-      uint32_t look = out | hit;   // nearly always 0: all four keep the reference
-      while (look) {
-        const int b = __ffs(look) - 1;
-        look &= look - 1u;
-        const uint32_t i = 4u * cc + (uint32_t)b;
-        // a row of a chunk whose bloom meets the dead slots', still in its
-        // reference interval: noted only if its own candidates' bloom does
-        if (!((out >> b) & 1u) && !(at<unsigned long long>(img, L.rowbl)[i] & bloom)) continue;
-        if (nslow < kDrawSlow) s_slow[nslow * (int)blockDim.x] = (uint16_t)i;
-        ++nslow;
+      for (int u = 0; u < N; ++u) r[u] = philox_at(pr, rch[x + u].head.x, key);
+#pragma unroll
+      for (int u = 0; u < N; ++u) {
+        const uint4 hd = rch[x + u].head, base = rch[x + u].base, span = rch[x + u].span;
+        const uint32_t hit = (hd.z & blo) | (hd.w & bhi);
+        // nearly always false: all four rows keep their reference
+        if (r[u].x - base.x > span.x || r[u].y - base.y > span.y || r[u].z - base.z > span.z ||
+            r[u].w - base.w > span.w || hit) {
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const uint32_t i = 4u * hd.x + (uint32_t)b;
+            bool look = word_of(r[u], b) - word_of(base, b) > word_of(span, b);
+            // a row of a chunk whose bloom meets the dead slots', still in
+            // its reference interval: noted only if its own bloom does
+            if (!look && hit && ((hd.y >> b) & 1u)) look = (rowbl[i] & bloom) != 0ull;
+            if (look) {
+              if (nslow < kDrawSlow) s_slow[nslow * bd] = (uint16_t)i;
+              ++nslow;
+            }
+          }
+        }
       }
     };
     int x = 0;
-    if (kDrawPairs) {
-      // three chunks per iteration: three independent Philox chains in flight
-      for (; x + 2 < nrca; x += 3) {
-        const uint32_t c0 = rch[x].head.x, c1 = rch[x + 1].head.x, c2 = rch[x + 2].head.x;
-        const uint4 r0 = philox_at(pr, c0, key);
-        const uint4 r1 = philox_at(pr, c1, key);
-        const uint4 r2 = philox_at(pr, c2, key);
-        test_chunk(x, c0, r0);
-        test_chunk(x + 1, c1, r1);
-        test_chunk(x + 2, c2, r2);
-      }
-    }
-    uint32_t cc_next = x < nrca ? rch[x].head.x : 0u;   // one iteration ahead
-    for (; x < nrca; ++x) {
-      const uint32_t cc = cc_next;
-      if (x + 1 < nrca) cc_next = rch[x + 1].head.x;
-      test_chunk(x, cc, philox_at(pr, cc, key));
-    }
+    for (; x + kDrawRows <= nrca; x += kDrawRows) chunks(x, Int<kDrawRows>());
+    for (; x < nrca; ++x) chunks(x, Int<1>());
   }
-  if (nslow > kDrawSlow) return false;
+  const size_t j = (size_t)h * md.h_up + n;
+  if (nslow > kDrawSlow) {
+    a.redo_list[atomicAdd(a.redo_count, 1u)] = (uint32_t)j;
+    return;
+  }
   // the deaths' score and key changes (a dead slot's change is its dead term)
   unsigned long long hsh = 0ull;
   long long delta = 0;
-  int dclut = 0, dninf = 0;
-  bool bad_row = false;
-  if (nd && nd <= kDrawDead) {
-    const long long* deadd = at<long long>(img, L.deadd);
-    const int8_t* dninf8 = at<int8_t>(img, L.dninf);
-    for (int q = 0; q < nd; ++q) {
-      const int t = s_dead[q * (int)blockDim.x];
-      hsh += dead_key(t);
-      delta += deadd[t];
-      dninf += dninf8[t];
+  int dninf = 0;
+  const long long* deadd = at<long long>(img, L.deadd);
+  const int8_t* dninf8 = at<int8_t>(img, L.dninf);
+  if (nd <= kDrawDead) {
+    // four deaths' loads in flight (the image's tables come from L2 or HBM)
+    for (int q0 = 0; q0 < nd; q0 += 4) {
+#pragma unroll
+      for (int q = q0; q < q0 + 4; ++q)
+        if (q < nd) {
+          const int t = s_dead[q * bd];
+          hsh += dead_key(t);
+          delta += deadd[t];
+          dninf += dninf8[t];
+        }
     }
-  } else if (nd) {
+  } else {
     // more deaths than the list holds: their draws again
-    const uint32_t* dpc = at<uint32_t>(img, L.dpc);
-    const uint32_t* dthr = at<uint32_t>(img, L.dthr);
     const PhiloxRun pd = philox_run((uint32_t)sc.uid, (uint32_t)(sc.uid >> 32), 2u * (uint32_t)n, key);
     const int ndpc = sc.ndpc;
-    int left = nd;
-    for (int x = 0; x < ndpc && left; ++x) {
+    for (int x = 0, left = nd; x < ndpc && left; ++x) {
       const uint32_t ent = dpc[x];
-      const uint32_t cc = ent >> 4, mask = ent & 15u;
-      const uint4 r = philox_at(pd, cc, key);
+      const uint4 r = philox_at(pd, ent >> 4, key), th = dth[x];
 #pragma unroll
       for (int b = 0; b < 4; ++b) {
-        const uint32_t t = 4u * cc + (uint32_t)b;
-        if (((mask >> b) & 1u) && (word_of(r, b) >> 8) < dthr[t]) {
+        const uint32_t t = 4u * (ent >> 4) + (uint32_t)b;
+        if (word_of(r, b) <= word_of(th, b) && ((ent >> b) & 1u)) {
           --left;
           hsh += dead_key((int)t);
-          delta += at<long long>(img, L.deadd)[t];
-          dninf += at<int8_t>(img, L.dninf)[t];
+          delta += deadd[t];
+          dninf += dninf8[t];
         }
       }
     }
   }
-  // the noted rows (out of line, once per child)
-  if (nslow) {
-    const SlowSum o = slow_rows<DZ>(&md, &a.pt, img, a.T_max, a.K_max, a.M_plan, s_slow, nslow, (int)blockDim.x, bloom,
-                                    (uint32_t)n, key);
-    hsh += o.hw;
-    dclut += o.clut;
-    delta += o.d;
-    dninf += o.ninf;
-    bad_row |= o.bad != 0;
-  }
-  const long long score = sc.ref_score + delta + (md.kappa_zero ? 0LL : (long long)dclut * md.fx_log_kappa);
-  const int ninf = sc.ninf_ref + dninf + (md.kappa_zero ? dclut : 0);
-  const bool valid = !bad_row && ninf == 0;
-  const size_t j = (size_t)h * md.h_up + n;
-  a.child_key[j] = valid ? score : kKeyInvalid;
   a.child_hash[j] = hsh;
-  a.child_status[j] = valid ? 1 : 0;
   a.child_alive[j] = (uint16_t)(sc.T - nd);
-  return true;
+  if (nslow) {
+    // the noted rows are left to finish_notes, with the deaths' sums
+    const unsigned act = __activemask();
+    const int lane = (int)threadIdx.x & 31, lead = __ffs(act) - 1;
+    unsigned k = 0;
+    if (lane == lead) k = atomicAdd(a.note_count, (unsigned)__popc(act));
+    k = __shfl_sync(act, k, lead) + __popc(act & ((1u << lane) - 1u));
+    DrawNote* o = reinterpret_cast<DrawNote*>(a.notes) + k;
+    o->child = (uint32_t)j;
+    o->n_rows = (uint16_t)nslow;
+    o->dninf = (int16_t)dninf;
+    o->bloom = bloom;
+    for (int q = 0; q < nslow; ++q) o->rows[q] = s_slow[q * bd];
+    a.child_key[j] = delta;
+    return;
+  }
+  const int ninf = sc.ninf_ref + dninf;
+  a.child_key[j] = ninf == 0 ? sc.ref_score + delta : kKeyInvalid;
+  a.child_status[j] = ninf == 0 ? 1 : 0;
+}
+
+// The noted children, one thread each.  In the draw kernel itself the few
+// lanes with noted rows would hold their warps through slow_rows' chains of
+// dependent loads; here the lanes are dense.
+template <int DZ>
+__device__ __noinline__ void finish_notes(const ExpandArgs& a, const Lay& L, const uint2 key) {
+  const Model& md = a.md;
+  const uint32_t count = *a.note_count;
+  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
+    const DrawNote* o = reinterpret_cast<const DrawNote*>(a.notes) + k;
+    const uint32_t j = o->child, h = j / (uint32_t)md.h_up;
+    const unsigned char* img = a.img + (size_t)h * a.img_stride;
+    const Scal& sc = *at<Scal>(img, L.scal);
+    const SlowSum d = slow_rows<DZ>(&md, &a.pt, img, a.T_max, a.K_max, a.M_plan, o->rows, o->n_rows, o->bloom,
+                                    j - h * (uint32_t)md.h_up, key);
+    const long long score =
+        sc.ref_score + a.child_key[j] + d.d + (md.kappa_zero ? 0LL : (long long)d.clut * md.fx_log_kappa);
+    const int ninf = sc.ninf_ref + o->dninf + d.ninf + (md.kappa_zero ? d.clut : 0);
+    const bool valid = !d.bad && ninf == 0;
+    a.child_key[j] = valid ? score : kKeyInvalid;
+    a.child_hash[j] += d.hw;
+    a.child_status[j] = valid ? 1 : 0;
+  }
 }
 
 int expand_stage_tail_bytes(int dz, int T_plan, int K_plan, int M_plan, int mode) {
   return make_stage_tail(dz, T_plan, K_plan, M_plan, mode).total;
 }
 
-int expand_draw_smem(int threads) { return threads * (kDrawSlow + kDrawDead) * (int)sizeof(uint16_t); }
+// lists of the threads, then (staged) the parents' records
+int expand_draw_smem(int threads, int h_up, int T, int M, bool staged) {
+  return threads * (kDrawSlow + kDrawDead) * (int)sizeof(uint16_t) +
+         (staged ? draw_parents(threads, h_up) * make_draw_rec(T, M).total : 0);
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
 
 // Persistent over the children of the frame, one thread per child in the
 // order parent * h_up + draw (a warp holds 32 consecutive children, of at
-// most two parents when h_up >= 32); no block-level synchronisation.
-template <int DZ>
+// most two parents when h_up >= 32).  STAGED: the CTA first copies what the
+// chunk loops read of its children's parents to shared memory, so that the
+// loops wait for no cache miss (a parent's records are read by three or four
+// warps only: from the image one load in four missed L1, half of those L2).
+// What bounds the loops is the integer pipes: 41 instructions per Philox call
+// (16 wide multiplications at half rate), issued on 57 % of the cycles.
+// Measured with the rows' follow-up moved to finish_notes, one launch of the
+// 3-D N = 200 scene at H_max = 5000: 295 -> 226 us (161 -> 127 M warp
+// instructions); two children per thread sharing the records' loads: 3-9 %
+// slower, 64 registers (four CTAs per SM, spilled): 4 % slower, 128 registers
+// (two CTAs): 4 % slower.
+template <int DZ, bool STAGED>
 __global__ void __launch_bounds__(256, 3) draw_kernel(const __grid_constant__ ExpandArgs a) {
   pdl_enter();
   extern __shared__ __align__(16) unsigned char sm[];
-  uint16_t* s_slow = reinterpret_cast<uint16_t*>(sm) + threadIdx.x;
-  uint16_t* s_dead = s_slow + kDrawSlow * blockDim.x;
+  const int bd = (int)blockDim.x, tid = (int)threadIdx.x;
+  uint16_t* s_slow = reinterpret_cast<uint16_t*>(sm) + tid;
+  uint16_t* s_dead = s_slow + kDrawSlow * bd;
+  unsigned char* s_rec = sm + bd * (kDrawSlow + kDrawDead) * (int)sizeof(uint16_t);
   const Lay L = make_lay(DZ, a.T_max, a.K_max, a.M_plan);
+  const DrawRec R = make_draw_rec(a.T_max, a.M_plan);
   const int H = a.fs->H, HU = a.md.h_up;
   const uint2 key = make_uint2(a.key_x, a.key_y);
   // a failed table or staging (the frame is redone or abandoned): the
   // images may be stale, so nothing is drawn
   if (*(volatile const unsigned*)a.err & kErrFatal) return;
   const long long total = (long long)H * HU;
-  for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < total;
-       j += (long long)gridDim.x * blockDim.x) {
-    const int h = (int)(j / HU);
-    const int n = (int)(j - (long long)h * HU);
-    const unsigned char* img = a.img + (size_t)h * a.img_stride;
-    if (at<Scal>(img, L.scal)->bad) continue;
-    if (!thread_child<DZ>(a, img, L, h, n, key, s_slow, s_dead))
-      a.redo_list[atomicAdd(a.redo_count, 1u)] = (uint32_t)j;
+  // children a CTA takes at a time: one per thread, or fewer (whole warps)
+  // when the children would leave CTAs without any
+  const int q = (int)min((long long)bd, ((total + gridDim.x - 1) / gridDim.x + 31) / 32 * 32);
+  for (long long j0 = (long long)blockIdx.x * q; j0 < total; j0 += (long long)gridDim.x * q) {
+    const int nk = (int)min((long long)q, total - j0);
+    const int h0 = (int)(j0 / HU);
+    const int n0 = (int)(j0 - (long long)h0 * HU);   // the first child's draw
+    if (STAGED) {
+      const int np = (n0 + nk - 1) / HU + 1;
+      __syncthreads();   // the last round's records are read
+      for (int p = 0; p < np; ++p) {
+        const unsigned char* img = a.img + (size_t)(h0 + p) * a.img_stride;
+        const Scal& sc = *at<Scal>(img, L.scal);
+        if (sc.bad) continue;
+        unsigned char* rec = s_rec + p * R.total;
+        const int nr = 3 * sc.nrca, nt = sc.ndpc, nc = (sc.ndpc + 3) >> 2;
+        for (int w = tid; w < nr; w += bd) cp_async16(rec + R.rch + 16 * w, img + L.rch + 16 * w);
+        for (int w = tid; w < nt; w += bd) cp_async16(rec + R.dth + 16 * w, img + L.dth + 16 * w);
+        for (int w = tid; w < nc; w += bd) cp_async16(rec + R.dpc + 16 * w, img + L.dpc + 16 * w);
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+    }
+    if (tid < nk) {
+      const int h = h0 + (n0 + tid) / HU;
+      const unsigned char* img = a.img + (size_t)h * a.img_stride;
+      if (!at<Scal>(img, L.scal)->bad) {
+        const unsigned char* rec = s_rec + (h - h0) * R.total;
+        thread_child<DZ>(a, img, L, h, n0 + tid - (h - h0) * HU, key, s_slow, s_dead,
+                         STAGED ? at<RowChunk>(rec, R.rch) : at<RowChunk>(img, L.rch),
+                         STAGED ? at<uint4>(rec, R.dth) : at<uint4>(img, L.dth),
+                         STAGED ? at<uint32_t>(rec, R.dpc) : at<uint32_t>(img, L.dpc));
+      }
+    }
   }
 }
 
@@ -1654,8 +1769,10 @@ __device__ void warp_child(const ExpandArgs& a, const View& v, const int T, cons
 
 // Persistent over a list of children, one group of a.warp_group warps each
 // (several when the children are few and long): the survivors (MAT), every
-// child of every parent (a.warp_all), or the draw kernel's overflow.
-template <int DZ, bool MAT, bool GRP>
+// child of every parent (a.warp_all), or the draw kernel's overflow (NOTES:
+// after its noted children; an instantiation of its own, because the calls'
+// stack costs the others 2 us a launch).
+template <int DZ, bool MAT, bool GRP, bool NOTES>
 __global__ void __launch_bounds__(512) warp_kernel(const __grid_constant__ ExpandArgs a) {
   pdl_enter();
   extern __shared__ __align__(16) unsigned char sm[];
@@ -1672,6 +1789,7 @@ __global__ void __launch_bounds__(512) warp_kernel(const __grid_constant__ Expan
   if (!MAT && (*(volatile const unsigned*)a.err & kErrFatal)) return;
   const long long count = MAT ? (long long)*a.n_surv
                               : (a.warp_all ? (long long)a.fs->H * HU : (long long)*a.redo_count);
+  if (NOTES) finish_notes<DZ>(a, L, key);
   // an empty list (the usual overflow case) costs no work-area set-up
   if ((long long)blockIdx.x * groups >= count) return;
   unsigned char* gb = sm + g * WL.total;
@@ -1866,14 +1984,18 @@ static KernelFn stage_fn(int dz, bool smem) {
   if (dz == 2) return smem ? stage_kernel<2, true> : stage_kernel<2, false>;
   return smem ? stage_kernel<3, true> : stage_kernel<3, false>;
 }
-static KernelFn draw_fn(int dz) { return dz == 2 ? draw_kernel<2> : draw_kernel<3>; }
-static KernelFn warp_fn(int dz, bool mat, bool grp = false) {
+static KernelFn draw_fn(int dz, bool staged) {
+  if (dz == 2) return staged ? draw_kernel<2, true> : draw_kernel<2, false>;
+  return staged ? draw_kernel<3, true> : draw_kernel<3, false>;
+}
+static KernelFn warp_fn(int dz, bool mat, bool grp = false, bool notes = false) {
+  if (notes) return dz == 2 ? warp_kernel<2, false, false, true> : warp_kernel<3, false, false, true>;
   if (grp) {
-    if (dz == 2) return mat ? warp_kernel<2, true, true> : warp_kernel<2, false, true>;
-    return mat ? warp_kernel<3, true, true> : warp_kernel<3, false, true>;
+    if (dz == 2) return mat ? warp_kernel<2, true, true, false> : warp_kernel<2, false, true, false>;
+    return mat ? warp_kernel<3, true, true, false> : warp_kernel<3, false, true, false>;
   }
-  if (dz == 2) return mat ? warp_kernel<2, true, false> : warp_kernel<2, false, false>;
-  return mat ? warp_kernel<3, true, false> : warp_kernel<3, false, false>;
+  if (dz == 2) return mat ? warp_kernel<2, true, false, false> : warp_kernel<2, false, false, false>;
+  return mat ? warp_kernel<3, true, false, false> : warp_kernel<3, false, false, false>;
 }
 static KernelFn prep_fn(int dz) { return dz == 2 ? mat_prep_kernel<2> : mat_prep_kernel<3>; }
 
@@ -1881,7 +2003,9 @@ void expand_init(int smem_limit) {
   for (int dz = 2; dz <= 3; ++dz) {
     cudaFuncSetAttribute(stage_fn(dz, true), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
     cudaFuncSetAttribute(stage_fn(dz, false), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
-    cudaFuncSetAttribute(draw_fn(dz), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
+    for (int st = 0; st < 2; ++st)
+      cudaFuncSetAttribute(draw_fn(dz, st), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
+    cudaFuncSetAttribute(warp_fn(dz, false, false, true), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
     for (int grp = 0; grp < 2; ++grp) {
       cudaFuncSetAttribute(warp_fn(dz, false, grp), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
       cudaFuncSetAttribute(warp_fn(dz, true, grp), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
@@ -1892,8 +2016,8 @@ void expand_init(int smem_limit) {
 static KernelFn kernel_of(const ExpandArgs& a, ExpandKernel k) {
   switch (k) {
     case ExpandKernel::kStage: return stage_fn(a.md.dz, a.stage_smem != 0);
-    case ExpandKernel::kDraw: return draw_fn(a.md.dz);
-    case ExpandKernel::kWarp: return warp_fn(a.md.dz, a.materialize != 0, a.warp_group > 1);
+    case ExpandKernel::kDraw: return draw_fn(a.md.dz, a.draw_staged != 0);
+    case ExpandKernel::kWarp: return warp_fn(a.md.dz, a.materialize != 0, a.warp_group > 1, !a.materialize && !a.warp_all);
     default: return prep_fn(a.md.dz);
   }
 }
@@ -1937,7 +2061,9 @@ int expand_warp_best_cta(int dz, int materialize, int T, int max_warps, int smem
 
 bool expand_kernel_takes_key(const void* fn) {
   for (int dz = 2; dz <= 3; ++dz)
-    if (fn == (const void*)draw_fn(dz) || fn == (const void*)warp_fn(dz, false) || fn == (const void*)warp_fn(dz, true) ||
+    if (fn == (const void*)draw_fn(dz, false) || fn == (const void*)draw_fn(dz, true) ||
+         fn == (const void*)warp_fn(dz, false, false, true) || fn == (const void*)warp_fn(dz, false) ||
+         fn == (const void*)warp_fn(dz, true) ||
         fn == (const void*)warp_fn(dz, false, true) || fn == (const void*)warp_fn(dz, true, true))
       return true;
   return false;
