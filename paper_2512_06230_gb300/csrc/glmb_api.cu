@@ -1060,7 +1060,9 @@ glmb_status enqueue_prune(glmb_handle* h, const Plan& p) {
   const int m_grid = p.fixed ? m_ctas * h->n_sm
                              : std::max(1, std::min((h->cap_h + p.Gm - 1) / p.Gm, m_ctas * h->n_sm));
   prof_begin(h, kStageMat);
-  launch_expand_kernel(a, ExpandKernel::kMatPrep, std::max(1, std::min((h->cap_h + 7) / 8, 2 * h->n_sm)),
+  // a warp per 32 slots of each survivor, up to two CTAs per SM
+  const long long prep_warps = (long long)h->cap_h * ((p.T + 31) / 32);
+  launch_expand_kernel(a, ExpandKernel::kMatPrep, (int)std::max(1LL, std::min((prep_warps + 7) / 8, 2LL * h->n_sm)),
                        256, 0, s);
   launch_expand_kernel(a, ExpandKernel::kWarp, m_grid, m_thr, m_smem, s);
   prof_end(h, kStageMat);
