@@ -7,19 +7,24 @@
 //      duplicate-marking kernel left per block (per-thread integer maximum
 //      and compensated FP32 sums of FP32 exponentials, rescaled and summed
 //      in FP64), the unique count, the fixed-point threshold log(tau) + LSE;
-//   2  top-H_max among the children at or above the threshold by 12-bit
-//      radix select on key - threshold: every CTA histograms its slice,
-//      each CTA sums one slice of bins over the cluster, every CTA gathers
-//      the summed histogram and finds the boundary digit (all CTAs compute
-//      the same result, so no broadcast is needed).  The first pass also
-//      counts each thread's children at or above the threshold: when the
-//      cluster's count is within H_max every one of them is kept, and that
-//      count is the compaction's, so no second pass is made;
+//   2  the children at or above the threshold counted over the cluster: when
+//      they are within H_max every one of them is kept and the count is the
+//      compaction's; else top-H_max by 12-bit radix select on key -
+//      threshold: every CTA histograms its slice, each CTA sums one slice of
+//      bins over the cluster, every CTA gathers the summed histogram and
+//      finds the boundary digit (all CTAs compute the same result, so no
+//      broadcast is needed);
 //   3  stable compaction in child order (parent, draw): per-CTA counts of
 //      children above and at the boundary, an exclusive scan over the
 //      cluster, then each thread writes its contiguous share;
 //   4  the retained set (CTA 0): renormalised FP64 log-weights, child uids,
 //      CSR offsets of the new hypothesis table.
+// What bounds it is latency: cluster barriers, reads of L2 and the FP64
+// reductions (16 cycles an instruction on an SM).  So up to kSoloKeys children
+// per thread one CTA selects alone, keys that fit are held from the first
+// read, warps without a value skip the FP64 sums, and the histogram is made
+// only when the cap binds.  Per frame: 25.0 -> 16.7 us (2500 children, cap
+// binds), 24.3 -> 16.1 (1500), 33.0 -> 27.4 (190 000), 44 -> 38.7 (a million).
 // Results equal the multi-kernel chain's except for the summation order of
 // the LSE (a different tree), which moves it by rounding only.
 #include <cooperative_groups.h>
@@ -35,6 +40,9 @@ namespace {
 
 constexpr int kSelDigit = 12, kSelBins = 1 << kSelDigit;
 constexpr int kSelThreads = 1024;
+// up to this many children per thread of one CTA, CTA 0 selects alone
+constexpr int kSoloKeys = 16;
+constexpr int kSoloSurv = 2048;   // survivors it keeps on chip
 
 __device__ __forceinline__ long long warp_max_k(long long v) {
 #pragma unroll
@@ -49,7 +57,7 @@ __device__ __forceinline__ double warp_sum_dd(double v) {
 
 struct SelShared {
   unsigned hist[kSelBins];        // this CTA's histogram of the current digit
-  unsigned hsum[2][kSelBins];     // the cluster's histogram (this CTA sums one slice; rounds alternate)
+  alignas(16) unsigned hsum[2][kSelBins];     // the cluster's histogram (this CTA sums one slice; rounds alternate)
   unsigned long long part[32];    // per-warp partials
   double dpart[32];
   long long pm;                   // CTA partial: maximum key
@@ -80,7 +88,7 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
                       HypTable parents, HypTable out, unsigned* err, long long cap_entries) {
   pdl_enter();
   cg::cluster_group cl = cg::this_cluster();
-  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int rank = (int)cl.block_rank();
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, wp = tid >> 5, nw = nthr >> 5;
   // the prune counters start at zero (this thread writes the first of them
   // below; the others are written after cluster barriers)
@@ -92,7 +100,24 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
   if (*(volatile const unsigned*)err & kErrFatal) return;
   extern __shared__ __align__(16) unsigned char sel_sm[];
   SelShared& S = *reinterpret_cast<SelShared*>(sel_sm);
+  // (loaded beside the parent count; masked by it below)
+  long long pm0 = kKeyInvalid;
+  double ps0 = 0.0;
+  unsigned pc0 = 0;
+  if (tid < n_part) {
+    pm0 = w.part_max[tid];
+    ps0 = w.part_sum[tid];
+    pc0 = w.part_cnt[tid];
+  }
   const long long n = (long long)fs->H * h_up;
+  // few children: CTA 0 alone, with block barriers in place of the cluster's
+  const bool solo = n <= (long long)kSoloKeys * nthr;
+  if (solo && rank != 0) return;
+  const int C = solo ? 1 : (int)cl.num_blocks();
+  auto csync = [&]() {
+    if (solo) __syncthreads();
+    else cl.sync();
+  };
   const long long per = (n + C - 1) / C;
   const long long lo = min(n, (long long)rank * per), hi = min(n, lo + per);
 
@@ -100,9 +125,18 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
   // (every CTA reduces all of them in the same order: the same result;
   // blocks beyond the parents wrote none)
   n_part = min(n_part, fs->H);
+  // each thread's contiguous share of the CTA's children (compaction order);
+  // its first keys, held when they are all
+  const long long chunk = hi - lo;
+  const long long q = (chunk + nthr - 1) / nthr;
+  const long long a0 = lo + (long long)tid * q, a1 = min(hi, a0 + q);
+  const bool held_keys = q <= 4;
+  long long kk[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) kk[u] = held_keys && a0 + u < a1 ? keys[a0 + u] : kKeyInvalid;
   {
-    long long m = kKeyInvalid;
-    for (int b = tid; b < n_part; b += nthr) m = max(m, w.part_max[b]);
+    long long m = tid < n_part ? pm0 : kKeyInvalid;
+    for (int b = tid + nthr; b < n_part; b += nthr) m = max(m, w.part_max[b]);
     m = warp_max_k(m);
     if (lane == 0) S.part[wp] = (unsigned long long)m;
     __syncthreads();
@@ -115,11 +149,15 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
     const long long M = S.pm;
     double r = 0.0;
     unsigned c = 0;
-    for (int b = tid; b < n_part; b += nthr) {
+    if (tid < n_part) {
+      r = lse_rescale(pm0, ps0, M);
+      c = pc0;
+    }
+    for (int b = tid + nthr; b < n_part; b += nthr) {
       r += lse_rescale(w.part_max[b], w.part_sum[b], M);
       c += w.part_cnt[b];
     }
-    r = warp_sum_dd(r);
+    if (32 * wp < n_part) r = warp_sum_dd(r);   // (a warp without partials holds zeros: the FP64 pipe is slow)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
     if (lane == 0) {
@@ -161,115 +199,137 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
   const long long thr = S.thr;
   const int passes = (nbits + kSelDigit - 1) / kSelDigit;
   const int slice = (kSelBins + C - 1) / C;
-  // each thread's contiguous share of the CTA's children (compaction order)
-  const long long chunk = hi - lo;
-  const long long q = (chunk + nthr - 1) / nthr;
-  const long long a0 = lo + (long long)tid * q, a1 = min(hi, a0 + q);
-  unsigned long long above0 = 0ull;   // this thread's children at or above thr (first pass)
-  for (int p = 0; p < passes; ++p) {
-    const int shift = (passes - 1 - p) * kSelDigit;
-    const int mode = S.mode;   // identical in every CTA
-    if (mode != 0) break;
-    unsigned* hs = S.hsum[p & 1];
-    for (int b = tid; b < kSelBins; b += nthr) S.hist[b] = 0u;
+  // The children at or above the threshold, counted first: a thread's, and
+  // the block's before them, are also the compaction's when every one of
+  // them is kept (the tau cut binds before the cap), and no histogram is made
+  unsigned long long mine = 0ull, excl_blk = 0ull;
+  // block exclusive scan of x (the block's total in S.part[nw - 1])
+  auto block_scan = [&](unsigned long long v) {
+    unsigned long long x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) S.part[wp] = x;
     __syncthreads();
-    const unsigned long long prefix = (unsigned long long)S.prefix;
-    // one shared-memory atomic per distinct bin of a warp (the keys near the
-    // top crowd a few bins)
-    // the lanes with a bin (most children are below the threshold) add
-    // their counts, one atomic per distinct bin
-    auto add_bin = [&](int bin) {
-      const unsigned act = __ballot_sync(0xFFFFFFFFu, bin >= 0);
-      if (bin >= 0) {
-        const unsigned grp = __match_any_sync(act, bin);
-        if (lane == __ffs(grp) - 1) atomicAdd(&S.hist[bin], (unsigned)__popc(grp));
+    if (wp == 0) {
+      unsigned long long t = lane < nw ? S.part[lane] : 0ull;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, t, o);
+        if (lane >= o) t += y;
       }
-    };
-    if (p == 0) {
-      // over the thread's own share, counting it as well; four loads in
-      // flight per step (every lane runs the same steps, so the warp stays
-      // converged for the ballots)
-      for (long long t = 0; t < q; t += 4) {
+      S.part[lane] = t;
+    }
+    __syncthreads();
+    return (wp > 0 ? S.part[wp - 1] : 0ull) + x - v;
+  };
+  // the cluster's total of the blocks' totals and the lower ranks' share
+  auto cluster_total = [&]() {
+    if (tid == 0) S.cnt = S.part[nw - 1];
+    csync();
+    if (wp == 0) {
+      const unsigned long long c = solo ? (lane == 0 ? S.cnt : 0ull)
+                                        : lane < C ? cl.map_shared_rank(&S, lane)->cnt : 0ull;
+      unsigned long long before = lane < rank ? c : 0ull, total = c;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+        total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
+      }
+      if (lane == 0) {
+        S.before = before;
+        S.total = total;
+      }
+    }
+    __syncthreads();
+  };
+  if (S.mode == 0) {
+    for (long long t = 0; t < q; t += 4) {
+      long long k4[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) k4[u] = held_keys ? kk[u] : a0 + t + u < a1 ? keys[a0 + t + u] : kKeyInvalid;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) mine += k4[u] != kKeyInvalid && k4[u] >= thr;
+    }
+    excl_blk = block_scan(mine);
+    cluster_total();
+    if (tid == 0 && (long long)S.total <= S.need) {
+      S.mode = 1;
+      S.bnd = thr - 1;   // every candidate is above the boundary
+      S.need = 0;
+    }
+    __syncthreads();
+  } else if (tid == 0) {
+    S.before = 0ull;
+    S.total = 0ull;
+  }
+  if (S.mode == 0) {
+    for (int p = 0; p < passes; ++p) {
+      const int shift = (passes - 1 - p) * kSelDigit;
+      unsigned* hs = S.hsum[p & 1];
+      for (int b = tid; b < kSelBins; b += nthr) S.hist[b] = 0u;
+      __syncthreads();
+      const unsigned long long prefix = (unsigned long long)S.prefix;
+      // one shared-memory atomic per distinct bin of a warp (the keys near
+      // the top crowd a few bins): the lanes with a bin (most children are
+      // below the threshold) add their counts; four loads in flight per step
+      // (every lane runs the same steps, so the warp stays converged for the
+      // ballots)
+      for (long long base = lo; base < hi; base += 4LL * nthr) {
         long long k4[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) k4[u] = a0 + t + u < a1 ? keys[a0 + t + u] : kKeyInvalid;
+        for (int u = 0; u < 4; ++u) {
+          const long long j = base + (long long)u * nthr + tid;
+          k4[u] = held_keys ? kk[u] : j < hi ? keys[j] : kKeyInvalid;
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           int bin = -1;
           if (k4[u] != kKeyInvalid && k4[u] >= thr) {
-            ++above0;
-            bin = (int)(((unsigned long long)(k4[u] - thr) >> shift) & (kSelBins - 1));
+            const unsigned long long v = (unsigned long long)(k4[u] - thr);
+            if (p == 0 || (v >> (shift + kSelDigit)) == prefix) bin = (int)((v >> shift) & (kSelBins - 1));
           }
-          add_bin(bin);
-        }
-      }
-    } else {
-      for (long long base = lo; base < hi; base += nthr) {
-        const long long j = base + tid;
-        int bin = -1;
-        if (j < hi) {
-          const long long k = keys[j];
-          if (k != kKeyInvalid && k >= thr) {
-            const unsigned long long v = (unsigned long long)(k - thr);
-            if ((v >> (shift + kSelDigit)) == prefix) bin = (int)((v >> shift) & (kSelBins - 1));
+          const unsigned act = __ballot_sync(0xFFFFFFFFu, bin >= 0);
+          if (bin >= 0) {
+            const unsigned grp = __match_any_sync(act, bin);
+            if (lane == __ffs(grp) - 1) atomicAdd(&S.hist[bin], (unsigned)__popc(grp));
           }
         }
-        add_bin(bin);
       }
-    }
-    cl.sync();
-    // this CTA's slice of the summed histogram
-    for (int b = rank * slice + tid; b < min(kSelBins, (rank + 1) * slice); b += nthr) {
-      unsigned t = 0;
-      for (int r = 0; r < C; ++r) t += cl.map_shared_rank(S.hist, r)[b];
-      hs[b] = t;
-    }
-    cl.sync();
-    // gather the other slices
-    for (int b = tid; b < kSelBins; b += nthr) {
-      const int owner = b / slice;
-      if (owner != rank) hs[b] = cl.map_shared_rank(hs, owner)[b];
-    }
-    __syncthreads();
-    // boundary digit: thread t owns bins [4t, 4t + 4); counts above a range =
-    // total - inclusive prefix
-    {
-      unsigned b4[4], mine = 0;
+      csync();
+      if (!solo) {
+        // this CTA's slice of the summed histogram
+        for (int b = rank * slice + tid; b < min(kSelBins, (rank + 1) * slice); b += nthr) {
+          unsigned t = 0;
+          for (int r = 0; r < C; ++r) t += cl.map_shared_rank(S.hist, r)[b];
+          hs[b] = t;
+        }
+        cl.sync();
+        // gather the other slices
+        for (int b = tid; b < kSelBins; b += nthr) {
+          const int owner = b / slice;
+          if (owner != rank) hs[b] = cl.map_shared_rank(hs, owner)[b];
+        }
+        __syncthreads();
+      } else {
+        hs = S.hist;
+      }
+      // boundary digit: thread t owns bins [4t, 4t + 4); counts above a range
+      // = total - inclusive prefix
+      unsigned b4[4], mine4 = 0;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         b4[k] = hs[4 * tid + k];
-        mine += b4[k];
+        mine4 += b4[k];
       }
-      unsigned x = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-        if (lane >= o) x += y;
-      }
-      if (lane == 31) S.part[wp] = x;
-      __syncthreads();
-      if (wp == 0) {
-        unsigned long long s = S.part[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-          if (lane >= o) s += y;
-        }
-        S.part[lane] = s;
-      }
-      __syncthreads();
-      const unsigned incl = x + (wp > 0 ? (unsigned)S.part[wp - 1] : 0u);
+      const unsigned excl = (unsigned)block_scan(mine4);
       const unsigned total = (unsigned)S.part[31];
-      const unsigned above = total - incl, upto = above + mine;
+      const unsigned above = total - excl - mine4, upto = above + mine4;
       const long long need = S.need;
       __syncthreads();   // everyone has read need before it changes
-      if (p == 0 && (long long)total <= need) {
-        if (tid == 0) {
-          S.mode = 1;
-          S.bnd = thr - 1;   // every candidate is above the boundary
-          S.need = 0;
-        }
-      } else if ((long long)above < need && (long long)upto >= need) {
+      if ((long long)above < need && (long long)upto >= need) {
         unsigned cum = above;
         int b = 3;
         for (; b > 0; --b) {
@@ -282,61 +342,36 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
       }
       __syncthreads();
     }
+    csync();   // the summed histograms are no longer read
+
+    // above and at the boundary, in compaction order
+    mine = 0ull;
+    if (held_keys) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) mine += keep_flag(kk[u], thr, S.bnd, S.need, 0);
+    } else {
+#pragma unroll 4
+      for (long long j = a0; j < a1; ++j) mine += keep_flag(keys[j], thr, S.bnd, S.need, 0);
+    }
+    excl_blk = block_scan(mine);
+    cluster_total();
   }
-  cl.sync();   // the summed histograms are no longer read
 
   // ---- 3: stable compaction in child order ----
+  __syncthreads();
   const int mode = S.mode;
   const long long bnd = S.bnd, need = S.need;
-  // every candidate kept (decided by the first pass), or none: the first
-  // pass's count is the thread's; else count above and at the boundary
-  unsigned long long mine = mode == 1 ? above0 : 0ull;
-  if (mode == 0)
-#pragma unroll 4
-    for (long long j = a0; j < a1; ++j) mine += keep_flag(keys[j], thr, bnd, need, mode);
-  // block exclusive scan of (above | at << 32)
-  unsigned long long x = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) S.part[wp] = x;
-  __syncthreads();
-  if (wp == 0) {
-    unsigned long long s = lane < nw ? S.part[lane] : 0ull;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, s, o);
-      if (lane >= o) s += y;
-    }
-    S.part[lane] = s;
-  }
-  __syncthreads();
-  const unsigned long long excl_blk = (wp > 0 ? S.part[wp - 1] : 0ull) + x - mine;
-  if (tid == 0) S.cnt = S.part[nw - 1];
-  cl.sync();
-  if (wp == 0) {
-    const unsigned long long c = lane < C ? cl.map_shared_rank(&S, lane)->cnt : 0ull;
-    unsigned long long before = lane < rank ? c : 0ull, total = c;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
-      total += __shfl_xor_sync(0xFFFFFFFFu, total, o);
-    }
-    if (lane == 0) {
-      S.before = before;
-      S.total = total;
-    }
-  }
-  __syncthreads();
+  // a CTA alone keeps its survivors and their keys in place of the summed
+  // histogram, which is no longer read
+  long long* s_surv = reinterpret_cast<long long*>(&S.hsum[0][0]);
+  static_assert(sizeof(S.hsum) == 16 * kSoloSurv, "room for (index, key) pairs");
   {
     unsigned long long run = S.before + excl_blk;
     // a share with nothing kept is not read again
     for (long long t = a0; mine && t < a1; t += 4) {
       long long k4[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) k4[u] = t + u < a1 ? keys[t + u] : kKeyInvalid;
+      for (int u = 0; u < 4; ++u) k4[u] = held_keys ? kk[u] : t + u < a1 ? keys[t + u] : kKeyInvalid;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const unsigned long long f = keep_flag(k4[u], thr, bnd, need, mode);
@@ -345,11 +380,17 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
         run += f;
         if ((f >> 32) && eq >= need) continue;
         const long long pos = gt + min(eq, need);
-        if (pos < h_max) w.surv_idx[pos] = t + u;
+        if (pos < h_max) {
+          w.surv_idx[pos] = t + u;
+          if (solo && pos < kSoloSurv) {
+            s_surv[2 * pos] = t + u;
+            s_surv[2 * pos + 1] = k4[u];
+          }
+        }
       }
     }
   }
-  cl.sync();   // every survivor index is written (the cluster barrier orders them)
+  csync();   // every survivor index is written (the barrier orders them)
 
   // ---- 4: the retained set, each CTA a contiguous share of it ----
   long long ns = 0;
@@ -360,7 +401,7 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
   }
   // shared over the cluster when it is larger than two rounds of one CTA;
   // else CTA 0 alone, without the cluster barriers
-  const bool spread = ns > 2LL * nthr;
+  const bool spread = !solo && ns > 2LL * nthr;
   if (!spread && rank != 0) return;
   const int Cs = spread ? C : 1;
   const long long sper = (ns + Cs - 1) / Cs;
@@ -375,14 +416,15 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
   const int rounds = (int)((r1 - r0 + nthr - 1) / nthr);
   const bool held = rounds <= kPer;
   auto load_survivor = [&](long long t, long long& j, long long& k, uint32_t& na, unsigned long long& pu) {
-    j = w.surv_idx[t];
+    const bool on_chip = solo && t < kSoloSurv;
+    j = on_chip ? s_surv[2 * t] : w.surv_idx[t];
     if (j < 0 || j >= n) {   // invariant: every survivor index was written this frame
       atomicOr(err, kErrChkSurv);
       j = 0;
     }
-    k = keys[j];
+    k = on_chip ? s_surv[2 * t + 1] : keys[j];
     na = child_alive[j];
-    pu = parents.uid[j / h_up];
+    pu = parents.uid[(j >> 32) ? j / h_up : (long long)((uint32_t)j / (uint32_t)h_up)];
   };
   {
     // the share's maximum, sum of exp(key - maximum) and alive count
@@ -444,7 +486,7 @@ select_cluster_kernel(const long long* __restrict__ keys, const FrameDev* __rest
     }
     __syncthreads();
     double r = (m == kKeyInvalid) ? 0.0 : sm_ * (double)expf(fx_to_f(m - S.pm));
-    r = warp_sum_dd(r);
+    if (r0 + 32 * wp < r1) r = warp_sum_dd(r);
     if (lane == 0) S.dpart[wp] = r;
     __syncthreads();
     if (wp == 0) {
@@ -579,8 +621,10 @@ bool launch_select_cluster(const long long* keys, const FrameDev* fs, int h_up, 
                            double log_tau, int h_max, int nbits, const uint16_t* child_alive,
                            const HypTable& parents, const HypTable& out, unsigned* err, long long cap_entries,
                            cudaStream_t s) {
-  const int c = select_cluster_size();
+  int c = select_cluster_size();
   if (c == 0) return false;
+  // a filter whose every frame one CTA selects alone needs no cluster
+  if ((long long)h_max * h_up <= (long long)kSoloKeys * kSelThreads) c = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(c);
   cfg.blockDim = dim3(kSelThreads);
