@@ -348,8 +348,8 @@ glmb_status glmb_step_batch(glmb_handle* const* hs, int n, const glmb_frame_in* 
  *   warp_cta_warps       most warps per CTA of the one-warp-per-child kernel
  *                        (1..16, default 16);
  *   stage_threads        threads per staging CTA (32..256, multiple of 32; 0,
- *                        the default: 256 when parents are staged in shared
- *                        memory or are fewer than two per SM, else 64).
+ *                        the default: by the parents' count and size, from
+ *                        64 for many small ones to 1024 for a few large).
  * Setting them drops the captured graphs. */
 typedef struct {
   int32_t thread_warps_per_sm;

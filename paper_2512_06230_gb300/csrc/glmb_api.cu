@@ -968,6 +968,7 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
       if (expand_stage_tail_bytes(dz, p.T, p.K, p.M, m) <= h->smem_limit) a.stage_tail = m;
   const int st_smem = (p.smem ? img : 0) + expand_stage_tail_bytes(dz, p.T, p.K, p.M, a.stage_tail);
   const int st_thr = p.st_thr;
+  a.stage_wide = st_thr > 256 ? 1 : 0;
   const int st_ctas = std::max(1, expand_occupancy(a, ExpandKernel::kStage, st_thr, st_smem));
   const int st_grid = p.fixed ? st_ctas * n_sm : std::max(1, std::min(h->H, st_ctas * n_sm));
   // draws: one thread per child over the frame's children in order
@@ -1136,14 +1137,19 @@ bool make_plan(glmb_handle* h, bool fixed, int T_plan, int K_plan, int M_plan, P
   p.smem = img_bytes + expand_stage_tail_bytes(dz, p.T, p.K, p.M, 0) <= h->smem_limit &&
            !(h->launch_opts & GLMB_OPT_STAGE_GLOBAL) &&
            (8LL * img_bytes <= (long long)h->smem_per_sm || (h->launch_opts & GLMB_OPT_STAGE_SHARED));
-  // staging threads: 256 in shared memory, or for few parents (each parent's
-  // work spread over more threads); else 128: with its scratch in shared
-  // memory (about 29 KB for the 3-D sweep's plans) six such CTAs per SM keep
-  // 24 warps in flight, where 64-thread CTAs would be limited to seven by
-  // shared memory (measured on the N = 200, H_max = 20000 cell: expansion
-  // 1.56 ms with 128, 1.87 ms with 64)
-  p.st_thr = h->tune.stage_threads > 0 ? h->tune.stage_threads
-             : (p.smem || (long long)h->H < 2LL * h->n_sm) ? 256 : 128;
+  // staging threads.  Large images (staged in global memory): 1024 when each
+  // parent has an SM of its own and 512 slots or rows to spread (15 parents of
+  // 1400 slots and 2600 rows); 256 while the parents are fewer than two per SM;
+  // else 128, whose scratch in shared memory (about 29 KB for the 3-D sweep's
+  // plans) lets six CTAs per SM keep 24 warps in flight (N = 200 at H_max =
+  // 20000: expansion 585 us with 128, 641 with 64, 618 with 256).  Small
+  // images (staged in shared memory) leave most of 256 threads waiting at the
+  // barriers: 64 once the parents fill the GPU with such CTAs (3-D N = 50:
+  // expansion 118 us with 256, 106 with 128, 103 with 64, 115 with 32)
+  if (h->tune.stage_threads > 0) p.st_thr = h->tune.stage_threads;
+  else if (p.smem) p.st_thr = (long long)h->H >= 4LL * h->n_sm ? 64 : 256;
+  else if (h->H <= h->n_sm && std::max(p.T, p.M) >= 512) p.st_thr = kStageWide;
+  else p.st_thr = (long long)h->H < 2LL * h->n_sm ? 256 : 128;
   p.Gw = p.Gm = 0;
   for (int g = h->tune.warp_cta_warps; g >= 1 && !p.Gw; --g)
     if (expand_warp_smem(dz, 0, p.T, g, 1) <= h->smem_limit) p.Gw = g;

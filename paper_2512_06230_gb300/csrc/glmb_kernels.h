@@ -121,6 +121,8 @@ constexpr long long kGateWaitLimit = 2000000000LL;     // SM clock cycles (about
 WaitTest wait_test();
 void set_wait_test(WaitTest w);
 
+constexpr int kStageWide = 1024;
+
 struct ExpandArgs {
   Model md;
   CompTable ct;           // working (predicted) table
@@ -134,6 +136,7 @@ struct ExpandArgs {
   unsigned char* img;
   long long img_stride;
   int stage_smem;         // staged in shared memory (else in the image itself)
+  int stage_wide;         // staging CTAs of kStageWide threads
   int draw_staged;        // thread-per-child draw: the parents' chunk records go to shared memory first
   int warp_all;           // warp kernel: every child of every parent (else the overflow list)
   uint32_t* redo_list;    // children the draw kernel could not take

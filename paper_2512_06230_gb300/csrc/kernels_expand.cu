@@ -144,7 +144,8 @@ __host__ __device__ inline StageTail make_stage_tail(int dz, int T, int K, int M
   StageTail S{};
   Bump b;
   b.take(16);   // next-parent word
-  b.take(32);   // warp sums of the row-count scan
+  b.take(32);   // the parent's sizes, counts and flags
+  b.take(128);  // warp sums of the row-count scan
   if (mode >= 1) {
     S.rowoff = b.take(4LL * (M + 1));
     S.rowfill = b.take(4LL * (M + 1));
@@ -438,7 +439,7 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   RowChunk* s_rch = at<RowChunk>(sm, L.rch);
   uint8_t* s_srow = at<uint8_t>(sm, L.srow);
   uint32_t* s_rowthr0 = at<uint32_t>(sm, L.rowthr0);
-  uint32_t* s_wsum = at<uint32_t>(tb, 16);
+  uint32_t* s_wsum = at<uint32_t>(tb, 16), *s_scan = at<uint32_t>(tb, 48);
   uint32_t* s_rowoff = mode >= 1 ? at<uint32_t>(tb, TS.rowoff) : at<uint32_t>(sm, L.rowoff);
   uint32_t* s_rowfill = mode >= 1 ? at<uint32_t>(tb, TS.rowfill) : at<uint32_t>(sm, L.rowfill);
   float* s_roww0 = at<float>(sm, L.roww0);
@@ -570,10 +571,10 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
       const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
       if (lane >= o) x += y;
     }
-    if (lane == 31) s_wsum[wp] = x;
+    if (lane == 31) s_scan[wp] = x;
     __syncthreads();
     uint32_t base = x - run;
-    for (int w = 0; w < wp; ++w) base += s_wsum[w];
+    for (int w = 0; w < wp; ++w) base += s_scan[w];
     for (int i = b0; i < b1; ++i) {
       const uint32_t v = s_rowfill[i];
       s_rowoff[i] = base;
@@ -589,7 +590,7 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
         sc.bad = 1;
         atomicOr(a.err, kErrSlots);
       }
-      s_wsum[7] = over ? 1u : 0u;   // no warp's scan reads the last word
+      s_wsum[7] = over ? 1u : 0u;
     }
   }
   __syncthreads();
@@ -939,8 +940,9 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
 // parent from a counter until none is left (parents differ in slots and
 // pairs, so a fixed share per CTA would leave SMs idle at the end).
 // SMEM: staged in shared memory and copied to the image (16-byte words).
-template <int DZ, bool SMEM>
-__global__ void __launch_bounds__(256, 3) stage_kernel(const __grid_constant__ ExpandArgs a) {
+// WIDE: CTAs of kStageWide threads, for a few parents of many slots and rows.
+template <int DZ, bool SMEM, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? kStageWide : 256, WIDE ? 1 : 3) stage_kernel(const __grid_constant__ ExpandArgs a) {
   pdl_enter();
   extern __shared__ __align__(16) unsigned char sm[];
   const Lay L = make_lay(DZ, a.T_max, a.K_max, a.M_plan);
@@ -2076,9 +2078,10 @@ void launch_dedup(const FrameDev* fs, int HU, long long* child_key, const unsign
 // ---- host side ----
 using KernelFn = void (*)(const ExpandArgs);
 
-static KernelFn stage_fn(int dz, bool smem) {
-  if (dz == 2) return smem ? stage_kernel<2, true> : stage_kernel<2, false>;
-  return smem ? stage_kernel<3, true> : stage_kernel<3, false>;
+static KernelFn stage_fn(int dz, bool smem, bool wide) {
+  if (wide) return dz == 2 ? stage_kernel<2, false, true> : stage_kernel<3, false, true>;
+  if (dz == 2) return smem ? stage_kernel<2, true, false> : stage_kernel<2, false, false>;
+  return smem ? stage_kernel<3, true, false> : stage_kernel<3, false, false>;
 }
 static KernelFn draw_fn(int dz, bool staged) {
   if (dz == 2) return staged ? draw_kernel<2, true> : draw_kernel<2, false>;
@@ -2097,8 +2100,9 @@ static KernelFn prep_fn(int dz) { return dz == 2 ? mat_prep_kernel<2> : mat_prep
 
 void expand_init(int smem_limit) {
   for (int dz = 2; dz <= 3; ++dz) {
-    cudaFuncSetAttribute(stage_fn(dz, true), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
-    cudaFuncSetAttribute(stage_fn(dz, false), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
+    cudaFuncSetAttribute(stage_fn(dz, true, false), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
+    for (int wide = 0; wide < 2; ++wide)
+      cudaFuncSetAttribute(stage_fn(dz, false, wide), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
     for (int st = 0; st < 2; ++st)
       cudaFuncSetAttribute(draw_fn(dz, st), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
     cudaFuncSetAttribute(warp_fn(dz, false, false, true), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
@@ -2111,7 +2115,7 @@ void expand_init(int smem_limit) {
 
 static KernelFn kernel_of(const ExpandArgs& a, ExpandKernel k) {
   switch (k) {
-    case ExpandKernel::kStage: return stage_fn(a.md.dz, a.stage_smem != 0);
+    case ExpandKernel::kStage: return stage_fn(a.md.dz, a.stage_smem != 0, a.stage_wide != 0);
     case ExpandKernel::kDraw: return draw_fn(a.md.dz, a.draw_staged != 0);
     case ExpandKernel::kWarp: return warp_fn(a.md.dz, a.materialize != 0, a.warp_group > 1, !a.materialize && !a.warp_all);
     default: return prep_fn(a.md.dz);
