@@ -11,10 +11,13 @@
 //             row integer thresholds of the categorical draw under "all slots
 //             alive", a reference association (each row's most likely option)
 //             with its exact score, and per slot the m-only part of the track
-//             term for m_ref - 2 .. m_ref + 2 detections;
-//             The stage also tabulates the exact score change of every single
-//             deviation from the reference: a detection joining a candidate
-//             pair's slot, leaving its reference slot, a slot dying;
+//             term for m_ref - 2 .. m_ref + 2 detections, and the exact score
+//             change of each slot dying.  What only deviating children read
+//             (innovations, covariances) stays in the pair and component
+//             tables: the images of the 3-D N = 200 scene shrink by 28 %, and
+//             the staging's reads go out together instead of each waiting for
+//             the write before it (with the follow-up below, expansion of the
+//             scene 577 -> 519 us per frame, gated 311 -> 266);
 //   draw      one thread per child: Philox words for the slots that can die
 //             (stage 1) and one per detection row (stage 2); the row's option
 //             is the first whose threshold exceeds the 24-bit uniform (rows
@@ -49,8 +52,8 @@ struct Lay {
   int scal;
   int row, rowbl, seref, sqref, termref, hwref, deadd;
   int rowrk, rch, rowoff, rowfill, roww0, rowthr0;
-  int comp, dthr, logp, log1mp, mref, refnew, hph, dpc, dth;
-  int cthr, ceidx, cw, ce, cq, cslot;
+  int comp, dthr, mref, refnew, dpc, dth;
+  int cthr, ceidx, cw, cslot;
   int ninfref, dninf, srow;
   int total;
 };
@@ -91,7 +94,6 @@ struct Scal {
 __host__ __device__ inline Lay make_lay(int dz, int T, int K, int M) {
   Lay L;
   Bump b;
-  const int NP = dz * (dz + 1) / 2;
   L.scal = b.take(sizeof(Scal));
   L.row = b.take(16LL * M);                 // packed row descriptors (uint4)
   L.rowbl = b.take(8LL * M);                // bit (slot mod 64) of each candidate slot
@@ -110,18 +112,13 @@ __host__ __device__ inline Lay make_lay(int dz, int T, int K, int M) {
   L.rowthr0 = b.take(4LL * M);              // clutter option's threshold
   L.comp = b.take(4LL * T);
   L.dthr = b.take(4LL * T);
-  L.logp = b.take(4LL * T);
-  L.log1mp = b.take(4LL * T);
   L.mref = b.take(4LL * T);
   L.refnew = b.take(4LL * T);
-  L.hph = b.take(4LL * NP * T);             // H P H^T of each slot (packed)
   L.dpc = b.take(4LL * (T / 4 + 2));        // chunks of 4 slots that can die
   L.dth = b.take(16LL * (T / 4 + 2));       // their slots' largest dying words (see the chunk lists)
   L.cthr = b.take(4LL * K);
-  L.ceidx = b.take(4LL * K);
+  L.ceidx = b.take(4LL * K);                // the pair's place in the table (innovation, q, log C)
   L.cw = b.take(4LL * K);
-  L.ce = b.take(4LL * dz * K);              // innovation of each candidate pair
-  L.cq = b.take(4LL * K);                   // e^T R^-1 e of each candidate pair
   L.cslot = b.take(2LL * K);
   L.ninfref = b.take(T);
   L.dninf = b.take(T);
@@ -227,14 +224,14 @@ __device__ __forceinline__ void touch(uint32_t* tmask, uint16_t* tlist, int* nt,
   if (!(old & bit)) tlist[atomicAdd(nt, 1)] = (uint16_t)t;
 }
 
+// H P H^T of component c
 template <int DZ>
-__device__ __forceinline__ void slot_HPH(const float* s_hph, int T, int t, float (&HPH)[DZ][DZ]) {
-  int k = 0;
+__device__ __forceinline__ void slot_HPH(const CompTable& ct, int dx, uint32_t c, float (&HPH)[DZ][DZ]) {
 #pragma unroll
   for (int x = 0; x < DZ; ++x)
 #pragma unroll
-    for (int y = x; y < DZ; ++y, ++k) {
-      const float v = s_hph[k * T + t];
+    for (int y = x; y < DZ; ++y) {
+      const float v = ct.cov[(size_t)pidx(dx, x, y) * ct.cap + c];
       HPH[x][y] = v;
       HPH[y][x] = v;
     }
@@ -266,14 +263,14 @@ struct SeVec {
 };
 
 template <int DZ>
-__device__ __noinline__ TermOut slot_term_full(const Model& md, const float* s_hph, const float* s_logp, int T,
-                                               int t, int m, const SeVec<DZ> se, long long sq) {
+__device__ __noinline__ TermOut slot_term_full(const Model& md, const CompTable& ct, uint32_t c, int m,
+                                               const SeVec<DZ> se, long long sq) {
   // the sums come and the result goes by value, so a caller keeps them in
   // registers (an array passed by reference would live in local memory)
   float HPH[DZ][DZ];
-  slot_HPH<DZ>(s_hph, T, t, HPH);
+  slot_HPH<DZ>(ct, md.dx, c, HPH);
   TermOut o;
-  o.term = alive_term<DZ>(md, HPH, s_logp[t], m, se.v, sq, o.ninf);
+  o.term = alive_term<DZ>(md, HPH, ct.logp[c], m, se.v, sq, o.ninf);
   return o;
 }
 
@@ -286,11 +283,10 @@ struct View {
   const unsigned long long* hwref;
   const RowChunk* rch;
   const uint4* dth;
-  const uint32_t *rowrk, *rowthr0, *comp, *dthr, *refnew, *dpc, *cthr;
-  const float *roww0, *logp, *log1mp, *hph, *cw, *ce, *cq;
-  const float* cslm;      // per-component m-only term parts (PairTable::slm)
-  const int8_t* csln;
-  int slm_cap;
+  const uint32_t *rowrk, *rowthr0, *comp, *dthr, *refnew, *dpc, *cthr, *ceidx;
+  const float *roww0, *cw;
+  const PairTable* pt;    // the pairs, and the per-component m-only term parts (slm)
+  const CompTable* ct;
   const int* mref;
   const uint16_t* cslot;
   const uint8_t* ninfref;
@@ -298,7 +294,7 @@ struct View {
   const uint8_t* srow;
 };
 
-__device__ __forceinline__ View make_view(const unsigned char* b, const Lay& L, const PairTable& pt) {
+__device__ __forceinline__ View make_view(const unsigned char* b, const Lay& L, const PairTable& pt, const CompTable& ct) {
   View v;
   v.sc = at<Scal>(b, L.scal);
   v.row = at<uint4>(b, L.row);
@@ -320,42 +316,42 @@ __device__ __forceinline__ View make_view(const unsigned char* b, const Lay& L, 
   v.dpc = at<uint32_t>(b, L.dpc);
   v.cthr = at<uint32_t>(b, L.cthr);
   v.roww0 = at<float>(b, L.roww0);
-  v.logp = at<float>(b, L.logp);
-  v.log1mp = at<float>(b, L.log1mp);
-  v.hph = at<float>(b, L.hph);
-  v.cslm = pt.slm;
-  v.csln = pt.sln;
-  v.slm_cap = pt.slm_cap;
+  v.ceidx = at<uint32_t>(b, L.ceidx);
+  v.pt = &pt;
+  v.ct = &ct;
   v.cw = at<float>(b, L.cw);
-  v.ce = at<float>(b, L.ce);
-  v.cq = at<float>(b, L.cq);
   v.mref = at<int>(b, L.mref);
   v.cslot = at<uint16_t>(b, L.cslot);
   v.ninfref = at<uint8_t>(b, L.ninfref);
   return v;
 }
 
-// a view for code that evaluates no track term (no per-component table)
-__device__ __forceinline__ View make_view(const unsigned char* b, const Lay& L) {
-  PairTable none{};
-  return make_view(b, L, none);
+// A candidate pair's innovation and e^T R^-1 e (the factorised mode sums log C
+// instead), in fixed point, from the table: few children need one, so the
+// images do not repeat them.
+template <int DZ>
+__device__ __forceinline__ void pair_sums(const Model& md, const View& v, uint32_t pos, long long (&e)[DZ],
+                                          long long& q) {
+  const uint32_t j = v.ceidx[pos];
+#pragma unroll
+  for (int d = 0; d < DZ; ++d) e[d] = fx_of(v.pt->e[(size_t)d * v.pt->cap_pairs + j]);
+  q = fx_of(md.score_mode == 1 ? v.pt->logC[j] : v.pt->q[j]);
 }
 
 // Term of slot t alive with m detections whose sums are (se, sq): the m-only
 // parts from the per-component table when it holds (component, m), else
 // built from H P H^T (the same function, so the same values).
 template <int DZ>
-__device__ __forceinline__ long long slot_term(const Model& md, const View& v, int T, int t, int m,
+__device__ __forceinline__ long long slot_term(const Model& md, const View& v, int t, int m,
                                                const long long (&se)[DZ], long long sq, int& ninf) {
-  if (md.score_mode == 1) return factor_term(md, v.logp[t], m, sq, ninf);
-  if (m >= 1 && m <= kSlmM) {
-    const uint32_t c = v.comp[t];
-    if (c < (uint32_t)v.slm_cap) return term_from<DZ>(md, load_cslm<DZ>(v.cslm, v.csln, v.slm_cap, m, c), m, se, sq, ninf);
-  }
+  const uint32_t c = v.comp[t];
+  if (md.score_mode == 1) return factor_term(md, v.ct->logp[c], m, sq, ninf);
+  if (m >= 1 && m <= kSlmM && c < (uint32_t)v.pt->slm_cap)
+    return term_from<DZ>(md, load_cslm<DZ>(v.pt->slm, v.pt->sln, v.pt->slm_cap, m, c), m, se, sq, ninf);
   SeVec<DZ> sv;
 #pragma unroll
   for (int d = 0; d < DZ; ++d) sv.v[d] = se[d];
-  const TermOut o = slot_term_full<DZ>(md, v.hph, v.logp, T, t, m, sv, sq);
+  const TermOut o = slot_term_full<DZ>(md, *v.ct, c, m, sv, sq);
   ninf = o.ninf;
   return o.term;
 }
@@ -447,20 +443,14 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   // death thresholds: written to the image, read back on chip
   uint32_t* g_dthr = at<uint32_t>(sm, L.dthr);
   uint32_t* s_dthr = in_tail ? at<uint32_t>(tb, TS.dthr) : g_dthr;
-  float* s_logp = at<float>(sm, L.logp);
-  float* s_log1mp = at<float>(sm, L.log1mp);
   int* s_mref = in_tail ? at<int>(tb, TS.mref) : at<int>(sm, L.mref);
-  float* s_hph = at<float>(sm, L.hph);
   uint32_t* s_dpc = at<uint32_t>(sm, L.dpc);
   uint4* s_dth = at<uint4>(sm, L.dth);
   uint32_t* s_cthr = at<uint32_t>(sm, L.cthr);
   uint32_t* s_ceidx = in_tail ? at<uint32_t>(tb, TS.ceidx) : at<uint32_t>(sm, L.ceidx);
   float* s_cw = at<float>(sm, L.cw);
-  float* s_ce = at<float>(sm, L.ce);
-  float* s_cq = at<float>(sm, L.cq);
   uint16_t* s_cslot = in_tail ? at<uint16_t>(tb, TS.cslot) : at<uint16_t>(sm, L.cslot);
   uint8_t* s_ninfref = in_tail ? at<uint8_t>(tb, TS.ninfref) : at<uint8_t>(sm, L.ninfref);
-  const int Kp = a.K_max;                   // stride of the candidate arrays
   const CompTable& ct = a.ct;
   const PairTable& pt = a.pt;
   const size_t capp = (size_t)pt.cap_pairs;
@@ -527,20 +517,9 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   for (int t = tid; t < T; t += nthr) {
     const uint32_t c = t < Town ? a.parents.comp[plo + t] : (uint32_t)(birth_base + (t - Town));
     s_comp[t] = c;
-    {
-      int k = 0;
-#pragma unroll
-      for (int x = 0; x < DZ; ++x)
-#pragma unroll
-        for (int y = x; y < DZ; ++y, ++k) s_hph[k * T + t] = ct.cov[(size_t)pidx(md.dx, x, y) * ct.cap + c];
-    }
-    {
-      const uint32_t dt = pt.dthr[c];
-      s_dthr[t] = dt;
-      if (in_tail) g_dthr[t] = dt;
-    }
-    s_logp[t] = ct.logp[c];
-    s_log1mp[t] = ct.log1mp[c];
+    const uint32_t dt = pt.dthr[c];
+    s_dthr[t] = dt;
+    if (in_tail) g_dthr[t] = dt;
     s_mref[t] = 0;
 #pragma unroll
     for (int d = 0; d < DZ; ++d) s_seref[d * T + t] = 0;
@@ -552,7 +531,14 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   for (int t = tid; t < T; t += nthr) {
     const uint32_t c = s_comp[t];
     const uint32_t n = pt.cnt[c], j0 = pt.ptr[c];
-    for (uint32_t j = j0; j < j0 + n; ++j) atomicAdd(&s_rowfill[pt.meas[j]], 1u);
+    for (uint32_t x = 0; x < n; x += 4) {   // four reads in flight
+      uint32_t i4[4];
+#pragma unroll
+      for (uint32_t y = 0; y < 4; ++y) i4[y] = x + y < n ? pt.meas[j0 + x + y] : 0u;
+#pragma unroll
+      for (uint32_t y = 0; y < 4; ++y)
+        if (x + y < n) atomicAdd(&s_rowfill[i4[y]], 1u);
+    }
     s_srow[t] = (n && s_dthr[t] > 0u) ? 1 : 0;
   }
   __syncthreads();
@@ -597,11 +583,18 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
   if (s_wsum[7]) return;
   for (int t = tid; t < T; t += nthr) {
     const uint32_t c = s_comp[t];
-    for (uint32_t j = pt.ptr[c], je = j + pt.cnt[c]; j < je; ++j) {
-      const uint32_t i = pt.meas[j];
-      const uint32_t pos = atomicAdd(&s_rowfill[i], 1u);
-      s_cslot[pos] = (uint16_t)t;
-      s_ceidx[pos] = j;
+    const uint32_t n = pt.cnt[c], j0 = pt.ptr[c];
+    for (uint32_t x = 0; x < n; x += 4) {
+      uint32_t i4[4];
+#pragma unroll
+      for (uint32_t y = 0; y < 4; ++y) i4[y] = x + y < n ? pt.meas[j0 + x + y] : 0u;
+#pragma unroll
+      for (uint32_t y = 0; y < 4; ++y)
+        if (x + y < n) {
+          const uint32_t pos = atomicAdd(&s_rowfill[i4[y]], 1u);
+          s_cslot[pos] = (uint16_t)t;
+          s_ceidx[pos] = j0 + x + y;
+        }
     }
   }
   __syncthreads();
@@ -683,16 +676,16 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
             }
         float lc[kRowReg];
         float smax = md.kappa_zero ? -INFINITY : md.log_kappa;
+        // (reads before the writes, which might otherwise be the same memory
+        // to the compiler and hold each read back for the write before it)
+#pragma unroll
+        for (int x = 0; x < kRowReg; ++x) lc[x] = x < nc ? pt.logC[ce[x]] : 0.f;
 #pragma unroll
         for (int x = 0; x < kRowReg; ++x) {
           if (x >= nc) break;
           s_cslot[off + x] = (uint16_t)cs[x];
           s_ceidx[off + x] = ce[x];
-          lc[x] = pt.logC[ce[x]];
           smax = fmaxf(smax, lc[x]);
-#pragma unroll
-          for (int d = 0; d < DZ; ++d) s_ce[d * Kp + off + x] = pt.e[d * capp + ce[x]];
-          s_cq[off + x] = md.score_mode == 1 ? lc[x] : pt.q[ce[x]];
         }
         const float w0 = md.kappa_zero ? 0.f : expf(md.log_kappa - smax);
         float wv[kRowReg];
@@ -733,7 +726,7 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
           prev = th;
           flag |= can_die;
         }
-        // the reference pair's innovation and q, read again (L1)
+        // the reference pair's innovation and q
         FVec<DZ> e_ref;
         float q_ref = 0.f;
 #pragma unroll
@@ -758,10 +751,6 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
       for (int j = 0; j < nc; ++j) {
         const uint32_t ei = s_ceidx[off + j];
         smax = fmaxf(smax, pt.logC[ei]);
-#pragma unroll
-        for (int d = 0; d < DZ; ++d) s_ce[d * Kp + off + j] = pt.e[d * capp + ei];
-        // e^T R^-1 e of the pair; the factorised mode sums log C instead
-        s_cq[off + j] = md.score_mode == 1 ? pt.logC[ei] : pt.q[ei];
       }
       const float w0 = md.kappa_zero ? 0.f : expf(md.log_kappa - smax);
       float sum = w0;
@@ -794,9 +783,11 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
       if (ref > 0) {
         const uint32_t pos = off + ref - 1;
         r = s_cslot[pos];
+        const uint32_t ei = s_ceidx[pos];
 #pragma unroll
-        for (int d = 0; d < DZ; ++d) e_ref.v[d] = s_ce[d * Kp + pos];
-        q_ref = s_cq[pos];
+        for (int d = 0; d < DZ; ++d) e_ref.v[d] = pt.e[d * capp + ei];
+        // e^T R^-1 e of the pair; the factorised mode sums log C instead
+        q_ref = md.score_mode == 1 ? pt.logC[ei] : pt.q[ei];
       }
       finish_row(ref, flag, thr0, lo, hi, bl, w0, r, e_ref, q_ref);
     };
@@ -877,8 +868,8 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
                              ninf);
       } else {
         float HPH[DZ][DZ];
-        slot_HPH<DZ>(s_hph, T, t, HPH);
-        term = alive_term<DZ>(md, HPH, s_logp[t], mr, se, s_sqref[t], ninf);
+        slot_HPH<DZ>(ct, md.dx, s_comp[t], HPH);
+        term = alive_term<DZ>(md, HPH, ct.logp[s_comp[t]], mr, se, s_sqref[t], ninf);
       }
       s_termref[t] = term;
       s_ninfref[t] = (uint8_t)ninf;
@@ -897,7 +888,7 @@ __device__ void stage_parent(const ExpandArgs& a, const int h, const Lay& L, uns
     int8_t* s_dninf = at<int8_t>(sm, L.dninf);
     for (int t = tid; t < T; t += nthr) {
       int ninf;
-      const long long term = dead_term(s_log1mp[t], ninf);
+      const long long term = dead_term(ct.log1mp[s_comp[t]], ninf);
       s_deadd[t] = term - s_termref[t];
       s_dninf[t] = (int8_t)(ninf - (int)s_ninfref[t]);
     }
@@ -982,15 +973,15 @@ __global__ void __launch_bounds__(WIDE ? kStageWide : 256, WIDE ? 1 : 3) stage_k
 // option when its 24-bit uniform falls in the reference interval and none
 // of its candidates died -- nearly always -- so the common path reads one
 // 48-byte chunk record and tests four intervals per call, and holds only
-// the chunk loop's state in registers.  Everything else about a row is out
-// of line (slow_rows): a row with a candidate that may have died is drawn
-// among the living, and a row that leaves the reference adds the staged
-// change of a single deviation.  Whether a slot died is answered by its
+// the chunk loop's state in registers.  Everything else about a row is left
+// to finish_notes: a row with a candidate that may have died is drawn
+// among the living, and a row that leaves the reference adds the change of
+// a single deviation.  Whether a slot died is answered by its
 // bloom bit and, when that is set, by regenerating the slot's death draw,
 // so a thread keeps no lists.  The slots a child's deviations meet are
 // kept as a 64-bit mask (bit slot mod 64): when a bit is met again (a slot
 // met twice, or two slots sharing a bit), the slots met more than once are
-// rescored exactly after the rows (slow_rows).
+// rescored exactly after the rows.
 
 // Whether slot t of the child whose death stream is pd died.
 __device__ __forceinline__ bool slot_died(const uint32_t* __restrict__ dthr, const PhiloxRun& pd, uint2 key,
@@ -999,211 +990,7 @@ __device__ __forceinline__ bool slot_died(const uint32_t* __restrict__ dthr, con
   return (word_of(r, (int)(t & 3u)) >> 8) < dthr[t];
 }
 
-// The rows a child's chunk loop noted, in one out-of-line call (the
-// parent's layout, view and generators are built once per child): each
-// row's uniform is regenerated; a row whose candidates' bloom meets the
-// child's dead slots is drawn among the living candidates in proportion to
-// their weights (clutter first), in the FP32 arithmetic of the warp kernel;
-// otherwise its option is the first whose cumulative threshold exceeds the
-// uniform.  A row that leaves its reference option adds the staged changes
-// of the slots it leaves and joins (a dead reference slot is not met: its
-// change is the death's).  When the deviations meet a slot more than once,
-// that slot's change is not the sum of the single changes but the exact
-// rescoring of the slot with every detection that joins and leaves it: the
-// slots met more than once are rescored with the warp kernel's functions
-// and inputs, so the keys are bit-identical.
-struct SlowSum {
-  long long d;
-  unsigned long long hw;
-  int ninf, clut, bad;
-};
-
-// The score change of one deviation, alone: candidate pair `pos` joining
-// (sg = 1) or leaving (sg = -1) slot t, from the slot's reference sums (the
-// same function and inputs as an exact rescoring of the slot, so the sums
-// are bit-identical); term = the change, ninf = the infinite-term count's.
-template <int DZ>
-__device__ __noinline__ TermOut single_deviation(const Model* md, const View* vp, int T, int Kp, int t, uint32_t pos,
-                                                 int sg) {
-  const View& v = *vp;
-  long long se[DZ];
-#pragma unroll
-  for (int d = 0; d < DZ; ++d) se[d] = v.seref[d * T + t] + (long long)sg * fx_of(v.ce[d * Kp + pos]);
-  int ninf;
-  const long long term =
-      slot_term<DZ>(*md, v, T, t, v.mref[t] + sg, se, v.sqref[t] + (long long)sg * fx_of(v.cq[pos]), ninf);
-  TermOut o;
-  o.term = term - v.termref[t];
-  o.ninf = ninf - (int)v.ninfref[t];
-  return o;
-}
-
-template <int DZ>
-__device__ __noinline__ SlowSum slow_rows(const Model* md, const PairTable* pt, const unsigned char* img,
-                                          const int Tp, const int Kp, const int Mp, const uint16_t* rows,
-                                          const int nslow, const unsigned long long bloom, const uint32_t n,
-                                          const uint2 key) {
-  constexpr int kE = 2 * 24;
-  const Lay L = make_lay(DZ, Tp, Kp, Mp);
-  const View v = make_view(img, L, *pt);
-  const Scal& sc = *v.sc;
-  const int T = sc.T;
-  const uint32_t uid_lo = (uint32_t)sc.uid, uid_hi = (uint32_t)(sc.uid >> 32);
-  const PhiloxRun pd = philox_run(uid_lo, uid_hi, 2u * n, key);
-  const PhiloxRun pr = philox_run(uid_lo, uid_hi, 2u * n + 1u, key);
-  SlowSum o{0, 0ull, 0, 0, 0};
-  uint16_t ep_slot[kE];
-  uint32_t ep_pos[kE];
-  int8_t ep_sg[kE], ep_dn[kE];
-  long long ep_d[kE];
-  int ne = 0;
-  auto single_dev = [&](int t, uint32_t pos, int sg, long long& d, int& dn) {
-    const TermOut r = single_deviation<DZ>(md, &v, T, Kp, t, pos, sg);
-    d = r.term;
-    dn = r.ninf;
-  };
-  unsigned long long metm = 0ull;
-  bool twice = false;
-  for (int q = 0; q < nslow; ++q) {
-    const int i = rows[q];
-    const uint4 rr = philox_at_rk(pr, (uint32_t)i >> 2, key);
-    const uint32_t k = word_of(rr, i & 3) >> 8;
-    const uint4 R = v.row[i];
-    const uint32_t off = R.x;
-    const int nc = (int)(R.y & 0x7FFFu);
-    const int ref = (int)(R.y >> 16);
-    int opt = -1;
-    if (v.rowbl[i] & bloom) {
-      auto is_dead = [&](int j) -> bool {
-        const uint32_t t = v.cslot[off + j];
-        return ((bloom >> (t & 63u)) & 1ull) && slot_died(v.dthr, pd, key, t);
-      };
-      uint32_t dm = 0u;
-      bool any = false;
-      for (int j = 0; j < nc; ++j)
-        if (is_dead(j)) {
-          any = true;
-          if (j < 32) dm |= 1u << j;
-        }
-      if (any) {
-        auto dead_j = [&](int j) -> bool { return j < 32 ? ((dm >> j) & 1u) != 0u : is_dead(j); };
-        const float w0 = md->kappa_zero ? 0.f : v.roww0[i];
-        float sum = w0;
-        for (int j = 0; j < nc; ++j)
-          if (!dead_j(j)) sum += v.cw[off + j];
-        if (!(sum > 0.f)) {
-          o.bad = 1;
-          opt = 0;
-        } else {
-          const float xk = (float)k * 5.9604644775390625e-8f * sum;
-          float cum = w0;
-          int last = w0 > 0.f ? 0 : -1;
-          if (w0 > 0.f && xk < cum) opt = 0;
-          for (int j = 0; j < nc; ++j) {
-            if (dead_j(j)) continue;
-            const float w = v.cw[off + j];
-            if (!(w > 0.f)) continue;
-            cum += w;
-            last = j + 1;
-            if (opt < 0 && xk < cum) opt = j + 1;
-          }
-          if (opt < 0) opt = last < 0 ? 0 : last;
-        }
-      }
-    }
-    if (opt < 0) {
-      if (k - R.z < R.w - R.z) continue;   // the reference option
-      if (k < v.rowthr0[i]) {
-        opt = 0;
-      } else {
-        int j = 0;
-        while (j < nc - 1 && k >= v.cthr[off + j]) ++j;
-        opt = j + 1;
-      }
-    }
-    if (opt == ref) continue;
-    uint32_t rs1 = ref > 0 ? (uint32_t)v.cslot[off + ref - 1] + 1u : 0u;
-    const uint32_t ns1 = opt > 0 ? (uint32_t)v.cslot[off + opt - 1] + 1u : 0u;
-    o.hw += row_key(i, (int)ns1) - row_key(i, (int)rs1);
-    o.clut += (opt == 0) - (ref == 0);
-    if (rs1 && ((bloom >> ((rs1 - 1u) & 63u)) & 1ull) && slot_died(v.dthr, pd, key, rs1 - 1u)) rs1 = 0u;
-    unsigned long long m1 = 0ull, m2 = 0ull;
-    if (rs1) {
-      long long d;
-      int dn;
-      single_dev((int)rs1 - 1, off + (uint32_t)ref - 1u, -1, d, dn);
-      o.d += d;
-      o.ninf += dn;
-      m1 = 1ull << ((rs1 - 1u) & 63u);
-      if (ne < kE) {
-        ep_slot[ne] = (uint16_t)rs1;
-        ep_sg[ne] = -1;
-        ep_pos[ne] = off + (uint32_t)ref - 1u;
-        ep_d[ne] = d;
-        ep_dn[ne] = (int8_t)dn;
-        ++ne;
-      }
-    }
-    if (ns1) {
-      long long d;
-      int dn;
-      single_dev((int)ns1 - 1, off + (uint32_t)opt - 1u, 1, d, dn);
-      o.d += d;
-      o.ninf += dn;
-      m2 = 1ull << ((ns1 - 1u) & 63u);
-      if (ne < kE) {
-        ep_slot[ne] = (uint16_t)ns1;
-        ep_sg[ne] = 1;
-        ep_pos[ne] = off + (uint32_t)opt - 1u;
-        ep_d[ne] = d;
-        ep_dn[ne] = (int8_t)dn;
-        ++ne;
-      }
-    }
-    twice |= (metm & (m1 | m2)) || (m1 & m2);
-    metm |= m1 | m2;
-  }
-  if (!twice) return o;
-  // slots met more than once: exact term minus reference term minus the
-  // single changes added above
-  for (int w = 0; w < ne; ++w) {
-    const uint16_t sp = ep_slot[w];
-    int cnt = 0;
-    bool first = true;
-    for (int w2 = 0; w2 < ne; ++w2)
-      if (ep_slot[w2] == sp) {
-        ++cnt;
-        if (w2 < w) first = false;
-      }
-    if (cnt < 2 || !first) continue;
-    int dcnt = 0, sninf = 0;
-    long long dse[DZ], dsq = 0, single = 0;
-#pragma unroll
-    for (int d = 0; d < DZ; ++d) dse[d] = 0;
-    for (int w2 = w; w2 < ne; ++w2) {
-      if (ep_slot[w2] != sp) continue;
-      const uint32_t pos = ep_pos[w2];
-      const int sg = ep_sg[w2];
-      single += ep_d[w2];
-      sninf += ep_dn[w2];
-      dcnt += sg;
-#pragma unroll
-      for (int d = 0; d < DZ; ++d) dse[d] += sg * fx_of(v.ce[d * Kp + pos]);
-      dsq += sg * fx_of(v.cq[pos]);
-    }
-    const int t = (int)sp - 1;
-    long long se[DZ];
-#pragma unroll
-    for (int d = 0; d < DZ; ++d) se[d] = v.seref[d * T + t] + dse[d];
-    int ninf;
-    const long long term = slot_term<DZ>(*md, v, T, t, v.mref[t] + dcnt, se, v.sqref[t] + dsq, ninf);
-    o.d += term - v.termref[t] - single;
-    o.ninf += ninf - (int)v.ninfref[t] - sninf;
-  }
-  return o;
-}
-
-// Rows a child's chunk loop sets aside for slow_rows (per-thread list in
+// Rows a child's chunk loop sets aside for finish_notes (per-thread list in
 // shared memory, entry q at [q * blockDim.x]); a child with more goes to
 // the warp kernel.
 constexpr int kDrawSlow = 24;
@@ -1252,7 +1039,7 @@ struct Int {
 // chunk loops only test the thresholds and intervals and note the slots that
 // die and the rows that need more (their uniform is regenerated afterwards),
 // so they hold nothing but their own state in registers.  Slots its
-// deviations meet more than once are rescored exactly (slow_rows).  A child
+// deviations meet more than once are rescored exactly (finish_notes).  A child
 // with more noted rows than the list holds is left to the warp kernel (the
 // redo list).
 template <int DZ>
@@ -1403,27 +1190,207 @@ __device__ __forceinline__ void thread_child(const ExpandArgs& a, const unsigned
   a.child_status[j] = ninf == 0 ? 1 : 0;
 }
 
-// The noted children, one thread each.  In the draw kernel itself the few
-// lanes with noted rows would hold their warps through slow_rows' chains of
-// dependent loads; here the lanes are dense.
+// The noted children, kNoteLanes lanes each, a row to a lane at a time.  In
+// the draw kernel itself the few lanes with noted rows would hold their warps
+// through the rows' chains of dependent loads (row, candidate, pair, slot,
+// term); here the lanes are dense and a child's chains run side by side
+// (the launch with a lane per child and its images' own copies of the pairs:
+// 25 us at 3-D N = 50, 51 at N = 200; now 14.6 and about 20).
+// Each row's uniform is regenerated; a row whose candidates' bloom meets the
+// child's dead slots is drawn among the living candidates in proportion to
+// their weights (clutter first), in the FP32 arithmetic of the warp kernel;
+// otherwise its option is the first whose cumulative threshold exceeds the
+// uniform.  A row that leaves its reference option adds the changes of the
+// slots it leaves and joins, each scored alone (a dead reference slot is not
+// met: its change is the death's).  When the deviations meet a slot more than
+// once, that slot's change is not the sum of the single changes but the exact
+// rescoring of the slot with every detection that joins and leaves it: such
+// slots are rescored with the warp kernel's functions and inputs, so the keys
+// are bit-identical.
+constexpr int kNoteLanes = 8, kNoteEnt = 2 * (kDrawSlow / kNoteLanes);
+static_assert(kDrawSlow % kNoteLanes == 0, "rows of a note over its lanes");
+
 template <int DZ>
 __device__ __noinline__ void finish_notes(const ExpandArgs& a, const Lay& L, const uint2 key) {
   const Model& md = a.md;
-  const uint32_t count = *a.note_count;
-  for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
+  const uint32_t count = *a.note_count, HU = (uint32_t)md.h_up;
+  const int lane = (int)threadIdx.x & 31, gl = lane & (kNoteLanes - 1);
+  const unsigned gm = ((1u << kNoteLanes) - 1u) << (lane - gl);
+  const uint32_t step = gridDim.x * blockDim.x / kNoteLanes;
+  for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) / kNoteLanes; k < count; k += step) {
     const DrawNote* o = reinterpret_cast<const DrawNote*>(a.notes) + k;
-    const uint32_t j = o->child, h = j / (uint32_t)md.h_up;
-    const unsigned char* img = a.img + (size_t)h * a.img_stride;
-    const Scal& sc = *at<Scal>(img, L.scal);
-    const SlowSum d = slow_rows<DZ>(&md, &a.pt, img, a.T_max, a.K_max, a.M_plan, o->rows, o->n_rows, o->bloom,
-                                    j - h * (uint32_t)md.h_up, key);
-    const long long score =
-        sc.ref_score + a.child_key[j] + d.d + (md.kappa_zero ? 0LL : (long long)d.clut * md.fx_log_kappa);
-    const int ninf = sc.ninf_ref + o->dninf + d.ninf + (md.kappa_zero ? d.clut : 0);
-    const bool valid = !d.bad && ninf == 0;
-    a.child_key[j] = valid ? score : kKeyInvalid;
-    a.child_hash[j] += d.hw;
-    a.child_status[j] = valid ? 1 : 0;
+    const uint32_t j = o->child, h = j / HU, n = j - h * HU;
+    const int n_rows = o->n_rows;
+    const unsigned long long bloom = o->bloom;
+    const View v = make_view(a.img + (size_t)h * a.img_stride, L, a.pt, a.ct);
+    const Scal& sc = *v.sc;
+    const int T = sc.T;
+    const PhiloxRun pd = philox_run((uint32_t)sc.uid, (uint32_t)(sc.uid >> 32), 2u * n, key);
+    const PhiloxRun pr = philox_run((uint32_t)sc.uid, (uint32_t)(sc.uid >> 32), 2u * n + 1u, key);
+    long long dsum = 0;
+    unsigned long long hw = 0ull, metm = 0ull;
+    int ninf = 0, clut = 0, ne = 0;
+    unsigned flags = 0u;   // 1: a row without a weight, 2: a slot met twice
+    // this lane's single deviations: slot + 1, leaving << 16, (infinite-term
+    // change + 128) << 17; the pair; the score change
+    uint32_t e_tag[kNoteEnt], e_pos[kNoteEnt];
+    long long e_d[kNoteEnt];
+    auto deviation = [&](uint32_t s1, uint32_t pos, int sg) {   // alone: joining (1) or leaving (-1) slot s1 - 1
+      const int t = (int)s1 - 1;
+      long long e[DZ], q, se[DZ];
+      pair_sums<DZ>(md, v, pos, e, q);
+#pragma unroll
+      for (int d = 0; d < DZ; ++d) se[d] = v.seref[d * T + t] + (long long)sg * e[d];
+      int ni;
+      const long long term = slot_term<DZ>(md, v, t, v.mref[t] + sg, se, v.sqref[t] + (long long)sg * q, ni);
+      const long long d = term - v.termref[t];
+      const int dn = ni - (int)v.ninfref[t];
+      dsum += d;
+      ninf += dn;
+      const unsigned long long m = 1ull << ((uint32_t)t & 63u);
+      if (metm & m) flags |= 2u;
+      metm |= m;
+      e_tag[ne] = s1 | (sg < 0 ? 1u << 16 : 0u) | ((uint32_t)(dn + 128) << 17);
+      e_pos[ne] = pos;
+      e_d[ne] = d;
+      ++ne;
+    };
+    for (int r = gl; r < n_rows; r += kNoteLanes) {
+      const int i = o->rows[r];
+      const uint4 rr = philox_at_rk(pr, (uint32_t)i >> 2, key);
+      const uint32_t u = word_of(rr, i & 3) >> 8;
+      const uint4 R = v.row[i];
+      const uint32_t off = R.x;
+      const int nc = (int)(R.y & 0x7FFFu);
+      const int ref = (int)(R.y >> 16);
+      int opt = -1;
+      if (v.rowbl[i] & bloom) {
+        auto is_dead = [&](int x) -> bool {
+          const uint32_t t = v.cslot[off + x];
+          return ((bloom >> (t & 63u)) & 1ull) && slot_died(v.dthr, pd, key, t);
+        };
+        uint32_t dm = 0u;
+        bool any = false;
+        for (int x = 0; x < nc; ++x)
+          if (is_dead(x)) {
+            any = true;
+            if (x < 32) dm |= 1u << x;
+          }
+        if (any) {
+          auto dead_x = [&](int x) -> bool { return x < 32 ? ((dm >> x) & 1u) != 0u : is_dead(x); };
+          const float w0 = md.kappa_zero ? 0.f : v.roww0[i];
+          float sum = w0;
+          for (int x = 0; x < nc; ++x)
+            if (!dead_x(x)) sum += v.cw[off + x];
+          if (!(sum > 0.f)) {
+            flags |= 1u;
+            opt = 0;
+          } else {
+            const float xk = (float)u * 5.9604644775390625e-8f * sum;
+            float cum = w0;
+            int last = w0 > 0.f ? 0 : -1;
+            if (w0 > 0.f && xk < cum) opt = 0;
+            for (int x = 0; x < nc; ++x) {
+              if (dead_x(x)) continue;
+              const float w = v.cw[off + x];
+              if (!(w > 0.f)) continue;
+              cum += w;
+              last = x + 1;
+              if (opt < 0 && xk < cum) opt = x + 1;
+            }
+            if (opt < 0) opt = last < 0 ? 0 : last;
+          }
+        }
+      }
+      if (opt < 0) {
+        if (u - R.z < R.w - R.z) continue;   // the reference option
+        if (u < v.rowthr0[i]) {
+          opt = 0;
+        } else {
+          int x = 0;
+          while (x < nc - 1 && u >= v.cthr[off + x]) ++x;
+          opt = x + 1;
+        }
+      }
+      if (opt == ref) continue;
+      uint32_t rs1 = ref > 0 ? (uint32_t)v.cslot[off + ref - 1] + 1u : 0u;
+      const uint32_t ns1 = opt > 0 ? (uint32_t)v.cslot[off + opt - 1] + 1u : 0u;
+      hw += row_key(i, (int)ns1) - row_key(i, (int)rs1);
+      clut += (opt == 0) - (ref == 0);
+      if (rs1 && ((bloom >> ((rs1 - 1u) & 63u)) & 1ull) && slot_died(v.dthr, pd, key, rs1 - 1u)) rs1 = 0u;
+      if (rs1) deviation(rs1, off + (uint32_t)ref - 1u, -1);
+      if (ns1) deviation(ns1, off + (uint32_t)opt - 1u, 1);
+    }
+    __syncwarp(gm);
+    // two lanes that met the same slot (or slots that share a bit)
+#pragma unroll
+    for (int x = 1; x < kNoteLanes; x <<= 1) {
+      const unsigned long long other = __shfl_xor_sync(gm, metm, x);
+      if (metm & other) flags |= 2u;
+      metm |= other;
+    }
+    flags = __reduce_or_sync(gm, flags);
+    if (flags & 2u) {
+      // slots met more than once, each by the lane of its first deviation:
+      // exact term minus reference term minus the single changes added above
+      const int most = (int)__reduce_max_sync(gm, (unsigned)ne);
+      for (int w = 0; w < most; ++w) {
+        const uint32_t mine = w < ne ? e_tag[w] & 0xFFFFu : 0u;
+        bool first = mine != 0u;
+        int cnt = 0, dcnt = 0, sninf = 0;
+        long long dse[DZ], dsq = 0, single = 0;
+#pragma unroll
+        for (int d = 0; d < DZ; ++d) dse[d] = 0;
+        for (int src = 0; src < kNoteLanes; ++src) {
+          const int from = lane - gl + src;
+          const int n_src = __shfl_sync(gm, ne, from);
+          for (int x = 0; x < n_src; ++x) {
+            const int y = min(x, kNoteEnt - 1);
+            const uint32_t tag = __shfl_sync(gm, e_tag[y], from), pos = __shfl_sync(gm, e_pos[y], from);
+            const long long d1 = __shfl_sync(gm, e_d[y], from);
+            if ((tag & 0xFFFFu) != mine) continue;
+            if (src < gl || (src == gl && x < w)) first = false;
+            if (!first) continue;
+            ++cnt;
+            const int sg = (tag >> 16) & 1u ? -1 : 1;
+            single += d1;
+            sninf += (int)(tag >> 17) - 128;
+            dcnt += sg;
+            long long e[DZ], q;
+            pair_sums<DZ>(md, v, pos, e, q);
+#pragma unroll
+            for (int d = 0; d < DZ; ++d) dse[d] += sg * e[d];
+            dsq += sg * q;
+          }
+        }
+        if (first && cnt >= 2) {
+          const int t = (int)mine - 1;
+          long long se[DZ];
+#pragma unroll
+          for (int d = 0; d < DZ; ++d) se[d] = v.seref[d * T + t] + dse[d];
+          int ni;
+          const long long term = slot_term<DZ>(md, v, t, v.mref[t] + dcnt, se, v.sqref[t] + dsq, ni);
+          dsum += term - v.termref[t] - single;
+          ninf += ni - (int)v.ninfref[t] - sninf;
+        }
+        __syncwarp(gm);
+      }
+    }
+#pragma unroll
+    for (int x = 1; x < kNoteLanes; x <<= 1) {
+      dsum += __shfl_xor_sync(gm, dsum, x);
+      hw += __shfl_xor_sync(gm, hw, x);
+      ninf += __shfl_xor_sync(gm, ninf, x);
+      clut += __shfl_xor_sync(gm, clut, x);
+    }
+    if (gl == 0) {
+      const long long score =
+          sc.ref_score + a.child_key[j] + dsum + (md.kappa_zero ? 0LL : (long long)clut * md.fx_log_kappa);
+      const bool valid = !(flags & 1u) && sc.ninf_ref + o->dninf + ninf + (md.kappa_zero ? clut : 0) == 0;
+      a.child_key[j] = valid ? score : kKeyInvalid;
+      a.child_hash[j] += hw;
+      a.child_status[j] = valid ? 1 : 0;
+    }
   }
 }
 
@@ -1512,7 +1479,7 @@ __global__ void __launch_bounds__(256, 3) draw_kernel(const __grid_constant__ Ex
 // The work area's sums, masks and touched list are zero on entry and are
 // left zero on return.
 template <int DZ, bool MAT, bool GRP>
-__device__ void warp_child(const ExpandArgs& a, const View& v, const int T, const int Kp, const int M,
+__device__ void warp_child(const ExpandArgs& a, const View& v, const int T, const int M,
                            const int h, const int n, const int s_out, const uint2 key, unsigned char* gb,
                            const WLay& WL, const int gsz_in, const int gid) {
   const int gsz = GRP ? gsz_in : 32;   // one warp: the group code folds away
@@ -1682,24 +1649,25 @@ __device__ void warp_child(const ExpandArgs& a, const View& v, const int T, cons
         int rs = -1;
         if (ref > 0) {
           rs = v.cslot[off + ref - 1];
-          const uint32_t pos = off + ref - 1;
+          long long e[DZ], q;
+          pair_sums<DZ>(md, v, off + ref - 1, e, q);
           atomicSub(&acc_cnt[rs], 1);
 #pragma unroll
           for (int d = 0; d < DZ; ++d)
-            atomicAdd((unsigned long long*)&acc_se[d * T + rs], (unsigned long long)(-fx_of(v.ce[d * Kp + pos])));
-          atomicAdd((unsigned long long*)&acc_sq[rs], (unsigned long long)(-fx_of(v.cq[pos])));
+            atomicAdd((unsigned long long*)&acc_se[d * T + rs], (unsigned long long)(-e[d]));
+          atomicAdd((unsigned long long*)&acc_sq[rs], (unsigned long long)(-q));
           if (MAT) atomicAdd(&acc_hw[rs], (unsigned long long)(0ULL - wset_key(i)));
           touch(tmask, tlist, ntp, rs);
         } else {
           --my_dclut;
         }
         if (opt > 0) {
-          const uint32_t pos = off + opt - 1;
+          long long e[DZ], q;
+          pair_sums<DZ>(md, v, off + opt - 1, e, q);
           atomicAdd(&acc_cnt[ns], 1);
 #pragma unroll
-          for (int d = 0; d < DZ; ++d)
-            atomicAdd((unsigned long long*)&acc_se[d * T + ns], (unsigned long long)fx_of(v.ce[d * Kp + pos]));
-          atomicAdd((unsigned long long*)&acc_sq[ns], (unsigned long long)fx_of(v.cq[pos]));
+          for (int d = 0; d < DZ; ++d) atomicAdd((unsigned long long*)&acc_se[d * T + ns], (unsigned long long)e[d]);
+          atomicAdd((unsigned long long*)&acc_sq[ns], (unsigned long long)q);
           if (MAT) atomicAdd(&acc_hw[ns], wset_key(i));
           touch(tmask, tlist, ntp, ns);
         } else {
@@ -1723,12 +1691,12 @@ __device__ void warp_child(const ExpandArgs& a, const View& v, const int T, cons
     int m = 0;
     const bool is_dead = bit_of(dmask, t);
     if (is_dead) {
-      term = dead_term(v.log1mp[t], ninf);
+      term = dead_term(v.ct->log1mp[v.comp[t]], ninf);
     } else {
       m = v.mref[t] + acc_cnt[t];
 #pragma unroll
       for (int d = 0; d < DZ; ++d) se[d] = v.seref[d * T + t] + acc_se[d * T + t];
-      term = slot_term<DZ>(md, v, T, t, m, se, v.sqref[t] + acc_sq[t], ninf);
+      term = slot_term<DZ>(md, v, t, m, se, v.sqref[t] + acc_sq[t], ninf);
     }
     my_delta += term - v.termref[t];
     my_dninf += ninf - (int)v.ninfref[t];
@@ -1860,9 +1828,9 @@ __global__ void __launch_bounds__(512) warp_kernel(const __grid_constant__ Expan
   for (long long c = (long long)blockIdx.x * groups + g; c < count; c += nw) {
     const long long ci = MAT ? a.surv_idx[c] : (a.warp_all ? c : (long long)a.redo_list[c]);
     const int h = (int)(ci / HU), n = (int)(ci % HU);
-    const View v = make_view(a.img + (size_t)h * a.img_stride, L, a.pt);
+    const View v = make_view(a.img + (size_t)h * a.img_stride, L, a.pt, a.ct);
     if (v.sc->bad) continue;
-    warp_child<DZ, MAT, GRP>(a, v, v.sc->T, a.K_max, M, h, n, (int)c, key, gb, WL, gsz, g);
+    warp_child<DZ, MAT, GRP>(a, v, v.sc->T, M, h, n, (int)c, key, gb, WL, gsz, g);
   }
 }
 

@@ -28,7 +28,7 @@ def test_staging_threads_do_not_change_the_children(glmb, preset, frames):  # no
     sc = scenes.make_scene(scenes.preset(preset), 22)
     fs = []
     for threads in (0, 32, 128):
-        f = glmb.Filter(sc.filter_config(h_max=min(2000, sc.filter_config()["h_max"])))
+        f = glmb.Filter(sc.filter_config(max_births=1016, max_tracks=3200, max_meas=4200))
         f.set_tuning(stage_threads=threads)
         fs.append(f)
     for k, fr in enumerate(sc.frames[:frames]):
