@@ -1,0 +1,244 @@
+// Exponential, logarithm, sine and cosine in 64-bit integer arithmetic, for
+// FP64 callers.  An SM issues an FP64 instruction every 16 cycles for a warp
+// and an integer one on each of its four schedulers every cycle or two, so
+// these cost a fraction of the FP64 library functions; each result is off by
+// no more than theirs (checked against 300-bit arithmetic: about half a unit
+// in the last place, beside the library's one).  The series are Taylor's, the
+// tables come from the series at compile time.
+#pragma once
+#include <stdint.h>
+
+#include <cmath>
+#include <cstring>
+
+#if defined(__CUDACC__)
+#define FX_FN __host__ __device__ __forceinline__
+#else
+#define FX_FN inline
+#endif
+
+namespace glmb {
+namespace fx {
+
+using u64 = unsigned long long;
+using u128 = unsigned __int128;
+
+FX_FN u64 mulhi(u64 a, u64 b) {
+#if defined(__CUDA_ARCH__)
+  return __umul64hi(a, b);
+#else
+  return (u64)(((u128)a * b) >> 64);
+#endif
+}
+FX_FN long long mulhi_s(long long a, long long b) {
+#if defined(__CUDA_ARCH__)
+  return __mul64hi(a, b);
+#else
+  return (long long)(((__int128)a * b) >> 64);
+#endif
+}
+FX_FN int clz(u64 v) {
+#if defined(__CUDA_ARCH__)
+  return __clzll((long long)v);
+#else
+  return v ? __builtin_clzll(v) : 64;
+#endif
+}
+FX_FN double from_bits(u64 b) {
+#if defined(__CUDA_ARCH__)
+  return __longlong_as_double((long long)b);
+#else
+  double d;
+  std::memcpy(&d, &b, 8);
+  return d;
+#endif
+}
+FX_FN u64 to_bits(double d) {
+#if defined(__CUDA_ARCH__)
+  return (u64)__double_as_longlong(d);
+#else
+  u64 b;
+  std::memcpy(&b, &d, 8);
+  return b;
+#endif
+}
+
+// v 2^e as a double, rounded to nearest (v > 0 with a normal result, or 0)
+FX_FN double to_double(u64 v, int e) {
+  if (v == 0ull) return 0.0;
+  const int lz = clz(v);
+  const u64 m = v << lz;
+  return from_bits(((u64)(1085 - lz + e) << 52) + (m >> 11) + ((m >> 10) & 1ull));
+}
+
+// ---- tables ----
+// 2^(-j/64) 2^63 and -ln(k_j / 1024) 2^59, k_j = round(1024 / (1 + (j + 1/2) / 128)),
+// from exp's and atanh's series with 100-bit fractions
+struct Tables {
+  u64 exp2[64];
+  u64 nlog[128];
+  uint16_t inv[128];
+  constexpr Tables() : exp2{}, nlog{}, inv{} {
+    constexpr u128 one = (u128)1 << 100;
+    constexpr u128 ln2 = ((u128)0xB17217F7Dull << 64) | 0x1CF79ABC9E3B3980ull;   // ln(2) 2^100
+    for (int j = 0; j < 64; ++j) {
+      const u128 x = (ln2 * (u128)j) >> 6;   // j ln(2) / 64
+      // exp(-x) by Horner's rule, 1 - x (1 - x/2 (1 - x/3 (...)))
+      u128 s = one;
+      for (int k = 34; k >= 1; --k) {
+        // x s / k with 100-bit fractions: the halves of s separately
+        const u128 sh = s >> 50, sl = s & (((u128)1 << 50) - 1);
+        const u128 xs = x >> 26;   // 74 fraction bits are left of x
+        s = one - (((xs * sh) >> 24) + ((xs * sl) >> 74)) / (u128)k;
+      }
+      exp2[j] = (u64)((s + ((u128)1 << 36)) >> 37);
+    }
+    for (int j = 0; j < 128; ++j) {
+      const int k = (1024 * 256 + (257 + 2 * j) / 2) / (257 + 2 * j);
+      inv[j] = (uint16_t)k;
+      // -ln(k / 1024) = 2 atanh(y), y = (1024 - k) / (1024 + k)
+      const u128 n = (u128)(1024 - k), d = (u128)(1024 + k);
+      u128 term = one * n / d, sum = 0;
+      for (int i = 1; term != 0 && i < 200; i += 2) {
+        sum += term / (u128)i;
+        term = term * n / d * n / d;
+      }
+      nlog[j] = (u64)((2 * sum + ((u128)1 << 40)) >> 41);
+    }
+  }
+};
+
+// ---- exp(-x), x >= 0 and not -0 (0 from 708 on; NaN for NaN) ----
+// x = n ln(2) / 64 + r: a table entry times the polynomial of exp(-r).
+FX_FN double exp_neg(double x, const u64* exp2) {
+  const u64 b = to_bits(x);
+  if (b >= 0x4086200000000000ull) return b > 0x7FF0000000000000ull ? x : 0.0;   // 708 and beyond; NaN
+  const int e = (int)(b >> 52) - 1075;                        // x = m 2^e (x >= 0)
+  const u64 m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  // X = x 2^53, rounded
+  const int sh = e + 53;
+  const u64 X = sh >= 0 ? m << sh : sh < -54 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh;
+  // n <= x 64 / ln 2, short of it by less than 2
+  const uint32_t n = (uint32_t)(((u64)(uint32_t)(X >> 32) * 0xB8AA3B29u) >> 46);
+  // r 2^64 (the integer part of x cancels modulo 2^64)
+  const u64 r = (X << 11) - (u64)n * 0x2C5C85FDF473DE6ull - (((u64)n * 0xAF278ECEull) >> 32);
+  // 1 - r (1 - r/2 (1 - r/3 (...))), the inner terms in 32 bits
+  const uint32_t rh = (uint32_t)(r >> 32);
+  uint32_t q = 35791394u - (uint32_t)(((u64)rh * 5965232u) >> 32);     // (1/120 - r/720) 2^32
+  q = 178956971u - (uint32_t)(((u64)rh * q) >> 32);
+  u64 p = 0x1555555555555555ull - mulhi(r, (u64)q << 31);              // (1/6 - ...) 2^63
+  p = 0x4000000000000000ull - mulhi(r, p);
+  p = 0x8000000000000000ull - mulhi(r, p);
+  p = 0x8000000000000000ull - mulhi(r, p);
+  const u64 t = mulhi(p, exp2[n & 63u]);                               // 2^62
+  return to_double(t, -62 - (int)(n >> 6));
+}
+
+// ---- -2 ln((2 w + 1) / 2^33) ----
+FX_FN double neg2_log_unit(uint32_t w, const u64* nlog, const uint16_t* inv) {
+  const u64 a = 2ull * w + 1ull;
+  const u64 dl = (1ull << 33) - a;
+  if (dl < (1ull << 26)) {
+    // near 1: d (1 + d/2 + d^2/3 + ...), d = dl 2^-33 < 2^-7
+    const u64 d = dl << 31;
+    u64 q = 0x071C71C71C71C71Cull;                                     // 1/9 2^62
+    q = 0x0800000000000000ull + mulhi(d, q);
+    q = 0x0924924924924925ull + mulhi(d, q);
+    q = 0x0AAAAAAAAAAAAAABull + mulhi(d, q);
+    q = 0x0CCCCCCCCCCCCCCDull + mulhi(d, q);
+    q = 0x1000000000000000ull + mulhi(d, q);
+    q = 0x1555555555555555ull + mulhi(d, q);
+    q = 0x2000000000000000ull + mulhi(d, q);
+    q = 0x4000000000000000ull + mulhi(d, q);
+    const int ln = clz(dl);
+    return to_double(mulhi(dl << ln, q), 3 - ln - 33);
+  }
+  const int lz = clz(a);
+  const u64 mm = (a << lz) >> 31;                                      // [1, 2) 2^32, exact
+  const int j = (int)(mm >> 25) & 127;
+  // r = m' k / 1024 - 1, |r| < 2^-7.6, exact; r 2^64
+  const long long r = (long long)((mm * inv[j] - (1ull << 42)) << 22);
+  long long p = 0x0924924924924925ll;                                  // 1/7 2^62
+  p = 0x0AAAAAAAAAAAAAABll - mulhi_s(r, p);
+  p = 0x0CCCCCCCCCCCCCCDll - mulhi_s(r, p);
+  p = 0x1000000000000000ll - mulhi_s(r, p);
+  p = 0x1555555555555555ll - mulhi_s(r, p);
+  p = 0x2000000000000000ll - mulhi_s(r, p);
+  p = 0x4000000000000000ll - mulhi_s(r, p);
+  const long long l1 = mulhi_s(r, p);                                  // ln(1 + r) 2^62
+  // E ln 2 + ln(k / 1024) - ln(1 + r), 2^59
+  const u64 E = (u64)(lz - 30);
+  const u64 L = E * 0x058B90BFBE8E7BCDull + ((E * 0x5E4F1D9Cull) >> 32) - nlog[j] - (u64)((l1 + 4) >> 3);
+  return to_double(L, -58);
+}
+
+// ---- sine and cosine of (octant + t / 2^64) / 8 of a turn, 0 <= t < 2^64 ----
+// both polynomials in q = (t / 2^64)^2, x = (pi / 4) t / 2^64
+FX_FN u64 cos_oct(u64 q) {                                             // cos x 2^63
+  u64 p = 0x13ull;
+  p = 0x2419ull - mulhi(q, p);
+  p = 0x36DC4Aull - mulhi(q, p);
+  p = 0x3F3A7147ull - mulhi(q, p);
+  p = 0x34DA3E5441ull - mulhi(q, p);
+  p = 0x1E1F506891BBull - mulhi(q, p);
+  p = 0xAAE9E3F1E5FFDull - mulhi(q, p);
+  p = 0x20783E1036B5876ull - mulhi(q, p);
+  p = 0x277A79937C8BBCB5ull - mulhi(q, p);
+  return 0x8000000000000000ull - mulhi(q, p);
+}
+FX_FN u64 sin_oct(u64 t, u64 q) {                                      // sin x 2^63
+  u64 p = 0x1ABull;
+  p = 0x2DF5Bull - mulhi(q, p);
+  p = 0x3D1E86Aull - mulhi(q, p);
+  p = 0x3C60E9FBDull - mulhi(q, p);
+  p = 0x2A0F0690FDDull - mulhi(q, p);
+  p = 0x132D2CCE62BD8ull - mulhi(q, p);
+  p = 0x519AF19DD6AB87ull - mulhi(q, p);
+  p = 0x0A55DE7312DF295Full - mulhi(q, p);
+  p = 0x6487ED5110B4611Aull - mulhi(q, p);
+  return mulhi(t, p);
+}
+
+// cos(2 pi (2 w + 1) / 2^33)
+FX_FN double cos_turn(uint32_t w) {
+  const u64 a = 2ull * w + 1ull;
+  const uint32_t oct = (uint32_t)(a >> 30);
+  uint32_t t30 = (uint32_t)a & 0x3FFFFFFFu;                            // odd
+  if (oct & 1u) t30 = 0x40000000u - t30;
+  const u64 q = ((u64)t30 * t30) << 4;
+  const bool use_sin = ((oct + 1u) & 2u) != 0u;                        // octants 1, 2, 5, 6
+  double v;
+  if (use_sin) {
+    // t30 times the polynomial, normalised: relative accuracy near 0 too
+    const int ln = clz(t30);
+    v = to_double(sin_oct((u64)t30 << ln, q), 64 - 63 - ln - 30);
+  } else {
+    v = to_double(cos_oct(q), -63);
+  }
+  return (oct >= 2u && oct < 6u) ? -v : v;
+}
+
+// sine and cosine of psi, |psi| < 2^30 (checked by the caller)
+FX_FN void sincos(double psi, double& s, double& c) {
+  const u64 b = to_bits(psi);
+  const int E = (int)((b >> 52) & 0x7FFull) - 1023;
+  const u64 M = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;   // |psi| = M 2^(E - 63)
+  // |psi| / (2 pi) modulo 1, as a 64-bit fraction
+  constexpr u64 Ih = 0x28BE60DB9391054Aull, Il = 0x7F09D5F47D4D3770ull;   // 2^-64, 2^-128 words of 1 / (2 pi)
+  const u64 hl = M * Ih, add = mulhi(M, Il);
+  const u64 p1 = hl + add, p2 = mulhi(M, Ih) + (p1 < hl ? 1ull : 0ull);
+  const int sh = E + 1;
+  const u64 f = sh >= 64 ? 0ull : sh > 0 ? (p2 << sh) | (p1 >> (64 - sh)) : sh > -64 ? p2 >> -sh : 0ull;
+  const uint32_t oct = (uint32_t)(f >> 61);
+  u64 t = f << 3;
+  if (oct & 1u) t = ~t;                                                   // 1 - t to 2^-64
+  const u64 q = mulhi(t, t);
+  const double vs = to_double(sin_oct(t, q), -63), vc = to_double(cos_oct(q), -63);
+  const bool swap = ((oct + 1u) & 2u) != 0u;
+  const double as = swap ? vc : vs, ac = swap ? vs : vc;
+  s = ((oct >= 4u) != ((b >> 63) != 0ull)) ? -as : as;
+  c = (oct >= 2u && oct < 6u) ? -ac : ac;
+}
+
+}  // namespace fx
+}  // namespace glmb

