@@ -970,7 +970,12 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
   const int st_thr = p.st_thr;
   a.stage_wide = st_thr > 256 ? 1 : 0;
   const int st_ctas = std::max(1, expand_occupancy(a, ExpandKernel::kStage, st_thr, st_smem));
-  const int st_grid = p.fixed ? st_ctas * n_sm : std::max(1, std::min(h->H, st_ctas * n_sm));
+  // grids: what the GPU holds at once, but no more CTAs than the work can fill
+  // (a graph's: the filter's caps; a CTA without work costs its launch, and
+  // room beside the graphs of other scenes)
+  const int hyp = p.fixed ? h->cap_h : std::max(1, h->H);
+  const long long kids = (long long)hyp * h_up;
+  const int st_grid = std::min(hyp, st_ctas * n_sm);
   // draws: one thread per child over the frame's children in order
   // (persistent grid)
   const int d_thr = h->tune.draw_threads > 0 ? h->tune.draw_threads : 256;
@@ -978,8 +983,8 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
   a.draw_staged = 2 * (expand_draw_smem(d_thr, h_up, p.T, p.M, true) + 1024) <= h->smem_per_sm ? 1 : 0;
   const int d_smem = expand_draw_smem(d_thr, h_up, p.T, p.M, a.draw_staged != 0);
   const int d_ctas = std::max(1, expand_occupancy(a, ExpandKernel::kDraw, d_thr, d_smem));
-  const long long d_need = ((long long)h->H * h_up + 63) / 64;   // (a CTA takes fewer than d_thr children when they are few)
-  const int d_grid = p.fixed ? d_ctas * n_sm : (int)std::max(1LL, std::min(d_need, (long long)d_ctas * n_sm));
+  // (a CTA takes fewer than d_thr children when they are few)
+  const int d_grid = (int)std::min((kids + 63) / 64, (long long)d_ctas * n_sm);
   // warp kernel: the overflow list, or every child
   int wg = p.wg;
   while (wg > 1 && p.Gw * wg > 16) wg >>= 1;   // a CTA holds at most 16 warps
@@ -987,10 +992,8 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
   const int w_smem = expand_warp_smem(dz, 0, p.T, p.Gw, wg > 1);
   a.warp_group = wg;
   const int w_ctas = std::max(1, expand_occupancy(a, ExpandKernel::kWarp, w_thr, w_smem));
-  int w_grid = w_ctas * n_sm;
-  if (p.thread) w_grid = std::min(w_ctas, 2) * n_sm;
-  else if (!p.fixed)
-    w_grid = (int)std::max(1LL, std::min(((long long)h->H * h_up + p.Gw - 1) / p.Gw, (long long)w_grid));
+  const int w_grid = p.thread ? std::min(w_ctas, 2) * n_sm
+                              : (int)std::min((kids + p.Gw - 1) / p.Gw, (long long)w_ctas * n_sm);
   h->exp_smem = p.thread ? img : w_smem;
   h->exp_ctas = p.thread ? d_ctas : w_ctas;
   h->exp_plan[0] = p.T;
@@ -1002,7 +1005,7 @@ glmb_status enqueue_expand(glmb_handle* h, const Plan& p, bool scal_zeroed = fal
   launch_expand_kernel(a, ExpandKernel::kStage, st_grid, st_thr, st_smem, s);
   if (p.thread) launch_expand_kernel(a, ExpandKernel::kDraw, d_grid, d_thr, d_smem, s);
   launch_expand_kernel(a, ExpandKernel::kWarp, w_grid, w_thr, w_smem, s);
-  h->lse_parts = std::min(kMaxLseParts, p.fixed ? 8 * n_sm : std::max(1, std::min(h->H, 8 * n_sm)));
+  h->lse_parts = std::min(kMaxLseParts, std::min(hyp, 8 * n_sm));
   launch_dedup(h->d_fs, h_up, h->child_key, h->child_hash, h->child_status, h->d_scal + S_ERR, h->pw,
                h->lse_parts, s);
   prof_end(h, kStageExpand);
@@ -1058,8 +1061,7 @@ glmb_status enqueue_prune(glmb_handle* h, const Plan& p) {
   const int m_smem = expand_warp_smem(h->md.dz, 1, p.T, p.Gm, mg > 1);
   a.warp_group = mg;
   const int m_ctas = std::max(1, expand_occupancy(a, ExpandKernel::kWarp, m_thr, m_smem));
-  const int m_grid = p.fixed ? m_ctas * h->n_sm
-                             : std::max(1, std::min((h->cap_h + p.Gm - 1) / p.Gm, m_ctas * h->n_sm));
+  const int m_grid = std::max(1, std::min((h->cap_h + p.Gm - 1) / p.Gm, m_ctas * h->n_sm));
   prof_begin(h, kStageMat);
   // a warp per 32 slots of each survivor, up to two CTAs per SM
   const long long prep_warps = (long long)h->cap_h * ((p.T + 31) / 32);

@@ -656,9 +656,10 @@ __global__ void __launch_bounds__(256, DZ == 2 ? 3 : 2) gc_remap_kernel(Model md
   }
   // the new hypothesis table's component indices: an old component to its
   // compacted position, a new one (tagged hash slot) to its update's
-  // position after the kept components (independent of the copies above)
+  // position after the kept components (independent of the copies above, and
+  // taken from the grid's other end, so that a thread seldom has both)
   const long long n_e = min((long long)*n_entries, cap_entries);
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n_e;
+  for (long long e = (long long)(gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x; e < n_e;
        e += (long long)gridDim.x * blockDim.x) {
     const uint32_t v = out_comp[e];
     if ((v & kNewTag) ? (v & ~kNewTag) > hmask : v >= (uint32_t)n_src) {
