@@ -1111,6 +1111,22 @@ void set_groups(glmb_handle* h, Plan& p, int wc, int mc) {
   p.mg = std::max(by_area(1), mc);
 }
 
+// Staging threads.  Large images (staged in global memory): 1024 when each
+// parent has an SM of its own and 512 slots or rows to spread (15 parents of
+// 1400 slots and 2600 rows); 256 while the parents are fewer than two per SM;
+// else 128, whose scratch in shared memory (about 29 KB for the 3-D sweep's
+// plans) lets six CTAs per SM keep 24 warps in flight (N = 200 at H_max =
+// 20000: expansion 585 us with 128, 641 with 64, 618 with 256).  Small images
+// (staged in shared memory) leave most of 256 threads waiting at the barriers:
+// 64 once the parents fill the GPU with such CTAs (3-D N = 50 when it staged
+// there: expansion 118 us with 256, 106 with 128, 103 with 64, 115 with 32).
+int stage_threads(const glmb_handle* h, const Plan& p, long long H) {
+  if (h->tune.stage_threads > 0) return h->tune.stage_threads;
+  if (p.smem) return H >= 4LL * h->n_sm ? 64 : 256;
+  if (H <= h->n_sm && std::max(p.T, p.M) >= 512) return kStageWide;
+  return H < 2LL * h->n_sm ? 256 : 128;
+}
+
 bool make_plan(glmb_handle* h, bool fixed, int T_plan, int K_plan, int M_plan, Plan& p) {
   p.fixed = fixed;
   p.T = std::max(1, T_plan);
@@ -1129,29 +1145,16 @@ bool make_plan(glmb_handle* h, bool fixed, int T_plan, int K_plan, int M_plan, P
   if (h->launch_opts & GLMB_OPT_DRAW_WARP) p.thread = false;
   p.thread = p.thread && p.K <= 65536;
   // parents are staged in shared memory (then copied out to their image)
-  // when eight staging CTAs fit on an SM; larger images are built in place
-  // in global memory, where many CTAs per SM keep more parents in flight
-  // (measured: on the 3-D sweep's N = 200 cell, 123 KB images, staging in
-  // global memory with 64-thread CTAs ran the expansion in 2.41 ms against
-  // 3.51 ms in shared memory at one CTA per SM; on the 2-D mid scene, 19 KB
-  // images, shared memory stayed faster)
+  // when sixteen images fit on an SM; larger ones are built in place in
+  // global memory, where more CTAs per SM keep more parents in flight and
+  // only what a parent uses is written (measured at 8, 16 and 40 images an
+  // SM: 3-D N = 50, images of 17 KB: 8.9, 8.4 and 8.4 ms a scene; batch of 16
+  // 2-D scenes 25.6, 24.8 and 24.8; the others the same)
   const int img_bytes = expand_image_bytes(dz, p.T, p.K, p.M);
   p.smem = img_bytes + expand_stage_tail_bytes(dz, p.T, p.K, p.M, 0) <= h->smem_limit &&
            !(h->launch_opts & GLMB_OPT_STAGE_GLOBAL) &&
-           (8LL * img_bytes <= (long long)h->smem_per_sm || (h->launch_opts & GLMB_OPT_STAGE_SHARED));
-  // staging threads.  Large images (staged in global memory): 1024 when each
-  // parent has an SM of its own and 512 slots or rows to spread (15 parents of
-  // 1400 slots and 2600 rows); 256 while the parents are fewer than two per SM;
-  // else 128, whose scratch in shared memory (about 29 KB for the 3-D sweep's
-  // plans) lets six CTAs per SM keep 24 warps in flight (N = 200 at H_max =
-  // 20000: expansion 585 us with 128, 641 with 64, 618 with 256).  Small
-  // images (staged in shared memory) leave most of 256 threads waiting at the
-  // barriers: 64 once the parents fill the GPU with such CTAs (3-D N = 50:
-  // expansion 118 us with 256, 106 with 128, 103 with 64, 115 with 32)
-  if (h->tune.stage_threads > 0) p.st_thr = h->tune.stage_threads;
-  else if (p.smem) p.st_thr = (long long)h->H >= 4LL * h->n_sm ? 64 : 256;
-  else if (h->H <= h->n_sm && std::max(p.T, p.M) >= 512) p.st_thr = kStageWide;
-  else p.st_thr = (long long)h->H < 2LL * h->n_sm ? 256 : 128;
+           (16LL * img_bytes <= (long long)h->smem_per_sm || (h->launch_opts & GLMB_OPT_STAGE_SHARED));
+  p.st_thr = stage_threads(h, p, h->H);
   p.Gw = p.Gm = 0;
   for (int g = h->tune.warp_cta_warps; g >= 1 && !p.Gw; --g)
     if (expand_warp_smem(dz, 0, p.T, g, 1) <= h->smem_limit) p.Gw = g;
@@ -1490,7 +1493,11 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
     int best = -1;
     for (int gi = 0; gi < (int)h->graphs.size(); ++gi) {
       const glmb_handle::CachedGraph& g = h->graphs[gi];
-      if (g.hcur != h->hcur || g.prof != h->prof_mask || g.plan.thread != p.thread || g.plan.st_thr != p.st_thr ||
+      // (staging threads: also what half or twice the parents would take, so
+      // that a scene whose hypotheses hover at a line keeps its graphs)
+      if (g.hcur != h->hcur || g.prof != h->prof_mask || g.plan.thread != p.thread ||
+          (g.plan.st_thr != p.st_thr && g.plan.st_thr != stage_threads(h, p, 2LL * h->H) &&
+           g.plan.st_thr != stage_threads(h, p, h->H / 2)) ||
           g.plan.wc != p.wc || g.plan.mc != p.mc ||
           g.plan.T < p.T || g.plan.K < p.K || g.plan.M < p.M)
         continue;
@@ -1498,11 +1505,16 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
     }
     if (best >= 0 && (long long)h->graphs[best].smem > 3LL * need_smem) best = -1;
     if (best < 0) {
+      // headroom of a half (a quarter for the rows), or less where it would
+      // take the images out of shared memory
       Plan q = p;
-      if (!make_plan(h, true, round_up(p.T + p.T / 2, 32), round_up(p.K + p.K / 2, 128), round_up(p.M + p.M / 4, 64), q) ||
-          q.thread != p.thread ||
-          (p.smem && !q.smem))
-        q = p;
+      bool roomy = false;
+      for (int part = 2; part <= 8 && !roomy; part *= 2)
+        roomy = make_plan(h, true, round_up(p.T + p.T / part, 32), round_up(p.K + p.K / part, 128),
+                          round_up(p.M + p.M / (2 * part), 64), q) &&
+                q.thread == p.thread && (!p.smem || q.smem);
+      if (!roomy) q = p;
+      q.st_thr = p.st_thr;   // the frame's, or the next frame would not find the graph
       set_groups(h, q, p.wc, p.mc);   // this frame's parts (q.T decides the rest)
       if ((st = ensure_img(h, q)) != GLMB_OK) {
         h->frame -= 1;
