@@ -71,6 +71,13 @@ FX_FN double to_double(u64 v, int e) {
   return from_bits(((u64)(1085 - lz + e) << 52) + (m >> 11) + ((m >> 10) & 1ull));
 }
 
+// a value v 2^e still in fixed point
+struct Val {
+  u64 v;
+  int e;
+};
+FX_FN double to_double(Val x) { return to_double(x.v, x.e); }
+
 // ---- tables ----
 // 2^(-j/64) 2^63 and -ln(k_j / 1024) 2^59, k_j = round(1024 / (1 + (j + 1/2) / 128)),
 // from exp's and atanh's series with 100-bit fractions
@@ -135,7 +142,7 @@ FX_FN double exp_neg(double x, const u64* exp2) {
 }
 
 // ---- -2 ln((2 w + 1) / 2^33) ----
-FX_FN double neg2_log_unit(uint32_t w, const u64* nlog, const uint16_t* inv) {
+FX_FN Val neg2_log_unit(uint32_t w, const u64* nlog, const uint16_t* inv) {
   const u64 a = 2ull * w + 1ull;
   const u64 dl = (1ull << 33) - a;
   if (dl < (1ull << 26)) {
@@ -151,7 +158,7 @@ FX_FN double neg2_log_unit(uint32_t w, const u64* nlog, const uint16_t* inv) {
     q = 0x2000000000000000ull + mulhi(d, q);
     q = 0x4000000000000000ull + mulhi(d, q);
     const int ln = clz(dl);
-    return to_double(mulhi(dl << ln, q), 3 - ln - 33);
+    return Val{mulhi(dl << ln, q), 3 - ln - 33};
   }
   const int lz = clz(a);
   const u64 mm = (a << lz) >> 31;                                      // [1, 2) 2^32, exact
@@ -169,7 +176,7 @@ FX_FN double neg2_log_unit(uint32_t w, const u64* nlog, const uint16_t* inv) {
   // E ln 2 + ln(k / 1024) - ln(1 + r), 2^59
   const u64 E = (u64)(lz - 30);
   const u64 L = E * 0x058B90BFBE8E7BCDull + ((E * 0x5E4F1D9Cull) >> 32) - nlog[j] - (u64)((l1 + 4) >> 3);
-  return to_double(L, -58);
+  return Val{L, -58};
 }
 
 // ---- sine and cosine of (octant + t / 2^64) / 8 of a turn, 0 <= t < 2^64 ----
@@ -199,36 +206,69 @@ FX_FN u64 sin_oct(u64 t, u64 q) {                                      // sin x 
   return mulhi(t, p);
 }
 
-// cos(2 pi (2 w + 1) / 2^33)
-FX_FN double cos_turn(uint32_t w) {
+// square root of x > 0, to about 2^-58 of its value: a 22-bit reciprocal root,
+// one correction of second order
+FX_FN Val root(Val x) {
+  const int lz = clz(x.v);
+  u64 M = x.v << lz;                                                   // x = M 2^E
+  int E = x.e - lz;
+  if (E & 1) {
+    M >>= 1;
+    ++E;
+  }
+  const float xf = (float)(uint32_t)(M >> 32) * 9.313225746154785e-10f;   // M 2^-62, in [1, 4)
+#if defined(__CUDA_ARCH__)
+  const float y = rsqrtf(xf);
+#else
+  const float y = 1.0f / std::sqrt(xf);
+#endif
+  const uint32_t Y = (uint32_t)(y * 2147483648.0f);                    // 1 / sqrt(x) 2^31
+  // r = 1 - x y^2 (2^-60 units); sqrt(x) = x y (1 + r/2 + 3 r^2 / 8 + ...)
+  const long long r = (long long)((1ull << 60) - mulhi(M, (u64)Y * Y));
+  const long long rh = r >> 20;
+  const long long c = (r >> 1) + ((3 * rh * rh) >> 23);
+  const u64 s0 = mulhi(M, (u64)Y << 32);                               // x y 2^61
+  return Val{s0 + (u64)mulhi_s((long long)s0, c << 4), E / 2 - 30};
+}
+
+// cos(2 pi (2 w + 1) / 2^33), its magnitude
+FX_FN Val cos_turn(uint32_t w, bool& neg) {
   const u64 a = 2ull * w + 1ull;
   const uint32_t oct = (uint32_t)(a >> 30);
   uint32_t t30 = (uint32_t)a & 0x3FFFFFFFu;                            // odd
   if (oct & 1u) t30 = 0x40000000u - t30;
   const u64 q = ((u64)t30 * t30) << 4;
-  const bool use_sin = ((oct + 1u) & 2u) != 0u;                        // octants 1, 2, 5, 6
-  double v;
-  if (use_sin) {
-    // t30 times the polynomial, normalised: relative accuracy near 0 too
-    const int ln = clz(t30);
-    v = to_double(sin_oct((u64)t30 << ln, q), 64 - 63 - ln - 30);
-  } else {
-    v = to_double(cos_oct(q), -63);
-  }
-  return (oct >= 2u && oct < 6u) ? -v : v;
+  neg = oct >= 2u && oct < 6u;
+  if (((oct + 1u) & 2u) == 0u) return Val{cos_oct(q), -63};
+  // octants 1, 2, 5, 6: t30 times the sine's polynomial, normalised, for
+  // relative accuracy near 0 too
+  const int ln = clz(t30);
+  return Val{sin_oct((u64)t30 << ln, q), 1 - ln - 30};
 }
 
-// sine and cosine of psi, |psi| < 2^30 (checked by the caller)
-FX_FN void sincos(double psi, double& s, double& c) {
-  const u64 b = to_bits(psi);
+// A standard normal of two words (Box and Muller's cosine branch):
+// sqrt(-2 ln u0) cos(2 pi u1), u = (word + 1/2) / 2^32, rounded once.
+FX_FN double normal(uint32_t w0, uint32_t w1, const u64* nlog, const uint16_t* inv) {
+  bool neg;
+  const Val s = root(neg2_log_unit(w0, nlog, inv)), c = cos_turn(w1, neg);
+  const double n = to_double(mulhi(s.v, c.v), s.e + c.e + 64);
+  return neg ? -n : n;
+}
+
+// x / (2 pi) modulo 1 as a 64-bit fraction, |x| < 2^30 (checked by the caller)
+FX_FN u64 turn(double x) {
+  const u64 b = to_bits(x);
   const int E = (int)((b >> 52) & 0x7FFull) - 1023;
-  const u64 M = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;   // |psi| = M 2^(E - 63)
-  // |psi| / (2 pi) modulo 1, as a 64-bit fraction
+  const u64 M = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;   // |x| = M 2^(E - 63)
   constexpr u64 Ih = 0x28BE60DB9391054Aull, Il = 0x7F09D5F47D4D3770ull;   // 2^-64, 2^-128 words of 1 / (2 pi)
   const u64 hl = M * Ih, add = mulhi(M, Il);
   const u64 p1 = hl + add, p2 = mulhi(M, Ih) + (p1 < hl ? 1ull : 0ull);
   const int sh = E + 1;
   const u64 f = sh >= 64 ? 0ull : sh > 0 ? (p2 << sh) | (p1 >> (64 - sh)) : sh > -64 ? p2 >> -sh : 0ull;
+  return b >> 63 ? 0ull - f : f;
+}
+// sine and cosine of f 2^-64 of a turn, to 2^-62 beside their rounding
+FX_FN void sincos_turn(u64 f, double& s, double& c) {
   const uint32_t oct = (uint32_t)(f >> 61);
   u64 t = f << 3;
   if (oct & 1u) t = ~t;                                                   // 1 - t to 2^-64
@@ -236,8 +276,26 @@ FX_FN void sincos(double psi, double& s, double& c) {
   const double vs = to_double(sin_oct(t, q), -63), vc = to_double(cos_oct(q), -63);
   const bool swap = ((oct + 1u) & 2u) != 0u;
   const double as = swap ? vc : vs, ac = swap ? vs : vc;
-  s = ((oct >= 4u) != ((b >> 63) != 0ull)) ? -as : as;
+  s = oct >= 4u ? -as : as;
   c = (oct >= 2u && oct < 6u) ? -ac : ac;
+}
+
+// sin(h) / h, |h| < 1/2 (checked by the caller)
+FX_FN double sinc(double h) {
+  const u64 b = to_bits(h) & 0x7FFFFFFFFFFFFFFFull;
+  const int sh = 1022 - (int)(b >> 52);                                   // |h| = M 2^-(sh + 64)
+  const u64 M = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
+  const u64 x = sh < 64 ? M >> sh : 0ull;
+  const u64 q = mulhi(x, x);
+  u64 p = 0x654Bull;                                                      // 1/17! 2^63
+  p = 0x6B9FD0ull - mulhi(q, p);
+  p = 0x5849184Full - mulhi(q, p);
+  p = 0x35CC8ACFEBull - mulhi(q, p);
+  p = 0x171DE3A556C7ull - mulhi(q, p);
+  p = 0x6806806806807ull - mulhi(q, p);
+  p = 0x111111111111111ull - mulhi(q, p);
+  p = 0x1555555555555555ull - mulhi(q, p);
+  return to_double(0x8000000000000000ull - mulhi(q, p), -63);
 }
 
 }  // namespace fx

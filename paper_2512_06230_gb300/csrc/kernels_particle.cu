@@ -39,13 +39,13 @@ __device__ __forceinline__ uint4 part_words(const PartModel& pm, int frame, uint
 // on an SM), so the functions run in integer arithmetic (fx_math.cuh) and what
 // is left in FP64 is the states' own arithmetic and the sums, which take a
 // fifth of the butterfly's additions (warp_sums).  Per frame, prediction and
-// update stages: 200 vehicles 85.9 -> 51.5 and 55.7 -> 46.7 us; a convoy of ten
-// 52.1 -> 33.2 and 50.1 -> 42.5.
+// update stages: 200 vehicles 85.9 -> 37.4 and 55.7 -> 46.7 us; a convoy of ten
+// 52.1 -> 28.9 and 50.1 -> 42.5.
 __device__ const fx::Tables kFx{};
 
 __device__ __forceinline__ void normal_pair(const uint4& w, double& n0, double& n1) {
-  n0 = sqrt(fx::neg2_log_unit(w.x, kFx.nlog, kFx.inv)) * fx::cos_turn(w.y);
-  n1 = sqrt(fx::neg2_log_unit(w.z, kFx.nlog, kFx.inv)) * fx::cos_turn(w.w);
+  n0 = fx::normal(w.x, w.y, kFx.nlog, kFx.inv);
+  n1 = fx::normal(w.z, w.w, kFx.nlog, kFx.inv);
 }
 
 // exp(l) of a log-weight difference, l <= 0 but for rounding
@@ -56,32 +56,31 @@ __device__ __forceinline__ double exp_weight(double l) {
 }
 
 // one CTRV step over dt; the arc (v / w)(sin(psi + w dt) - sin psi, ...)
-// as v dt sinc(h)(cos, sin)(psi + h), h = w dt / 2, valid at w = 0.  The
-// half-angle terms sin h, cos h and sinc h come from their Taylor series
-// when |h| < 0.03 (the first omitted terms, h^8 / 9! and h^8 / 8!, are
-// below 1e-16 of the sums) and (cos, sin)(psi + h) from the angle sum, so
-// a particle takes one sincos instead of three transcendental calls.
+// as v dt sinc(h)(cos, sin)(psi + h), h = w dt / 2, valid at w = 0.  Heading
+// and half angle are added as fractions of a turn, so that the FP64 pipe sees
+// 17 operations a particle instead of about 60 (for headings or half angles
+// beyond the fixed-point range: the library's functions).
 __device__ __forceinline__ void ctrv(const double (&x)[5], double dt, double a, double al, double (&y)[5]) {
   const double h = 0.5 * x[4] * dt;
-  double sh, ch, sinc;
-  if (fabs(h) < 0.03) {
-    const double h2 = h * h;
-    sinc = 1.0 - h2 / 6.0 * (1.0 - h2 / 20.0 * (1.0 - h2 / 42.0));
-    sh = h * sinc;
-    ch = 1.0 - 0.5 * h2 * (1.0 - h2 / 12.0 * (1.0 - h2 / 30.0));
+  double s0, c0, s1, c1, sc;
+  if (fabs(h) < 0.5 && fabs(x[3]) < 1e9) {
+    const fx::u64 f = fx::turn(x[3]);
+    fx::sincos_turn(f, s0, c0);
+    fx::sincos_turn(f + fx::turn(h), s1, c1);
+    sc = fx::sinc(h);
   } else {
+    double sh, ch;
     sincos(h, &sh, &ch);
-    sinc = sh / h;
+    sincos(x[3], &s0, &c0);
+    sc = h == 0.0 ? 1.0 : sh / h;
+    s1 = s0 * ch + c0 * sh;
+    c1 = c0 * ch - s0 * sh;
   }
-  const double vdt = x[2] * dt * sinc;
-  double s0, c0;
-  if (fabs(x[3]) < 1e9) fx::sincos(x[3], s0, c0);
-  else sincos(x[3], &s0, &c0);
-  const double s1 = s0 * ch + c0 * sh, c1 = c0 * ch - s0 * sh;
-  y[0] = x[0] + vdt * c1 + 0.5 * dt * dt * c0 * a;
-  y[1] = x[1] + vdt * s1 + 0.5 * dt * dt * s0 * a;
+  const double vdt = x[2] * dt * sc, hd = 0.5 * dt * dt;
+  y[0] = x[0] + vdt * c1 + hd * c0 * a;
+  y[1] = x[1] + vdt * s1 + hd * s0 * a;
   y[2] = x[2] + dt * a;
-  y[3] = x[3] + x[4] * dt + 0.5 * dt * dt * al;
+  y[3] = x[3] + x[4] * dt + hd * al;
   y[4] = x[4] + dt * al;
 }
 

@@ -15,9 +15,23 @@ SRC = """
 using namespace glmb;
 static constexpr fx::Tables T{};
 extern "C" void f_exp(const double* x, double* y, int n) { for (int i = 0; i < n; ++i) y[i] = fx::exp_neg(x[i], T.exp2); }
-extern "C" void f_log(const unsigned* w, double* y, int n) { for (int i = 0; i < n; ++i) y[i] = fx::neg2_log_unit(w[i], T.nlog, T.inv); }
-extern "C" void f_cos(const unsigned* w, double* y, int n) { for (int i = 0; i < n; ++i) y[i] = fx::cos_turn(w[i]); }
-extern "C" void f_sc(const double* x, double* s, double* c, int n) { for (int i = 0; i < n; ++i) fx::sincos(x[i], s[i], c[i]); }
+extern "C" void f_log(const unsigned* w, double* y, double* r, int n) {
+  for (int i = 0; i < n; ++i) {
+    const fx::Val v = fx::neg2_log_unit(w[i], T.nlog, T.inv);
+    y[i] = fx::to_double(v);
+    r[i] = fx::to_double(fx::root(v));
+  }
+}
+extern "C" void f_cos(const unsigned* w, double* y, int n) {
+  for (int i = 0; i < n; ++i) {
+    bool neg;
+    const double v = fx::to_double(fx::cos_turn(w[i], neg));
+    y[i] = neg ? -v : v;
+  }
+}
+extern "C" void f_norm(const unsigned* w, const unsigned* u, double* y, int n) { for (int i = 0; i < n; ++i) y[i] = fx::normal(w[i], u[i], T.nlog, T.inv); }
+extern "C" void f_sc(const double* x, double* s, double* c, int n) { for (int i = 0; i < n; ++i) fx::sincos_turn(fx::turn(x[i]), s[i], c[i]); }
+extern "C" void f_sinc(const double* x, double* y, int n) { for (int i = 0; i < n; ++i) y[i] = fx::sinc(x[i]); }
 """
 LD = np.longdouble
 if np.finfo(LD).nmant < 63:
@@ -63,11 +77,22 @@ def test_exp(lib):
 
 def test_log(lib):
     w = _words()
-    y = np.empty(len(w))
-    lib.f_log(_p(w), _p(y), len(w))
+    y, r = np.empty(len(w)), np.empty(len(w))
+    lib.f_log(_p(w), _p(y), _p(r), len(w))
     d = (LD(2) ** 33 - (LD(2) * w.astype(LD) + 1)) / LD(2) ** 33   # 1 - u, exact
     want = -2 * np.log1p(-d)
     assert np.all(np.abs(y.astype(LD) / want - 1) <= TOL)
+    assert np.all(np.abs(r.astype(LD) / np.sqrt(want) - 1) <= TOL)
+
+
+def test_normal(lib):
+    w = _words()
+    u = np.roll(w, 17)
+    y = np.empty(len(w))
+    lib.f_norm(_p(w), _p(u), _p(y), len(w))
+    d = (LD(2) ** 33 - (LD(2) * w.astype(LD) + 1)) / LD(2) ** 33
+    size, c = np.sqrt(-2 * np.log1p(-d)), np.cos(2 * PI * ((LD(2) * u.astype(LD) + 1) / LD(2) ** 33))
+    assert np.all(np.abs(y.astype(LD) - size * c) <= TOL * size * np.maximum(np.abs(c), LD(2) ** -8))
 
 
 def test_cos_of_a_turn(lib):
@@ -86,3 +111,13 @@ def test_sincos(lib):
     lib.f_sc(_p(x), _p(s), _p(c), len(x))
     assert np.all(np.abs(s.astype(LD) - np.sin(x.astype(LD))) <= TOL)
     assert np.all(np.abs(c.astype(LD) - np.cos(x.astype(LD))) <= TOL)
+
+
+def test_sinc(lib):
+    rng = np.random.default_rng(6)
+    x = np.concatenate([rng.uniform(-0.4999, 0.4999, 2000), 2.0 ** rng.uniform(-200, -2, 500), [0.0, -0.0, 0.49999999]])
+    y = np.empty_like(x)
+    lib.f_sinc(_p(x), _p(y), len(x))
+    xl = x.astype(LD)
+    want = np.where(np.abs(xl) < 1e-12, LD(1), np.sin(xl) / np.where(xl == 0, LD(1), xl))
+    assert np.all(np.abs(y.astype(LD) / want - 1) <= TOL)
