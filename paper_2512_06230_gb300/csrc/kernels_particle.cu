@@ -257,7 +257,8 @@ __global__ void __launch_bounds__(kPartThreads) particle_step_kernel(Model md, P
   }
 }
 
-// The working table's moments: one block of 64 threads per component,
+// The working table's moments: one block of 128 threads per component (64: 3 us
+// more for a convoy of ten, the same for 200 vehicles),
 // threads over its particles, one pass with offsets from its particle 0, d_p = x_p - x_0:
 // mean = x_0 + sum w d, covariance = sum w d d^T - (sum w d)(sum w d)^T
 // (the weights sum to one), mean rounded to FP32 with a zero low part.
@@ -306,7 +307,8 @@ __global__ void __launch_bounds__(kPartThreads) particle_moments_kernel(PartMode
   }
 }
 
-// Compatibility entries: one warp per component, lanes over particles;
+// Compatibility entries: the warps of a block on one component, a pair to a
+// warp at a time, lanes over particles;
 // log C = log P_D + log sum_p w_p N(z; (px, py)_p, R) for each of the
 // component's gated pairs (the table kernels wrote the pairs, gated on
 // the moments), then the death probability from these entries.  The
@@ -318,18 +320,25 @@ __global__ void __launch_bounds__(kPartThreads) particle_moments_kernel(PartMode
 // FP32 too (log C is stored in FP32).  Particles beyond kRegP per lane
 // are re-read from the particle rows.
 constexpr int kRegP = 8;   // particles held in registers per lane (256 per warp)
+// A component's pairs are few (up to a dozen or two), but with one warp each
+// they follow one another through shuffles and exponentials, and the frame
+// waits for its longest list: four warps share a component, and the death
+// probability's sum over the pairs, whose order is the pairs', follows.  Table
+// stage with one, two and four warps: 22.7, 17.8 and 16.1 us (convoy of ten),
+// 25.9, 20.8 and 20.0 (200 vehicles).
+constexpr int kLogcWarps = 4;
 
-__global__ void __launch_bounds__(256) particle_logc_kernel(Model md, PartModel pm, CompTable ct, PairTable pt,
-                                                            const FrameDev* fs) {
+__global__ void __launch_bounds__(32 * kLogcWarps) particle_logc_kernel(Model md, PartModel pm, CompTable ct,
+                                                                        PairTable pt, const FrameDev* fs) {
   pdl_enter();
-  const int T = fs->T, np = pm.np, lane = threadIdx.x & 31;
+  __shared__ float s_logc[32];
+  const int T = fs->T, np = pm.np, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   if (fs->M > 0 && !__isGlobal(fs->Z)) return;   // flagged by the count kernel
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
   const unsigned cap_p = (unsigned)min(pt.cap_pairs, (long long)0xFFFFFFFF);
   const size_t capp = (size_t)pt.cap_pairs;
   const float r0 = (float)pm.Rinv[0], r1 = (float)(pm.Rinv[1] + pm.Rinv[2]), r3 = (float)pm.Rinv[3];
   const float lc0 = (float)(pm.log_pd - pm.lnorm);
-  for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < T; c += nwarps) {
+  for (int c = blockIdx.x; c < T; c += gridDim.x) {
     const unsigned k0 = min(pt.ptr[c], cap_p), k1 = min(k0 + pt.cnt[c], cap_p);
     const double mx = (double)ct.mhi[c], my = (double)ct.mhi[(size_t)ct.cap + c];
     float ox[kRegP], oy[kRegP], ow[kRegP];
@@ -343,7 +352,9 @@ __global__ void __launch_bounds__(256) particle_logc_kernel(Model md, PartModel 
     }
     float lm = -INFINITY, ls = 0.f;
     bool any = false;
-    for (unsigned k = k0; k < k1; ++k) {
+    for (unsigned kb = k0; kb < k1; kb += 32) {   // 32 pairs, then their part of the sum
+    const unsigned ke = min(kb + 32u, k1);
+    for (unsigned k = kb + wp; k < ke; k += kLogcWarps) {
       const float ex = pt.e[k], ey = pt.e[capp + k];
       // the register-held particles' terms are independent: their maximum,
       // then the sum of their exponentials (no dependent chain through expf)
@@ -381,11 +392,20 @@ __global__ void __launch_bounds__(256) particle_logc_kernel(Model md, PartModel 
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) sw += __shfl_xor_sync(0xFFFFFFFFu, sw, o);
       const float logC = mw == -INFINITY ? -INFINITY : lc0 + mw + logf(sw);
-      if (lane == 0) pt.logC[k] = logC;
-      any = true;
-      if (!md.kappa_zero) lse_push(lm, ls, logC - md.log_kappa);
+      if (lane == 0) {
+        pt.logC[k] = logC;
+        s_logc[k - kb] = logC;
+      }
     }
-    if (lane == 0) death_prob(md, ct.logp[c], ct.log1mp[c], lm, ls, any, pt.dprob[c], pt.dthr[c]);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      any = true;
+      if (!md.kappa_zero)
+        for (unsigned k = kb; k < ke; ++k) lse_push(lm, ls, s_logc[k - kb] - md.log_kappa);
+    }
+    __syncthreads();
+    }
+    if (threadIdx.x == 0) death_prob(md, ct.logp[c], ct.log1mp[c], lm, ls, any, pt.dprob[c], pt.dthr[c]);
   }
 }
 
@@ -539,12 +559,12 @@ __global__ void __launch_bounds__(kPartThreads) particle_remap_kernel(
 void launch_particle_predict(const Model& md, const PartModel& pm, const CompTable& src, const CompTable& dst,
                              const FrameDev* fs, const double* births_dev, int grid, cudaStream_t s) {
   launch_k(particle_step_kernel, grid, kPartThreads, 0, s, md, pm, src, dst, fs, births_dev);
-  launch_k(particle_moments_kernel, 4 * grid, 64, 0, s, pm, dst, fs);
+  launch_k(particle_moments_kernel, 4 * grid, 128, 0, s, pm, dst, fs);
 }
 
 void launch_particle_logc(const Model& md, const PartModel& pm, const CompTable& ct, const PairTable& pt,
                           const FrameDev* fs, int grid, cudaStream_t s) {
-  launch_k(particle_logc_kernel, grid, 256, 0, s, md, pm, ct, pt, fs);
+  launch_k(particle_logc_kernel, 4 * grid, 32 * kLogcWarps, 0, s, md, pm, ct, pt, fs);
 }
 
 void launch_particle_remap(const Model& md, const PartModel& pm, const CompTable& src, const CompTable& dst,
