@@ -1077,7 +1077,7 @@ glmb_status enqueue_prune(glmb_handle* h, const Plan& p) {
   if (h->md.particle)
     launch_particle_remap(h->md, h->pm, B, A, h->gc_newpos, h->gc_flag, h->d_fs, h->d_scal + S_NKEEP, h->upd_src,
                           h->upd_m, h->upd_se, (int)h->cap_upd, h->d_scal + S_NUPD, h->pw.counts,
-                          h->d_scal + S_ERR, 4 * h->n_sm, s);
+                          h->d_scal + S_ERR, 4 * h->n_sm, h->cap_h, s);
   launch_gc_remap(h->md, B, A, h->gc_newpos, h->gc_flag, h->d_fs, h->d_scal + S_NKEEP, h->upd_src, h->upd_m,
                   h->upd_se, (int)h->cap_upd, h->d_scal + S_NUPD, h->pw.counts, h->d_scal + S_ERR, O.comp,
                   h->pw.counts + 1, h->cap_entries, h->hvals, h->hmask, h->d_hprev, ggc, s);

@@ -101,7 +101,7 @@ void launch_particle_remap(const Model& md, const PartModel& pm, const CompTable
                            const uint32_t* newpos, const uint32_t* flag, const FrameDev* fs,
                            const unsigned* n_keep_dev, const uint32_t* upd_src, const uint32_t* upd_m,
                            const long long* upd_se, int cap_upd, const unsigned* n_upd_dev,
-                           const unsigned* n_surv_dev, unsigned* err, int grid, cudaStream_t s);
+                           const unsigned* n_surv_dev, unsigned* err, int grid, int h_max, cudaStream_t s);
 int particle_remap_smem(int np);
 
 // ---- expansion / materialisation (kernels_expand.cu) ----

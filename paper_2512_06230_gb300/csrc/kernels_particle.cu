@@ -160,14 +160,27 @@ __device__ double block_max(double v, double* red) {
   return m;
 }
 
+// A block's particles, PER a thread in registers (particle threadIdx.x + i *
+// blockDim.x), or, PER = 0, in global memory: the update of a component reads
+// and sums them several times.
+template <int PER>
+__device__ __forceinline__ int particles_of(int np) {
+  return PER > 0 ? PER : (np - (int)threadIdx.x + (int)blockDim.x - 1) / (int)blockDim.x;
+}
+
 // weighted mean and covariance of component c's particles into its moment
-// fields (mean rounded to FP32, mlo = 0); wv holds the particles' weights
-__device__ void write_moments(const CompTable& ct, int np, int c, const double* wv, double* red, double* tot) {
+// fields (mean rounded to FP32, mlo = 0); x(i, k) and w(i) give row k and the
+// weight of the thread's particle i
+template <int PER, typename X, typename W>
+__device__ __forceinline__ void write_moments(const CompTable& ct, int np, int c, X x, W w, double* red, double* tot) {
+  const int n = particles_of<PER>(np), lane = (int)threadIdx.x;
   double s[5] = {0, 0, 0, 0, 0};
-  for (int p = threadIdx.x; p < np; p += blockDim.x) {
-    const double w = wv[p];
+#pragma unroll PER > 0 ? PER : 1
+  for (int i = 0; i < n; ++i) {
+    if (lane + i * (int)blockDim.x >= np) break;
+    const double wi = w(i);
 #pragma unroll
-    for (int k = 0; k < 5; ++k) s[k] += w * prow(ct, np, c, k)[p];
+    for (int k = 0; k < 5; ++k) s[k] += wi * x(i, k);
   }
   block_sum<5>(s, red, tot);
 #pragma unroll
@@ -175,18 +188,19 @@ __device__ void write_moments(const CompTable& ct, int np, int c, const double* 
   double q[15];
 #pragma unroll
   for (int k = 0; k < 15; ++k) q[k] = 0.0;
-  for (int p = threadIdx.x; p < np; p += blockDim.x) {
-    const double w = wv[p];
+#pragma unroll PER > 0 ? PER : 1
+  for (int i = 0; i < n; ++i) {
+    if (lane + i * (int)blockDim.x >= np) break;
+    const double wi = w(i);
     double d[5];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) d[k] = prow(ct, np, c, k)[p] - s[k];
+    for (int k = 0; k < 5; ++k) d[k] = x(i, k) - s[k];
     int k = 0;
 #pragma unroll
-    for (int i = 0; i < 5; ++i)
+    for (int a = 0; a < 5; ++a)
 #pragma unroll
-      for (int j = i; j < 5; ++j, ++k) q[k] += w * d[i] * d[j];
+      for (int b = a; b < 5; ++b, ++k) q[k] += wi * d[a] * d[b];
   }
-  const int lane = (int)threadIdx.x;
   const size_t cap = ct.cap;
   if (lane < 5) {
     ct.mhi[lane * cap + c] = (float)tot[lane];
@@ -194,7 +208,7 @@ __device__ void write_moments(const CompTable& ct, int np, int c, const double* 
   }
   block_sum<15>(q, red, tot + 5);
   if (lane < 15) ct.cov[(size_t)lane * cap + c] = (float)tot[5 + lane];
-  __syncthreads();   // wv and the totals are reused by the next component
+  __syncthreads();   // the weights and the totals are reused by the next component
 }
 
 // Prediction, particle by particle (a flat grid over the working table's
@@ -409,25 +423,33 @@ __global__ void __launch_bounds__(32 * kLogcWarps) particle_logc_kernel(Model md
   }
 }
 
-// Regeneration: one block (64 threads) per kept component (copied to its compacted
+// Regeneration: one block per kept component (copied to its compacted
 // position) and per distinct (component, detection set) update (written
 // after the kept ones): log w_p -= (m / 2) (zbar - h_p)^T R^-1 (zbar - h_p)
 // (the product of the m detections' likelihoods up to a factor common to
 // all particles), normalised; systematic resampling when the effective
-// sample size is below ess_frac * P.  Dynamic shared memory: P doubles
-// (cumulative weights).
-__global__ void __launch_bounds__(kPartThreads) particle_remap_kernel(
+// sample size is below ess_frac * P.  Dynamic shared memory: 2 P doubles
+// (log-weights; weights, then cumulative weights).
+// What bounds it is the chain of block reductions and, with many updates, the
+// FP64 pipe: the particles stay in registers (PER a thread) between the
+// passes, the runs of the cumulative weights are scanned across the warps,
+// the search compares the weights' bits, and what all threads share is formed
+// by one.
+template <int PER>
+__global__ void __launch_bounds__(kPartThreads, 2) particle_remap_kernel(
     Model md, PartModel pm, CompTable src, CompTable dst, const uint32_t* __restrict__ newpos,
     const uint32_t* __restrict__ flag, const FrameDev* __restrict__ fs, const unsigned* __restrict__ n_keep_dev,
     const uint32_t* __restrict__ upd_src, const uint32_t* __restrict__ upd_m, const long long* __restrict__ upd_se,
     int cap_upd, const unsigned* __restrict__ n_upd_dev, const unsigned* __restrict__ n_surv_dev, unsigned* err) {
   pdl_enter();
-  extern __shared__ double cum[];
+  extern __shared__ double s_dyn[];
   __shared__ double red[(kPartThreads / 32) * 15], tot[20];
-  __shared__ double s_lse, s_inv;
-  __shared__ double runs[kPartThreads];
+  __shared__ double s_wsum[kPartThreads / 32];
   if (*n_surv_dev == 0u || (*(volatile unsigned*)err & kErrFatal)) return;
   const int n_src = fs->T, np = pm.np, frame = fs->frame;
+  double* s_l = s_dyn;         // log-weights
+  double* cum = s_dyn + np;    // weights, then cumulative weights
+  const int tid = (int)threadIdx.x, bd = (int)blockDim.x;
   const unsigned n_keep = *n_keep_dev;
   const unsigned n_upd = min(*n_upd_dev, (unsigned)cap_upd);
   if ((long long)n_keep + n_upd > dst.cap) return;   // flagged by the remap kernel
@@ -467,85 +489,121 @@ __global__ void __launch_bounds__(kPartThreads) particle_remap_kernel(
 #pragma unroll
     for (int a = 0; a < 2; ++a)
       zb[a] = (double)src.mhi[a * (size_t)src.cap + c] + (double)upd_se[(size_t)a * cap_upd + u] * kFxInv / m;
-    // reweight (kept in the destination's weight row), then normalise
+    // reweight, then normalise
+    constexpr int kHeld = PER > 0 ? PER : 1;
+    double xr[kHeld][5];
     double mx = -INFINITY;
-    for (int p = threadIdx.x; p < np; p += blockDim.x) {
-      const double ex = zb[0] - prow(src, np, c, 0)[p], ey = zb[1] - prow(src, np, c, 1)[p];
-      const double l = prow(src, np, c, 5)[p] -
-                       0.5 * m * (pm.Rinv[0] * ex * ex + (pm.Rinv[1] + pm.Rinv[2]) * ex * ey + pm.Rinv[3] * ey * ey);
-      prow(dst, np, d, 5)[p] = l;
+    const int n = particles_of<PER>(np);
+#pragma unroll PER > 0 ? PER : 1
+    for (int i = 0; i < n; ++i) {
+      const int p = tid + i * bd;
+      if (p >= np) break;
+      double px = prow(src, np, c, 0)[p], py = prow(src, np, c, 1)[p];
+      const double l0 = prow(src, np, c, 5)[p];
+      if (PER > 0) {
+        xr[i % kHeld][0] = px;
+        xr[i % kHeld][1] = py;
+#pragma unroll
+        for (int k = 2; k < 5; ++k) xr[i % kHeld][k] = prow(src, np, c, k)[p];
+      }
+      const double ex = zb[0] - px, ey = zb[1] - py;
+      const double l =
+          l0 - 0.5 * m * (pm.Rinv[0] * ex * ex + (pm.Rinv[1] + pm.Rinv[2]) * ex * ey + pm.Rinv[3] * ey * ey);
+      s_l[p] = l;
       mx = fmax(mx, l);
     }
     mx = block_max(mx, red);
     double sv[1] = {0.0};
-    for (int p = threadIdx.x; p < np; p += blockDim.x) {
-      const double e = exp_weight(prow(dst, np, d, 5)[p] - mx);
+    for (int p = tid; p < np; p += bd) {
+      const double e = exp_weight(s_l[p] - mx);
       cum[p] = e;
       sv[0] += e;
     }
     block_sum<1>(sv, red, tot, [&](double t) {   // (one warp's FP64 work, not every warp's)
-      s_lse = mx + log(t);
-      s_inv = 1.0 / t;
+      tot[1] = mx + log(t);
+      tot[2] = 1.0 / t;
     });
-    const double lse = s_lse, inv = s_inv;
-    // normalised weights cum[p] = exp(l_p - mx) / sum; the log-weights
-    // l_p - lse stay in the destination row
+    const double lse = tot[1], inv = tot[2];
+    // normalised weights cum[p] = exp(l_p - mx) / sum, log-weights l_p - lse
     double s2[1] = {0.0};
-    for (int p = threadIdx.x; p < np; p += blockDim.x) {
-      prow(dst, np, d, 5)[p] -= lse;
+    for (int p = tid; p < np; p += bd) {
       const double w = cum[p] * inv;
       cum[p] = w;
       s2[0] += w * w;
     }
-    block_sum<1>(s2, red, tot, [&](double t) { tot[1] = 1.0 / t; });
-    if (tot[1] < pm.ess_frac * np) {
+    block_sum<1>(s2, red, tot, [&](double t) {
+      tot[1] = 1.0 / t;
+      if (tot[1] < pm.ess_frac * np) {
+        tot[2] = -log((double)np);
+        tot[3] = 1.0 / np;
+      }
+    });
+    const bool resample = tot[1] < pm.ess_frac * np;
+    const double lw_r = tot[2], w_r = tot[3];
+    if (resample) {
       // cumulative weights: each thread scans a contiguous run, then the
-      // runs' totals are scanned by thread 0
-      const int per = (np + blockDim.x - 1) / blockDim.x, b0 = threadIdx.x * per, b1 = min(np, b0 + per);
+      // runs' totals are scanned over the block
+      const int per = (np + bd - 1) / bd, b0 = min(np, tid * per), b1 = min(np, b0 + per);
       double run = 0.0;
       for (int p = b0; p < b1; ++p) {
         run += cum[p];
         cum[p] = run;
       }
-      runs[threadIdx.x] = run;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double acc = 0.0;
-        for (int t = 0; t < (int)blockDim.x; ++t) {
-          const double v = runs[t];
-          runs[t] = acc;
-          acc += v;
-        }
+      const int lane = tid & 31, wp = tid >> 5;
+      double incl = run;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
       }
+      if (lane == 31) s_wsum[wp] = incl;
       __syncthreads();
-      const double off = runs[threadIdx.x];
+      // (the exclusive scan from the lower lanes' totals: no rounding of incl - run)
+      double off = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
+      if (lane == 0) off = 0.0;
+      double before = 0.0;
+      for (int w = 0; w < wp; ++w) before += s_wsum[w];
+      off += before;
       for (int p = b0; p < b1; ++p) cum[p] += off;
       __syncthreads();
       const double u0 = unit_open(part_words(pm, frame, src.lk[c], src.lb[c], 0u, 3u, 0u).x);
-      const double lw_r = -log((double)np);
-      for (int r = threadIdx.x; r < np; r += blockDim.x) {
-        const double target = (u0 + r) / np;
+      const bool pow2 = (np & (np - 1)) == 0;   // then 1 / np is exact
+      const unsigned long long* bits = reinterpret_cast<const unsigned long long*>(cum);
+#pragma unroll PER > 0 ? PER : 1
+      for (int i = 0; i < n; ++i) {
+        const int r = tid + i * bd;
+        if (r >= np) break;
+        const double target = pow2 ? (u0 + r) * w_r : (u0 + r) / np;
+        const unsigned long long tb = fx::to_bits(target);
         int lo = 0, hi = np - 1;   // first k with cum[k] > target, else np - 1
-        while (lo < hi) {
+        while (lo < hi) {          // (doubles that are not negative compare as their bits)
           const int mid = (lo + hi) >> 1;
-          if (cum[mid] > target) hi = mid;
+          if (bits[mid] > tb) hi = mid;
           else lo = mid + 1;
         }
 #pragma unroll
-        for (int k = 0; k < 5; ++k) prow(dst, np, d, k)[r] = prow(src, np, c, k)[lo];
-      }
-      __syncthreads();   // every cumulative weight read before it is overwritten
-      for (int r = threadIdx.x; r < np; r += blockDim.x) {
+        for (int k = 0; k < 5; ++k) {
+          const double v = prow(src, np, c, k)[lo];
+          if (PER > 0) xr[i % kHeld][k] = v;
+          prow(dst, np, d, k)[r] = v;
+        }
         prow(dst, np, d, 5)[r] = lw_r;
-        cum[r] = 1.0 / np;
       }
     } else {
-      for (int k = 0; k < 5; ++k)
-        for (int p = threadIdx.x; p < np; p += blockDim.x) prow(dst, np, d, k)[p] = prow(src, np, c, k)[p];
+#pragma unroll PER > 0 ? PER : 1
+      for (int i = 0; i < n; ++i) {
+        const int p = tid + i * bd;
+        if (p >= np) break;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) prow(dst, np, d, k)[p] = PER > 0 ? xr[i % kHeld][k] : prow(src, np, c, k)[p];
+        prow(dst, np, d, 5)[p] = s_l[p] - lse;
+      }
     }
-    __syncthreads();
-    write_moments(dst, np, d, cum, red, tot);
-    if (threadIdx.x == 0) {
+    write_moments<PER>(
+        dst, np, d,
+        [&](int i, int k) { return PER > 0 ? xr[i % kHeld][k] : prow(dst, np, d, k)[tid + i * bd]; },
+        [&](int i) { return resample ? w_r : cum[tid + i * bd]; }, red, tot);
+    if (tid == 0) {
       dst.lk[d] = src.lk[c];
       dst.lb[d] = src.lb[c];
       dst.logp[d] = src.logp[c];
@@ -571,13 +629,22 @@ void launch_particle_remap(const Model& md, const PartModel& pm, const CompTable
                            const uint32_t* newpos, const uint32_t* flag, const FrameDev* fs,
                            const unsigned* n_keep_dev, const uint32_t* upd_src, const uint32_t* upd_m,
                            const long long* upd_se, int cap_upd, const unsigned* n_upd_dev,
-                           const unsigned* n_surv_dev, unsigned* err, int grid, cudaStream_t s) {
-  // 64-thread blocks: several updates in flight per SM, each with short
-  // block reductions
-  launch_k(particle_remap_kernel, 4 * grid, 64, (size_t)pm.np * sizeof(double), s, md, pm, src, dst, newpos,
-           flag, fs, n_keep_dev, upd_src, upd_m, upd_se, cap_upd, n_upd_dev, n_surv_dev, err);
+                           const unsigned* n_surv_dev, unsigned* err, int grid, int h_max, cudaStream_t s) {
+  // a thread per four particles, which it then holds: several updates in
+  // flight per SM, each with short block reductions; a thread per two where
+  // few hypotheses make few updates, whose chains the frame waits for (above
+  // 1024 particles 64 threads, the particles in memory).  Update stage with 256
+  // particles, before and with 64 and 128 threads: convoy of ten (h_max 100)
+  // 42.6, 35.1 and 30.4 us; 200 vehicles (h_max 1000) 47.5, 39.6 and 41.9
+  const size_t smem = particle_remap_smem(pm.np);
+  int threads = pm.np <= 256 ? 64 : pm.np <= 512 ? 128 : pm.np <= 1024 ? 256 : 64;
+  if (h_max <= 256 && pm.np > threads && pm.np <= 512) threads *= 2;
+  auto k = pm.np <= 1024 ? particle_remap_kernel<4> : particle_remap_kernel<0>;
+  if (smem > 40 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  launch_k(k, 4 * grid, threads, smem, s, md, pm, src, dst, newpos, flag, fs, n_keep_dev, upd_src, upd_m, upd_se, cap_upd,
+           n_upd_dev, n_surv_dev, err);
 }
 
-int particle_remap_smem(int np) { return np * (int)sizeof(double); }
+int particle_remap_smem(int np) { return 2 * np * (int)sizeof(double); }
 
 }  // namespace glmb
