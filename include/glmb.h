@@ -237,6 +237,14 @@ glmb_status glmb_step(glmb_handle* h, const glmb_birth* births, int n_births, co
 glmb_status glmb_estimates(glmb_handle* h, glmb_track* out, int cap, int* n_out,
                            double* card_pmf, int pmf_cap);
 
+/* The same estimates where they lie: the tracks (n_out <= cap) and the
+ * cardinality distribution (pmf_n values) in the handle's result block, which
+ * stays where it is and holds them until the next call that steps, updates,
+ * prunes, resets, imports a state or destroys the handle.  For callers that
+ * copy the fields out themselves.  Errors: those of glmb_estimates. */
+glmb_status glmb_estimates_ref(glmb_handle* h, int cap, const glmb_track** tracks, int* n_out,
+                               const double** card_pmf, int* pmf_n);
+
 /* For each detection i of the last update, the total weight of retained
  * hypotheses that assign it to clutter (r_u[i], i < M <= cap). Synchronises. */
 glmb_status glmb_meas_assoc(glmb_handle* h, double* r_u, int cap);

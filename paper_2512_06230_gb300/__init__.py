@@ -170,7 +170,8 @@ def load() -> C.CDLL:
     sig = {
         "glmb_create": [P, P], "glmb_destroy": [P], "glmb_reset": [P],
         "glmb_predict": [P, P, I], "glmb_update": [P, P, I, I], "glmb_prune": [P],
-        "glmb_estimates": [P, P, I, P, P, I], "glmb_meas_assoc": [P, P, I],
+        "glmb_estimates": [P, P, I, P, P, I], "glmb_estimates_ref": [P, I, P, P, P, P],
+        "glmb_meas_assoc": [P, P, I],
         "glmb_get_info": [P, P], "glmb_export_state": [P, P, C.c_size_t, P],
         "glmb_import_state": [P, P, C.c_size_t],
         "glmb_get_hypotheses": [P, P, P, P, P, P, P, I, L, P],
@@ -461,22 +462,32 @@ class Filter:
     # ---- outputs ----
     def estimates(self, cap: int = 4096, pmf_cap: int = 4096):
         """MAP tracks (labels, existence, mean, cov) and the cardinality pmf."""
-        # the output buffers and their pointers are kept between calls (this
-        # runs once per frame; building ctypes pointers costs microseconds)
-        buf = getattr(self, "_est_buf", None)
-        if buf is None or len(buf[0]) < cap or len(buf[1]) < pmf_cap:
-            o, q, n = np.zeros(cap, TRACK_DTYPE), np.zeros(pmf_cap), C.c_int()
-            buf = (o, q, _ptr(o), _ptr(q), n, C.byref(n))
-            self._est_buf = buf
-        out, pmf, p_out, p_pmf, n, n_ref = buf
-        self._check(self.lib.glmb_estimates(self.h, p_out, cap, n_ref, p_pmf, pmf_cap))
+        # the records are read where the library keeps them and copied once
+        # (this runs once per frame: ctypes pointers and NumPy views of the
+        # result block, which does not move, are kept between calls)
+        ref = getattr(self, "_est_ref", None)
+        if ref is None:
+            p, n, q, m = C.c_void_p(), C.c_int(), C.c_void_p(), C.c_int()
+            ref = self._est_ref = [n, C.byref(p), C.byref(n), C.byref(q), C.byref(m), p, q, m, None, None]
+        n, rp, rn, rq, rm, p, q, m, tracks, dist = ref
+        self._check(self.lib.glmb_estimates_ref(self.h, cap, rp, rn, rq, rm))
+        if tracks is None:
+            rows = m.value   # a record and a cardinality for up to max_tracks tracks
+            tracks = np.ndarray((rows,), TRACK_DTYPE, (C.c_char * (rows * TRACK_DTYPE.itemsize)).from_address(p.value))
+            dist = np.ndarray((rows,), np.float64, (C.c_char * (8 * rows)).from_address(q.value))
+            ref[8], ref[9] = tracks, dist
         k, dx = n.value, self.dx
-        t = out[:k].copy()
+        t = tracks[:k].copy()
+        if pmf_cap <= len(dist):
+            pmf = dist[:pmf_cap].copy()
+        else:
+            pmf = np.zeros(pmf_cap)
+            pmf[: len(dist)] = dist
         # every field is a view of this call's own copy of the records;
         # labels: (k, 2) of (label_k, label_b), the records' first two words
         words = t.view(np.uint32).reshape(k, TRACK_DTYPE.itemsize // 4)
         return dict(n=k, labels=words[:, :2], r=t["r"], mean=t["mean"][:, :dx],
-                    cov=t["cov"][:, : dx * dx].reshape(k, dx, dx), pmf=pmf[:pmf_cap].copy())
+                    cov=t["cov"][:, : dx * dx].reshape(k, dx, dx), pmf=pmf)
 
     STAGES = ("predict", "table", "expand", "select", "materialize", "update_gc", "estimates")
 

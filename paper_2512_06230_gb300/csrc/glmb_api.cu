@@ -1729,12 +1729,11 @@ glmb_status glmb_get_info(glmb_handle* h, glmb_info* info) {
   return GLMB_OK;
 }
 
-glmb_status glmb_estimates(glmb_handle* h, glmb_track* out, int cap, int* n_out, double* card_pmf,
-                           int pmf_cap) {
-  if (!h || !n_out || (cap > 0 && !out)) return GLMB_E_INVALID;
+glmb_status glmb_estimates_ref(glmb_handle* h, int cap, const glmb_track** tracks, int* n_out,
+                               const double** card_pmf, int* pmf_n) {
+  if (!h || !tracks || !n_out || !card_pmf || !pmf_n) return GLMB_E_INVALID;
   if (h->stage >= 2) return fail(h, GLMB_E_STATE, "estimates: call glmb_prune (or glmb_step_finish) first");
   cudaStream_t s = h->stream;
-  const int pcap = h->max_tracks + 1;
   if (h->est_gen != h->gen) {   // not computed with this state's step
     enqueue_estimates(h, h->hyps[h->hcur], h->comps[h->cur], nullptr, h->H);
     CU(cudaGetLastError());
@@ -1742,16 +1741,27 @@ glmb_status glmb_estimates(glmb_handle* h, glmb_track* out, int cap, int* n_out,
     CU(cudaStreamSynchronize(s));
     h->est_gen = h->gen;
   }
-  int nb[2];
-  std::memcpy(nb, h->h_est, sizeof nb);
-  const int nhat = nb[0];
+  int nhat;
+  std::memcpy(&nhat, h->h_est, sizeof nhat);
   *n_out = nhat;
-  const double* pmf = (const double*)(h->h_est + h->est_off_pmf);
-  if (card_pmf)
-    for (int k = 0; k < pmf_cap; ++k) card_pmf[k] = k < pcap ? pmf[k] : 0.0;
+  *tracks = (const glmb_track*)(h->h_est + h->est_off_tr);
+  *card_pmf = (const double*)(h->h_est + h->est_off_pmf);
+  *pmf_n = h->max_tracks + 1;
   if (nhat > cap) return fail(h, GLMB_E_CAPACITY, "estimates: %d tracks > cap %d", nhat, cap);
-  if (nhat > 0) std::memcpy(out, h->h_est + h->est_off_tr, (size_t)nhat * sizeof(glmb_track));
   return GLMB_OK;
+}
+
+glmb_status glmb_estimates(glmb_handle* h, glmb_track* out, int cap, int* n_out, double* card_pmf,
+                           int pmf_cap) {
+  if (!h || !n_out || (cap > 0 && !out)) return GLMB_E_INVALID;
+  const glmb_track* tracks;
+  const double* pmf = nullptr;
+  int pcap = 0;
+  const glmb_status st = glmb_estimates_ref(h, cap, &tracks, n_out, &pmf, &pcap);
+  if (pmf && card_pmf)
+    for (int k = 0; k < pmf_cap; ++k) card_pmf[k] = k < pcap ? pmf[k] : 0.0;
+  if (st == GLMB_OK && *n_out > 0) std::memcpy(out, tracks, (size_t)*n_out * sizeof(glmb_track));
+  return st;
 }
 
 glmb_status glmb_meas_assoc(glmb_handle* h, double* r_u, int cap) {
