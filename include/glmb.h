@@ -391,7 +391,7 @@ glmb_status glmb_get_tuning(glmb_handle* h, glmb_tuning* t);
  *                          large plan leave an SM fewer than 16 warps, or
  *                          when a plan of 768 slots or more has too few
  *                          children to fill the GPU's warps).
- * Default 0: shared-memory staging when eight staging CTAs fit on an SM
+ * Default 0: shared-memory staging when sixteen images fit on an SM
  * (else in global memory, with as much of the staging's scratch in shared
  * memory as fits), one thread per child once the children give every SM
  * four warps. */

@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
     ("tiny", 40, 100, {}),           # one block, at most 4000 children
     ("tiny", 100, 150, {}),          # one block, keys read again
     ("tiny", 20, 823, {}),           # past one block's children by a few
+    ("tiny", 4, 5000, {}),           # duplicate marking with one table
+    ("tiny", 4, 1500, {}),           # tables of 48 KB
     ("sweep_N50", 60, 100, {}),      # 3-D, cap binds
     ("sweep_N50", 400, 331, {}),     # cluster, keys read again, cap binds
     ("sweep_N50", 3000, 100, {}),    # cluster, the cap does not bind at first
