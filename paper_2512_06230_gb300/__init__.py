@@ -365,6 +365,7 @@ class Filter:
         if getattr(self, "h", None):
             self.lib.glmb_destroy(self.h)
             self.h = None
+            self._est_ref = None   # views of the freed result block
 
     def __del__(self):
         try:
