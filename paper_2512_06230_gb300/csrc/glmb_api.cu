@@ -1252,6 +1252,7 @@ glmb_status finish_frame(glmb_handle* h, bool copies_enqueued = false, bool est_
   auto abandon = [&](glmb_status st, const char* msg) {
     h->frame -= 1;
     h->stage = 0;
+    h->est_gen = -1;   // the frame's estimates may have replaced the state's in the result block
     return fail(h, st, "prune: %s", msg);
   };
   glmb_status st;
