@@ -622,6 +622,9 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
   cudaDeviceGetAttribute(&h->smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, dev);
   expand_init(h->smem_limit);
+  table_init(h->smem_limit);
+  particle_init(h->smem_limit);
+  prune_init(h->smem_limit);
   if (c.stream) {
     h->stream = (cudaStream_t)c.stream;
   } else {

@@ -31,6 +31,21 @@ inline void launch_k(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
   ++g_launches;
 }
 
+// Lets kernel k use all the shared memory a block may have (`limit`, the
+// device's opt-in size; its static part counts too).  Done once, when a filter
+// is created: a launch that set the attribute to its own need would take it
+// away from a larger filter's launch in another thread.
+template <typename K>
+inline void opt_in_smem(K* k, int limit) {
+  cudaFuncAttributes fa{};
+  if (cudaFuncGetAttributes(&fa, k) == cudaSuccess)
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit - (int)fa.sharedSizeBytes);
+}
+// the kernels of a file whose shared memory follows the filter's sizes
+void table_init(int smem_limit);
+void particle_init(int smem_limit);
+void prune_init(int smem_limit);
+
 // ---- prediction, births, table (kernels_table.cu) ----
 // Sizes come from the device FrameDev; grid is the number of blocks of a
 // grid-stride launch.

@@ -2037,8 +2037,6 @@ void launch_dedup(const FrameDev* fs, int HU, long long* child_key, const unsign
   while (ts < 2 * HU) ts <<= 1;
   const int tables = 2 * ts * 12 <= 96 * 1024 ? 2 : 1;   // (8192 draws: 196 KB a table)
   const int smem = tables * ts * 12;
-  if (smem > 40 * 1024)   // (the block holds static shared memory too)
-    cudaFuncSetAttribute(dedup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   launch_k(dedup_kernel, std::min(grid, kMaxLseParts), kDedupThreads, smem, s, fs, HU, child_key, child_hash, child_status,
            err, w.part_max, w.part_sum, w.part_cnt, tables);
 }
@@ -2067,6 +2065,7 @@ static KernelFn warp_fn(int dz, bool mat, bool grp = false, bool notes = false) 
 static KernelFn prep_fn(int dz) { return dz == 2 ? mat_prep_kernel<2> : mat_prep_kernel<3>; }
 
 void expand_init(int smem_limit) {
+  opt_in_smem(dedup_kernel, smem_limit);
   for (int dz = 2; dz <= 3; ++dz) {
     cudaFuncSetAttribute(stage_fn(dz, true, false), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
     for (int wide = 0; wide < 2; ++wide)

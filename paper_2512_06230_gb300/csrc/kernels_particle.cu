@@ -614,6 +614,11 @@ __global__ void __launch_bounds__(kPartThreads, 2) particle_remap_kernel(
 
 }  // namespace
 
+void particle_init(int smem_limit) {
+  opt_in_smem(particle_remap_kernel<4>, smem_limit);
+  opt_in_smem(particle_remap_kernel<0>, smem_limit);
+}
+
 void launch_particle_predict(const Model& md, const PartModel& pm, const CompTable& src, const CompTable& dst,
                              const FrameDev* fs, const double* births_dev, int grid, cudaStream_t s) {
   launch_k(particle_step_kernel, grid, kPartThreads, 0, s, md, pm, src, dst, fs, births_dev);
@@ -640,7 +645,6 @@ void launch_particle_remap(const Model& md, const PartModel& pm, const CompTable
   int threads = pm.np <= 256 ? 64 : pm.np <= 512 ? 128 : pm.np <= 1024 ? 256 : 64;
   if (h_max <= 256 && pm.np > threads && pm.np <= 512) threads *= 2;
   auto k = pm.np <= 1024 ? particle_remap_kernel<4> : particle_remap_kernel<0>;
-  if (smem > 40 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   launch_k(k, 4 * grid, threads, smem, s, md, pm, src, dst, newpos, flag, fs, n_keep_dev, upd_src, upd_m, upd_se, cap_upd,
            n_upd_dev, n_surv_dev, err);
 }

@@ -961,14 +961,11 @@ __global__ void __launch_bounds__(kEstThreads) est_tracks_kernel(const __grid_co
 // beside the cardinality bins; else a second launch spreads the tracks over
 // blocks (N = 1000, one block for all tracks: 52 us).
 constexpr int kEstFuseTracks = 512;
+void prune_init(int smem_limit) { opt_in_smem(est_sums_kernel, smem_limit); }
+
 void launch_estimates(EstArgs a, int H_bound, int n_sm, cudaStream_t s) {
   a.fused = H_bound <= 4096 && a.pcap <= kEstFuseTracks ? 1 : 0;
   const int words = std::max(std::min(kEstPriv, a.ct.cap), a.fused ? 2 * a.pcap : a.pcap);
-  static int attr_words = 48 * 1024 / 8;   // the limit only grows (graphs of larger filters stay valid)
-  if (words > attr_words) {
-    cudaFuncSetAttribute(est_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, words * 8);
-    attr_words = words;
-  }
   // block 0: the cardinality; blocks 1..: one warp per hypothesis
   const int blocks = std::max(1, std::min((H_bound + 31) / 32, n_sm));
   launch_k(est_sums_kernel, 1 + blocks, 1024, (size_t)words * 8, s, a);

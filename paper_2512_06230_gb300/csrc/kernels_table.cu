@@ -378,11 +378,15 @@ __global__ void __launch_bounds__(32 * kTabWarps)
   }
 }
 
+void table_init(int smem_limit) {
+  opt_in_smem(table_kernel<2>, smem_limit);
+  opt_in_smem(table_kernel<3>, smem_limit);
+}
+
 void launch_table(TableArgs a, int cap_meas, int grid, cudaStream_t s) {
   a.words = table_words(cap_meas);
   const int smem = kTabWarps * a.words * (int)sizeof(uint32_t);
   auto k = a.md.dz == 2 ? table_kernel<2> : table_kernel<3>;
-  if (smem > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   launch_k(k, grid, 32 * kTabWarps, smem, s, a);
 }
 

@@ -1,4 +1,6 @@
-"""Estimates after a frame that was abandoned: those of the frame before."""
+"""Estimates where their handling can go wrong: after a frame that was
+abandoned, and at result blocks around 48 KB (where the launch's shared memory
+passes the default limit only with the kernel's static part)."""
 from __future__ import annotations
 
 import numpy as np
@@ -50,3 +52,28 @@ def test_abandoned_frame_keeps_the_estimates(glmb, how):
     assert _same(g.estimates(), before)
     f.close()
     g.close()
+
+
+def _small(max_tracks, **kw):
+    rng = np.random.default_rng(11)
+    births = [(0.7, np.concatenate([rng.uniform(0, 100, 2), rng.normal(size=2)]), np.diag([9.0, 9.0, 1.0, 1.0]))
+              for _ in range(6)]
+    Z = np.array([b[1][:2] for b in births[:5]], np.float32)
+    cfg = dict(dim_x=4, dim_z=2, dt=1.0, q=1.0, R=4.0 * np.eye(2), p_s=0.99, p_d=0.9, lambda_d=1.0, clutter_rate=2.0,
+               volume=1e4, gate=18.4, h_max=4, h_up=8, tau=1e-6, seed=3, score_mode=0, max_tracks=max_tracks,
+               max_meas=64, max_births=8, max_components=256, max_pairs=4096)
+    cfg.update(kw)
+    return cfg, births, Z
+
+
+@pytest.mark.parametrize("max_tracks", [511, 512, 4095, 4096, 6045, 6046, 6100, 6143, 6144, 6200, 20000])
+def test_result_blocks_of_every_size(glmb, max_tracks):
+    cfg, births, Z = _small(max_tracks)
+    ref, f = glmb.Filter(_small(64)[0]), glmb.Filter(cfg)
+    for k in range(3):
+        for x in (ref, f):
+            x.step(births if k == 0 else [], Z)
+        a, b = ref.estimates(pmf_cap=65), f.estimates(pmf_cap=65)
+        assert a["n"] > 0 and _same(a, b)
+    ref.close()
+    f.close()
