@@ -264,6 +264,7 @@ bool halloc(glmb_handle* h, T** p, long long n) {
   void* q = nullptr;
   if (n <= 0) n = 1;
   if (cudaMallocHost(&q, (size_t)n * sizeof(T)) != cudaSuccess) return false;
+  std::memset(q, 0, (size_t)n * sizeof(T));   // as the device's: results are never read before they are written
   h->host_allocs.push_back(q);
   *p = (T*)q;
   return true;
@@ -1527,7 +1528,17 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
       cudaGraph_t graph = nullptr;
       cudaGraphExec_t exec = nullptr;
       const auto t_cap = std::chrono::steady_clock::now();
-      CU(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+      const long long launches = g_launches;
+      // a capture that is not whole is not kept: the frame did not run
+      auto refuse = [&](const char* what, cudaError_t e) {
+        if (graph) cudaGraphDestroy(graph);
+        cudaGetLastError();
+        g_launches = launches;
+        h->frame -= 1;
+        return fail(h, GLMB_E_CUDA, "step: %s: %s", what, cudaGetErrorString(e));
+      };
+      const cudaError_t be = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+      if (be != cudaSuccess) return refuse("graph capture", be);
       h->capturing = true;
       // zero scalars, sizes and host detections (and the particle model's
       // births) in one copy of the input block
@@ -1551,7 +1562,10 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
       else
         enqueue_results(h);
       h->capturing = false;
-      CU(cudaStreamEndCapture(h->stream, &graph));
+      const cudaError_t le = cudaGetLastError();   // a launch that was refused left no node
+      const cudaError_t ce = cudaStreamEndCapture(h->stream, &graph);
+      if (le != cudaSuccess || ce != cudaSuccess)
+        return refuse("graph capture", le != cudaSuccess ? le : ce);
       size_t n_nodes = 0;
       cudaGraphGetNodes(graph, nullptr, &n_nodes);
       std::vector<cudaGraphNode_t> nodes(n_nodes);
@@ -1578,10 +1592,7 @@ glmb_status glmb_step_enqueue(glmb_handle* h, const glmb_birth* births, int n_bi
         key_nodes.push_back(kn);
       }
       const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
-      if (ie != cudaSuccess) {
-        cudaGraphDestroy(graph);
-        return fail(h, GLMB_E_CUDA, "step: graph instantiation: %s", cudaGetErrorString(ie));
-      }
+      if (ie != cudaSuccess) return refuse("graph instantiation", ie);
       if (h->graphs.size() >= 32) {
         // evict the least recently replayed graph
         int lru = 0;

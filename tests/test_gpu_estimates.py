@@ -1,6 +1,7 @@
 """Estimates where their handling can go wrong: after a frame that was
-abandoned, and at result blocks around 48 KB (where the launch's shared memory
-passes the default limit only with the kernel's static part)."""
+abandoned, at result blocks around 48 KB (where the launch's shared memory
+passes the default limit only with the kernel's static part), and where the
+estimates' kernel cannot be launched at all."""
 from __future__ import annotations
 
 import numpy as np
@@ -77,3 +78,25 @@ def test_result_blocks_of_every_size(glmb, max_tracks):
         assert a["n"] > 0 and _same(a, b)
     ref.close()
     f.close()
+
+
+def test_frame_whose_estimates_cannot_be_launched(glmb):
+    """More tracks than a block can count in shared memory: each step reports
+    the refused launch and leaves the state, and frames without the estimates
+    run."""
+    cfg, births, Z = _small(40000)
+    f, ref = glmb.Filter(cfg), glmb.Filter(_small(64)[0])
+    frame = f.info()["frame"]
+    for _ in range(3):
+        with pytest.raises(glmb.GlmbError) as ei:
+            f.step(births, Z)
+        assert ei.value.status == 4          # GLMB_E_CUDA
+        info = f.info()
+        assert info["frame"] == frame and info["n_graph_captures"] == 0 and info["n_graph_launches"] == 0
+    f.set_step_estimates(False)
+    for k in range(2):
+        f.step(births if k == 0 else [], Z)
+        ref.step(births if k == 0 else [], Z)
+    assert f.export_state() == ref.export_state()
+    f.close()
+    ref.close()
