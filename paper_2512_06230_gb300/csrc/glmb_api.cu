@@ -106,7 +106,8 @@ struct glmb_handle {
   unsigned char* notes = nullptr;
   PruneWork pw{};
   unsigned long long* hkeys = nullptr;
-  uint32_t* hvals = nullptr;
+  uint32_t* hvals = nullptr;        // (between frames the rows of the inspection calls)
+  long long row_words = 0;          // its words: one per slot of the table, or more for those calls
   uint32_t* upd_src = nullptr;
   uint32_t* upd_slot = nullptr;   // update id -> hash slot
   unsigned* d_hprev = nullptr;     // updates the last materialisation inserted
@@ -553,6 +554,7 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
   h->cap_upd = std::min(h->cap_entries, h->cap_comp);
   const long long hcap = next_pow2(2 * h->cap_entries);
   h->hmask = (uint32_t)(hcap - 1);
+  h->row_words = std::max(hcap, 1LL << 15);
   if (h->cap_comp >= (1LL << 31) || hcap > (1LL << 31) || h->cap_pairs >= (1LL << 32)) {
     delete h;
     return GLMB_E_INVALID;
@@ -658,7 +660,7 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
             dalloc(h, &h->pw.flags, h->cap_children) &&
             dalloc(h, &h->pw.flags_tmp, scan_tmp_elems(h->cap_children)) &&
             dalloc(h, &h->pw.surv_idx, h->cap_h) &&
-            dalloc(h, &h->hkeys, hcap) && dalloc(h, &h->hvals, hcap) &&
+            dalloc(h, &h->hkeys, hcap) && dalloc(h, &h->hvals, h->row_words) &&
             dalloc(h, &h->upd_src, h->cap_upd) && dalloc(h, &h->upd_m, h->cap_upd) &&
             dalloc(h, &h->upd_slot, h->cap_upd) && dalloc(h, &h->d_hprev, 1) &&
             dalloc(h, &h->upd_se, h->cap_upd * dz) && dalloc(h, &h->gc_flag, h->cap_comp) &&
@@ -1316,40 +1318,32 @@ glmb_status finish_frame(glmb_handle* h, bool copies_enqueued = false, bool est_
   return GLMB_OK;
 }
 
-extern "C++" {
-// Pairs of table P in table order (component, then detection): their storage
-// positions, and the CSR offsets by component.
-glmb_status pair_order(glmb_handle* h, const PairTable& P, std::vector<uint32_t>& csr, std::vector<uint32_t>& at) {
-  const int T = h->T_work;
-  unsigned K32 = 0;
-  CU(cudaMemcpy(&K32, P.total, sizeof K32, cudaMemcpyDeviceToHost));
-  std::vector<uint32_t> cnt(std::max(T, 1)), ptr(std::max(T, 1));
-  if (T > 0) {
-    CU(cudaMemcpy(cnt.data(), P.cnt, (size_t)T * 4, cudaMemcpyDeviceToHost));
-    CU(cudaMemcpy(ptr.data(), P.ptr, (size_t)T * 4, cudaMemcpyDeviceToHost));
-  }
-  csr.assign((size_t)T + 1, 0u);
-  at.clear();
-  at.reserve(K32);
-  for (int c = 0; c < T; ++c) {
-    for (uint32_t j = 0; j < cnt[c]; ++j) at.push_back(ptr[c] + j);
-    csr[c + 1] = (uint32_t)at.size();
-  }
+// The inspection calls' copies of a pair table, in table order (component,
+// then detection).  Their work areas are the regeneration's, which holds
+// nothing between frames: the scan of the counts in gc_newpos, the rows on
+// their way to the host in hvals.
+glmb_status pair_count(glmb_handle* h, const PairTable& P, uint32_t& n) {
+  CU(cudaMemcpy(&n, P.total, sizeof n, cudaMemcpyDeviceToHost));
   return GLMB_OK;
 }
-
-// rows of `width` device elements at the storage positions `at`, in that
-// order, `stride` elements apart in out (positions beyond the n stored rows,
-// of a table that overflowed, give zeros)
-template <typename T>
-glmb_status gather_pairs(glmb_handle* h, T* out, int stride, const T* src, int width, const std::vector<uint32_t>& at,
-                         long long n) {
-  std::vector<T> col((size_t)n * width);
-  CU(cudaMemcpy(col.data(), src, col.size() * sizeof(T), cudaMemcpyDeviceToHost));
-  for (size_t k = 0; k < at.size(); ++k)
-    for (int a = 0; a < width; ++a) out[k * stride + a] = at[k] < n ? col[(size_t)at[k] * width + a] : T(0);
-  return GLMB_OK;
+void pair_order(glmb_handle* h, const PairTable& P) {
+  scan_u32(P.cnt, h->gc_newpos, &h->d_fs->T, 1, std::max(h->T_work, 1), nullptr, false, h->scan_tmp32, h->scan_cap32,
+           h->d_scal + S_ERR, h->stream);
 }
+// the first n rows, after pair_order: out[k * width + a], element a of pair p
+// at src[p * ps + a * as]
+glmb_status copy_pairs(glmb_handle* h, const PairTable& P, void* out, const void* src, int bytes, long long ps,
+                       long long as, int width, long long n) {
+  const long long step = h->row_words * 4 / (width * bytes);
+  for (long long k = 0; k < n; k += step) {
+    const long long m = std::min(step, n - k);
+    launch_pair_rows(P, h->gc_newpos, h->T_work, src, bytes, ps, as, width, h->hvals, k, m, h->stream);
+    CU(cudaGetLastError());
+    CU(cudaMemcpyAsync((unsigned char*)out + (size_t)k * width * bytes, h->hvals, (size_t)m * width * bytes,
+                       cudaMemcpyDeviceToHost, h->stream));
+  }
+  CU(cudaStreamSynchronize(h->stream));
+  return GLMB_OK;
 }
 
 }  // namespace
@@ -2129,21 +2123,24 @@ glmb_status glmb_get_pairs(glmb_handle* h, uint32_t* comp_ptr, uint32_t* meas, f
   if (!h->have_update) return fail(h, GLMB_E_STATE, "get_pairs: no update");
   CU(cudaStreamSynchronize(h->stream));
   const int T = h->T_work, dz = h->md.dz;
-  std::vector<uint32_t> csr, at;
-  glmb_status st = pair_order(h, h->pt, csr, at);
+  const PairTable& P = h->pt;
+  uint32_t K32 = 0;
+  glmb_status st = pair_count(h, P, K32);
   if (st != GLMB_OK) return st;
-  const long long K = std::min<long long>((long long)at.size(), h->cap_pairs);
+  const long long K = std::min<long long>(K32, h->cap_pairs);
   *n_pairs = K;
   if (T + 1 > cap_comp || K > cap_pairs) return fail(h, GLMB_E_CAPACITY, "get_pairs: caps");
-  if (comp_ptr) std::memcpy(comp_ptr, csr.data(), (size_t)(T + 1) * 4);
-  at.resize(K);
+  pair_order(h, P);
+  if (comp_ptr) {
+    CU(cudaMemcpyAsync(comp_ptr, h->gc_newpos, (size_t)T * 4, cudaMemcpyDeviceToHost, h->stream));
+    CU(cudaStreamSynchronize(h->stream));
+    comp_ptr[T] = K32;
+  }
   if (K == 0) return GLMB_OK;
-  if (meas && (st = gather_pairs(h, meas, 1, h->pt.meas, 1, at, K)) != GLMB_OK) return st;
-  if (logC && (st = gather_pairs(h, logC, 1, h->pt.logC, 1, at, K)) != GLMB_OK) return st;
-  if (q && (st = gather_pairs(h, q, 1, h->pt.q, 1, at, K)) != GLMB_OK) return st;
-  if (e)
-    for (int a = 0; a < dz; ++a)
-      if ((st = gather_pairs(h, e + a, dz, h->pt.e + (size_t)a * h->cap_pairs, 1, at, K)) != GLMB_OK) return st;
+  if (meas && (st = copy_pairs(h, P, meas, P.meas, 4, 1, 0, 1, K)) != GLMB_OK) return st;
+  if (logC && (st = copy_pairs(h, P, logC, P.logC, 4, 1, 0, 1, K)) != GLMB_OK) return st;
+  if (q && (st = copy_pairs(h, P, q, P.q, 4, 1, 0, 1, K)) != GLMB_OK) return st;
+  if (e) return copy_pairs(h, P, e, P.e, 4, 1, P.cap_pairs, dz, K);
   return GLMB_OK;
 }
 
@@ -2232,17 +2229,17 @@ glmb_status glmb_gate_features(glmb_handle* h, float* X, int64_t cap, int64_t* n
   if (!h->have_update) return fail(h, GLMB_E_STATE, "gate_features: no update");
   CU(cudaStreamSynchronize(h->stream));
   const PairTable& P0 = pregate_table(h);
-  std::vector<uint32_t> csr, at;
-  glmb_status st = pair_order(h, P0, csr, at);
+  uint32_t K32 = 0;
+  const glmb_status st = pair_count(h, P0, K32);
   if (st != GLMB_OK) return st;
-  *n = (int64_t)at.size();
+  *n = K32;
   if (*n > cap)
     return fail(h, GLMB_E_CAPACITY, "gate_features: %lld pairs, cap %lld", (long long)*n, (long long)cap);
   if (*n == 0) return GLMB_OK;
   if (!h->gate_X && !dalloc(h, &h->gate_X, h->cap_pairs * 5)) return fail(h, GLMB_E_OOM, "gate_features: scratch");
   launch_gate_features(h->md, h->comps[1 - h->cur], P0, h->d_fs, h->gate_X, h->cap_pairs, 2 * h->n_sm, h->stream);
-  CU(cudaStreamSynchronize(h->stream));
-  return gather_pairs(h, X, 5, h->gate_X, 5, at, std::min<long long>(*n, h->cap_pairs));
+  pair_order(h, P0);
+  return copy_pairs(h, P0, X, h->gate_X, 4, 5, 1, 5, *n);
 }
 
 glmb_status glmb_gate_logits(glmb_handle* h, float* logit, int64_t cap, int64_t* n) {
@@ -2250,13 +2247,15 @@ glmb_status glmb_gate_logits(glmb_handle* h, float* logit, int64_t cap, int64_t*
   if (!h->have_update || h->gate_mode_frame == GLMB_GATE_OFF)
     return fail(h, GLMB_E_STATE, "gate_logits: no update with the gate on");
   CU(cudaStreamSynchronize(h->stream));
-  std::vector<uint32_t> csr, at;
-  glmb_status st = pair_order(h, pregate_table(h), csr, at);
+  const PairTable& P0 = pregate_table(h);
+  uint32_t K32 = 0;
+  const glmb_status st = pair_count(h, P0, K32);
   if (st != GLMB_OK) return st;
-  *n = (int64_t)at.size();
+  *n = K32;
   if (*n > cap) return fail(h, GLMB_E_CAPACITY, "gate_logits: cap");
   if (*n == 0) return GLMB_OK;
-  return gather_pairs(h, logit, 1, h->gate_logit, 1, at, std::min<long long>(*n, h->cap_pairs));
+  pair_order(h, P0);
+  return copy_pairs(h, P0, logit, h->gate_logit, 4, 1, 0, 1, *n);
 }
 
 glmb_status glmb_gate_usage(glmb_handle* h, uint8_t* used, int64_t cap_pairs, uint8_t* hyp_flag, int cap_h,
@@ -2266,10 +2265,9 @@ glmb_status glmb_gate_usage(glmb_handle* h, uint8_t* used, int64_t cap_pairs, ui
     return fail(h, GLMB_E_STATE, "gate_usage: no pruned frame");
   if (h->gate_mode_frame == GLMB_GATE_PRUNE) return fail(h, GLMB_E_STATE, "gate_usage: the gate pruned the table");
   CU(cudaStreamSynchronize(h->stream));
-  std::vector<uint32_t> csr, at;
-  glmb_status st = pair_order(h, h->pt, csr, at);
+  uint32_t K32 = 0;
+  const glmb_status st = pair_count(h, h->pt, K32);
   if (st != GLMB_OK) return st;
-  const uint32_t K32 = (uint32_t)at.size();
   *n_pairs = K32;
   *n_hyp = h->H;
   if ((used && (int64_t)K32 > cap_pairs) || (hyp_flag && h->H > cap_h))
@@ -2285,7 +2283,10 @@ glmb_status glmb_gate_usage(glmb_handle* h, uint8_t* used, int64_t cap_pairs, ui
                     h->gate_used, h->gate_hflag, capT, std::max(1, std::min(h->H, 8 * h->n_sm)), h->stream);
   if (hyp_flag && h->H) CU(cudaMemcpyAsync(hyp_flag, h->gate_hflag, (size_t)h->H, cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
-  if (used && K32) return gather_pairs(h, used, 1, h->gate_used, 1, at, std::min<long long>(K32, h->cap_pairs));
+  if (used && K32) {
+    pair_order(h, h->pt);
+    return copy_pairs(h, h->pt, used, h->gate_used, 1, 1, 0, 1, K32);
+  }
   return GLMB_OK;
 }
 

@@ -74,6 +74,12 @@ struct TableArgs {
   int cap_upd;
 };
 void launch_table(TableArgs a, int cap_meas, int grid, cudaStream_t s);
+// rows [k0, k0 + n) of a pair table in table order (component, then detection)
+// into dst: element a of pair p is src[p * ps + a * as], a < width (1 or 4
+// bytes each); csr: exclusive scan of pt.cnt over the T components.  A pair
+// beyond the table's capacity gives zeros.
+void launch_pair_rows(const PairTable& pt, const uint32_t* csr, int T, const void* src, int bytes, long long ps,
+                      long long as, int width, void* dst, long long k0, long long n, cudaStream_t s);
 void launch_parent_stats(const HypTable& hp, const FrameDev* fs, const PairTable& pt,
                          unsigned* max_T, unsigned* max_K, int grid, cudaStream_t s);
 

@@ -378,6 +378,37 @@ __global__ void __launch_bounds__(32 * kTabWarps)
   }
 }
 
+// Pairs lie where their component's piece was taken; the inspection calls give
+// them in table order.  A thread per row finds its component by bisection in
+// the scan of the counts (in L1 after the first rows) and copies the row.
+template <typename T>
+__global__ void __launch_bounds__(256) pair_rows_kernel(PairTable pt, const uint32_t* __restrict__ csr, int n_comp,
+                                                        const T* __restrict__ src, long long ps, long long as, int width,
+                                                        T* __restrict__ dst, long long k0, long long n) {
+  pdl_enter();
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const uint32_t k = (uint32_t)(k0 + i);
+    int lo = 0, hi = n_comp;   // the last component that starts at or before k
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (csr[mid] <= k) lo = mid; else hi = mid;
+    }
+    const long long p = (long long)pt.ptr[lo] + (k - csr[lo]);
+    for (int a = 0; a < width; ++a) dst[i * width + a] = p < pt.cap_pairs ? src[p * ps + a * as] : T(0);
+  }
+}
+
+void launch_pair_rows(const PairTable& pt, const uint32_t* csr, int T, const void* src, int bytes, long long ps,
+                      long long as, int width, void* dst, long long k0, long long n, cudaStream_t s) {
+  const int grid = (int)std::min((n + 255) / 256, 4096LL);
+  if (bytes == 1)
+    launch_k(pair_rows_kernel<uint8_t>, grid, 256, 0, s, pt, csr, T, (const uint8_t*)src, ps, as, width, (uint8_t*)dst,
+             k0, n);
+  else
+    launch_k(pair_rows_kernel<uint32_t>, grid, 256, 0, s, pt, csr, T, (const uint32_t*)src, ps, as, width,
+             (uint32_t*)dst, k0, n);
+}
+
 void table_init(int smem_limit) {
   opt_in_smem(table_kernel<2>, smem_limit);
   opt_in_smem(table_kernel<3>, smem_limit);
