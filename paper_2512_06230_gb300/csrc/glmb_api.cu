@@ -837,7 +837,8 @@ glmb_status enqueue_predict(glmb_handle* h, const Plan& p) {
 
 // fuse: the table kernel predicts the components it gates (a frame graph
 // without enqueue_predict), from the pinned birth records
-glmb_status enqueue_table(glmb_handle* h, const Plan& p, bool fuse = false) {
+// (place: see TableArgs)
+glmb_status enqueue_table(glmb_handle* h, const Plan& p, bool fuse = false, const uint32_t* place = nullptr) {
   const CompTable& B = h->comps[1 - h->cur];
   const int T = h->T_work;
   prof_begin(h, kStageTable);
@@ -854,6 +855,7 @@ glmb_status enqueue_table(glmb_handle* h, const Plan& p, bool fuse = false) {
   ta.fs = h->d_fs;
   ta.births = fuse ? h->h_births : h->d_births;
   ta.fuse = fuse ? 1 : 0;
+  ta.place = place;
   ta.n_fp64 = h->d_scal + S_FP64;
   ta.err = h->d_scal + S_ERR;
   ta.hkeys = h->hkeys;
@@ -1251,6 +1253,47 @@ glmb_status clear_hash_if_dirty(glmb_handle* h) {
   return GLMB_OK;
 }
 
+// The inspection calls' copies of a pair table, in table order (component,
+// then detection).  Their work areas are the regeneration's, which holds
+// nothing between frames: the scan of the counts in gc_newpos, the rows on
+// their way to the host in hvals.
+glmb_status pair_count(glmb_handle* h, const PairTable& P, uint32_t& n) {
+  CU(cudaMemcpy(&n, P.total, sizeof n, cudaMemcpyDeviceToHost));
+  return GLMB_OK;
+}
+void pair_order(glmb_handle* h, const PairTable& P) {
+  scan_u32(P.cnt, h->gc_newpos, &h->d_fs->T, 1, std::max(h->T_work, 1), nullptr, false, h->scan_tmp32, h->scan_cap32,
+           h->d_scal + S_ERR, h->stream);
+}
+// the first n rows, after pair_order: out[k * width + a], element a of pair p
+// at src[p * ps + a * as]
+glmb_status copy_pairs(glmb_handle* h, const PairTable& P, void* out, const void* src, int bytes, long long ps,
+                       long long as, int width, long long n) {
+  const long long step = h->row_words * 4 / (width * bytes);
+  for (long long k = 0; k < n; k += step) {
+    const long long m = std::min(step, n - k);
+    launch_pair_rows(P, h->gc_newpos, h->T_work, src, bytes, ps, as, width, h->hvals, k, m, h->stream);
+    CU(cudaGetLastError());
+    CU(cudaMemcpyAsync((unsigned char*)out + (size_t)k * width * bytes, h->hvals, (size_t)m * width * bytes,
+                       cudaMemcpyDeviceToHost, h->stream));
+  }
+  CU(cudaStreamSynchronize(h->stream));
+  return GLMB_OK;
+}
+
+// A frame with more pairs than the table holds fails, but its first pairs can
+// be inspected: which ones the table kept is a matter of the pieces' order, so
+// they are written again in table order, while the detections are there.
+glmb_status order_overflow(glmb_handle* h, const Plan& p) {
+  const bool prune = h->gate_mode_frame == GLMB_GATE_PRUNE;
+  pair_order(h, prune ? h->pt_full : h->pt);
+  CU(cudaMemsetAsync(h->d_scal + S_FP64, 0, sizeof(unsigned), h->stream));   // counted again
+  if (prune) CU(cudaMemsetAsync(h->d_scal + S_K, 0, sizeof(unsigned), h->stream));
+  const glmb_status st = enqueue_table(h, p, false, h->gc_newpos);
+  CU(cudaStreamSynchronize(h->stream));
+  return st;
+}
+
 // results: the counters were copied by the frame's launches when
 // copies_enqueued (with the estimates when est_enqueued); redo, abandon or
 // commit
@@ -1289,6 +1332,8 @@ glmb_status finish_frame(glmb_handle* h, bool copies_enqueued = false, bool est_
     est_enqueued = false;   // the estimates copied with the first pass are stale
   }
   if (e & kErrInput) return abandon(GLMB_E_INVALID, "non-finite detection");
+  // (glmb_update has done this for glmb_prune)
+  if ((e & kErrPairs) && copies_enqueued && (st = order_overflow(h, h->plan)) != GLMB_OK) return st;
   if (e & (kErrGate | kErrTimeout)) return abandon(GLMB_E_TIMEOUT, err_text(e));
   if (e & kErrFatal) return abandon(e & kErrNumeric ? GLMB_E_NUMERIC : GLMB_E_CAPACITY, err_text(e));
   h->n_pairs = h->h_scal[S_K];
@@ -1315,34 +1360,6 @@ glmb_status finish_frame(glmb_handle* h, bool copies_enqueued = false, bool est_
   h->stage = 0;
   ++h->gen;
   if (est_enqueued) h->est_gen = h->gen;
-  return GLMB_OK;
-}
-
-// The inspection calls' copies of a pair table, in table order (component,
-// then detection).  Their work areas are the regeneration's, which holds
-// nothing between frames: the scan of the counts in gc_newpos, the rows on
-// their way to the host in hvals.
-glmb_status pair_count(glmb_handle* h, const PairTable& P, uint32_t& n) {
-  CU(cudaMemcpy(&n, P.total, sizeof n, cudaMemcpyDeviceToHost));
-  return GLMB_OK;
-}
-void pair_order(glmb_handle* h, const PairTable& P) {
-  scan_u32(P.cnt, h->gc_newpos, &h->d_fs->T, 1, std::max(h->T_work, 1), nullptr, false, h->scan_tmp32, h->scan_cap32,
-           h->d_scal + S_ERR, h->stream);
-}
-// the first n rows, after pair_order: out[k * width + a], element a of pair p
-// at src[p * ps + a * as]
-glmb_status copy_pairs(glmb_handle* h, const PairTable& P, void* out, const void* src, int bytes, long long ps,
-                       long long as, int width, long long n) {
-  const long long step = h->row_words * 4 / (width * bytes);
-  for (long long k = 0; k < n; k += step) {
-    const long long m = std::min(step, n - k);
-    launch_pair_rows(P, h->gc_newpos, h->T_work, src, bytes, ps, as, width, h->hvals, k, m, h->stream);
-    CU(cudaGetLastError());
-    CU(cudaMemcpyAsync((unsigned char*)out + (size_t)k * width * bytes, h->hvals, (size_t)m * width * bytes,
-                       cudaMemcpyDeviceToHost, h->stream));
-  }
-  CU(cudaStreamSynchronize(h->stream));
   return GLMB_OK;
 }
 
@@ -1413,6 +1430,7 @@ glmb_status glmb_update(glmb_handle* h, const float* Z, int M, int z_is_device) 
   CU(cudaStreamSynchronize(h->stream));
   unsigned sc[4] = {0, 0, 0, 0};
   CU(cudaMemcpy(sc, h->d_scal, sizeof sc, cudaMemcpyDeviceToHost));
+  if ((sc[S_ERR] & kErrPairs) && !(sc[S_ERR] & kErrInput) && (st = order_overflow(h, p)) != GLMB_OK) return st;
   if ((sc[S_ERR] & kErrSlots) && !(sc[S_ERR] & (kErrFatal & ~kErrSlots))) {
     Plan q;
     unsigned mt = 0, mk = 0;

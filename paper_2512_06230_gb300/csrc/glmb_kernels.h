@@ -66,6 +66,7 @@ struct TableArgs {
   const double* births;   // birth records (fuse; device or pinned host memory)
   int fuse;
   int words;              // set by launch_table
+  const uint32_t* place;  // nullable: the components' places in the pair arrays, instead of the order they come in
   unsigned* n_fp64;
   unsigned* err;
   unsigned long long* hkeys;

@@ -204,7 +204,8 @@ __device__ __forceinline__ bool pair_eval(const Model& md, const CompGeom<DZ>& g
 template <int DZ>
 __device__ __forceinline__ void table_write_comp(const Model& md, const CompTable& ct, const PairTable& pt, int c,
                                  const CompGeom<DZ>& g, const float* __restrict__ Z,
-                                 const uint32_t* bits, int words, unsigned* n_fp64, unsigned* err) {
+                                 const uint32_t* bits, int words, const uint32_t* place, unsigned* n_fp64,
+                                 unsigned* err) {
   const int lane = threadIdx.x & 31;
   if (!g.ok) {
     if (lane == 0) {
@@ -224,7 +225,7 @@ __device__ __forceinline__ void table_write_comp(const Model& md, const CompTabl
   unsigned base = 0;
   if (lane == 0) {
     if (g.fp64) atomicAdd(n_fp64, 1u);
-    base = cnt ? atomicAdd(pt.total, cnt) : 0u;
+    base = place ? place[c] : cnt ? atomicAdd(pt.total, cnt) : 0u;
     pt.cnt[c] = cnt;
     pt.ptr[c] = base;
   }
@@ -354,7 +355,7 @@ __global__ void __launch_bounds__(32 * kTabWarps)
         }
     }
     __syncthreads();
-    if (in && wi == 0) table_write_comp<DZ>(md, ct, pt, c, g, Z, bits, words, a.n_fp64, a.err);
+    if (in && wi == 0) table_write_comp<DZ>(md, ct, pt, c, g, Z, bits, words, a.place, a.n_fp64, a.err);
     // the m-only parts of the component's alive term, m = lane + 1
     if (in && wi == W - 1 && md.score_mode == 0 && (uint32_t)c < (uint32_t)pt.slm_cap && lane < kSlmM) {
       constexpr int NP = DZ * (DZ + 1) / 2;

@@ -1,6 +1,7 @@
 """The inspection calls of the pair table (pairs, gate features, logits and
 usage), whose order is the table's (component, then detection) whatever place
-the pairs took, over tables larger than the calls' work area."""
+the pairs took: after a frame whose pairs overflowed the table, and over
+tables larger than the calls' work area."""
 from __future__ import annotations
 
 import ctypes as C
@@ -34,6 +35,57 @@ def _cfg(dim, n, M, max_pairs, **kw):
                max_tracks=n + 4, max_meas=M, max_births=n, max_pairs=max_pairs)
     cfg.update(kw)
     return cfg
+
+
+def _particle(cfg):
+    out = dict(cfg, dim_x=5, model=1, n_particles=64, sigma_a=1.0, sigma_w=0.05, ess_frac=0.5, score_mode=1)
+    return out
+
+
+def _particle_births(births):
+    return [(r, np.array([m[0], m[1], 3.0, 0.3, 0.01]), np.diag([30.0, 30.0, 1.0, 0.1, 0.01])) for r, m, _ in births]
+
+
+@pytest.mark.parametrize("kind", ["2d", "3d", "particles"])
+@pytest.mark.parametrize("frame", ["update", "step"])
+@pytest.mark.parametrize("n,M", [(40, 33), (300, 70)])
+def test_pairs_of_an_overflowed_frame(glmb, kind, frame, n, M):
+    """The frame fails, and the table's first max_pairs pairs are still
+    those of a filter with room for all."""
+    dim = 3 if kind == "3d" else 2
+    births, Z = _frame(dim, n, M, n + M)
+    big = _cfg(dim, n, M, n * M)
+    if kind == "particles":
+        big, births = _particle(big), _particle_births(births)
+    a = glmb.Filter(big)
+    a.predict(births)
+    a.update(Z)
+    ref, comps = a.pairs(), a.components()
+    K = len(ref["meas"])
+    cap = K // 3
+    assert cap > 50
+    b = glmb.Filter(dict(big, max_pairs=cap))
+    for _ in range(2):                     # the frame is refused, and refused again
+        if frame == "update":
+            b.predict(births)
+            b.update(Z)
+        else:
+            with pytest.raises(glmb.GlmbError) as ei:
+                b.step(births, Z)
+            assert ei.value.status == 3
+        got = b.pairs()
+        assert len(got["meas"]) == cap and np.array_equal(got["ptr"], ref["ptr"])
+        for k in ("meas", "logC", "q", "e"):
+            assert np.array_equal(got[k], ref[k][:cap]), k
+        whole = ref["ptr"][1:].astype(np.int64) <= cap      # components with all their pairs
+        assert whole.any() and np.array_equal(b.components()["dprob"][whole], comps["dprob"][whole])
+        if frame == "update":
+            with pytest.raises(glmb.GlmbError) as ei:
+                b.prune()
+            assert ei.value.status == 3
+    b.step(births, Z[:0])                  # a frame without detections runs
+    a.close()
+    b.close()
 
 
 def test_capacity_is_checked_before_anything_is_built(glmb):
