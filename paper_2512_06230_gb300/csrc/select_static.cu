@@ -23,9 +23,9 @@
 // operations a clock on an SM) and the number of launches.  Therefore the
 // keys and the exponentials are formed in integer arithmetic (fx_exp), and
 // what one block has to decide between two passes is done by the last block
-// of the first (five launches instead of twelve).  Measured, 10^6 children,
+// of the first (six launches instead of twelve).  Measured, 10^6 children,
 // h_max 20000: 413 us with an FP64 exponential per child and per kept child
-// in one block (twelve launches), 64 us with these.
+// in one block (twelve launches), 65 us with these.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -54,14 +54,26 @@ constexpr size_t kScratchBytes = kOffScal + 256;
 static_assert(kScratchBytes == 41216, "scratch size changed: update glmb.h");
 // keys of the boundary bin that fit in the histogram's place
 constexpr unsigned kListS = kBinsS / 2;
-// up to this many children the boundary bin of the first histogram is listed
-// and finished by one block; beyond it the bin outgrows the list, and each
-// digit takes a histogram pass over the children
-constexpr long long kListN = 1LL << 22;
+// A boundary bin with no more keys than that is listed and finished by one
+// block.  A bin with more (equal or nearly equal weights, or a cap that
+// crowds it) takes its next digits, of up to 13 bits, from histograms over
+// the grid until it does fit: the passes for them are always launched and
+// return at once when the list was enough (1 us of a call).  One block that
+// read all the children again for each digit took 1.4 ms for a million and
+// 5.6 ms for four million equal weights; now 65 and 135 us, as other weights.
+constexpr int kWideBits = 13, kWideBins = 1 << kWideBits;
+static_assert(4 * kWideBins <= kOffScal, "the wide histogram takes the place of the partials and the first one");
+// Up to this many children one block does read them again, and the passes are
+// not launched: 5000 children, equal or smooth weights, 37.2 and 34.3 us with
+// one block and 38.3 and 35.0 with the passes; 16384, 50.2 and 36.5 against
+// 40.6 and 37.3.
+constexpr long long kSoloN = 1LL << 13;
 
 struct SelScal {
-  unsigned done[3];     // last-block counters (histogram, boundary list, count)
-  unsigned n_list;      // keys in the boundary list (may exceed kListS)
+  unsigned done[3];     // last-block counters (histogram, boundary, count)
+  unsigned n_list;      // keys in the boundary list
+  unsigned n_bin;       // keys in the boundary bin
+  int left;             // bits of the boundary key still to be found
   double lse;           // log-sum-exp over valid children
   double lse_kept;      // log-sum-exp of the kept log-weights less lse
   long long thr;        // fixed-point threshold
@@ -80,13 +92,14 @@ struct Ptrs {
   unsigned* blk_gt;
   unsigned* blk_eq;
   unsigned* hist;
+  unsigned* wide;
   long long* list;
   SelScal* sc;
 };
 
 __host__ __device__ inline Ptrs ptrs_of(unsigned char* base) {
   return Ptrs{(long long*)(base + kOffBlkM), (double*)(base + kOffBlkS), (unsigned*)(base + kOffBlkGt),
-              (unsigned*)(base + kOffBlkEq), (unsigned*)(base + kOffHist), (long long*)(base + kOffHist),
+              (unsigned*)(base + kOffBlkEq), (unsigned*)(base + kOffHist), (unsigned*)base, (long long*)(base + kOffHist),
               (SelScal*)(base + kOffScal)};
 }
 
@@ -230,6 +243,8 @@ __global__ void __launch_bounds__(kThreads) sel_lse(const double* __restrict__ l
     if (threadIdx.x == 0) {
       p.sc->done[0] = p.sc->done[1] = p.sc->done[2] = 0u;
       p.sc->n_list = 0u;
+      p.sc->n_bin = 0u;
+      p.sc->left = 0;
       p.sc->need = h_max;
       p.sc->prefix = 0;
       p.sc->bound = 0;
@@ -272,24 +287,28 @@ __global__ void __launch_bounds__(kThreads) sel_lse(const double* __restrict__ l
   }
 }
 
-// Boundary digit of histogram h (kBinsS bins, shared memory) by a block of
-// kBinsS / 4 threads: the digit and the elements still needed in its bin;
+// Boundary digit of histogram h (BINS bins, shared memory) by a block of 1024
+// threads: the digit, the elements in its bin and those still needed of them;
 // `all`: the whole histogram is within `need`.
 struct Digit {
   int digit;
+  unsigned count;
   long long need;
   bool all;
 };
+template <int BINS>
 __device__ Digit find_digit(const unsigned* h, long long need) {
+  constexpr int kPer = BINS / 1024;
   __shared__ unsigned wsum[32];
   __shared__ int s_digit;
+  __shared__ unsigned s_count;
   __shared__ long long s_need;
   const int t = threadIdx.x, lane = t & 31, wp = t >> 5;
-  unsigned b4[4], mine = 0;
+  unsigned b[kPer], mine = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    b4[k] = h[4 * t + k];
-    mine += b4[k];
+  for (int k = 0; k < kPer; ++k) {
+    b[k] = h[kPer * t + k];
+    mine += b[k];
   }
   const unsigned x = warp_incl(mine);
   if (lane == 31) wsum[wp] = x;
@@ -299,19 +318,39 @@ __device__ Digit find_digit(const unsigned* h, long long need) {
   const unsigned before = __shfl_sync(0xFFFFFFFFu, ws, max(wp - 1, 0));
   const unsigned above = total - x - (wp > 0 ? before : 0u), upto = above + mine;
   if ((long long)above < need && (long long)upto >= need) {
-    unsigned cum = above;
-    int b = 3;
-    for (; b > 0; --b) {
-      if ((long long)(cum + b4[b]) >= need) break;
-      cum += b4[b];
+    unsigned cum = above, in = 0;
+    int at = 0;
+    bool found = false;
+#pragma unroll
+    for (int k = kPer - 1; k >= 0; --k) {
+      if (found) continue;
+      if ((long long)(cum + b[k]) >= need) {
+        found = true;
+        at = k;
+        in = b[k];
+      } else {
+        cum += b[k];
+      }
     }
-    s_digit = 4 * t + b;
+    s_digit = kPer * t + at;
+    s_count = in;
     s_need = need - cum;
   }
   __syncthreads();
-  const Digit d{s_digit, s_need, (long long)total <= need};
+  const Digit d{s_digit, s_count, s_need, (long long)total <= need};
   __syncthreads();
   return d;
+}
+
+// one more key in bin `bin` (< 0: none) of a histogram in shared memory; a
+// warp whose keys share their bin (equal weights) adds them at once
+__device__ __forceinline__ void hist_add(unsigned* hist, int bin) {
+  const unsigned act = __ballot_sync(__activemask(), bin >= 0);
+  if (bin < 0) return;
+  int same;
+  __match_all_sync(act, bin, &same);
+  if (!same) atomicAdd(&hist[bin], 1u);
+  else if ((int)(threadIdx.x & 31) == __ffs(act) - 1) atomicAdd(&hist[bin], (unsigned)__popc(act));
 }
 
 // true in every thread of the grid's last block to get here
@@ -325,20 +364,19 @@ __device__ bool last_block(unsigned* done) {
   return last;
 }
 
-// Pass 2 (and, for large n, once per further digit): histogram of the digit
-// of `width` bits at `shift` of the keys at or above the threshold that share the prefix; the
-// last block finds the boundary digit.  On the first digit every block forms
-// the log-sum-exp and the threshold from pass 1's partials (the same in all).
-__global__ void __launch_bounds__(1024) sel_hist(const double* __restrict__ lw, long long n, int shift, int width, int first,
+// Pass 2: histogram of the first digit, of `width` bits at `shift`, of the
+// keys at or above the threshold; the last block finds the boundary digit.
+// Every block forms the log-sum-exp and the threshold from pass 1's partials
+// (the same in all).
+__global__ void __launch_bounds__(1024) sel_hist(const double* __restrict__ lw, long long n, int shift, int width,
                                                  int nblk_lse, double log_tau, unsigned char* base) {
   load_exp_tab();
   pdl_enter();
   __shared__ unsigned hist[kBinsS];
   __shared__ long long s_thr;
   Ptrs p = ptrs_of(base);
-  if (p.sc->mode != 0) return;
   for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) hist[b] = 0;
-  if (first) {
+  {
     const int b = threadIdx.x;   // one partial per thread (kMaxBlocks = blockDim)
     const LseS u = block_lse(b < nblk_lse ? LseS{p.blk_m[b], p.blk_s[b]} : LseS{kKeyInvalid, 0.0});
     const bool none = u.m == kKeyInvalid || !(u.s > 0.0);
@@ -356,12 +394,9 @@ __global__ void __launch_bounds__(1024) sel_hist(const double* __restrict__ lw, 
         p.sc->top = u.m;
       }
     }
-  } else if (threadIdx.x == 0) {
-    s_thr = p.sc->thr;
   }
   __syncthreads();
   const long long thr = s_thr;
-  const unsigned long long prefix = (unsigned long long)p.sc->prefix;
   long long lo, hi;
   chunk_of(n, lo, hi);
 #pragma unroll 4
@@ -369,80 +404,118 @@ __global__ void __launch_bounds__(1024) sel_hist(const double* __restrict__ lw, 
     const long long k = key_of(lw[j]);
     if (k == kKeyInvalid || k < thr) continue;
     const unsigned long long v = (unsigned long long)(k - thr);
-    if ((v >> (shift + width)) != prefix) continue;
+    if ((v >> (shift + width)) != 0ull) continue;
     atomicAdd(&hist[(v >> shift) & ((1u << width) - 1u)], 1u);
   }
   __syncthreads();
   for (int b = threadIdx.x; b < kBinsS; b += blockDim.x)
     if (hist[b]) atomicAdd(&p.hist[b], hist[b]);
   if (!last_block(&p.sc->done[0])) return;
-  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) {
-    hist[b] = __ldcg(&p.hist[b]);
-    p.hist[b] = 0u;
-  }
+  for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) hist[b] = __ldcg(&p.hist[b]);
   __syncthreads();
-  const long long need = p.sc->need;
-  const Digit d = find_digit(hist, need);
+  const Digit d = find_digit<kBinsS>(hist, p.sc->need);
+  // the next digit's bins, in place of the partials and of this histogram
+  if (d.count > kListS)
+    for (int b = threadIdx.x; b < kWideBins; b += blockDim.x) p.wide[b] = 0u;
   if (threadIdx.x != 0) return;
-  p.sc->done[0] = 0u;
   if (thr == LLONG_MAX) {
     p.sc->mode = 2;
-  } else if (first && d.all) {
+  } else if (d.all) {
     p.sc->mode = 1;
     p.sc->bound = thr - 1;
     p.sc->need = 0;
   } else {
-    const long long pre = (long long)((prefix << width) | (unsigned)d.digit);
-    p.sc->prefix = pre;
+    p.sc->prefix = d.digit;
     p.sc->need = d.need;
-    if (shift == 0) p.sc->bound = thr + pre;
+    p.sc->n_bin = d.count;
+    p.sc->left = shift;
+    if (shift == 0) p.sc->bound = thr + d.digit;
   }
 }
 
-// Pass 3 (n <= kListN): the keys of the boundary bin are listed, and the last
-// block finds the boundary key among them digit by digit in shared memory.  A
-// bin that outgrows the list (many equal or nearly equal keys) is read from
-// the children again by that block.
-__global__ void __launch_bounds__(1024) sel_boundary(const double* __restrict__ lw, long long n, int shift,
+// Pass 3, once or, for more than kSoloN children, once per kWideBits bits that
+// may be left: the rest of the boundary key.  A boundary bin that fits the
+// list is listed, and the last block finds the key among its keys digit by
+// digit in shared memory; a larger one takes one digit from a histogram over
+// the grid (`solo`: the last block reads the children again for each digit).
+// A million children, whole call: h_max 20000 of smooth, equal, nearly equal
+// weights 65, 65, 72 us, h_max 400000 of smooth ones 68 us; four million,
+// h_max a million 169 us (in one block 5.3 ms).
+__global__ void __launch_bounds__(1024) sel_boundary(const double* __restrict__ lw, long long n, int solo,
                                                      unsigned char* base) {
   pdl_enter();
-  __shared__ unsigned hist[kBinsS];
+  __shared__ unsigned hist[kWideBins];
   Ptrs p = ptrs_of(base);
-  if (p.sc->mode != 0) return;
+  const int left = p.sc->left;
+  if (p.sc->mode != 0 || left == 0) return;
   const long long thr = p.sc->thr;
   unsigned long long prefix = (unsigned long long)p.sc->prefix;
   const int lane = threadIdx.x & 31;
+  const bool listed = p.sc->n_bin <= kListS, wide = !listed && !solo;
+  const int width_w = min(kWideBits, left), shift_w = left - width_w;   // a wide digit
   long long lo, hi;
   chunk_of(n, lo, hi);
-  for (long long j0 = lo; j0 < hi; j0 += blockDim.x) {
-    const long long j = j0 + threadIdx.x;
-    const long long k = j < hi ? key_of(lw[j]) : kKeyInvalid;
-    const bool in = k != kKeyInvalid && k >= thr && ((unsigned long long)(k - thr) >> shift) == prefix;
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, in);
-    if (!bal) continue;
-    unsigned at = 0;
-    if (lane == __ffs(bal) - 1) at = atomicAdd(&p.sc->n_list, (unsigned)__popc(bal));
-    at = __shfl_sync(0xFFFFFFFFu, at, __ffs(bal) - 1) + __popc(bal & ((1u << lane) - 1u));
-    if (in && at < kListS) p.list[at] = k;
-  }
-  if (!last_block(&p.sc->done[1])) return;
-  const unsigned nl = __ldcg(&p.sc->n_list);
-  const bool listed = nl <= kListS;
-  const long long total = listed ? (long long)nl : n;
-  long long need = p.sc->need;
-  for (int above = shift; above > 0;) {
-    const int width = min(kDigitS, above), sh = above - width;
-    for (int b = threadIdx.x; b < kBinsS; b += blockDim.x) hist[b] = 0u;
+  if (wide) {
+    for (int b = threadIdx.x; b < kWideBins; b += blockDim.x) hist[b] = 0u;
     __syncthreads();
-    for (long long j = threadIdx.x; j < total; j += blockDim.x) {
-      const long long k = listed ? __ldcg(&p.list[j]) : key_of(lw[j]);
+#pragma unroll 4
+    for (long long j = lo + threadIdx.x; j < hi; j += blockDim.x) {
+      const long long k = key_of(lw[j]);
       if (k == kKeyInvalid || k < thr) continue;
       const unsigned long long v = (unsigned long long)(k - thr);
-      if ((v >> above) != prefix) continue;
-      atomicAdd(&hist[(v >> sh) & ((1u << width) - 1u)], 1u);
+      if ((v >> left) != prefix) continue;
+      atomicAdd(&hist[(v >> shift_w) & ((1u << width_w) - 1u)], 1u);
     }
     __syncthreads();
-    const Digit d = find_digit(hist, need);
+    for (int b = threadIdx.x; b < kWideBins; b += blockDim.x)
+      if (hist[b]) atomicAdd(&p.wide[b], hist[b]);
+  } else if (listed) {
+    for (long long j0 = lo; j0 < hi; j0 += blockDim.x) {
+      const long long j = j0 + threadIdx.x;
+      const long long k = j < hi ? key_of(lw[j]) : kKeyInvalid;
+      const bool in = k != kKeyInvalid && k >= thr && ((unsigned long long)(k - thr) >> left) == prefix;
+      const unsigned bal = __ballot_sync(0xFFFFFFFFu, in);
+      if (!bal) continue;
+      unsigned at = 0;
+      if (lane == __ffs(bal) - 1) at = atomicAdd(&p.sc->n_list, (unsigned)__popc(bal));
+      at = __shfl_sync(0xFFFFFFFFu, at, __ffs(bal) - 1) + __popc(bal & ((1u << lane) - 1u));
+      if (in && at < kListS) p.list[at] = k;
+    }
+  }
+  if (!last_block(&p.sc->done[1])) return;
+  long long need = p.sc->need;
+  if (wide) {
+    for (int b = threadIdx.x; b < kWideBins; b += blockDim.x) {
+      hist[b] = __ldcg(&p.wide[b]);
+      p.wide[b] = 0u;   // for the next digit
+    }
+    __syncthreads();
+    const Digit d = find_digit<kWideBins>(hist, need);
+    if (threadIdx.x == 0) {
+      prefix = (prefix << width_w) | (unsigned)d.digit;
+      p.sc->done[1] = 0u;
+      p.sc->prefix = (long long)prefix;
+      p.sc->need = d.need;
+      p.sc->n_bin = d.count;
+      p.sc->left = shift_w;
+      if (shift_w == 0) p.sc->bound = thr + (long long)prefix;
+    }
+    return;
+  }
+  const long long total = listed ? (long long)min(__ldcg(&p.sc->n_list), kListS) : n;
+  for (int above = left; above > 0;) {
+    const int width = min(kWideBits, above), sh = above - width;
+    for (int b = threadIdx.x; b < kWideBins; b += blockDim.x) hist[b] = 0u;
+    __syncthreads();
+    for (long long j0 = 0; j0 < total; j0 += blockDim.x) {
+      const long long j = j0 + threadIdx.x;
+      const long long k = j >= total ? kKeyInvalid : listed ? __ldcg(&p.list[j]) : key_of(lw[j]);
+      const unsigned long long v = (unsigned long long)(k - thr);
+      const bool in = k != kKeyInvalid && k >= thr && (v >> above) == prefix;
+      hist_add(hist, in ? (int)((v >> sh) & ((1u << width) - 1u)) : -1);
+    }
+    __syncthreads();
+    const Digit d = find_digit<kWideBins>(hist, need);
     prefix = (prefix << width) | (unsigned)d.digit;
     need = d.need;
     above = sh;
@@ -450,6 +523,7 @@ __global__ void __launch_bounds__(1024) sel_boundary(const double* __restrict__ 
   if (threadIdx.x == 0) {
     p.sc->need = need;
     p.sc->bound = thr + (long long)prefix;
+    p.sc->left = 0;
   }
 }
 
@@ -649,16 +723,10 @@ extern "C" glmb_status glmb_select_top_static(const double* logw_dev, int64_t n,
   // digits from the top of the nbits bits of key - threshold
   const int width = std::min(kDigitS, nbits), top = nbits - width;
   launch_sel(sel_lse, nblk, kThreads, s, logw_dev, n, h_max, base);
-  launch_sel(sel_hist, hblk, 1024, s, logw_dev, n, top, width, 1, nblk, log_tau, base);
-  if (n <= kListN) {
-    if (top > 0) launch_sel(sel_boundary, hblk, 1024, s, logw_dev, n, top, base);
-  } else {
-    for (int above = top; above > 0;) {
-      const int w = std::min(kDigitS, above);
-      above -= w;
-      launch_sel(sel_hist, hblk, 1024, s, logw_dev, n, above, w, 0, nblk, log_tau, base);
-    }
-  }
+  launch_sel(sel_hist, hblk, 1024, s, logw_dev, n, top, width, nblk, log_tau, base);
+  const int solo = n <= kSoloN ? 1 : 0;
+  for (int above = top; above > 0; above -= solo ? above : kWideBits)
+    launch_sel(sel_boundary, hblk, 1024, s, logw_dev, n, solo, base);
   launch_sel(sel_count, nblk, kThreads, s, logw_dev, n, h_max, n_out_dev, base);
   launch_sel(sel_write, nblk, kThreads, s, logw_dev, n, h_max, (long long*)idx_out_dev, logw_out_dev, base);
   return cudaGetLastError() == cudaSuccess ? GLMB_OK : GLMB_E_CUDA;
