@@ -115,6 +115,18 @@ struct Tables {
   }
 };
 
+// exp(-r 2^-64) 2^63 for r 2^-64 < 0.022, by Taylor's series
+FX_FN u64 exp_poly(u64 r) {
+  // 1 - r (1 - r/2 (1 - r/3 (...))), the inner terms in 32 bits
+  const uint32_t rh = (uint32_t)(r >> 32);
+  uint32_t q = 35791394u - (uint32_t)(((u64)rh * 5965232u) >> 32);     // (1/120 - r/720) 2^32
+  q = 178956971u - (uint32_t)(((u64)rh * q) >> 32);
+  u64 p = 0x1555555555555555ull - mulhi(r, (u64)q << 31);              // (1/6 - ...) 2^63
+  p = 0x4000000000000000ull - mulhi(r, p);
+  p = 0x8000000000000000ull - mulhi(r, p);
+  return 0x8000000000000000ull - mulhi(r, p);
+}
+
 // ---- exp(-x), x >= 0 and not -0 (0 from 708 on; NaN for NaN) ----
 // x = n ln(2) / 64 + r: a table entry times the polynomial of exp(-r).
 FX_FN double exp_neg(double x, const u64* exp2) {
@@ -129,16 +141,49 @@ FX_FN double exp_neg(double x, const u64* exp2) {
   const uint32_t n = (uint32_t)(((u64)(uint32_t)(X >> 32) * 0xB8AA3B29u) >> 46);
   // r 2^64 (the integer part of x cancels modulo 2^64)
   const u64 r = (X << 11) - (u64)n * 0x2C5C85FDF473DE6ull - (((u64)n * 0xAF278ECEull) >> 32);
-  // 1 - r (1 - r/2 (1 - r/3 (...))), the inner terms in 32 bits
-  const uint32_t rh = (uint32_t)(r >> 32);
-  uint32_t q = 35791394u - (uint32_t)(((u64)rh * 5965232u) >> 32);     // (1/120 - r/720) 2^32
-  q = 178956971u - (uint32_t)(((u64)rh * q) >> 32);
-  u64 p = 0x1555555555555555ull - mulhi(r, (u64)q << 31);              // (1/6 - ...) 2^63
-  p = 0x4000000000000000ull - mulhi(r, p);
-  p = 0x8000000000000000ull - mulhi(r, p);
-  p = 0x8000000000000000ull - mulhi(r, p);
-  const u64 t = mulhi(p, exp2[n & 63u]);                               // 2^62
+  const u64 t = mulhi(exp_poly(r), exp2[n & 63u]);                     // 2^62
   return to_double(t, -62 - (int)(n >> 6));
+}
+
+// ---- exp(-d 2^-32), d >= 0: sums of many such values beside a large one ----
+// d log2(e) = i + j/64 + r / ln 2: the table's 2^(-j/64) times the polynomial
+// of exp(-r).  t 2^(-62 - i), t in [2^61, 2^62], is the value to 2^-54 of it.
+struct ExpParts {
+  u64 t;
+  int i;
+};
+FX_FN ExpParts exp_parts(u64 d, const u64* exp2) {                     // d < 2^39
+  const u64 y = mulhi(d << 25, 0x5C551D94AE0BF85Eull);                 // d log2(e) 2^(55 - 32)
+  const u64 r = mulhi((y & 0x1FFFFFFFFFFFFull) << 9, 0xB17217F7D1CF79ACull);
+  return ExpParts{mulhi(exp_poly(r), exp2[(y >> 49) & 63u]), (int)(y >> 55)};
+}
+// Up to 31 values summed in units of 2^-90: of 2^30 values beside one of 1 the
+// sum is off by 2^-60 (0 from d = 63 2^32 on, where the value is below 2^-90).
+struct ExpSum {
+  u64 hi = 0ull, lo = 0ull;                                            // 2^-58 and 2^-90 units (lo: carries above bit 32)
+  FX_FN void add(u64 d, const u64* exp2) {
+    if (d >= (63ull << 32)) return;
+    const ExpParts e = exp_parts(d, exp2);                             // 0 <= i <= 90
+    if (e.i < 60) {
+      hi += e.t >> (4 + e.i);
+      lo += (e.t << (60 - e.i)) >> 32;
+    } else {
+      lo += (e.t >> (e.i - 60)) >> 32;
+    }
+  }
+  FX_FN bool any() const { return (hi | lo) != 0ull; }
+  FX_FN double value() const {
+    const u64 h = hi + (lo >> 32), l = lo << 32;
+    if (h == 0ull) return to_double(l >> 32, -90);
+    const int lz = clz(h);
+    return to_double((h << lz) | ((l >> 1) >> (63 - lz)), -58 - lz);
+  }
+};
+// one value, rounded (d < 2^39, beyond it 0: the value is below 2^-184)
+FX_FN double exp_fixed(u64 d, const u64* exp2) {
+  if (d >> 39) return 0.0;
+  const ExpParts e = exp_parts(d, exp2);
+  return to_double(e.t, -62 - e.i);
 }
 
 // ---- -2 ln((2 w + 1) / 2^33) ----

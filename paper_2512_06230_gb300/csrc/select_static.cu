@@ -14,23 +14,24 @@
 // children below tau are dropped, the h_max largest are kept (ties by
 // index), the kept ones are listed in index order and their log-weights
 // renormalised.  The log-sum-exp is summed differently (exponentials to
-// 2^-55 here, FP32 exponentials with compensated sums there), so the two
+// 2^-54 here, FP32 exponentials with compensated sums there), so the two
 // agree up to its rounding: a child whose normalised weight lies within that
 // rounding of tau may land on either side of the cut.
 //
 // What bounds it: at a million children the 8 MB of log-weights stay in L2,
 // so a pass is a few microseconds and the cost is the FP64 pipe (about two
 // operations a clock on an SM) and the number of launches.  Therefore the
-// keys and the exponentials are formed in integer arithmetic (fx_exp), and
+// keys and the exponentials are formed in integer arithmetic (fx_math.cuh), and
 // what one block has to decide between two passes is done by the last block
 // of the first (six launches instead of twelve).  Measured, 10^6 children,
 // h_max 20000: 413 us with an FP64 exponential per child and per kept child
-// in one block (twelve launches), 65 us with these.
+// in one block (twelve launches), 66 us with these.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
 
 #include "../../include/glmb.h"
+#include "fx_math.cuh"
 #include "glmb_dev.cuh"
 
 namespace {
@@ -60,7 +61,7 @@ constexpr unsigned kListS = kBinsS / 2;
 // the grid until it does fit: the passes for them are always launched and
 // return at once when the list was enough (1 us of a call).  One block that
 // read all the children again for each digit took 1.4 ms for a million and
-// 5.6 ms for four million equal weights; now 65 and 135 us, as other weights.
+// 5.6 ms for four million equal weights; now 65 and 138 us, as other weights.
 constexpr int kWideBits = 13, kWideBins = 1 << kWideBits;
 static_assert(4 * kWideBins <= kOffScal, "the wide histogram takes the place of the partials and the first one");
 // Up to this many children one block does read them again, and the passes are
@@ -127,55 +128,17 @@ __device__ __forceinline__ long long key_of(double lw) {
   return (b >> 63) ? -(long long)v : (long long)v;
 }
 
-// 2^(-j/64) as 63-bit fractions, from exp's Taylor series at compile time
-struct Exp2Tab {
-  unsigned long long v[64];
-  constexpr Exp2Tab() : v{} {
-    for (int j = 0; j < 64; ++j) {
-      const double x = -0.69314718055994530942 * j / 64.0;
-      double t = 1.0, s = 0.0;
-      for (int k = 24; k >= 1; --k) s = (s + 1.0) * x / k;   // x (1 + x/2 (1 + x/3 (...)))
-      t += s;
-      v[j] = (unsigned long long)(t * 9223372036854775808.0);
-    }
-  }
-};
-__device__ const Exp2Tab kExp2Tab{};
-// the block's copy (lanes read different entries); every kernel that forms
-// exponentials fills it first
+__device__ const fx::Tables kFx{};
+// the block's copy of 2^(-j/64) (lanes read different entries); every kernel
+// that forms exponentials fills it first
 __device__ __forceinline__ unsigned long long* exp_tab() {
   __shared__ unsigned long long t[64];
   return t;
 }
 __device__ __forceinline__ void load_exp_tab() {
-  if (threadIdx.x < 64) exp_tab()[threadIdx.x] = kExp2Tab.v[threadIdx.x];
+  if (threadIdx.x < 64) exp_tab()[threadIdx.x] = kFx.exp2[threadIdx.x];
   __syncthreads();
 }
-
-// exp(-d 2^-32) 2^58 for d >= 0, to about 2^-51 of its value, in integer
-// arithmetic: d log2(e) = i + j/64 + r, then the table's 2^(-j/64) times the
-// Taylor polynomial of 2^-r (z = r ln 2 < 0.011, six terms: z^7/7! < 2^-57).
-__device__ __forceinline__ unsigned long long fx_exp(unsigned long long d) {
-  if (d >= (42ull << 32)) return 0ull;                         // below 2^-60
-  constexpr unsigned long long kLog2e = 0x5C551D94AE0BF85Eull; // log2(e) 2^62
-  constexpr unsigned long long kLn2 = 0xB17217F7D1CF79ACull;   // ln(2) 2^64
-  const unsigned long long y = __umul64hi(d << 25, kLog2e);    // 2^-55 units
-  const int i = (int)(y >> 55), j = (int)(y >> 49) & 63;
-  const unsigned long long z = __umul64hi((y & 0x1FFFFFFFFFFFFull) << 9, kLn2);   // z 2^64
-  // 1 - z (1 - z (1/2 - z (1/6 - z (1/24 - z (1/120 - z/720))))), the inner
-  // terms in 32 bits (z 2^32 < 2^26), the outer ones scaled by 2^63
-  const uint32_t zh = (uint32_t)(z >> 32);
-  uint32_t q = 35791394u - __umulhi(zh, 5965232u);             // (1/120 - z/720) 2^32
-  q = 178956971u - __umulhi(zh, q);                            // 1/24
-  q = 715827883u - __umulhi(zh, q);                            // 1/6
-  unsigned long long p = 0x4000000000000000ull - __umul64hi(z, (unsigned long long)q << 31);
-  p = 0x8000000000000000ull - __umul64hi(z, p);
-  p = 0x8000000000000000ull - __umul64hi(z, p);
-  const unsigned long long t = __umul64hi(p, exp_tab()[j]);   // 2^62 scale
-  const int s = 4 + i;
-  return (t + (1ull << (s - 1))) >> s;
-}
-constexpr double kExpInv = 3.4694469519536141888e-18;          // 2^-58
 
 __device__ __forceinline__ long long warp_max_ll(long long v) {
 #pragma unroll
@@ -216,7 +179,7 @@ __device__ LseS block_lse(LseS v) {
   const long long M = warp_max_ll(lane < nw ? sm[lane] : kKeyInvalid);
   const double r = v.m == kKeyInvalid ? 0.0
                    : v.m == M         ? v.s
-                                      : v.s * ((double)fx_exp((unsigned long long)(M - v.m)) * kExpInv);
+                                      : v.s * fx::exp_fixed((unsigned long long)(M - v.m), exp_tab());
   const double ws = warp_sum_of(r);
   if (lane == 0) ss[w] = ws;
   __syncthreads();
@@ -271,14 +234,14 @@ __global__ void __launch_bounds__(kThreads) sel_lse(const double* __restrict__ l
     m = warp_max_ll(m);
     if (m == kKeyInvalid) continue;
     if (m != v.m) {
-      if (v.m != kKeyInvalid) v.s *= (double)fx_exp((unsigned long long)(m - v.m)) * kExpInv;
+      if (v.m != kKeyInvalid) v.s *= fx::exp_fixed((unsigned long long)(m - v.m), exp_tab());
       v.m = m;
     }
-    unsigned long long s = 0ull;   // at most 8 terms of 2^58
+    fx::ExpSum s;
 #pragma unroll
     for (int u = 0; u < kU; ++u)
-      if (k[u] != kKeyInvalid) s += fx_exp((unsigned long long)(m - k[u]));
-    if (s) v.s += (double)s * kExpInv;
+      if (k[u] != kKeyInvalid) s.add((unsigned long long)(m - k[u]), exp_tab());
+    if (s.any()) v.s += s.value();
   }
   v = block_lse(v);
   if (threadIdx.x == 0) {
@@ -439,8 +402,8 @@ __global__ void __launch_bounds__(1024) sel_hist(const double* __restrict__ lw, 
 // digit in shared memory; a larger one takes one digit from a histogram over
 // the grid (`solo`: the last block reads the children again for each digit).
 // A million children, whole call: h_max 20000 of smooth, equal, nearly equal
-// weights 65, 65, 72 us, h_max 400000 of smooth ones 68 us; four million,
-// h_max a million 169 us (in one block 5.3 ms).
+// weights 66, 65, 73 us, h_max 400000 of smooth ones 70 us; four million,
+// h_max a million 177 us (in one block 5.3 ms).
 __global__ void __launch_bounds__(1024) sel_boundary(const double* __restrict__ lw, long long n, int solo,
                                                      unsigned char* base) {
   pdl_enter();
@@ -554,7 +517,7 @@ __global__ void __launch_bounds__(kThreads) sel_count(const double* __restrict__
   double sum = 0.0;
   constexpr int kU = 4;
   for (long long j0 = lo; j0 < hi; j0 += kU * kThreads) {
-    unsigned long long f = 0ull;
+    fx::ExpSum f;
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const long long j = j0 + u * kThreads + threadIdx.x;
@@ -562,9 +525,9 @@ __global__ void __launch_bounds__(kThreads) sel_count(const double* __restrict__
       bool gt, eq;
       keep_kind(k, s, gt, eq);
       c += (gt ? 1ull : 0ull) + (eq ? 1ull << 32 : 0ull);
-      if (gt) f += fx_exp((unsigned long long)(s.top - k));
+      if (gt) f.add((unsigned long long)(s.top - k), exp_tab());
     }
-    if (f) sum += (double)f * kExpInv;
+    if (f.any()) sum += f.value();
   }
   c = warp_sum_of(c);
   sum = warp_sum_of(sum);
@@ -619,7 +582,7 @@ __global__ void __launch_bounds__(kThreads) sel_count(const double* __restrict__
     *n_out = (int)kept;
     for (int w = 1; w < kWarps; ++w) sum += wd[w];
     if (s.mode == 0 && s.need > 0)
-      sum += (double)min(eq, s.need) * ((double)fx_exp((unsigned long long)(s.top - s.bound)) * kExpInv);
+      sum += (double)min(eq, s.need) * fx::exp_fixed((unsigned long long)(s.top - s.bound), exp_tab());
     p.sc->lse_kept = kept > 0 ? ((double)s.top * kFxInv - s.lse) + log(sum) : 0.0;
   }
 }

@@ -1,6 +1,7 @@
 """glmb_select_top_static where the boundary bin of its first histogram
 outgrows the list one block finishes (equal and nearly equal weights, large
-caps), on both sides of the sizes where the grid takes the digits over."""
+caps), on both sides of the sizes where the grid takes the digits over, and its sums
+where many small weights stand beside a large one."""
 from __future__ import annotations
 
 import numpy as np
@@ -72,3 +73,21 @@ def test_ties_take_little_longer_than_other_weights(select):  # noqa: F811
 
     rng = np.random.default_rng(1)
     assert best(_case("equal", 1_000_000, rng)) < 5 * best(_case("smooth", 1_000_000, rng))
+
+
+@pytest.mark.parametrize("tail", [-16.0, -24.5, -30.25, -41.3, -41.8, -44.0])
+def test_a_million_small_weights_beside_a_large_one(select, tail):  # noqa: F811
+    """The log-sum-exp is log(1 + (n - 1) e^tail): its sum is rounded to 2^-53
+    by each of at most 32 additions on the way to the largest weight's
+    partial, once over all and once over the kept (whose sum is the same), so
+    the largest weight's result is off by at most 64 units of 2^-53."""
+    n = 1_000_000
+    lw = np.full(n, tail)
+    lw[n // 3] = 0.0
+    idx, out = select(lw, 1, 1e-30)
+    assert list(idx) == [n // 3] and abs(out[0]) <= 2.0 ** -52      # alone after the second normalisation
+    idx, out = select(lw, n, 1e-30)
+    key = np.longdouble(np.rint(tail * 2.0 ** 32)) * np.longdouble(2.0) ** -32
+    s = float(np.log1p((n - 1) * np.exp(key)))
+    assert len(idx) == n
+    assert abs(out[n // 3] + s) <= 64 * 2.0 ** -53
