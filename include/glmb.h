@@ -172,7 +172,11 @@ typedef struct {
 } glmb_info;
 
 /* Creates a filter holding the initial GLMB: one hypothesis with no tracks
- * and weight one.  All device memory is allocated here from the capacities.
+ * and weight one.  The device memory that follows the capacities is allocated
+ * here.  64 bytes of it per child slot (h_max x h_up) are the notes of the
+ * one-thread-per-child draw: only filters whose children can be drawn so have
+ * them (from 128 children per SM, unless the tuning says otherwise), and one
+ * for which they cannot be allocated runs without, more slowly.
  * Errors: GLMB_E_INVALID (bad model or capacity), GLMB_E_OOM, GLMB_E_CUDA. */
 glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out);
 

@@ -103,7 +103,11 @@ struct glmb_handle {
   unsigned char* img = nullptr;
   size_t img_alloc = 0;
   uint32_t* redo_list = nullptr;
+  // room for every child's noted rows, once children are drawn one to a
+  // thread (ensure_notes); none: such children go to the redo list
   unsigned char* notes = nullptr;
+  unsigned note_cap = 0;
+  bool notes_tried = false;
   PruneWork pw{};
   unsigned long long* hkeys = nullptr;
   uint32_t* hvals = nullptr;        // (between frames the rows of the inspection calls)
@@ -292,6 +296,23 @@ void free_all(glmb_handle* h) {
   for (void* p : h->host_allocs) cudaFreeHost(p);
   h->allocs.clear();
   h->host_allocs.clear();
+}
+
+// one thread per child once the children give every SM enough warps
+bool draws_by_thread(const glmb_handle* h, long long children) {
+  return children >= (long long)h->tune.thread_warps_per_sm * 32 * h->n_sm;
+}
+
+// The draw kernel's notes, 64 bytes per child slot: allocated at create for a
+// filter that can have enough children to be drawn so, else at the first plan
+// that does (launch options, tuning), so that the others do not hold them.
+// Without room the children's noted rows are redone by the warp kernel: the
+// same results, later.
+void ensure_notes(glmb_handle* h) {
+  if (h->notes_tried) return;
+  h->notes_tried = true;
+  if (dalloc(h, &h->notes, h->cap_children * (long long)expand_note_bytes()))
+    h->note_cap = (unsigned)std::min<long long>(h->cap_children, 0xFFFFFFFFLL);
 }
 
 size_t round_up64(size_t x) { return (x + 63) / 64 * 64; }
@@ -651,7 +672,6 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
             dalloc(h, &h->child_hash, h->cap_children) &&
             dalloc(h, &h->child_alive, h->cap_children) &&
             dalloc(h, &h->redo_list, h->cap_children) &&
-            dalloc(h, &h->notes, h->cap_children * (long long)expand_note_bytes()) &&
             dalloc(h, &h->pw.blk_max, 4097) && dalloc(h, &h->pw.blk_sum, 4097) &&
             dalloc(h, &h->pw.blk_done, 4) && dalloc(h, &h->pw.lse, 2) && dalloc(h, &h->pw.thr, 1) &&
             dalloc(h, &h->pw.part_max, kMaxLseParts) && dalloc(h, &h->pw.part_sum, kMaxLseParts) &&
@@ -666,6 +686,7 @@ glmb_status glmb_create(const glmb_config* cfg, glmb_handle** out) {
             dalloc(h, &h->upd_se, h->cap_upd * dz) && dalloc(h, &h->gc_flag, h->cap_comp) &&
             dalloc(h, &h->gc_newpos, h->cap_comp) && dalloc(h, &h->d_ru, h->cap_meas);
   if (ok) {
+    if (draws_by_thread(h, h->cap_children)) ensure_notes(h);
     h->pw.err = h->d_scal + S_ERR;
     h->pw.flags_tmp_cap = h->cap_children;
     h->scan_cap32 = scan_n;
@@ -893,6 +914,7 @@ ExpandArgs expand_args(glmb_handle* h, const Plan& p, bool mat) {
   a.redo_list = h->redo_list;
   a.redo_count = h->d_scal + S_REDO;
   a.notes = h->notes;
+  a.note_cap = h->note_cap;
   a.note_count = h->d_scal + S_NOTE;
   a.stage_next = h->d_scal + S_STAGE;
   a.materialize = mat ? 1 : 0;
@@ -909,6 +931,7 @@ ExpandArgs expand_args(glmb_handle* h, const Plan& p, bool mat) {
 // the image buffer holds cap_h parents of plan p; growing it invalidates the
 // captured graphs (they hold its address)
 glmb_status ensure_img(glmb_handle* h, const Plan& p) {
+  if (p.thread) ensure_notes(h);
   const size_t need = (size_t)h->cap_h * (size_t)expand_image_bytes(h->md.dz, p.T, p.K, p.M);
   if (need <= h->img_alloc) return GLMB_OK;
   CU(cudaStreamSynchronize(h->stream));
@@ -1148,7 +1171,7 @@ bool make_plan(glmb_handle* h, bool fixed, int T_plan, int K_plan, int M_plan, P
   const int dz = h->md.dz;
   // one thread per child once the children give every SM four warps (the
   // register lists address pairs with 16 bits); else one warp per child
-  p.thread = (long long)h->H * h->cfg.h_up >= (long long)h->tune.thread_warps_per_sm * 32 * h->n_sm;
+  p.thread = draws_by_thread(h, (long long)h->H * h->cfg.h_up);
   if (h->launch_opts & GLMB_OPT_DRAW_THREAD) p.thread = true;
   if (h->launch_opts & GLMB_OPT_DRAW_WARP) p.thread = false;
   p.thread = p.thread && p.K <= 65536;

@@ -163,7 +163,8 @@ struct ExpandArgs {
   int warp_all;           // warp kernel: every child of every parent (else the overflow list)
   uint32_t* redo_list;    // children the draw kernel could not take
   unsigned* redo_count;
-  unsigned char* notes;   // children with noted rows (expand_note_bytes each)
+  unsigned char* notes;   // children with noted rows (expand_note_bytes each; beyond note_cap: redo list)
+  unsigned note_cap;
   unsigned* note_count;
   unsigned* stage_next;   // staging: next parent to take (zero at the launch)
   int stage_tail;         // staging in global memory: what it keeps in shared memory (expand_stage_tail_bytes)

@@ -1176,6 +1176,10 @@ __device__ __forceinline__ void thread_child(const ExpandArgs& a, const unsigned
     unsigned k = 0;
     if (lane == lead) k = atomicAdd(a.note_count, (unsigned)__popc(act));
     k = __shfl_sync(act, k, lead) + __popc(act & ((1u << lane) - 1u));
+    if (k >= a.note_cap) {
+      a.redo_list[atomicAdd(a.redo_count, 1u)] = (uint32_t)j;
+      return;
+    }
     DrawNote* o = reinterpret_cast<DrawNote*>(a.notes) + k;
     o->child = (uint32_t)j;
     o->n_rows = (uint16_t)nslow;
@@ -1213,7 +1217,7 @@ static_assert(kDrawSlow % kNoteLanes == 0, "rows of a note over its lanes");
 template <int DZ>
 __device__ __noinline__ void finish_notes(const ExpandArgs& a, const Lay& L, const uint2 key) {
   const Model& md = a.md;
-  const uint32_t count = *a.note_count, HU = (uint32_t)md.h_up;
+  const uint32_t count = min(*a.note_count, a.note_cap), HU = (uint32_t)md.h_up;
   const int lane = (int)threadIdx.x & 31, gl = lane & (kNoteLanes - 1);
   const unsigned gm = ((1u << kNoteLanes) - 1u) << (lane - gl);
   const uint32_t step = gridDim.x * blockDim.x / kNoteLanes;
