@@ -2,9 +2,10 @@
 // FP64 callers.  An SM issues an FP64 instruction every 16 cycles for a warp
 // and an integer one on each of its four schedulers every cycle or two, so
 // these cost a fraction of the FP64 library functions; each result is off by
-// no more than theirs (checked against 300-bit arithmetic: about half a unit
-// in the last place, beside the library's one).  The series are Taylor's, the
-// tables come from the series at compile time.
+// no more than theirs (about half a unit in the last place of the result, the
+// library's being one; tests/test_fx_*.py check them against extended and
+// 70-digit arithmetic).  The series are Taylor's, the tables come from the
+// series at compile time.
 #pragma once
 #include <stdint.h>
 
@@ -300,25 +301,79 @@ FX_FN double normal(uint32_t w0, uint32_t w1, const u64* nlog, const uint16_t* i
   return neg ? -n : n;
 }
 
-// x / (2 pi) modulo 1 as a 64-bit fraction, |x| < 2^30 (checked by the caller)
-FX_FN u64 turn(double x) {
+// A fraction of a turn, (hi 2^64 + lo) 2^-128.
+struct Turn {
+  u64 hi, lo;
+};
+FX_FN Turn operator+(Turn a, Turn b) {
+  const u64 lo = a.lo + b.lo;
+  return Turn{a.hi + b.hi + (lo < a.lo ? 1ull : 0ull), lo};
+}
+
+// 0, or a magnitude from 2^-60 up to below `limit`: what the functions below
+// take without losing more than 2^-57 of the result (a smaller angle would
+// have its own bits below 2^-128 of a turn)
+FX_FN bool in_turn_range(double x, double limit) {
+  const u64 b = to_bits(x) & 0x7FFFFFFFFFFFFFFFull;
+  return b == 0ull || b - 0x3C30000000000000ull < to_bits(limit) - 0x3C30000000000000ull;
+}
+
+// x / (2 pi) modulo 1, x in range (below 2^30): the significand times 192 bits
+// of 1 / (2 pi), so that the distance from a zero of the sine or the cosine,
+// however small, has its full precision too
+FX_FN Turn turn(double x) {
   const u64 b = to_bits(x);
   const int E = (int)((b >> 52) & 0x7FFull) - 1023;
   const u64 M = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;   // |x| = M 2^(E - 63)
-  constexpr u64 Ih = 0x28BE60DB9391054Aull, Il = 0x7F09D5F47D4D3770ull;   // 2^-64, 2^-128 words of 1 / (2 pi)
-  const u64 hl = M * Ih, add = mulhi(M, Il);
-  const u64 p1 = hl + add, p2 = mulhi(M, Ih) + (p1 < hl ? 1ull : 0ull);
+  constexpr u64 I2 = 0x28BE60DB9391054Aull, I1 = 0x7F09D5F47D4D3770ull, I0 = 0x36D8A5664F10E410ull;
+  // M I, from the units down: w2 (the integer part), w1, w0 (2^-128)
+  u64 w0 = M * I1, w1 = M * I2, w2 = mulhi(M, I2);
+  const u64 c0 = mulhi(M, I0), c1 = mulhi(M, I1);
+  w0 += c0;
+  const u64 k0 = w0 < c0 ? 1ull : 0ull;
+  w1 += c1;
+  w2 += w1 < c1 ? 1ull : 0ull;
+  w1 += k0;
+  w2 += w1 < k0 ? 1ull : 0ull;
+  // times 2^(E + 1) (b == 0: nothing, E = -1023)
   const int sh = E + 1;
-  const u64 f = sh >= 64 ? 0ull : sh > 0 ? (p2 << sh) | (p1 >> (64 - sh)) : sh > -64 ? p2 >> -sh : 0ull;
-  return b >> 63 ? 0ull - f : f;
+  Turn f;
+  if (sh >= 0) {
+    f.hi = (w2 << sh) | ((w1 >> 1) >> (63 - sh));
+    f.lo = (w1 << sh) | ((w0 >> 1) >> (63 - sh));
+  } else if (sh > -64) {
+    f.hi = w2 >> -sh;
+    f.lo = (w2 << (64 + sh)) | (w1 >> -sh);
+  } else {
+    f.hi = f.lo = 0ull;
+  }
+  if (b >> 63) {
+    f.lo = 0ull - f.lo;
+    f.hi = 0ull - f.hi - (f.lo != 0ull ? 1ull : 0ull);
+  }
+  return f;
 }
-// sine and cosine of f 2^-64 of a turn, to 2^-62 beside their rounding
-FX_FN void sincos_turn(u64 f, double& s, double& c) {
-  const uint32_t oct = (uint32_t)(f >> 61);
-  u64 t = f << 3;
-  if (oct & 1u) t = ~t;                                                   // 1 - t to 2^-64
-  const u64 q = mulhi(t, t);
-  const double vs = to_double(sin_oct(t, q), -63), vc = to_double(cos_oct(q), -63);
+// sine and cosine of a fraction of a turn, each to 2^-57 of itself beside its
+// rounding
+FX_FN void sincos_turn(Turn f, double& s, double& c) {
+  const uint32_t oct = (uint32_t)(f.hi >> 61);
+  u64 t1 = (f.hi << 3) | (f.lo >> 61), t0 = f.lo << 3;                    // (t1 2^64 + t0) 2^-128 of an octant
+  if (oct & 1u) {
+    t1 = ~t1;                                                             // 1 - t to 2^-128
+    t0 = ~t0;
+  }
+  const u64 q = mulhi(t1, t1);
+  // the sine's polynomial times t, normalised: the zero it has at t = 0 is the
+  // sine's own or, in the swapped octants, the cosine's
+  int e = -63;
+  if (t1 == 0ull) {
+    t1 = t0;
+    t0 = 0ull;
+    e = -127;
+  }
+  const int lz = clz(t1) & 63;                                            // (t = 0 stays 0)
+  const u64 tn = (t1 << lz) | ((t0 >> 1) >> (63 - lz));
+  const double vs = to_double(sin_oct(tn, q), e - lz), vc = to_double(cos_oct(q), -63);
   const bool swap = ((oct + 1u) & 2u) != 0u;
   const double as = swap ? vc : vs, ac = swap ? vs : vc;
   s = oct >= 4u ? -as : as;

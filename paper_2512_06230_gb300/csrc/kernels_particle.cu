@@ -63,8 +63,8 @@ __device__ __forceinline__ double exp_weight(double l) {
 __device__ __forceinline__ void ctrv(const double (&x)[5], double dt, double a, double al, double (&y)[5]) {
   const double h = 0.5 * x[4] * dt;
   double s0, c0, s1, c1, sc;
-  if (fabs(h) < 0.5 && fabs(x[3]) < 1e9) {
-    const fx::u64 f = fx::turn(x[3]);
+  if (fx::in_turn_range(h, 0.5) && fx::in_turn_range(x[3], 1e9)) {
+    const fx::Turn f = fx::turn(x[3]);
     fx::sincos_turn(f, s0, c0);
     fx::sincos_turn(f + fx::turn(h), s1, c1);
     sc = fx::sinc(h);
