@@ -129,6 +129,7 @@ FX_FN u64 exp_poly(u64 r) {
 }
 
 // ---- exp(-x), x >= 0 and not -0 (0 from 708 on; NaN for NaN) ----
+// (exp_weight below goes on to the last subnormal)
 // x = n ln(2) / 64 + r: a table entry times the polynomial of exp(-r).
 FX_FN double exp_neg(double x, const u64* exp2) {
   const u64 b = to_bits(x);
@@ -144,6 +145,19 @@ FX_FN double exp_neg(double x, const u64* exp2) {
   const u64 r = (X << 11) - (u64)n * 0x2C5C85FDF473DE6ull - (((u64)n * 0xAF278ECEull) >> 32);
   const u64 t = mulhi(exp_poly(r), exp2[n & 63u]);                     // 2^62
   return to_double(t, -62 - (int)(n >> 6));
+}
+
+// exp(l) of a log-weight difference, l <= 0 but for rounding; the library's
+// function above 0 and where the result is below the normal range or near it
+// (-708 down to -746, from where it is 0)
+FX_FN double exp_weight(double l, const u64* exp2) {
+  const u64 b = to_bits(l);
+  if ((b << 1) == 0ull) return 1.0;
+  if (b >> 63) {
+    if (b < 0xC086200000000000ull) return exp_neg(-l, exp2);
+    if (b >= 0xC087500000000000ull && b <= 0xFFF0000000000000ull) return 0.0;
+  }
+  return exp(l);
 }
 
 // ---- exp(-d 2^-32), d >= 0: sums of many such values beside a large one ----

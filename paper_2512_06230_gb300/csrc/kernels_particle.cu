@@ -48,12 +48,7 @@ __device__ __forceinline__ void normal_pair(const uint4& w, double& n0, double& 
   n1 = fx::normal(w.z, w.w, kFx.nlog, kFx.inv);
 }
 
-// exp(l) of a log-weight difference, l <= 0 but for rounding
-__device__ __forceinline__ double exp_weight(double l) {
-  const fx::u64 b = fx::to_bits(l);
-  if ((b << 1) == 0ull) return 1.0;
-  return b >> 63 ? fx::exp_neg(-l, kFx.exp2) : exp(l);
-}
+__device__ __forceinline__ double exp_weight(double l) { return fx::exp_weight(l, kFx.exp2); }
 
 // one CTRV step over dt; the arc (v / w)(sin(psi + w dt) - sin psi, ...)
 // as v dt sinc(h)(cos, sin)(psi + h), h = w dt / 2, valid at w = 0.  Heading
