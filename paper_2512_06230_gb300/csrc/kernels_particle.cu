@@ -635,10 +635,16 @@ void launch_particle_remap(const Model& md, const PartModel& pm, const CompTable
   // few hypotheses make few updates, whose chains the frame waits for (above
   // 1024 particles 64 threads, the particles in memory).  Update stage with 256
   // particles, before and with 64 and 128 threads: convoy of ten (h_max 100)
-  // 42.6, 35.1 and 30.4 us; 200 vehicles (h_max 1000) 47.5, 39.6 and 41.9
+  // 42.6, 35.1 and 30.4 us; 200 vehicles (h_max 1000) 47.5, 39.6 and 41.9.
+  // Over the range, four and two a thread: 20 and 60 vehicles at h_max 25 to
+  // 256, 36.2 and 32.0 (256 particles), 31.6 and 29.1 (100), 37.5 and 38.7
+  // (512: blocks of 256 threads spend more in their barriers, so four a thread
+  // from 257 particles on; 200 vehicles with 512: 49 and 57); 200 vehicles with
+  // 256, h_max 25, 100, 256, 500: 39.0 and 36.7, 39.1 and 38.1, 39.7 and 40.4,
+  // 39.2 and 40.7
   const size_t smem = particle_remap_smem(pm.np);
   int threads = pm.np <= 256 ? 64 : pm.np <= 512 ? 128 : pm.np <= 1024 ? 256 : 64;
-  if (h_max <= 256 && pm.np > threads && pm.np <= 512) threads *= 2;
+  if (h_max <= 256 && pm.np > threads && pm.np <= 256) threads *= 2;
   auto k = pm.np <= 1024 ? particle_remap_kernel<4> : particle_remap_kernel<0>;
   launch_k(k, 4 * grid, threads, smem, s, md, pm, src, dst, newpos, flag, fs, n_keep_dev, upd_src, upd_m, upd_se, cap_upd,
            n_upd_dev, n_surv_dev, err);
