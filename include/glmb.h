@@ -532,10 +532,11 @@ glmb_status glmb_select_top_static(const double* logw_dev, int64_t n, int32_t h_
  * leaving the previous frame's state intact.  This call makes one such
  * wait run out on purpose, without any GPU fault:
  *   GLMB_WAIT_TEST_SCAN  the first tile of every one-pass scan (of the
- *                        kept-component flags, in filters with room for more
- *                        than 16384 components) withholds its prefix, so the
- *                        look-back waits of the later tiles give up after `limit`
- *                        polls;
+ *                        kept-component flags, in frames with more than 16384
+ *                        working components: while a wait test is set, frames
+ *                        run without a graph, each sized by itself) withholds
+ *                        its prefix, so the look-back waits of the later tiles
+ *                        give up after `limit` polls;
  *   GLMB_WAIT_TEST_GATE  CTA 0 of the learned gate's forward pass issues no
  *                        tensor-core work for its first tile (nothing is in
  *                        flight), so its completion wait gives up after

@@ -1151,6 +1151,12 @@ void set_groups(glmb_handle* h, Plan& p, int wc, int mc) {
 // (staged in shared memory) leave most of 256 threads waiting at the barriers:
 // 64 once the parents fill the GPU with such CTAs (3-D N = 50 when it staged
 // there: expansion 118 us with 256, 106 with 128, 103 with 64, 115 with 32).
+// Both sides of the first line, expansion with 1024, 256 and 128 threads, 3-D:
+// 100 slots and 448 rows (below it), 100 parents 58, 57, 57 us; 250 and 667,
+// 15 parents 46, 48, 57 and 150 parents 125, 126, 134; 401 and 1077, 43 parents
+// 183, 187, 200; 701 and 1839, 32 parents 104, 116, 136; 1000 and 2563, 3
+// parents 94, 109, 139.  More parents than SMs: 250 slots, 200 parents 104, 92,
+// 99 and 600 parents 154, 134, 128 (where the second line lies).
 int stage_threads(const glmb_handle* h, const Plan& p, long long H) {
   if (h->tune.stage_threads > 0) return h->tune.stage_threads;
   if (p.smem) return H >= 4LL * h->n_sm ? 64 : 256;

@@ -113,7 +113,7 @@ constexpr int kBirthRec = 58;
 void launch_particle_predict(const Model& md, const PartModel& pm, const CompTable& src, const CompTable& dst,
                              const FrameDev* fs, const double* births_dev, int grid, cudaStream_t s);
 // log C of every gated pair from the particles, then the death probability
-// (after launch_table_write, which wrote the pairs)
+// (after launch_table, which wrote the pairs)
 void launch_particle_logc(const Model& md, const PartModel& pm, const CompTable& ct, const PairTable& pt,
                           const FrameDev* fs, int grid, cudaStream_t s);
 // the regeneration's component work: kept components copied to their

@@ -238,7 +238,7 @@ __device__ __forceinline__ void slot_HPH(const CompTable& ct, int dx, uint32_t c
 }
 
 // The m-only parts of component c's alive term with m detections, from the
-// frame's per-component table (built by the table's count kernel).
+// frame's per-component table (built by the table kernel).
 template <int DZ>
 __device__ __forceinline__ SlotM<DZ> load_cslm(const float* slm, const int8_t* sln, int cap, int m, uint32_t c) {
   constexpr int NP = DZ * (DZ + 1) / 2;

@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(32 * kLogcWarps) particle_logc_kernel(Model md
   pdl_enter();
   __shared__ float s_logc[32];
   const int T = fs->T, np = pm.np, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  if (fs->M > 0 && !__isGlobal(fs->Z)) return;   // flagged by the count kernel
+  if (fs->M > 0 && !__isGlobal(fs->Z)) return;   // flagged by the table kernel
   const unsigned cap_p = (unsigned)min(pt.cap_pairs, (long long)0xFFFFFFFF);
   const size_t capp = (size_t)pt.cap_pairs;
   const float r0 = (float)pm.Rinv[0], r1 = (float)(pm.Rinv[1] + pm.Rinv[2]), r3 = (float)pm.Rinv[3];
